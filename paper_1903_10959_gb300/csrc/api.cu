@@ -140,7 +140,8 @@ constexpr bool kMatrixFreeDefault = true;
 // blocks, projector and binary64 staging buffers); later calls regrow it.
 void release_scratch(chfsi_ctx* ctx) {
   cudaStreamSynchronize(ctx->stream);
-  for (DevBuf* b : {&ctx->T1, &ctx->Wb, &ctx->NLb, &ctx->Zb, &ctx->Rb, &ctx->rot, &ctx->cmaxb, &ctx->pjb, &ctx->tinv}) {
+  for (DevBuf* b : {&ctx->T1, &ctx->Wb, &ctx->NLb, &ctx->Zb, &ctx->Rb, &ctx->rot, &ctx->cmaxb, &ctx->pjb, &ctx->tinv,
+                    &ctx->exb}) {
     dfree(ctx, b->ptr, b->bytes);
     b->ptr = nullptr;
     b->bytes = 0;
@@ -171,6 +172,10 @@ void free_device_data(chfsi_ctx* ctx) {
   ctx->dev_bytes -= (int64_t)(ctx->tc.bytes + ctx->tc.bf_bytes + ctx->tc.f16_bytes + ctx->tc.nl_bytes +
                               ctx->tc.pj_bytes);   // packed copies
   tc_free(ctx->tc);
+  release(ctx, ctx->ex.words, ctx->ex.word_bytes);
+  release(ctx, ctx->ex.hsum, ctx->ex.exp_bytes);
+  ctx->ex = ExCellData();
+  ctx->ex_off = false;
   ctx->kpack_valid = false;   // the mixed Bloch packs hold the old cell matrices
   release(ctx, ctx->d_site_ptr, ctx->hproj.site_ptr.size() * 8);
   release(ctx, ctx->d_site_dof, ctx->hproj.site_dof.size() * 4);
@@ -406,8 +411,11 @@ chfsi_status check_x(chfsi_ctx* ctx, const void* X, int64_t ldx, int ncol, chfsi
 
 // Device-side bounded waits report through a status word; map it to an error.
 chfsi_status check_device_status(chfsi_ctx* ctx, chfsi_precision prec) {
-  if (!is_mixed(prec)) return CHFSI_OK;
-  int v = tc_read_status(ctx->stream);
+  int v = is_mixed(prec) ? tc_read_status(ctx->stream) : 0;
+  if (!v && ctx->ex_used) {
+    v = ex_read_status(ctx->stream);
+    ctx->ex_used = false;
+  }
   if (v) return fail(ctx, CHFSI_ERR_TIMEOUT, "device wait timed out (site " + std::to_string(v) + ")");
   return CHFSI_OK;
 }
@@ -545,7 +553,14 @@ chfsi_status gram_impl(chfsi_ctx* ctx, chfsi_precision prec, const void* A, int6
   const HostMesh& m = ctx->mesh;
   chfsi_status st;
   if (prec == CHFSI_FP64) {
-    size_t want = (size_t)8 * 8 * n1 * n2;
+    size_t want = ex_gram_work_bytes(m.ndofs, n1, n2, lower);
+    if ((st = grow(ctx, ctx->part, want)) == CHFSI_OK) {
+      ctx->ex_used = true;
+      CK(ex_gram((const double*)A, lda, (const double*)Bm, ldb, m.ndofs, n1, n2, C, ldc, lower, ctx->part.ptr,
+                 ctx->part.bytes, ctx->stream));
+      return CHFSI_OK;
+    }
+    want = (size_t)8 * 8 * n1 * n2;
     if ((st = grow(ctx, ctx->part, want)) != CHFSI_OK) return st;
     CK(launch_gram_fp64((const double*)A, lda, (const double*)Bm, ldb, m.ndofs, n1, n2, C, ldc,
                         lower, (double*)ctx->part.ptr, ctx->part.bytes, ctx->stream));
@@ -559,6 +574,21 @@ chfsi_status gram_impl(chfsi_ctx* ctx, chfsi_precision prec, const void* A, int6
   return CHFSI_OK;
 }
 
+// C = X U in binary64 (M x n2, U n1 x n2 column-major).
+chfsi_status tall64_impl(chfsi_ctx* ctx, const double* X, int64_t ldx, int n1, int n2, const double* U, int64_t ldu,
+                         double* C, int64_t ldc, int upper, int trans) {
+  const HostMesh& m = ctx->mesh;
+  const std::string err = ctx->err;
+  if (grow(ctx, ctx->work, ex_tall_work_bytes(m.ndofs, n1, n2)) == CHFSI_OK) {
+    ctx->ex_used = true;
+    CK(ex_tall(X, ldx, U, ldu, m.ndofs, n1, n2, C, ldc, upper, trans, ctx->work.ptr, ctx->stream));
+    return CHFSI_OK;
+  }
+  ctx->err = err;
+  CK(launch_tallgemm_fp64(X, ldx, U, ldu, m.ndofs, n1, n2, C, ldc, upper, trans, ctx->stream));
+  return CHFSI_OK;
+}
+
 // X <- X U (U n x n column-major; trans / upper flags as launch_tallgemm_fp64).
 chfsi_status rotate_impl(chfsi_ctx* ctx, chfsi_precision prec, void* X, int64_t ldx, int n,
                          const double* U, int upper, int trans) {
@@ -567,8 +597,8 @@ chfsi_status rotate_impl(chfsi_ctx* ctx, chfsi_precision prec, void* X, int64_t 
   chfsi_status st;
   if ((st = grow(ctx, ctx->rot, (size_t)m.ndofs * n * es)) != CHFSI_OK) return st;
   if (prec == CHFSI_FP64) {
-    CK(launch_tallgemm_fp64((const double*)X, ldx, U, n, m.ndofs, n, n, (double*)ctx->rot.ptr, n,
-                            upper, trans, ctx->stream));
+    if ((st = tall64_impl(ctx, (const double*)X, ldx, n, n, U, n, (double*)ctx->rot.ptr, n, upper, trans)) != CHFSI_OK)
+      return st;
   } else {
     if ((st = grow(ctx, ctx->work, tc_tallgemm_work_bytes(n, n))) != CHFSI_OK) return st;
     CK(tc_tallgemm_mixed((const float*)X, ldx, U, n, m.ndofs, n, n, (float*)ctx->rot.ptr, n, upper,
@@ -903,7 +933,7 @@ chfsi_status chfsi_destroy(chfsi_ctx* ctx) {
     if (q) cudaFree(q);
   for (DevBuf* b : {&ctx->T1, &ctx->Wb, &ctx->NLb, &ctx->Zb, &ctx->rot, &ctx->Ssq, &ctx->work,
                     &ctx->part, &ctx->vec, &ctx->lam, &ctx->Rb, &ctx->Db, &ctx->pol, &ctx->scfb, &ctx->scfq,
-                    &ctx->cmaxb, &ctx->pjb, &ctx->tinv,
+                    &ctx->cmaxb, &ctx->pjb, &ctx->tinv, &ctx->exb,
                     &ctx->scfr, &ctx->scfw, &ctx->kW, &ctx->kT1, &ctx->kG, &ctx->kS, &ctx->kwork,
                     &ctx->kY, &ctx->kvec})
     dfree(ctx, b->ptr, b->bytes);
@@ -1190,7 +1220,9 @@ chfsi_status chfsi_apply(chfsi_ctx* ctx, const void* X, int64_t ldx, void* Y, in
   if (st != CHFSI_OK) return st;
   if (ncol > 0 && (!Y || ldy < ncol)) return fail(ctx, CHFSI_ERR_ARG, "bad Y / ldy");
   st = apply_blocks(ctx, prec, X, ldx, Y, ldy, ncol);
-  if (st == CHFSI_OK) st = check_device_status(ctx, prec);
+  // a binary64 application stays asynchronous: a wait that gave up in it is
+  // reported by the next call that synchronises
+  if (st == CHFSI_OK && is_mixed(prec)) st = check_device_status(ctx, prec);
   return st;
 }
 
@@ -1342,8 +1374,7 @@ chfsi_status chfsi_rayleigh_ritz_split(chfsi_ctx* ctx, const void* X, int64_t ld
                                         ", eigenpairs " + std::to_string(meig));
   // 3. X_fr = X Q_fr (the n x n_fr leading block of H^, leading dimension n)
   if (prec == CHFSI_FP64) {
-    CK(launch_tallgemm_fp64((const double*)X, ldx, Hh, n, m.ndofs, n, n_fr, (double*)Xfr, ldfr, 0, 0,
-                            ctx->stream));
+    if ((st = tall64_impl(ctx, (const double*)X, ldx, n, n_fr, Hh, n, (double*)Xfr, ldfr, 0, 0)) != CHFSI_OK) return st;
   } else {
     if ((st = grow(ctx, ctx->work, tc_tallgemm_work_bytes(n, n_fr))) != CHFSI_OK) return st;
     CK(tc_tallgemm_mixed((const float*)X, ldx, Hh, n, m.ndofs, n, n_fr, (float*)Xfr, ldfr, 0, 0, 0,
@@ -1398,7 +1429,8 @@ chfsi_status chfsi_residuals(chfsi_ctx* ctx, const void* X, int64_t ldx, int n, 
   chfsi_status st = check_x(ctx, X, ldx, n, prec);
   if (st != CHFSI_OK) return st;
   if (n > 0 && !evals_host) return fail(ctx, CHFSI_ERR_ARG, "evals required");
-  return residual_impl(ctx, X, ldx, n, prec, evals_host, res_host, gres_host);
+  st = residual_impl(ctx, X, ldx, n, prec, evals_host, res_host, gres_host);
+  return st == CHFSI_OK ? check_device_status(ctx, CHFSI_FP64) : st;
 }
 
 chfsi_status chfsi_bounds(chfsi_ctx* ctx, int lanczos_steps, uint64_t seed, double* b_out) {
@@ -1470,7 +1502,7 @@ chfsi_status chfsi_bounds(chfsi_ctx* ctx, int lanczos_steps, uint64_t seed, doub
     else lo = mid;
   }
   *b_out = hi + std::fabs(be[k - 1]);
-  return CHFSI_OK;
+  return check_device_status(ctx, CHFSI_FP64);
 }
 
 chfsi_status chfsi_solve(chfsi_ctx* ctx, void* X, int64_t ldx, int n, int iters, int degree, double b,
@@ -1547,7 +1579,7 @@ chfsi_status chfsi_solve_polish(chfsi_ctx* ctx, float* X, int64_t ldx, int n, in
   CK(cudaStreamSynchronize(ctx->stream));
   std::memcpy(evals_host, D.data(), (size_t)n * 8);
   if (iters_done) *iters_done = it;
-  return CHFSI_OK;
+  return check_device_status(ctx, CHFSI_FP64);
 }
 
 chfsi_status chfsi_step_host(chfsi_ctx* ctx, void* X_host, int64_t ldh, void* X, int64_t ldx, int n,

@@ -6,6 +6,7 @@
 
 #include <cusolverDn.h>
 
+#include "ex.h"
 #include "internal.h"
 #include "tc.h"
 
@@ -35,6 +36,11 @@ struct chfsi_ctx {
   std::vector<double> fac;
   int fp64_op = -1;                // binary64 cell operator: 0 cell matrices, 1 matrix-free, -1 auto
   chfsi::TcCellData tc;                   // tensor-core copies (mixed precisions)
+  // digit slices of the binary64 cell matrices (packed on first binary64 use;
+  // ex_off: they did not fit, the binary64 operator stays on the ALUs until
+  // the next build); ex_used: a digit-slice kernel ran since the last status read
+  chfsi::ExCellData ex;
+  bool ex_off = false, ex_used = false;
   int32_t* d_dofmap = nullptr;
   uint8_t* d_modes = nullptr;
   int32_t* d_cells = nullptr;
@@ -51,6 +57,7 @@ struct chfsi_ctx {
   float* d_dof_c32 = nullptr;
   // grown scratch
   chfsi::DevBuf T1, Wb, NLb, Zb, rot, Ssq, work, part, vec, lam, Rb;
+  chfsi::DevBuf exb;               // digit slices: the block's words and scales
   chfsi::DevBuf pol;               // binary64 staging block of the polish
   chfsi::DevBuf scfb, scfq, scfr, scfw;   // Poisson / SCF work arrays (scf.cu)
   chfsi::DevBuf kW, kT1, kG, kS, kwork, kY, kvec;   // Bloch (k-point) work arrays (kpoint.cu)
