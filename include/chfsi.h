@@ -186,14 +186,19 @@ chfsi_status chfsi_set_cell_gather(chfsi_ctx* ctx, int mode);
 /* Cell operator of the binary64 path (every CHFSI_FP64 apply, and the
  * binary64 products of the mixed precisions' last Rayleigh-Ritz, residuals
  * and polish): 0 = the stored cell matrices H~_e (dense n_e x n_e products,
- * Sec. 3.3.1); 1 = matrix-free, H_e applied by sum factorisation over the
- * tensor-product cell (1-D mass / stiffness / Gauss-point factors, the
- * alternative the paper notes for the cell-level products), 3.2x (p = 6) to
- * 5.5x (p = 8) fewer flops; -1 = the library's default: matrix-free where it
- * exists, else the cell matrices.  The matrix-free form
- * needs 2 <= p <= 8 and quad_points = p + 2 (CHFSI_ERR_ARG otherwise).  Both
- * give the same operator to rounding.  chfsi_fp64_operator returns the one in
- * use (0 or 1). */
+ * Sec. 3.3.1), evaluated on the tensor cores as exact products of 8-bit digit
+ * slices (a library-owned copy of the matrices as 64-bit digit words, 8 B per
+ * entry, made on first use; the ALUs take over when it does not fit); 1 =
+ * matrix-free, H_e applied by sum factorisation over the tensor-product cell
+ * (1-D mass / stiffness / Gauss-point factors, the alternative the paper notes
+ * for the cell-level products), 3.2x (p = 6) to 5.5x (p = 8) fewer flops, on
+ * the ALUs; -1 = the library's default: matrix-free, where it exists, for
+ * blocks of up to 12 columns (15 for p >= 7) of meshes that fill the GPU and
+ * when there are no cell matrices (chfsi_set_potential_qp_device), else the
+ * cell matrices.  The matrix-free form needs 2 <= p <= 8 and quad_points =
+ * p + 2 (CHFSI_ERR_ARG otherwise).  Both give the same operator to rounding.
+ * chfsi_fp64_operator returns 1 when the matrix-free form is selected or, by
+ * default, available, else 0. */
 chfsi_status chfsi_set_fp64_operator(chfsi_ctx* ctx, int op);
 int          chfsi_fp64_operator(const chfsi_ctx* ctx);
 

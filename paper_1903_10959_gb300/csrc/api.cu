@@ -250,6 +250,56 @@ chfsi_status ensure_tc_data(chfsi_ctx* ctx, chfsi_precision prec) {
   return CHFSI_OK;
 }
 
+// Columns up to which a binary64 step stays on the matrix-free kernel: the
+// digit-slice kernel always computes 128-column tiles, so a narrow block wastes
+// them unless the whole launch is only a few tiles per SM (4^3 cells, p = 4, one
+// column: 0.045 ms against 0.168 ms in eight colour launches).  8^3 cells, p = 6:
+// matrix-free 0.42 ms (8 columns), 0.74 (12, 13), digit slices 0.51; 16^3 cells:
+// 2.9, 4.0, 5.0 against 3.8; 8^3 cells, p = 7: 0.62, 0.89, 1.72 (16) against 1.13.
+int narrow_columns(const chfsi_ctx* ctx) { return ctx->mesh.p >= 7 ? 15 : 12; }
+constexpr int64_t kFewTiles = 4 * 152;
+bool stays_matrix_free(const chfsi_ctx* ctx, int ncol) {
+  return use_matrix_free(ctx) &&
+         (ctx->fp64_op == 1 || (ncol <= narrow_columns(ctx) &&
+                                ex_cell_tiles(ctx->mesh.ncells, ctx->mesh.ne, ncol) > kFewTiles));
+}
+
+// Whether a binary64 step of ncol columns takes the digit-slice cell products
+// (kernels_ex.cu): the cell matrices are resident, the block is not one for the
+// matrix-free kernel, and the words of the matrices, of the block and its dense
+// cell blocks fit in memory.  Otherwise the colour-ordered ALU kernels run.
+bool ensure_ex(chfsi_ctx* ctx, int ncol, int64_t* ldr) {
+  const HostMesh& m = ctx->mesh;
+  if (!ctx->d_Ht || ctx->ex_off || stays_matrix_free(ctx, ncol)) return false;
+  *ldr = (ncol + 1) & ~1;
+  if (!ctx->ex.words) {
+    ExCellData& d = ctx->ex;
+    ex_cell_bytes(m.ncells, m.ne, &d.word_bytes, &d.exp_bytes);
+    if (dalloc(ctx, (void**)&d.words, d.word_bytes) != cudaSuccess) d.words = nullptr;
+    if (d.words && dalloc(ctx, (void**)&d.hsum, d.exp_bytes) != cudaSuccess) d.hsum = nullptr;
+    if (!d.hsum || ex_pack_cells(d, ctx->d_Ht, m.ncells, m.ne, ctx->stream) != cudaSuccess) {
+      cudaGetLastError();
+      release(ctx, d.words, d.word_bytes);
+      release(ctx, d.hsum, d.exp_bytes);
+      d = ExCellData();
+      ctx->ex_off = true;
+      return false;
+    }
+  }
+  const std::string err = ctx->err;
+  // the partial sums of the narrow blocks that follow on the matrix-free kernel
+  // are allocated with the first block of any width, as one call always did
+  const int nw = std::min(ncol, narrow_columns(ctx));
+  if ((stays_matrix_free(ctx, nw) && grow(ctx, ctx->Wb, (size_t)m.ndofs * nw * sizeof(double)) != CHFSI_OK) ||
+      grow(ctx, ctx->exb, ex_cell_work_bytes(m.ncells, m.ne, ncol)) != CHFSI_OK ||
+      grow(ctx, ctx->Rb, (size_t)m.ncells * m.ne * *ldr * sizeof(double)) != CHFSI_OK) {
+    ctx->err = err;   // no room: the ALU kernels until the next build
+    ctx->ex_off = true;
+    return false;
+  }
+  return true;
+}
+
 // One recurrence step over the ncol columns of a block:
 // Yout = alpha (H~ Yin - shift Yin) + beta Yprev, colour by colour.
 chfsi_status apply_step(chfsi_ctx* ctx, chfsi_precision prec, const void* Yin, int64_t ld_in,
@@ -260,7 +310,9 @@ chfsi_status apply_step(chfsi_ctx* ctx, chfsi_precision prec, const void* Yin, i
   const int B = std::max(ncol, 1);
   const size_t es = esize(prec);
   chfsi_status st;
-  if (prec == CHFSI_FP64 && (st = grow(ctx, ctx->Wb, (size_t)m.ndofs * B * es)) != CHFSI_OK) return st;
+  int64_t ldr = 0;
+  const bool ex = prec == CHFSI_FP64 && ncol > 0 && ensure_ex(ctx, ncol, &ldr);
+  if (prec == CHFSI_FP64 && !ex && (st = grow(ctx, ctx->Wb, (size_t)m.ndofs * B * es)) != CHFSI_OK) return st;
   const bool nl = ctx->hproj.nsite > 0;
   if (nl) {
     if (prec == CHFSI_FP64 && (st = grow(ctx, ctx->NLb, (size_t)m.ndofs * B * es)) != CHFSI_OK) return st;
@@ -273,6 +325,23 @@ chfsi_status apply_step(chfsi_ctx* ctx, chfsi_precision prec, const void* Yin, i
                                 (const double*)Yin, ld_in, ncol, (double*)ctx->Zb.ptr, ctx->stream));
       CK(launch_nl_expand_fp64(ctx->d_dof_ptr, ctx->d_dof_site, ctx->d_dof_c, m.ndofs,
                                (const double*)ctx->Zb.ptr, ncol, (double*)ctx->NLb.ptr, B, ctx->stream));
+    }
+    if (ex) {   // every cell's dense block in one launch, then the fixed-order assembly
+      ctx->ex_used = true;
+      {
+        KTimer kt(ctx, 0);
+        CK(ex_cell_launch(ctx->ex, ExCellArgs{ctx->d_dofmap, m.ncells, m.ne, ncol, (const double*)Yin, ld_in,
+                                              (double*)ctx->Rb.ptr, ldr, ctx->exb.ptr},
+                          ctx->stream));
+      }
+      KTimer kt(ctx, 1);
+      CK(ex_assemble_launch(ExAssembleArgs{ctx->d_node_ptr, ctx->d_node_ent, m.ndofs, ncol,
+                                           (const double*)ctx->Rb.ptr, ldr,
+                                           nl ? (const double*)ctx->NLb.ptr : nullptr, B, (const double*)Yin, ld_in,
+                                           (double*)Yout, ld_out, beta != 0.0 ? (const double*)Yprev : nullptr,
+                                           ld_prev, alpha, beta, shift},
+                            ctx->stream));
+      return CHFSI_OK;
     }
     const bool mf = use_matrix_free(ctx);
     if (!mf && !ctx->d_Ht) return fail(ctx, CHFSI_ERR_STATE, "no cell matrices for the binary64 operator");

@@ -93,7 +93,15 @@ size_t estimate_bytes(const chfsi_request& r) {
   b += M * n * es;                                                  // X
   b += std::max(M * n * es, M * B * 16);                            // rotation / binary64 pair
   b += M * B * es + M * B * 8;                                      // filter block, binary64 apply
-  if (mixed) b += ncells * ne * B * 4;                              // dense cell blocks R_e
+  b += ncells * ne * ((B + 1) & ~(size_t)1) * 8;                    // dense cell blocks R_e (binary64 applications)
+  {                                                                 // digit words of the binary64 products
+    size_t words = 0, scales = 0;
+    chfsi::ex_cell_bytes((int64_t)ncells, (int)ne, &words, &scales);
+    b += words + scales + chfsi::ex_cell_work_bytes((int64_t)ncells, (int)ne, (int)B);
+    if (!mixed || r.polish_iters > 0)
+      b += std::max(chfsi::ex_gram_work_bytes((int64_t)M, r.n, r.n, 1), chfsi::ex_gram_work_bytes((int64_t)M, r.n, (int)B, 1)) +
+           chfsi::ex_tall_work_bytes((int64_t)M, r.n, r.n);
+  }
   b += std::max(n * n * 128 + (mixed ? ((size_t)64 << 20) : 0), n * 12288);  // Gram partials
   b += n * n * 8 * 5 + n * 64 + 4096;                               // N x N (S / H^, L^{-1}), solver workspace
   b += M * 24 + ((size_t)16 << 20);                                 // vectors, library slack
