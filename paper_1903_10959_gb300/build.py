@@ -21,7 +21,7 @@ LIB = os.path.join(HERE, "libchfsi.so")
 CUDA_HOME = os.environ.get("CUDA_HOME", "/usr/local/cuda")
 NVCC = os.path.join(CUDA_HOME, "bin", "nvcc")
 GENCODE = ["-gencode", "arch=compute_103a,code=sm_103a"]
-CUDA_SOURCES = ["kernels_fp64.cu", "kernels_tc.cu", "kernels_mf.cu", "kernels_ex.cu", "api.cu", "batch.cu", "server.cu",
+CUDA_SOURCES = ["kernels_fp64.cu", "kernels_tc.cu", "kernels_mf.cu", "kernels_ex.cu", "cellmat.cu", "api.cu", "batch.cu", "server.cu",
                 "density.cu", "scf.cu", "kpoint.cu"]
 CXX_SOURCES = ["mesh.cpp", "partition.cpp"]
 
@@ -34,7 +34,7 @@ def _stale() -> bool:
     if not os.path.exists(LIB):
         return True
     t = os.path.getmtime(LIB)
-    deps = _sources() + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".h")]
+    deps = _sources() + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".h", ".cuh"))]
     deps.append(os.path.join(ROOT, "include", "chfsi.h"))
     return any(os.path.getmtime(d) > t for d in deps)
 

@@ -164,17 +164,24 @@ bool use_matrix_free(const chfsi_ctx* ctx) {
   return ctx->fp64_op == 1 || (ctx->fp64_op < 0 && kMatrixFreeDefault);
 }
 
-void free_device_data(chfsi_ctx* ctx) {
+// Drop the cell data of the present potential.  keep: a rebuild follows, and
+// the buffers whose size the mesh alone fixes (cell matrices, potential and 1-D
+// factors, BF16x3 terms, digit words) stay for it.
+void free_device_data(chfsi_ctx* ctx, bool keep = false) {
   const HostMesh& m = ctx->mesh;
-  release(ctx, ctx->d_Ht, (size_t)m.ncells * m.ne * m.ne * 8);
-  release(ctx, ctx->d_wv, ctx->wv.size() * 8);
-  release(ctx, ctx->d_fac, ctx->fac.size() * 8);
-  ctx->dev_bytes -= (int64_t)(ctx->tc.bytes + ctx->tc.bf_bytes + ctx->tc.f16_bytes + ctx->tc.nl_bytes +
-                              ctx->tc.pj_bytes);   // packed copies
-  tc_free(ctx->tc);
-  release(ctx, ctx->ex.words, ctx->ex.word_bytes);
-  release(ctx, ctx->ex.hsum, ctx->ex.exp_bytes);
-  ctx->ex = ExCellData();
+  if (!keep) {
+    release(ctx, ctx->d_Ht, (size_t)m.ncells * m.ne * m.ne * 8);
+    release(ctx, ctx->d_wv, (size_t)ctx->nwv * 8);
+    release(ctx, ctx->d_fac, ctx->fac.size() * 8);
+    release(ctx, ctx->ex.words, ctx->ex.word_bytes);
+    release(ctx, ctx->ex.hsum, ctx->ex.exp_bytes);
+    ctx->ex = ExCellData();
+    ctx->dev_bytes -= (int64_t)ctx->tc.bf_bytes;
+    if (ctx->tc.bf) cudaFree(ctx->tc.bf);
+    ctx->tc.bf = nullptr;
+  }
+  tc_build(ctx->tc, m.ncells, m.ne, &ctx->dev_bytes);   // the other packed copies
+  ctx->ex_ready = false;
   ctx->ex_off = false;
   ctx->kpack_valid = false;   // the mixed Bloch packs hold the old cell matrices
   release(ctx, ctx->d_site_ptr, ctx->hproj.site_ptr.size() * 8);
@@ -209,7 +216,7 @@ chfsi_status ensure_tc_data(chfsi_ctx* ctx, chfsi_precision prec) {
                   std::string("FP16x2 cell data: ") + cudaGetErrorString(pe));
     }
   }
-  if (bf16 && !ctx->tc.bf) {
+  if (bf16 && !ctx->tc.bf_ready) {
     cudaError_t pe = tc_pack_bf16_from_device(ctx->tc, ctx->d_Ht, ctx->stream, &ctx->dev_bytes);
     if (pe != cudaSuccess) {
       cudaGetLastError();
@@ -272,12 +279,14 @@ bool ensure_ex(chfsi_ctx* ctx, int ncol, int64_t* ldr) {
   const HostMesh& m = ctx->mesh;
   if (!ctx->d_Ht || ctx->ex_off || stays_matrix_free(ctx, ncol)) return false;
   *ldr = (ncol + 1) & ~1;
-  if (!ctx->ex.words) {
+  if (!ctx->ex_ready) {
     ExCellData& d = ctx->ex;
-    ex_cell_bytes(m.ncells, m.ne, &d.word_bytes, &d.exp_bytes);
-    if (dalloc(ctx, (void**)&d.words, d.word_bytes) != cudaSuccess) d.words = nullptr;
-    if (d.words && dalloc(ctx, (void**)&d.hsum, d.exp_bytes) != cudaSuccess) d.hsum = nullptr;
-    if (!d.hsum || ex_pack_cells(d, ctx->d_Ht, m.ncells, m.ne, ctx->stream) != cudaSuccess) {
+    if (!d.hsum) {
+      ex_cell_bytes(m.ncells, m.ne, &d.word_bytes, &d.exp_bytes);
+      if (dalloc(ctx, (void**)&d.words, d.word_bytes) != cudaSuccess) d.words = nullptr;
+      if (d.words && dalloc(ctx, (void**)&d.hsum, d.exp_bytes) != cudaSuccess) d.hsum = nullptr;
+    }
+    if (!d.hsum || ex_pack_cells(d, ctx->cellmat, m.ne, ctx->stream) != cudaSuccess) {
       cudaGetLastError();
       release(ctx, d.words, d.word_bytes);
       release(ctx, d.hsum, d.exp_bytes);
@@ -285,6 +294,7 @@ bool ensure_ex(chfsi_ctx* ctx, int ncol, int64_t* ldr) {
       ctx->ex_off = true;
       return false;
     }
+    ctx->ex_ready = true;
   }
   const std::string err = ctx->err;
   // the partial sums of the narrow blocks that follow on the matrix-free kernel
@@ -996,6 +1006,8 @@ chfsi_status chfsi_destroy(chfsi_ctx* ctx) {
   release(ctx, ctx->d_node_ptr, m.node_ptr.size() * 4);
   release(ctx, ctx->d_node_ent, m.node_ent.size() * 4);
   release(ctx, ctx->d_msq, m.mass.size() * 8);
+  release(ctx, ctx->d_K, ((size_t)2 * m.ne * m.ne + 3 * m.n1 + 2 * m.q + (size_t)m.q * m.n1) * 8);
+  dfree(ctx, ctx->wellb.ptr, ctx->wellb.bytes);
   if (ctx->d_kfac) cudaFree(ctx->d_kfac);
   ctx->d_kfac = nullptr;
   for (void* q : {(void*)ctx->d_kA, (void*)ctx->d_kG, (void*)ctx->kbf, (void*)ctx->kgbf})
@@ -1117,20 +1129,73 @@ chfsi_status chfsi_set_projectors(chfsi_ctx* ctx, int n, const double* xyz, cons
 chfsi_status chfsi_build(chfsi_ctx* ctx) {
   CHECK_CTX();
   CK(cudaStreamSynchronize(ctx->stream));
-  free_device_data(ctx);
+  free_device_data(ctx, true);
   const HostMesh& m = ctx->mesh;
-  std::vector<double> Ht;
-  build_cell_matrices(m, ctx->wells, Ht, &ctx->wv);
-  build_mf_factors(m, ctx->fac);
-  build_projectors(m, ctx->proj, ctx->hproj);
-  cudaError_t e;
-  if ((e = upload(ctx, &ctx->d_Ht, Ht)) != cudaSuccess ||
-      (e = upload(ctx, &ctx->d_wv, ctx->wv)) != cudaSuccess ||
-      (e = upload(ctx, &ctx->d_fac, ctx->fac)) != cudaSuccess) {
+  const int nq = m.q * m.q * m.q;
+  auto oom = [&](cudaError_t e) {
     cudaGetLastError();
+    free_device_data(ctx);
     return fail(ctx, e == cudaErrorMemoryAllocation ? CHFSI_ERR_OOM : CHFSI_ERR_CUDA,
                 std::string("cell matrices: ") + cudaGetErrorString(e));
+  };
+  cudaError_t e;
+  // what the mesh alone fixes, on the first build
+  std::vector<double> K;
+  if (!ctx->d_K) {
+    std::vector<double> s1;
+    build_kinetic(m, K, s1);
+    K.insert(K.end(), s1.begin(), s1.end());
+    K.insert(K.end(), m.gq_x.begin(), m.gq_x.end());
+    K.insert(K.end(), m.gq_w.begin(), m.gq_w.end());
+    K.insert(K.end(), m.B.begin(), m.B.end());
+    if ((e = upload(ctx, &ctx->d_K, K)) != cudaSuccess) return oom(e);
   }
+  if (!ctx->d_fac) {
+    build_mf_factors(m, ctx->fac);
+    if ((e = upload(ctx, &ctx->d_fac, ctx->fac)) != cudaSuccess) return oom(e);
+  }
+  if (!ctx->d_Ht && (e = dalloc(ctx, (void**)&ctx->d_Ht, (size_t)m.ncells * m.ne * m.ne * 8)) != cudaSuccess) {
+    ctx->d_Ht = nullptr;
+    return oom(e);
+  }
+  if (!ctx->d_wv) {
+    ctx->nwv = m.ncells * (int64_t)nq;
+    if ((e = dalloc(ctx, (void**)&ctx->d_wv, (size_t)ctx->nwv * 8)) != cudaSuccess) {
+      ctx->d_wv = nullptr;
+      return oom(e);
+    }
+  }
+  // the wells, then the given values, in one upload
+  build_well_images(m, ctx->wells, ctx->wellh);
+  const int nwell = (int)(ctx->wellh.size() / 5);
+  ctx->wellh.insert(ctx->wellh.end(), ctx->wells.vqp.begin(), ctx->wells.vqp.end());
+  chfsi_status gs = grow(ctx, ctx->wellb, ctx->wellh.size() * 8 + 16);
+  if (gs != CHFSI_OK) return gs;
+  if (!ctx->wellh.empty())
+    CK(cudaMemcpyAsync(ctx->wellb.ptr, ctx->wellh.data(), ctx->wellh.size() * 8, cudaMemcpyHostToDevice, ctx->stream));
+  CellMatArgs& ca = ctx->cellmat;
+  ca = CellMatArgs{};
+  for (int a = 0; a < 3; ++a) {
+    ca.n[a] = m.n[a];
+    ca.h[a] = m.h[a];
+  }
+  ca.n1 = m.n1;
+  ca.q = m.q;
+  ca.jac = m.h[0] * m.h[1] * m.h[2] / 8.0;
+  ca.ncells = m.ncells;
+  ca.wells = (const double*)ctx->wellb.ptr;
+  ca.nwell = nwell;
+  ca.vqp = ctx->wells.vqp.empty() ? nullptr : ca.wells + 5 * (int64_t)nwell;
+  ca.K = ctx->d_K;
+  ca.s1 = ctx->d_K + (size_t)2 * m.ne * m.ne;
+  ca.gx = ca.s1 + 3 * m.n1;
+  ca.gw = ca.gx + m.q;
+  ca.B = ca.gw + m.q;
+  ca.dofmap = ctx->d_dofmap;
+  ca.wv = ctx->d_wv;
+  ca.Ht = ctx->d_Ht;
+  CK(launch_cell_matrices(ca, ctx->stream));
+  build_projectors(m, ctx->proj, ctx->hproj);
   if (ctx->hproj.nsite > 0) {
     std::vector<float> sc32(ctx->hproj.site_c.begin(), ctx->hproj.site_c.end());
     std::vector<float> dc32(ctx->hproj.dof_c.begin(), ctx->hproj.dof_c.end());
@@ -1143,12 +1208,6 @@ chfsi_status chfsi_build(chfsi_ctx* ctx) {
     CK(upload(ctx, &ctx->d_site_c32, sc32));
     CK(upload(ctx, &ctx->d_dof_c32, dc32));
     CK(cudaStreamSynchronize(ctx->stream));
-  }
-  cudaError_t te = tc_build(ctx->tc, Ht, m.ncells, m.ne, ctx->stream, &ctx->dev_bytes);   // packed lazily
-  if (te != cudaSuccess) {
-    cudaGetLastError();
-    return fail(ctx, te == cudaErrorMemoryAllocation ? CHFSI_ERR_OOM : CHFSI_ERR_CUDA,
-                std::string("tensor-core cell data: ") + cudaGetErrorString(te));
   }
   CK(cudaStreamSynchronize(ctx->stream));
   ctx->built = true;

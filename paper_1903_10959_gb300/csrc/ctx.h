@@ -32,7 +32,11 @@ struct chfsi_ctx {
   double* d_wv = nullptr;          // matrix-free apply: w jac V at the Gauss points per cell
   double* d_fac = nullptr;         // matrix-free apply: 1-D factors
   double* d_msq = nullptr;         // M^{-1/2} per unknown
-  std::vector<double> wv;          // host copy of d_wv (sizes)
+  int64_t nwv = 0;                 // its entries
+  double* d_K = nullptr;           // the cells' scaled kinetic matrix, the 1-D scales, the Gauss rule and B (constant per mesh)
+  chfsi::CellMatArgs cellmat{};    // what the present cell data was formed from
+  chfsi::DevBuf wellb;             // chfsi_build: well images, given potential values
+  std::vector<double> wellh;       // host side of the upload
   std::vector<double> fac;
   int fp64_op = -1;                // binary64 cell operator: 0 cell matrices, 1 matrix-free, -1 auto
   chfsi::TcCellData tc;                   // tensor-core copies (mixed precisions)
@@ -40,7 +44,7 @@ struct chfsi_ctx {
   // ex_off: they did not fit, the binary64 operator stays on the ALUs until
   // the next build); ex_used: a digit-slice kernel ran since the last status read
   chfsi::ExCellData ex;
-  bool ex_off = false, ex_used = false;
+  bool ex_ready = false, ex_off = false, ex_used = false;
   int32_t* d_dofmap = nullptr;
   uint8_t* d_modes = nullptr;
   int32_t* d_cells = nullptr;

@@ -19,8 +19,9 @@ struct ExCellData {
 // Output tiles of a cell launch (one CTA per SM takes them in turn).
 int64_t ex_cell_tiles(int64_t ncells, int ne, int ncol);
 void ex_cell_bytes(int64_t ncells, int ne, size_t* words, size_t* ex);
-// Fill d (buffers allocated by the caller) from the binary64 cell matrices (device).
-cudaError_t ex_pack_cells(const ExCellData& d, const double* dHt, int64_t ncells, int ne, cudaStream_t s);
+// Fill d (buffers allocated by the caller) for the cell data that m describes
+// (m.Ht, formed before, gives the scales).
+cudaError_t ex_pack_cells(const ExCellData& d, const CellMatArgs& m, int ne, cudaStream_t s);
 
 // R (cell, local node) rows x ncol (row stride ldr) = H~_e Y_e for every cell.
 // work: ex_cell_work_bytes of scratch.

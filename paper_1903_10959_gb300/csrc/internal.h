@@ -81,11 +81,37 @@ struct Projectors {
   double sigma = 0.8, rcut = 3.0;
 };
 
-// Cell matrices H~_e (binary64, row-major ne x ne per cell) for all cells;
-// wv (optional): per cell, w_a w_b w_c jac V at the q^3 Gauss points (the
-// potential factor of the matrix-free apply).
-void build_cell_matrices(const HostMesh& m, const Wells& w, std::vector<double>& Ht,
-                         std::vector<double>* wv = nullptr);
+// The cells' shared scaled kinetic matrix D^{-1/2} 1/2 K D^{-1/2} (ne x ne,
+// row-major, the binary64 values and then what they leave of twice that
+// precision) and the 1-D factors s1 (3 x n1) of D^{-1/2}: on a uniform mesh the
+// assembled GLL mass at a cell's nodes is a product over the axes, the same for
+// every cell.
+void build_kinetic(const HostMesh& m, std::vector<double>& K, std::vector<double>& s1);
+// The wells with their images along the periodic axes as explicit centres:
+// 5 values each (centre, depth, 1 / (2 width^2)).
+void build_well_images(const HostMesh& m, const Wells& w, std::vector<double>& out);
+// Cell matrices H~_e (binary64, row-major ne x ne per cell) and the potential
+// factor of the matrix-free apply (per cell, w_a w_b w_c jac V at the q^3 Gauss
+// points) for all cells, on the device (cellmat.cu).
+struct CellMatArgs {
+  int n[3], n1, q;
+  double h[3], jac;
+  int64_t ncells;
+  const double* wells;       // nwell x 5
+  int nwell;
+  const double* vqp;         // optional given values, ncells x q^3
+  const double *gx, *gw;     // Gauss rule
+  const double* B;           // q x n1 basis values
+  const double *K, *s1;      // build_kinetic
+  const int32_t* dofmap;
+  double* wv;                // out
+  double* Ht;                // out
+};
+cudaError_t launch_cell_matrices(const CellMatArgs& P, cudaStream_t s);
+// The same matrices as digit words (ex.h) under the row scales hexp, into W
+// (K-major, row stride ldw): the kinetic part enters with twice the precision of
+// binary64, so that the words carry no rounding of the sum.
+cudaError_t launch_cell_words(const CellMatArgs& P, const int16_t* hexp, uint64_t* W, int ldw, cudaStream_t s);
 // 1-D factors of the matrix-free apply: A_x, A_y, A_z, S_x, S_y, S_z (n1 x n1,
 // consistent mass and stiffness by the Gauss rule), B (q x n1) and B^T.
 void build_mf_factors(const HostMesh& m, std::vector<double>& fac);

@@ -20,7 +20,10 @@
 // any order (g = 6, 7 can round at 2^-60 of the largest product).  After a
 // segment the groups are combined in 64-bit integers, V = sum_g I_g 2^(41 - 8 g),
 // and V is rounded once to binary64 when the contraction ends (or every 960
-// terms, so that |V| < 2^63).
+// terms, so that |V| < 2^63).  The cell products cancel (||H~|| is hundreds of
+// times the low eigenvalues), so their sums keep four more bits, 2^(45 - 8 g):
+// the scale of a row of the cell matrix is raised where its first digits would
+// add up to more than 2^11.
 //
 //  ex_kernel<CELL>  R_e = H~_e Y_e for every cell (M: columns of Y, N: rows of
 //                   the cell matrix)
@@ -45,6 +48,7 @@
 
 #include <cuda_fp16.h>
 
+#include "digits.cuh"
 #include "ex.h"
 #include "tc_ptx.cuh"
 
@@ -75,7 +79,6 @@ constexpr int EX_THREADS = 640;
 constexpr int EX_SMEM = STAGES * B_STAGE + 8 * A_DEP * A_WORDS + 3 * B_DEP * B_WORDS + 512;
 constexpr int kNonFinite = 1 << 20;         // scale mark of a vector holding an infinity or a NaN
 constexpr int kNoScale = -(1 << 20);        // scale of a vector of zeros
-constexpr uint64_t kZeroWord = 0x8080808080808080ull;
 // Scratch of one launch's words: the operands are processed in slices of at
 // most this size (cells, or rows of the block).
 constexpr size_t kWordBytes = (size_t)512 << 20;
@@ -111,16 +114,6 @@ struct ExParams {
 __device__ __forceinline__ int elem_off(int r, int k) {   // 16-bit elements, K-major core matrices
   return (r >> 3) * 128 + (k >> 3) * 64 + (r & 7) * 8 + (k & 7);
 }
-__device__ __forceinline__ int expo(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
-
-// Digit word of v under the scale s = (vector's exponent field - v's own).
-__device__ __forceinline__ uint64_t word_of(double v, int s) {
-  const int hi = __double2hiint(v);
-  if (!(hi & 0x7ff00000)) return kZeroWord;         // zeros and subnormal numbers vanish
-  const uint64_t m = (uint64_t)(uint32_t)((hi & 0xfffff) | 0x100000) << 32 | (uint32_t)__double2loint(v);
-  const int64_t t = (int64_t)(m << 9);
-  return (uint64_t)((hi < 0 ? -t : t) >> min(s, 63)) + kZeroWord;
-}
 
 // fp16 pair (bytes picked by sel from x, minus 128): PRMT makes 1024 + byte.
 __device__ __forceinline__ uint32_t half_pair(uint32_t x, uint32_t sel) {
@@ -144,29 +137,34 @@ __device__ __forceinline__ void expand_pair(uint64_t w0, uint64_t w1, uint32_t* 
   if (ND == 8) out[7 * stride] = half_pair(lb, 0x4140);
 }
 
-// V += I_g 2^(41 - 8 g) for a drained group sum f = I_g, plus a constant per
-// segment (kGroupOffset over the eight groups).  The sums of at most 2^22 (g =
+// V += I_g 2^(SH - 8 g) for a drained group sum f = I_g, plus a constant per
+// segment (group_offset over the eight groups).  The sums of at most 2^22 (g =
 // 0, 1) and those that may be rounded (g = 6, 7: to units of V) are converted by
 // adding 1.5 2^23, whose low mantissa bits then hold the integer: the conversion
 // instruction runs at an eighth of the rate of the adds and, used for all
 // groups, bounds the drain.
 constexpr float kMagic = 12582912.f;
 constexpr uint64_t kMagicBits = 0x4B400000u;
-constexpr uint64_t kGroupOffset = (kMagicBits << 41) + (kMagicBits << 33) + 2 * kMagicBits;
+template <int SH>
+__device__ constexpr uint64_t group_offset() {
+  return (kMagicBits << SH) + (kMagicBits << (SH - 8)) + 2 * kMagicBits;
+}
+template <int SH>
 __device__ __forceinline__ void add_group(int64_t& V, float f, int g) {
   if (g < 2) {
     const uint32_t b = __float_as_uint(f + kMagic);
-    V += (int64_t)((uint64_t)(b << (g == 0 ? 9 : 1)) << 32);
+    V += (int64_t)((uint64_t)(b << (SH - 32 - 8 * g)) << 32);
   } else if (g < 6) {
-    V += (int64_t)__float2int_rn(f) * (1ll << (41 - 8 * (g < 6 ? g : 5)));
+    V += (int64_t)__float2int_rn(f) * (1ll << (SH - 8 * (g < 6 ? g : 5)));
   } else {
-    V += (int64_t)(uint64_t)__float_as_uint(fmaf(f, g == 6 ? 1.f / 128.f : 1.f / 32768.f, kMagic));
+    V += (int64_t)(uint64_t)__float_as_uint(fmaf(f, 1.f / (float)(1 << (g < 6 ? 0 : 8 * g - SH)), kMagic));
   }
 }
 
-// V 2^(ex - 2097) rounded to binary64 (ex: sum of the two scales); integer
+// V 2^(ex - 2056 - SH) rounded to binary64 (ex: sum of the two scales); integer
 // arithmetic only, since the conversion and the scaling would take two
 // binary64-pipe operations per output.
+template <int SH>
 __device__ __forceinline__ double compose(int64_t v, int ex) {
   if (v == 0) return 0.0;
   const uint64_t a = v < 0 ? (uint64_t)(-v) : (uint64_t)v;
@@ -174,7 +172,7 @@ __device__ __forceinline__ double compose(int64_t v, int ex) {
   const uint64_t t = a << lz;                        // top bit set
   uint64_t m = t >> 11;
   m += ((t & 0x7ff) + (m & 1)) > 0x400;              // to nearest, ties to even
-  const int f = 63 - lz + ex - 1074;                 // exponent field
+  const int f = 63 - lz + ex - 1033 - SH;                 // exponent field
   const uint64_t sg = v < 0 ? 0x8000000000000000ull : 0ull;
   if (f <= 0) return __longlong_as_double((long long)sg);
   if (f >= 2047) return __longlong_as_double((long long)(sg | 0x7ff0000000000000ull));
@@ -280,6 +278,7 @@ __device__ __forceinline__ void cp_async_wait() {
 
 template <int MODE>
 __global__ void __launch_bounds__(EX_THREADS, 1) ex_kernel(const __grid_constant__ ExParams P) {
+  constexpr int SH = MODE == EX_CELL ? 45 : 41;   // units of the integer sums
   extern __shared__ __align__(1024) unsigned char smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   unsigned char* wordsA = smem + STAGES * B_STAGE;
@@ -319,7 +318,7 @@ __global__ void __launch_bounds__(EX_THREADS, 1) ex_kernel(const __grid_constant
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  const int seg = MODE == EX_CELL && *P.hsum <= (1 << 24) ? 1 << 20 : SEG;   // chunks per segment
+  const int seg = MODE == EX_CELL && *P.hsum <= (1 << 24) - (1 << 18) ? 1 << 20 : SEG;   // chunks per segment
   // A role whose wait gives up records it and leaves; the waits of the roles
   // that depend on it then run out in turn, so that every warp reaches the end.
   auto give_up = [&](int site) { atomicExch(&g_ex_status, site); };
@@ -350,7 +349,7 @@ __global__ void __launch_bounds__(EX_THREADS, 1) ex_kernel(const __grid_constant
           __syncwarp();
           if (lane == 0) mbar_arrive(ge(g));
 #pragma unroll
-          for (int j = 0; j < HN; ++j) add_group(V[j], f[j], g);
+          for (int j = 0; j < HN; ++j) add_group<SH>(V[j], f[j], g);
         }
         if (!ok) break;
         if (sg % FLUSH != FLUSH - 1 && sg != nseg - 1) continue;
@@ -376,7 +375,7 @@ __global__ void __launch_bounds__(EX_THREADS, 1) ex_kernel(const __grid_constant
           out = P.C + (P.r0 + I.row + m) * P.ldc + I.n0 + j0;
           so = 1;
         }
-        const int64_t off = (int64_t)(kGroupOffset * (uint64_t)(sg % FLUSH + 1));   // segments in V
+        const int64_t off = (int64_t)(group_offset<SH>() * (uint64_t)(sg % FLUSH + 1));   // segments in V
         constexpr int bad = MODE == EX_TALL ? kNonFinite : 2047;
 #pragma unroll
         for (int j = 0; j < HN; ++j) {
@@ -384,7 +383,7 @@ __global__ void __launch_bounds__(EX_THREADS, 1) ex_kernel(const __grid_constant
           if (j0 + j < I.nv && m < I.mv) {
             double v;
             if (e == bad || em == bad) v = quiet_nan();
-            else v = compose(V[j] - off, e + em);     // a vector of zeros has V = 0
+            else v = compose<SH>(V[j] - off, e + em);     // a vector of zeros has V = 0
             if (!first) v += *out;
             *out = v;
           }
@@ -722,7 +721,8 @@ __global__ void __launch_bounds__(256) ex_u_words_kernel(const double* __restric
   W[(int64_t)k * ldw + j] = w;
 }
 
-// Scales of the cell matrices' rows, one warp per row, and the largest over all
+// Scales of the cell matrices' rows, one warp per row (the exponent of the
+// largest entry, raised until the first digits add up to at most 2,040), and the largest over all
 // rows (atomicMax into hsum, zeroed by the caller) of the bounds of their group
 // sums g <= 5: the sums of |digits| of the row against the largest digits any M
 // vector can have (64 for the first, else 128).  Up to 2^24 one FP32 segment
@@ -735,50 +735,30 @@ __global__ void __launch_bounds__(256) ex_h_scale_kernel(const double* __restric
   int m = 0;
   for (int k = lane; k < ne; k += 32) m = max(m, expo(Ht[r * ne + k]));
   m = __reduce_max_sync(0xffffffffu, m);
-  int a[6] = {0, 0, 0, 0, 0, 0};
-  for (int k = lane; k < ne; k += 32) {
-    const double v = Ht[r * ne + k];
-    const uint64_t w = word_of(v, m - expo(v));
+  int a[6];
+  for (int up = 0;; ++up) {
 #pragma unroll
-    for (int d = 0; d < 6; ++d) a[d] += abs((int)((w >> (56 - 8 * d)) & 0xff) - 128);
+    for (int d = 0; d < 6; ++d) a[d] = 0;
+    for (int k = lane; k < ne; k += 32) {
+      const double v = Ht[r * ne + k];
+      const uint64_t w = word_of(v, m - expo(v));
+#pragma unroll
+      for (int d = 0; d < 6; ++d) a[d] += abs((int)((w >> (56 - 8 * d)) & 0xff) - 128);
+    }
+#pragma unroll
+    for (int d = 0; d < 6; ++d) a[d] = __reduce_add_sync(0xffffffffu, a[d]);
+    if (a[0] <= 2040 || m >= 2040 || up == 8) break;   // |V| <= 64 a[0] 2^45 + ... < 2^63
+    ++m;
   }
   int bound = 0, below = 0;
 #pragma unroll
   for (int g = 0; g < 6; ++g) {
-    a[g] = __reduce_add_sync(0xffffffffu, a[g]);
     bound = max(bound, (64 * a[g] + 128 * below) * (g < 2 ? 4 : 1));
     below += a[g];
   }
   if (lane == 0) {
     hexp[r] = (int16_t)m;
     atomicMax(hsum, bound);
-  }
-}
-
-// Words of the cell matrices, K-major with rows padded to rp: block (32, 8)
-// per 32 x 32 tile of a cell.
-__global__ void __launch_bounds__(256) ex_h_words_kernel(const double* __restrict__ Ht, int ne, int rp,
-                                                         const int16_t* __restrict__ hexp,
-                                                         uint64_t* __restrict__ W) {
-  __shared__ uint64_t t[32][33];
-  const int64_t e = blockIdx.z * (int64_t)gridDim.y + blockIdx.y;
-  const int nt = (ne + 31) / 32;
-  const int l0 = (int)(blockIdx.x % nt) * 32, k0 = (int)(blockIdx.x / nt) * 32;
-#pragma unroll
-  for (int i = 0; i < 32; i += 8) {
-    const int l = l0 + threadIdx.y + i, k = k0 + threadIdx.x;
-    uint64_t w = kZeroWord;
-    if (l < ne && k < ne) {
-      const double v = Ht[(e * ne + l) * (int64_t)ne + k];
-      w = word_of(v, hexp[e * ne + l] - expo(v));
-    }
-    t[threadIdx.y + i][threadIdx.x] = w;
-  }
-  __syncthreads();
-#pragma unroll
-  for (int i = 0; i < 32; i += 8) {
-    const int k = k0 + threadIdx.y + i, l = l0 + threadIdx.x;
-    if (k < ne && l < ne) W[(e * ne + k) * (int64_t)rp + l] = t[threadIdx.x][threadIdx.y + i];
   }
 }
 
@@ -955,20 +935,14 @@ void ex_cell_bytes(int64_t ncells, int ne, size_t* words, size_t* ex) {
   *ex = 16 + (size_t)ncells * ne * sizeof(int16_t);
 }
 
-cudaError_t ex_pack_cells(const ExCellData& d, const double* dHt, int64_t ncells, int ne, cudaStream_t s) {
-  const int64_t rows = ncells * ne;
+cudaError_t ex_pack_cells(const ExCellData& d, const CellMatArgs& m, int ne, cudaStream_t s) {
+  const int64_t rows = m.ncells * ne;
   cudaError_t e = cudaMemsetAsync(d.hsum, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
   note_launch();
-  ex_h_scale_kernel<<<(unsigned)((rows + 7) / 8), 256, 0, s>>>(dHt, rows, ne, d.hexp(), d.hsum);
-  const int nt = (ne + 31) / 32;
-  for (int64_t e0 = 0; e0 < ncells; e0 += 32768) {
-    const unsigned n = (unsigned)std::min<int64_t>(32768, ncells - e0);
-    note_launch();
-    ex_h_words_kernel<<<dim3(nt * nt, n), dim3(32, 8), 0, s>>>(dHt + e0 * ne * (int64_t)ne, ne, pad2(ne),
-                                                               d.hexp() + e0 * ne, d.words + e0 * ne * (int64_t)pad2(ne));
-  }
-  return cudaGetLastError();
+  ex_h_scale_kernel<<<(unsigned)((rows + 7) / 8), 256, 0, s>>>(m.Ht, rows, ne, d.hexp(), d.hsum);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  return launch_cell_words(m, d.hexp(), d.words, pad2(ne), s);
 }
 
 size_t ex_cell_work_bytes(int64_t ncells, int ne, int ncol) {

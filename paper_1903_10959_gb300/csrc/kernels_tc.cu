@@ -84,17 +84,19 @@ __global__ void tc_pack_kernel(const double* __restrict__ Ht, float* __restrict_
   base[mt * 1024 + t * 1024 + o] = lo;
 }
 
-cudaError_t tc_build(TcCellData& d, const std::vector<double>&, int64_t ncells, int ne,
-                     cudaStream_t s, int64_t* dev_bytes) {
-  // the device copy of the binary64 cell matrices is packed by tc_pack_from_device
-  (void)s;
-  (void)dev_bytes;
-  d = TcCellData();
+void tc_build(TcCellData& d, int64_t ncells, int ne, int64_t* dev_bytes) {
+  // the device copy of the binary64 cell matrices is packed on first use
+  uint16_t* bf = d.bf;
+  const size_t bf_bytes = d.bf_bytes;
+  if (dev_bytes) *dev_bytes -= (int64_t)(d.bytes + d.f16_bytes + d.nl_bytes + d.pj_bytes);
+  d.bf = nullptr;
+  tc_free(d);
+  d.bf = bf;
+  d.bf_bytes = bf ? bf_bytes : 0;
   d.ncells = ncells;
   d.ne = ne;
   d.mt = (ne + 127) / 128;
   d.kt = (ne + CELL_KC - 1) / CELL_KC * CELL_KC;
-  return cudaSuccess;
 }
 
 cudaError_t tc_pack_from_device(TcCellData& d, const double* dHt, cudaStream_t s,
@@ -141,12 +143,27 @@ __device__ __host__ __forceinline__ int bf_elem_off(int r, int k) {   // in bf16
   return (r >> 3) * 128 + (k >> 3) * 64 + (r & 7) * 8 + (k & 7);
 }
 
+// The split of a binary64 value in binary32 arithmetic: v = f + e with f =
+// float(v) and the remainder e, both from the bits of v (its first 24
+// significant bits and the other 29), so that no conversion or addition runs on
+// the binary64 pipe, which has a sixty-fourth of the rate.  b1, f - b1 and
+// f - b1 - b2 are exact; values below 2^-126 vanish.
 __device__ __forceinline__ void bf16_split3(double v, uint16_t& b1, uint16_t& b2, uint16_t& b3) {
-  const __nv_bfloat16 h1 = __float2bfloat16_rn((float)v);
-  const double r1 = v - (double)__bfloat162float(h1);
-  const __nv_bfloat16 h2 = __float2bfloat16_rn((float)r1);
-  const double r2 = r1 - (double)__bfloat162float(h2);
-  const __nv_bfloat16 h3 = __float2bfloat16_rn((float)r2);
+  const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+  const int ex = (int)((hi >> 20) & 0x7ff) - 896;                // binary32 exponent field
+  const uint32_t sg = hi & 0x80000000u;
+  float t = __uint_as_float(sg | 0x7f800000u), r = 0.f;           // beyond the range of binary32
+  if (ex <= 0) {
+    t = 0.f;
+  } else if (ex < 255) {
+    t = __uint_as_float(sg | (uint32_t)ex << 23 | (hi & 0xfffffu) << 3 | lo >> 29);
+    if (ex > 52) r = (float)(lo & 0x1fffffffu) * __uint_as_float(sg | (uint32_t)(ex - 52) << 23);
+  }
+  const float f = t + r, e = (t - f) + r;
+  const __nv_bfloat16 h1 = __float2bfloat16_rn(f);
+  const float r1 = f - __bfloat162float(h1);
+  const __nv_bfloat16 h2 = __float2bfloat16_rn(r1 + e);
+  const __nv_bfloat16 h3 = __float2bfloat16_rn((r1 - __bfloat162float(h2)) + e);
   b1 = __bfloat16_as_ushort(h1);
   b2 = __bfloat16_as_ushort(h2);
   b3 = __bfloat16_as_ushort(h3);
@@ -198,30 +215,46 @@ __device__ __forceinline__ void f16_split2_pair(float x0, float x1, uint32_t& w1
   w2 = cvt_f16x2(r1, r0);
 }
 
-// add (optional): an n_e x n_e matrix added to every cell's matrix first.
-__global__ void tc_pack_bf16_kernel(const double* __restrict__ Ht, uint16_t* __restrict__ out,
-                                    int64_t ncells, int ne, int mt, int nk16,
-                                    const double* __restrict__ add = nullptr) {
-  const int64_t per_chunk = (int64_t)mt * 2048;   // elements of one term, all tiles
-  const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (idx >= ncells * nk16 * per_chunk) return;
-  // one thread per (cell, chunk, tile, row, k); writes the three terms
-  const int64_t e = idx / (nk16 * per_chunk);
-  int64_t rem = idx - e * nk16 * per_chunk;
-  const int kc = (int)(rem / per_chunk);
-  rem -= (int64_t)kc * per_chunk;
-  const int t = (int)(rem / 2048);
-  const int w = (int)(rem - t * 2048);
-  const int r = w / BF_KC, k = w % BF_KC;
-  const int row = t * 128 + r, col = kc * BF_KC + k;
-  double v = (row < ne && col < ne) ? Ht[(e * ne + row) * (int64_t)ne + col] : 0.0;
-  if (add && row < ne && col < ne) v += add[(int64_t)row * ne + col];
-  uint16_t b1, b2, b3;
-  bf16_split3(v, b1, b2, b3);
-  uint16_t* base = out + (e * nk16 + kc) * 3 * per_chunk + (int64_t)t * 2048 + bf_elem_off(r, k);
-  base[0] = b1;
-  base[per_chunk] = b2;
-  base[2 * per_chunk] = b3;
+// add (optional): an n_e x n_e matrix added to every cell's matrix first.  One
+// thread per (cell, chunk, 16-byte unit of a term): eight values of a row, read
+// as one stretch, written as one unit of each of the three terms.
+__global__ void __launch_bounds__(256) tc_pack_bf16_kernel(const double* __restrict__ Ht, uint16_t* __restrict__ out,
+                                                           int64_t ncells, int ne, int mt, int nk16,
+                                                           const double* __restrict__ add = nullptr) {
+  const int units = mt * 256;                     // 16-byte units of one term, all tiles
+  const int u = blockIdx.x * 256 + threadIdx.x;
+  if (u >= units * nk16) return;
+  const int64_t e = blockIdx.y + (int64_t)blockIdx.z * gridDim.y;
+  if (e >= ncells) return;
+  const int kc = u / units, w = u % units;
+  const int row = (w >> 8) * 128 + ((w & 255) >> 4) * 8 + (w & 7), k0 = kc * BF_KC + ((w >> 3) & 1) * 8;
+  uint32_t b[3][4] = {};
+  if (row < ne) {
+    const double* h = Ht + (e * ne + row) * (int64_t)ne;
+    double v[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      v[j] = k0 + j < ne ? h[k0 + j] : 0.0;
+      if (add && k0 + j < ne) v[j] += add[(int64_t)row * ne + k0 + j];
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      uint16_t t[3];
+      bf16_split3(v[j], t[0], t[1], t[2]);
+#pragma unroll
+      for (int p = 0; p < 3; ++p) b[p][j >> 1] |= (uint32_t)t[p] << (16 * (j & 1));
+    }
+  }
+  uint4* base = reinterpret_cast<uint4*>(out) + ((e * nk16 + kc) * 3) * (int64_t)units + w;
+#pragma unroll
+  for (int p = 0; p < 3; ++p) base[(int64_t)p * units] = make_uint4(b[p][0], b[p][1], b[p][2], b[p][3]);
+}
+static void pack_bf16(const double* dHt, uint16_t* out, int64_t ncells, int ne, int mt, int nk16, const double* add,
+                      cudaStream_t s) {
+  const unsigned ny = (unsigned)std::min<int64_t>(ncells, 32768);
+  note_launch();
+  tc_pack_bf16_kernel<<<dim3((unsigned)(mt * nk16), ny, (unsigned)((ncells + ny - 1) / ny)), 256, 0, s>>>(
+      dHt, out, ncells, ne, mt, nk16, add);
 }
 
 cudaError_t tc_pack_bf16_matrices(const double* dH, const double* dadd, int64_t ncells, int ne, uint16_t** out,
@@ -236,26 +269,25 @@ cudaError_t tc_pack_bf16_matrices(const double* dH, const double* dadd, int64_t 
     }
     *bytes = need;
   }
-  const int64_t n = ncells * (int64_t)nk16 * mt * 2048;
-  note_launch();
-  tc_pack_bf16_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(dH, *out, ncells, ne, mt, nk16, dadd);
+  if (ncells > 0) pack_bf16(dH, *out, ncells, ne, mt, nk16, dadd, s);
   return cudaGetLastError();
 }
 
 cudaError_t tc_pack_bf16_from_device(TcCellData& d, const double* dHt, cudaStream_t s,
                                      int64_t* dev_bytes) {
   const int nk16 = (d.ne + BF_KC - 1) / BF_KC;
-  d.bf_bytes = (size_t)d.ncells * nk16 * 3 * d.mt * 2048 * sizeof(uint16_t);
-  cudaError_t e = cudaMalloc(&d.bf, d.bf_bytes);
-  if (e != cudaSuccess) {
-    d.bf = nullptr;
-    d.bf_bytes = 0;
-    return e;
+  if (!d.bf) {
+    d.bf_bytes = (size_t)d.ncells * nk16 * 3 * d.mt * 2048 * sizeof(uint16_t);
+    cudaError_t e = cudaMalloc(&d.bf, d.bf_bytes);
+    if (e != cudaSuccess) {
+      d.bf = nullptr;
+      d.bf_bytes = 0;
+      return e;
+    }
+    if (dev_bytes) *dev_bytes += (int64_t)d.bf_bytes;
   }
-  if (dev_bytes) *dev_bytes += (int64_t)d.bf_bytes;
-  const int64_t n = d.ncells * (int64_t)nk16 * d.mt * 2048;
-  note_launch();
-  tc_pack_bf16_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(dHt, d.bf, d.ncells, d.ne, d.mt, nk16);
+  d.bf_ready = true;
+  pack_bf16(dHt, d.bf, d.ncells, d.ne, d.mt, nk16, nullptr, s);
   return cudaGetLastError();
 }
 

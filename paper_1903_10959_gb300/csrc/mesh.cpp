@@ -247,144 +247,71 @@ void build_mesh(const chfsi_mesh_desc& d, HostMesh& m) {
         }
 }
 
-// Potential of the wells at a point (wells pre-filtered to those in range).
-static inline double well_sum(const double* x, const std::vector<double>& cx,
-                              const std::vector<double>& dd, const std::vector<double>& inv2w2) {
-  double v = 0.0;
-  for (size_t a = 0; a < dd.size(); ++a) {
-    double dx = x[0] - cx[3 * a], dy = x[1] - cx[3 * a + 1], dz = x[2] - cx[3 * a + 2];
-    v -= dd[a] * std::exp(-(dx * dx + dy * dy + dz * dz) * inv2w2[a]);
+namespace {
+// Sums and products as unevaluated pairs (error-free transformations of Dekker
+// and Knuth with a fused multiply-add).
+struct Pair {
+  double hi, lo;
+};
+inline Pair two_sum(double a, double b) {
+  const double s = a + b, t = s - a;
+  return {s, (a - (s - t)) + (b - t)};
+}
+inline Pair mul(Pair a, double b) {
+  const double p = a.hi * b;
+  return two_sum(p, std::fma(a.hi, b, -p) + a.lo * b);
+}
+inline Pair add(Pair a, Pair b) {
+  const Pair s = two_sum(a.hi, b.hi);
+  return two_sum(s.hi, s.lo + (a.lo + b.lo));
+}
+}  // namespace
+
+void build_kinetic(const HostMesh& m, std::vector<double>& K, std::vector<double>& s1) {
+  const int n1 = m.n1, ne = m.ne, nn = n1 * n1;
+  std::vector<double> fac;
+  build_mf_factors(m, fac);   // A_x, A_y, A_z, S_x, S_y, S_z
+  const double* A[3] = {&fac[0], &fac[nn], &fac[2 * nn]};
+  const double* S[3] = {&fac[3 * nn], &fac[4 * nn], &fac[5 * nn]};
+  // a node on a cell face is shared by two cells (a face node of one cell only
+  // lies on a Dirichlet boundary and is eliminated)
+  auto shared = [&](int i) { return i == 0 || i == m.p ? 2.0 : 1.0; };
+  s1.resize(3 * n1);
+  for (int ax = 0; ax < 3; ++ax)
+    for (int i = 0; i < n1; ++i) s1[ax * n1 + i] = 1.0 / std::sqrt(m.gll_w[i] * shared(i) * m.h[ax] / 2.0);
+  const double jac = m.h[0] * m.h[1] * m.h[2] / 8.0;
+  std::vector<double> s(ne);   // M^{-1/2} as the assembled mass gives it
+  for (int k = 0; k < n1; ++k)
+    for (int j = 0; j < n1; ++j)
+      for (int i = 0; i < n1; ++i)
+        s[i + n1 * (j + n1 * k)] =
+            1.0 / std::sqrt(m.gll_w[i] * m.gll_w[j] * m.gll_w[k] * jac * (shared(i) * shared(j) * shared(k)));
+  K.assign((size_t)2 * ne * ne, 0.0);
+#pragma omp parallel for schedule(static)
+  for (int r = 0; r < ne; ++r) {
+    const int i = r % n1, j = r / n1 % n1, k = r / nn;
+    for (int c = 0; c < ne; ++c) {
+      const int il = i * n1 + c % n1, jm = j * n1 + c / n1 % n1, kn = k * n1 + c / nn;
+      const Pair t = add(add(mul(mul({S[0][il], 0.0}, A[1][jm]), A[2][kn]), mul(mul({A[0][il], 0.0}, S[1][jm]), A[2][kn])),
+                         mul(mul({A[0][il], 0.0}, A[1][jm]), S[2][kn]));
+      const Pair v = mul(mul(t, 0.5 * s[r]), s[c]);
+      K[(size_t)r * ne + c] = v.hi;
+      K[(size_t)ne * ne + (size_t)r * ne + c] = v.lo;
+    }
   }
-  return v;
 }
 
-void build_cell_matrices(const HostMesh& m, const Wells& wl, std::vector<double>& Ht,
-                         std::vector<double>* wv) {
-  const int n1 = m.n1, ne = m.ne, q = m.q;
-  const int nn = n1 * n1;
-  Ht.assign((size_t)m.ncells * ne * ne, 0.0);
-  if (wv) wv->assign((size_t)m.ncells * q * q * q, 0.0);
-
-  // 1-D consistent mass A and stiffness S per axis (Gauss rule, exact)
-  std::vector<double> A[3], S[3];
-  for (int ax = 0; ax < 3; ++ax) {
-    A[ax].assign(nn, 0.0);
-    S[ax].assign(nn, 0.0);
-    for (int i = 0; i < n1; ++i)
-      for (int l = 0; l < n1; ++l) {
-        double sa = 0.0, ss = 0.0;
-        for (int a = 0; a < q; ++a) {
-          sa += m.gq_w[a] * m.B[a * n1 + i] * m.B[a * n1 + l];
-          ss += m.gq_w[a] * m.D[a * n1 + i] * m.D[a * n1 + l];
-        }
-        A[ax][i * n1 + l] = sa * m.h[ax] / 2.0;
-        S[ax][i * n1 + l] = ss * 2.0 / m.h[ax];
-      }
-  }
-  // shared kinetic matrix 1/2 K (identical for every cell of the uniform mesh)
-  std::vector<double> K(ne * ne);
-  for (int k = 0; k < n1; ++k) for (int j = 0; j < n1; ++j) for (int i = 0; i < n1; ++i)
-    for (int c = 0; c < n1; ++c) for (int b = 0; b < n1; ++b) for (int a = 0; a < n1; ++a) {
-      int r = i + n1 * (j + n1 * k), s = a + n1 * (b + n1 * c);
-      K[r * ne + s] = 0.5 * (S[0][i * n1 + a] * A[1][j * n1 + b] * A[2][k * n1 + c] +
-                             A[0][i * n1 + a] * S[1][j * n1 + b] * A[2][k * n1 + c] +
-                             A[0][i * n1 + a] * A[1][j * n1 + b] * S[2][k * n1 + c]);
-    }
-  // BB[a][i*n1+l] = w_a B[a][i] B[a][l]
-  std::vector<double> BB(q * nn);
-  for (int a = 0; a < q; ++a)
-    for (int i = 0; i < n1; ++i)
-      for (int l = 0; l < n1; ++l) BB[a * nn + i * n1 + l] = m.gq_w[a] * m.B[a * n1 + i] * m.B[a * n1 + l];
-
-  // wells: images along the periodic axes as explicit centres; cut off where
-  // the Gaussian is < 1e-18 D
-  std::vector<double> ic, idp, iw;
-  const int nw = (int)wl.depth.size();
-  for (int a = 0; a < nw; ++a) {
+void build_well_images(const HostMesh& m, const Wells& wl, std::vector<double>& out) {
+  out.clear();
+  for (size_t a = 0; a < wl.depth.size(); ++a)
     for (int sz = -1; sz <= 1; ++sz) for (int sy = -1; sy <= 1; ++sy) for (int sx = -1; sx <= 1; ++sx) {
       if ((!m.per[0] && sx) || (!m.per[1] && sy) || (!m.per[2] && sz)) continue;
-      ic.push_back(wl.xyz[3 * a] + sx * m.len[0]);
-      ic.push_back(wl.xyz[3 * a + 1] + sy * m.len[1]);
-      ic.push_back(wl.xyz[3 * a + 2] + sz * m.len[2]);
-      idp.push_back(wl.depth[a]);
-      iw.push_back(wl.width[a]);
+      out.push_back(wl.xyz[3 * a] + sx * m.len[0]);
+      out.push_back(wl.xyz[3 * a + 1] + sy * m.len[1]);
+      out.push_back(wl.xyz[3 * a + 2] + sz * m.len[2]);
+      out.push_back(wl.depth[a]);
+      out.push_back(1.0 / (2.0 * wl.width[a] * wl.width[a]));
     }
-  }
-  const double jac = m.h[0] * m.h[1] * m.h[2] / 8.0;
-
-#pragma omp parallel
-  {
-    std::vector<double> cx, dd, inv2w2, V(q * q * q), T1(q * q * nn), T2(q * nn * nn), He(ne * ne);
-    double xq[3];
-#pragma omp for schedule(dynamic, 4)
-    for (int64_t e = 0; e < m.ncells; ++e) {
-      int c3[3] = {(int)(e % m.n[0]), (int)((e / m.n[0]) % m.n[1]), (int)(e / ((int64_t)m.n[0] * m.n[1]))};
-      double lo[3], hi[3];
-      for (int ax = 0; ax < 3; ++ax) { lo[ax] = c3[ax] * m.h[ax]; hi[ax] = lo[ax] + m.h[ax]; }
-      cx.clear(); dd.clear(); inv2w2.clear();
-      for (size_t a = 0; a < idp.size(); ++a) {
-        double r2 = 0.0;
-        for (int ax = 0; ax < 3; ++ax) {
-          double c = ic[3 * a + ax];
-          double dlt = c < lo[ax] ? lo[ax] - c : (c > hi[ax] ? c - hi[ax] : 0.0);
-          r2 += dlt * dlt;
-        }
-        if (r2 * 1.0 / (2.0 * iw[a] * iw[a]) > 41.5) continue;   // exp(-41.5) < 1e-18
-        cx.push_back(ic[3 * a]); cx.push_back(ic[3 * a + 1]); cx.push_back(ic[3 * a + 2]);
-        dd.push_back(idp[a]);
-        inv2w2.push_back(1.0 / (2.0 * iw[a] * iw[a]));
-      }
-      const double* vq = wl.vqp.empty() ? nullptr : wl.vqp.data() + e * (int64_t)q * q * q;
-      for (int c = 0; c < q; ++c) for (int b = 0; b < q; ++b) for (int a = 0; a < q; ++a) {
-        xq[0] = lo[0] + (m.gq_x[a] + 1.0) * m.h[0] / 2.0;
-        xq[1] = lo[1] + (m.gq_x[b] + 1.0) * m.h[1] / 2.0;
-        xq[2] = lo[2] + (m.gq_x[c] + 1.0) * m.h[2] / 2.0;
-        const int pt = (c * q + b) * q + a;
-        V[pt] = (well_sum(xq, cx, dd, inv2w2) + (vq ? vq[pt] : 0.0)) * jac;
-        if (wv) (*wv)[(size_t)e * q * q * q + pt] = V[pt] * m.gq_w[a] * m.gq_w[b] * m.gq_w[c];
-      }
-      // T1[c][b][il] = sum_a BB[a][il] V[c][b][a]
-      for (int cb = 0; cb < q * q; ++cb)
-        for (int il = 0; il < nn; ++il) {
-          double s = 0.0;
-          for (int a = 0; a < q; ++a) s += BB[a * nn + il] * V[cb * q + a];
-          T1[cb * nn + il] = s;
-        }
-      // T2[c][jm][il] = sum_b BB[b][jm] T1[c][b][il]
-      for (int c = 0; c < q; ++c)
-        for (int jm = 0; jm < nn; ++jm)
-          for (int il = 0; il < nn; ++il) {
-            double s = 0.0;
-            for (int b = 0; b < q; ++b) s += BB[b * nn + jm] * T1[(c * q + b) * nn + il];
-            T2[(c * nn + jm) * nn + il] = s;
-          }
-      // V_e[(i j k),(l m n)] = sum_c BB[c][kn] T2[c][jm][il]
-      for (int k = 0; k < n1; ++k) for (int nk = 0; nk < n1; ++nk) {
-        int kn = k * n1 + nk;
-        for (int j = 0; j < n1; ++j) for (int mj = 0; mj < n1; ++mj) {
-          int jm = j * n1 + mj;
-          for (int i = 0; i < n1; ++i) for (int li = 0; li < n1; ++li) {
-            int il = i * n1 + li;
-            double s = 0.0;
-            for (int c = 0; c < q; ++c) s += BB[c * nn + kn] * T2[(c * nn + jm) * nn + il];
-            int r = i + n1 * (j + n1 * k), col = li + n1 * (mj + n1 * nk);
-            He[r * ne + col] = s;
-          }
-        }
-      }
-      // H~_e = D^{-1/2} (1/2 K + V_e) D^{-1/2}; rows/cols of eliminated nodes zero
-      double* out = &Ht[(size_t)e * ne * ne];
-      const int32_t* dm = &m.dofmap[e * ne];
-      for (int r = 0; r < ne; ++r) {
-        if (dm[r] < 0) continue;
-        double sr = 1.0 / std::sqrt(m.mass[dm[r]]);
-        for (int c = 0; c < ne; ++c) {
-          if (dm[c] < 0) continue;
-          out[(size_t)r * ne + c] = (K[r * ne + c] + He[r * ne + c]) * sr / std::sqrt(m.mass[dm[c]]);
-        }
-      }
-    }
-  }
 }
 
 void build_mf_factors(const HostMesh& m, std::vector<double>& fac) {
@@ -414,6 +341,7 @@ void build_projectors(const HostMesh& m, const Projectors& pr, HostProjectors& o
   const int ns = (int)pr.h.size() / 4;
   const int n1 = m.n1, ne = m.ne, q = m.q;
   out = HostProjectors();
+  if (ns == 0) return;
   out.nsite = ns;
   out.site_ptr.assign(ns + 1, 0);
   const double jac = m.h[0] * m.h[1] * m.h[2] / 8.0;

@@ -478,23 +478,30 @@ chfsi_status chfsi_set_potential_qp_device(chfsi_ctx* ctx, const double* v) {
     ctx->dev_bytes -= (int64_t)m.ncells * m.ne * m.ne * 8;
     ctx->d_Ht = nullptr;
   }
+  for (auto b : {std::make_pair((void*)ctx->ex.words, ctx->ex.word_bytes), std::make_pair((void*)ctx->ex.hsum, ctx->ex.exp_bytes)})
+    if (b.first) {
+      cudaFree(b.first);
+      ctx->dev_bytes -= (int64_t)b.second;
+    }
+  ctx->ex = ExCellData();
+  ctx->ex_ready = false;
   ctx->dev_bytes -= (int64_t)(ctx->tc.bytes + ctx->tc.bf_bytes + ctx->tc.f16_bytes + ctx->tc.nl_bytes +
                               ctx->tc.pj_bytes);
   ctx->kpack_valid = false;
   tc_free(ctx->tc);
   ctx->tc.ncells = m.ncells;
   ctx->tc.ne = m.ne;
-  if (!ctx->d_wv || ctx->wv.size() != (size_t)n) {
+  if (!ctx->d_wv || ctx->nwv != n) {
     if (ctx->d_wv) {
       cudaFree(ctx->d_wv);
-      ctx->dev_bytes -= (int64_t)ctx->wv.size() * 8;
+      ctx->dev_bytes -= ctx->nwv * 8;
       ctx->d_wv = nullptr;
     }
-    ctx->wv.assign((size_t)n, 0.0);
+    ctx->nwv = n;
     if (cudaMalloc(&ctx->d_wv, (size_t)n * 8) != cudaSuccess) {
       cudaGetLastError();
       ctx->d_wv = nullptr;
-      ctx->wv.clear();
+      ctx->nwv = 0;
       return sfail(ctx, CHFSI_ERR_OOM, "potential factor");
     }
     ctx->dev_bytes += n * 8;

@@ -18,6 +18,7 @@ struct TcCellData {
   // BF16x3 copy (three bf16 terms per value), packed on first use
   uint16_t* bf = nullptr;
   size_t bf_bytes = 0;
+  bool bf_ready = false;   // false after a rebuild: the buffer waits for the new matrices
   // FP16x2 copy (two fp16 terms of 2^s_e H~_e per value) and the per-cell
   // inverse scales 2^-s_e (float), packed on first use; f16_bytes covers both
   uint16_t* f16 = nullptr;
@@ -153,8 +154,9 @@ cudaError_t tc_cell_f16_launch(const TcCellData& d, const TcApplyArgs& a, const 
 cudaError_t tc_pack_f16_from_device(TcCellData& d, const double* dHt, cudaStream_t s,
                                     int64_t* dev_bytes);
 
-cudaError_t tc_build(TcCellData& d, const std::vector<double>& Ht, int64_t ncells, int ne,
-                     cudaStream_t s, int64_t* dev_bytes);
+// Start over for new cell matrices of the same mesh: every packed copy is freed
+// (and taken off *dev_bytes) but the BF16x3 buffer, which the next pack fills.
+void tc_build(TcCellData& d, int64_t ncells, int ne, int64_t* dev_bytes);
 // Split the binary64 device cell matrices into three bf16 terms (BF16x3 layout).
 cudaError_t tc_pack_bf16_from_device(TcCellData& d, const double* dHt, cudaStream_t s,
                                      int64_t* dev_bytes);
