@@ -140,7 +140,7 @@ constexpr bool kMatrixFreeDefault = true;
 // blocks, projector and binary64 staging buffers); later calls regrow it.
 void release_scratch(chfsi_ctx* ctx) {
   cudaStreamSynchronize(ctx->stream);
-  for (DevBuf* b : {&ctx->T1, &ctx->Wb, &ctx->NLb, &ctx->Zb, &ctx->Rb, &ctx->rot, &ctx->cmaxb, &ctx->pjb, &ctx->tinv,
+  for (DevBuf* b : {&ctx->T1, &ctx->T2, &ctx->Wb, &ctx->NLb, &ctx->Zb, &ctx->Rb, &ctx->rot, &ctx->cmaxb, &ctx->pjb, &ctx->tinv,
                     &ctx->exb}) {
     dfree(ctx, b->ptr, b->bytes);
     b->ptr = nullptr;
@@ -413,7 +413,8 @@ chfsi_status apply_step(chfsi_ctx* ctx, chfsi_precision prec, const void* Yin, i
   }
   // owner-computes: dense cell blocks R_e (one launch over all cells), then the
   // fixed-order assembly fused with the Chebyshev update
-  if ((st = grow(ctx, ctx->Rb, (size_t)m.ncells * m.ne * ncol * sizeof(float))) != CHFSI_OK) return st;
+  const int64_t ldr4 = (ncol + 3) & ~3;   // 16-byte rows of R
+  if ((st = grow(ctx, ctx->Rb, (size_t)m.ncells * m.ne * ldr4 * sizeof(float))) != CHFSI_OK) return st;
   TcApplyArgs ra{};
   ra.dofmap = ctx->d_dofmap;
   ra.ncells = m.ncells;
@@ -421,6 +422,7 @@ chfsi_status apply_step(chfsi_ctx* ctx, chfsi_precision prec, const void* Yin, i
   ra.Yin = (const float*)Yin;
   ra.ld_in = ld_in;
   ra.R = (float*)ctx->Rb.ptr;
+  ra.ldr = ldr4;
   ra.split3 = prec == CHFSI_MIXED_TF32X3;
   ra.tile = ctx->cell_tile;
   ra.gather = ctx->cell_gather;
@@ -447,6 +449,7 @@ chfsi_status apply_step(chfsi_ctx* ctx, chfsi_precision prec, const void* Yin, i
   ap.M = m.ndofs;
   ap.ncol = ncol;
   ap.R = (const float*)ctx->Rb.ptr;
+  ap.ldr = ldr4;
   ap.Yin = (const float*)Yin;
   ap.ld_in = ld_in;
   ap.Yout = (float*)Yout;
@@ -510,6 +513,7 @@ void toc(chfsi_ctx* ctx, int slot) {
 
 // The filter of the columns [0, ncol) of X in blocks of the filter block size
 // (every step on ctx->stream, scratch in ctx->T1 / Rb / Zb).
+constexpr int kPadDegree = 6;
 chfsi_status filter_range(chfsi_ctx* ctx, void* X, int64_t ldx, int ncol, int degree, double a,
                           double b, double a0, chfsi_precision prec) {
   const HostMesh& m = ctx->mesh;
@@ -525,6 +529,32 @@ chfsi_status filter_range(chfsi_ctx* ctx, void* X, int64_t ldx, int ncol, int de
     // Y0 = Xb, Y1 -> T1, then Y_{k+1} overwrites Y_{k-1}
     void* bufs[2] = {Xb, ctx->T1.ptr};
     int64_t lds[2] = {ldx, (int64_t)nb};
+    // Mixed precisions, rows of X not on 16 bytes or a ragged width: the steps
+    // run on copies padded with zero columns to whole 16-byte quads, so that the
+    // assembly takes 16-byte accesses (7^3 cells, p = 5, 77 columns: 20.7 -> 16.5
+    // us a step; 10^3, p = 6, 1,001: 751 -> 669).  Not FP16x2, whose
+    // column scales come with the block, nor a few steps, which the two copies
+    // would cost.
+    int ncs = nb;   // columns of the steps
+    bool pad = is_mixed(prec) && prec != CHFSI_MIXED_F16X2 && degree >= kPadDegree &&
+               ((nb & 3) || (ldx & 3) || (reinterpret_cast<uintptr_t>(Xb) & 15));
+    if (pad) {
+      const std::string err = ctx->err;
+      const int n4 = (nb + 3) & ~3;
+      if (grow(ctx, ctx->T2, (size_t)m.ndofs * n4 * es) == CHFSI_OK &&
+          grow(ctx, ctx->T1, (size_t)m.ndofs * n4 * es) == CHFSI_OK) {
+        ncs = n4;
+        bufs[0] = ctx->T2.ptr;
+        bufs[1] = ctx->T1.ptr;
+        lds[0] = lds[1] = n4;
+        CK(launch_copy_pad((const float*)Xb, ldx, nb, (float*)ctx->T2.ptr, n4, m.ndofs, ctx->stream));
+      } else {
+        ctx->err = err;
+        pad = false;
+        if ((st = grow(ctx, ctx->T1, (size_t)m.ndofs * nb * es)) != CHFSI_OK) return st;
+        bufs[1] = ctx->T1.ptr;
+      }
+    }
     int cur = 0;  // buffer holding Y_k
     double sig = s1;
     // FP16x2: each step's assembly leaves the column maxima of its output, the
@@ -547,12 +577,14 @@ chfsi_status filter_range(chfsi_ctx* ctx, void* X, int64_t ldx, int ncol, int de
         sig = sn;
       }
       const int nxt = 1 - cur;  // holds Y_{k-2} (or is free at k = 1)
-      st = apply_step(ctx, prec, bufs[cur], lds[cur], bufs[nxt], lds[nxt], bufs[nxt], lds[nxt], nb,
+      st = apply_step(ctx, prec, bufs[cur], lds[cur], bufs[nxt], lds[nxt], bufs[nxt], lds[nxt], ncs,
                       alpha, beta, c, k == 1 ? nullptr : cm[cur], k == degree ? nullptr : cm[nxt]);
       if (st != CHFSI_OK) return st;
       cur = nxt;
     }
-    if (cur == 1)
+    if (pad)
+      CK(launch_copy_pad((const float*)bufs[cur], lds[cur], nb, (float*)Xb, ldx, m.ndofs, ctx->stream, false));
+    else if (cur == 1)
       CK(cudaMemcpy2DAsync(Xb, ldx * es, ctx->T1.ptr, nb * es, nb * es, m.ndofs,
                            cudaMemcpyDeviceToDevice, ctx->stream));
   }
@@ -569,6 +601,7 @@ struct LaneScope {
     if (l == 0) return;
     ctx->stream = ctx->lane_stream[l];
     std::swap(ctx->T1, ctx->laneT1[l]);
+    std::swap(ctx->T2, ctx->laneT2[l]);
     std::swap(ctx->Rb, ctx->laneR[l]);
     std::swap(ctx->Zb, ctx->laneZ[l]);
     std::swap(ctx->cmaxb, ctx->laneC[l]);
@@ -577,6 +610,7 @@ struct LaneScope {
   ~LaneScope() {
     if (l == 0) return;
     std::swap(ctx->T1, ctx->laneT1[l]);
+    std::swap(ctx->T2, ctx->laneT2[l]);
     std::swap(ctx->Rb, ctx->laneR[l]);
     std::swap(ctx->Zb, ctx->laneZ[l]);
     std::swap(ctx->cmaxb, ctx->laneC[l]);
@@ -1012,14 +1046,14 @@ chfsi_status chfsi_destroy(chfsi_ctx* ctx) {
   ctx->d_kfac = nullptr;
   for (void* q : {(void*)ctx->d_kA, (void*)ctx->d_kG, (void*)ctx->kbf, (void*)ctx->kgbf})
     if (q) cudaFree(q);
-  for (DevBuf* b : {&ctx->T1, &ctx->Wb, &ctx->NLb, &ctx->Zb, &ctx->rot, &ctx->Ssq, &ctx->work,
+  for (DevBuf* b : {&ctx->T1, &ctx->T2, &ctx->Wb, &ctx->NLb, &ctx->Zb, &ctx->rot, &ctx->Ssq, &ctx->work,
                     &ctx->part, &ctx->vec, &ctx->lam, &ctx->Rb, &ctx->Db, &ctx->pol, &ctx->scfb, &ctx->scfq,
                     &ctx->cmaxb, &ctx->pjb, &ctx->tinv, &ctx->exb,
                     &ctx->scfr, &ctx->scfw, &ctx->kW, &ctx->kT1, &ctx->kG, &ctx->kS, &ctx->kwork,
                     &ctx->kY, &ctx->kvec})
     dfree(ctx, b->ptr, b->bytes);
   for (int l = 0; l < chfsi_ctx::kMaxLanes; ++l) {
-    for (DevBuf* b : {&ctx->laneT1[l], &ctx->laneR[l], &ctx->laneZ[l], &ctx->laneC[l], &ctx->laneP[l]})
+    for (DevBuf* b : {&ctx->laneT1[l], &ctx->laneT2[l], &ctx->laneR[l], &ctx->laneZ[l], &ctx->laneC[l], &ctx->laneP[l]})
       dfree(ctx, b->ptr, b->bytes);
     if (ctx->lane_stream[l]) cudaStreamDestroy(ctx->lane_stream[l]);
     if (ctx->lane_ev[l]) cudaEventDestroy(ctx->lane_ev[l]);

@@ -60,7 +60,7 @@ struct chfsi_ctx {
   float* d_site_c32 = nullptr;
   float* d_dof_c32 = nullptr;
   // grown scratch
-  chfsi::DevBuf T1, Wb, NLb, Zb, rot, Ssq, work, part, vec, lam, Rb;
+  chfsi::DevBuf T1, T2, Wb, NLb, Zb, rot, Ssq, work, part, vec, lam, Rb;
   chfsi::DevBuf exb;               // digit slices: the block's words and scales
   chfsi::DevBuf pol;               // binary64 staging block of the polish
   chfsi::DevBuf scfb, scfq, scfr, scfw;   // Poisson / SCF work arrays (scf.cu)
@@ -86,7 +86,7 @@ struct chfsi_ctx {
   int filter_lanes = 1;
   cudaStream_t lane_stream[kMaxLanes] = {};   // lane 0 runs on `stream`
   cudaEvent_t lane_ev[kMaxLanes] = {};
-  chfsi::DevBuf laneT1[kMaxLanes], laneR[kMaxLanes], laneZ[kMaxLanes], laneC[kMaxLanes], laneP[kMaxLanes];
+  chfsi::DevBuf laneT1[kMaxLanes], laneT2[kMaxLanes], laneR[kMaxLanes], laneZ[kMaxLanes], laneC[kMaxLanes], laneP[kMaxLanes];
   chfsi::DevBuf cmaxb;             // FP16x2: column maxima of the filter's blocks (3 x ncol words)
   chfsi::DevBuf pjb;               // partial projections of the cells (pj_rows x ncol)
   chfsi::DevBuf tinv;              // CholGS: L^{-1} (n x n binary64)

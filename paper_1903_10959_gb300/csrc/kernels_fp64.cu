@@ -440,6 +440,22 @@ __global__ void copy_cols_kernel(const void* src, int64_t lds, void* dst, int64_
   else ((float*)dst)[r * ldd + c] = (float)v;
 }
 
+__global__ void __launch_bounds__(256) copy_pad_kernel(const float* __restrict__ src, int64_t lds, int ncol,
+                                                       float* __restrict__ dst, int64_t ldd, int64_t rows, int wd) {
+  const int64_t r = (int64_t)blockIdx.x * 8 + threadIdx.y;
+  if (r >= rows) return;
+#pragma unroll 4
+  for (int c = threadIdx.x; c < wd; c += 32) dst[r * ldd + c] = c < ncol ? src[r * lds + c] : 0.f;
+}
+cudaError_t launch_copy_pad(const float* src, int64_t lds, int ncol, float* dst, int64_t ldd, int64_t rows,
+                            cudaStream_t s, bool fill) {
+  if (rows <= 0 || ncol <= 0) return cudaSuccess;
+  note_launch();
+  copy_pad_kernel<<<(unsigned)((rows + 7) / 8), dim3(32, 8), 0, s>>>(src, lds, ncol, dst, ldd, rows,
+                                                                    fill ? (int)ldd : ncol);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_copy_cols(const void* src, int64_t lds, void* dst, int64_t ldd, int64_t rows,
                              int ncol, int src_double, int dst_double, cudaStream_t s) {
   const int64_t tot = rows * ncol;

@@ -28,6 +28,7 @@
 #include <algorithm>
 #include <cstdio>
 #include <mutex>
+#include <type_traits>
 
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -592,7 +593,6 @@ struct RParams {
   const int64_t* pj_row;
   int pj_npmax;
   int tpc;                  // multi-tile kernel: column tiles per CTA
-  int r_evict;              // write R under an evict_first L2 policy (R much larger than L2)
 };
 
 template <int BN, bool MULTI>
@@ -814,7 +814,7 @@ cudaError_t tc_cell_r_launch(const TcCellData& d, const TcApplyArgs& a, cudaStre
   // measured slower than both variants here: the two halves gather Y twice)
   const int bn = a.tile == 128 ? 128 : 64;
   RParams P{d.hi, a.dofmap, a.Yin, a.R, a.ld_in, a.ncol, d.ne, d.mt, d.kt / CELL_KC, a.split3,
-            nullptr, 0, 0, a.ncol, 0};
+            nullptr, 0, 0, a.ldr, 0};
   tc_cell_prepare();
   const CellSmem L = cell_smem(d.mt, a.split3, bn);
   for (int64_t e0 = 0; e0 < a.ncells; e0 += 65535) {   // grid y is limited to 65535
@@ -884,6 +884,38 @@ __host__ __device__ inline BfPlan bf_plan(int ne) {
   b.stages = S;
   b.total = S * stage + kCellSmemTail;
   return b;
+}
+
+// Epilogue of the BF16x3 / FP16x2 cell kernels: the warp's 32 accumulator lanes
+// (one column of the block each), rows [0, nrow) of the tile, rows below rend and
+// lanes with `on` stored to dst + row * ld, times `scale`: 128 contiguous bytes
+// per warp and row.  Sixteen rows at a time without a test per row but at the
+// tail: a CTA has nothing else to do here, and the tests, the 64-bit products of
+// the addresses and a per-row choice of cache policy were a tenth of the launch
+// (16^3 cells, p = 6, 1,100 columns: 5.34 -> 5.03 ms; 7^3, p = 5, 77: 43 -> 37 us;
+// rows staged in shared memory and sent by bulk copies under an evict-first
+// policy: 5.34 ms).
+__device__ __forceinline__ void store_rows(uint32_t taddr, int nrow, int rend, float* dst, int64_t ld, bool on,
+                                           float scale = 1.f) {
+#pragma unroll 1
+  for (int cb = 0; cb < nrow; cb += 16) {
+    float acc[16];
+    __syncwarp();
+    tmem_ld16(taddr + cb, acc);
+    tmem_wait_ld();
+    if (!on) continue;
+    if (cb + 16 <= rend) {
+#pragma unroll
+      for (int j = 0; j < 16; ++j) {
+        *dst = acc[j] * scale;
+        dst += ld;
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < 16; ++j)
+        if (cb + j < rend) dst[j * ld] = acc[j] * scale;
+    }
+  }
 }
 
 __global__ void __launch_bounds__(CELL_THREADS, 2) tc_cell_bf16_kernel(RParams P) {
@@ -1035,18 +1067,7 @@ __global__ void __launch_bounds__(CELL_THREADS, 2) tc_cell_bf16_kernel(RParams P
     const bool run = __all_sync(0xffffffffu, okacc && !*(volatile int*)abort_flag);
     const int c = warp * 32 + lane;
     float* dst = P.R + ((int64_t)e * ne + r0) * P.ldr + c0 + c;
-    for (int cb = 0; cb < B.nh; cb += 16) {
-      float acc[16];
-      __syncwarp();
-      if (run) {
-        tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + cb, acc);
-        tmem_wait_ld();
-      }
-      if (!run || c >= ncv) continue;
-#pragma unroll
-      for (int j = 0; j < 16; ++j)
-        if (r0 + cb + j < ne) dst[(int64_t)(cb + j) * P.ldr] = acc[j];
-    }
+    if (run) store_rows(tmem + ((uint32_t)(warp * 32) << 16), B.nh, ne - r0, dst, P.ldr, c < ncv);
   }
   tc_fence_before();
   __syncthreads();
@@ -1284,18 +1305,7 @@ __global__ void __launch_bounds__(BFA_THREADS, 2) tc_cell_bf16_async_kernel(RPar
     const bool run = __all_sync(0xffffffffu, okacc && !*(volatile int*)abort_flag);
     const int c = warp * 32 + lane;
     float* dst = P.R + ((int64_t)e * ne + r0) * P.ldr + c0 + c;
-    for (int cb = 0; cb < B.nh; cb += 16) {
-      float acc[16];
-      __syncwarp();
-      if (run) {
-        tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + cb, acc);
-        tmem_wait_ld();
-      }
-      if (!run || c >= ncv) continue;
-#pragma unroll
-      for (int j = 0; j < 16; ++j)
-        if (r0 + cb + j < ne) dst[(int64_t)(cb + j) * P.ldr] = acc[j];
-    }
+    if (run) store_rows(tmem + ((uint32_t)(warp * 32) << 16), B.nh, ne - r0, dst, P.ldr, c < ncv);
   }
   tc_fence_before();
   __syncthreads();
@@ -1475,7 +1485,7 @@ __global__ void __launch_bounds__((2 * NPAIR + 2) * 32, 2) tc_cell_bf16_rings_ke
         for (int i = max(0, issued - SM); i < issued; ++i) mbar_wait(fa(i % SM), (i / SM) & 1);
     }
   } else if (warp == WMMA) {
-    if (lane == 0) {
+    if (elect_one()) {
       const uint32_t idesc = NT == 3 ? idesc_bf16(128, nrow) : idesc_f16(128, nrow);
       for (int i = 0; i < nkt; ++i) {
         const int sa = i % SM, sy = i % SY;
@@ -1524,33 +1534,33 @@ __global__ void __launch_bounds__((2 * NPAIR + 2) * 32, 2) tc_cell_bf16_rings_ke
         if (c < ncv) tsc[u] = f16_scale_of(__uint_as_float(P.cmax[c0 + c]));
       }
     }
-    for (int i = pair; i < nkt; i += NPAIR) {
+    // one chunk: 8 rows x 4 columns per lane; KIND 1: a projector chunk (rows of
+    // Z), 2: a Bloch chunk (the cell's rows again, (re, im) -> (im, -re): the swap
+    // in the address and the sign in a select).  The kinds are compiled apart, so
+    // that the 32 loads of a chunk stay together (512 cells, p = 6, 220 columns,
+    // Bloch chunks with a branch around each load: 711 us, now 290).
+    auto chunk = [&](int i, auto kind) {
+      constexpr int KIND = decltype(kind)::value;
       const int s = i % SY;
       float v[8][4];
-      const bool zc = NLC && i >= nk;   // a projector chunk: rows of Z
-      const bool sw = KPT && i >= nk;   // a Bloch chunk: the cell's rows again, columns swapped
 #pragma unroll
       for (int a = 0; a < 8; ++a) {
-        const int l = (sw ? i - nk : i) * BF_KC + q * 8 + a;
-        const int g = zc ? P.nl_zrow[(int64_t)(nl0 + i - nk) * BF_KC + q * 8 + a] : (l < ne ? dm[l] : -1);
-        const float* src = zc ? P.Z + (int64_t)(g < 0 ? 0 : g) * P.ldz + c0
-                              : P.Yin + (int64_t)(g < 0 ? 0 : g) * P.ld_in + c0;
+        const int l = (KIND == 2 ? i - nk : i) * BF_KC + q * 8 + a;
+        const int g = KIND == 1 ? P.nl_zrow[(int64_t)(nl0 + i - nk) * BF_KC + q * 8 + a] : (l < ne ? dm[l] : -1);
+        const float* src = KIND == 1 ? P.Z + (int64_t)(g < 0 ? 0 : g) * P.ldz + c0
+                                     : P.Yin + (int64_t)(g < 0 ? 0 : g) * P.ld_in + c0;
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           const int c = lane + 32 * u;
-          if (KPT && sw) {   // (re, im) -> (im, -re)
-            const float y = (g >= 0 && c < ncv) ? __ldg(src + (c ^ 1)) : 0.f;
-            v[a][u] = (c & 1) ? -y : y;
-          } else {
-            v[a][u] = (g >= 0 && c < ncv) ? __ldg(src + c) : 0.f;
-          }
+          const float y = (g >= 0 && c < ncv) ? __ldg(src + (KIND == 2 ? c ^ 1 : c)) : 0.f;
+          v[a][u] = KIND == 2 && (c & 1) ? -y : y;
         }
       }
       if (i >= SY && !mbar_wait(ey(s), ((i / SY) - 1) & 1)) {
         atomicExch(&g_tc_status, 43);
         *(volatile int*)abort_flag = 1;
       }
-      if (*(volatile int*)abort_flag) break;
+      if (*(volatile int*)abort_flag) return false;
       uint16_t* ys = reinterpret_cast<uint16_t*>(ybase + s * YT);
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
@@ -1569,7 +1579,13 @@ __global__ void __launch_bounds__((2 * NPAIR + 2) * 32, 2) tc_cell_bf16_rings_ke
       }
       fence_proxy_async_smem();
       if (!(withhold && warp == 0 && i == 0)) mbar_arrive(fy(s));
-    }
+      return true;
+    };
+    int i = pair;
+    bool go = true;
+    for (; go && i < nk; i += NPAIR) go = chunk(i, std::integral_constant<int, 0>());
+    if (NLC || KPT)
+      for (; go && i < nkt; i += NPAIR) go = chunk(i, std::integral_constant<int, NLC ? 1 : 2>());
     // epilogue: warps 0-3 (TMEM lane quarter = warp % 4); further gather warps are done
     if (warp < 4) {
     const bool okacc = mbar_wait(accb, 0);
@@ -1584,62 +1600,7 @@ __global__ void __launch_bounds__((2 * NPAIR + 2) * 32, 2) tc_cell_bf16_rings_ke
     const int rend = min(nrow, PROJ ? nrow : ne - r0);   // rows of this CTA's result
     // FP16x2: undo the cell's and the column's scales (exact powers of two)
     const float back = NT == 2 && c < ncv ? P.cinv[e] / f16_scale_of(__uint_as_float(P.cmax[c0 + c])) : 1.f;
-    // The result leaves through the rings, now idle (every MMA has completed):
-    // the four warps write groups of up to `cap` rows into shared memory, row
-    // r at [r][128 columns], and each thread then sends rows r = c (mod 128)
-    // with one bulk copy of ncv columns; the warps wait only until the copies
-    // have read shared memory, not for their writes to reach memory.
-    // Without 16-byte rows (ld or ncv not a multiple of 4) the threads store
-    // their column of each row directly.
-    const int cap = (SM * mstage + SY * YT) / 512 / 16 * 16;
-    if ((P.ldr & 3) == 0 && (ncv & 3) == 0 && cap >= 16) {
-      float* stage = reinterpret_cast<float*>(smem);
-      for (int g0 = 0; g0 < nrow; g0 += cap) {
-        const int g1 = min(nrow, g0 + cap);
-        for (int cb = g0; cb < g1; cb += 16) {
-          float acc[16];
-          __syncwarp();
-          if (run) {
-            tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + cb, acc);
-            tmem_wait_ld();
-#pragma unroll
-            for (int j = 0; j < 16; ++j)
-              if (cb + j < g1) stage[(cb - g0 + j) * 128 + c] = NT == 2 ? acc[j] * back : acc[j];
-          }
-        }
-        fence_proxy_async_smem();
-        named_bar_sync(1, 128);
-        if (run) {
-          // R is read once, by the next launch: when it cannot stay in L2 it
-          // is written as the first to be evicted, ahead of the Y rows and
-          // cell matrices the other CTAs still read
-          const uint64_t pol = l2_evict_first();
-          for (int r = g0 + c; r < min(g1, rend); r += 128) {
-            float* d = rbase + (int64_t)r * P.ldr;
-            const uint32_t sa = smem_u32(stage + (r - g0) * 128);
-            if (P.r_evict) bulk_s2g_hint(d, sa, (uint32_t)ncv * 4, pol);
-            else bulk_s2g(d, sa, (uint32_t)ncv * 4);
-          }
-          bulk_commit();
-          bulk_wait_read0();
-        }
-        named_bar_sync(1, 128);   // the staging rows are free again
-      }
-    } else {
-      float* dst = rbase + c;
-      for (int cb = 0; cb < nrow; cb += 16) {
-        float acc[16];
-        __syncwarp();
-        if (run) {
-          tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + cb, acc);
-          tmem_wait_ld();
-        }
-        if (!run || c >= ncv) continue;
-#pragma unroll
-        for (int j = 0; j < 16; ++j)
-          if (cb + j < rend) dst[(int64_t)(cb + j) * P.ldr] = NT == 2 ? acc[j] * back : acc[j];
-      }
-    }
+    if (run) store_rows(tmem + ((uint32_t)(warp * 32) << 16), nrow, rend, rbase + c, P.ldr, c < ncv, back);
     }
   }
   tc_fence_before();
@@ -1660,7 +1621,6 @@ __global__ void __launch_bounds__((2 * NPAIR + 2) * 32, 2) tc_cell_bf16_rings_ke
 // 256 (t % 2) ..), so the MMAs of tile t + 1 run while the epilogue drains
 // tile t, deeper rings (the whole shared memory) and NPAIR gather pairs.
 constexpr int kTilesPerCta = 3;
-constexpr double kL2Bytes = 129.0 * 1024 * 1024;   // GB300 L2
 template <int NPAIR, int NACC>
 __global__ void __launch_bounds__((2 * NPAIR + 6) * 32, NACC == 1 ? 2 : 1) tc_cell_bf16_tiles_kernel(RParams P) {
   constexpr int NT = 3, WPROD = 2 * NPAIR, WMMA = 2 * NPAIR + 1, WEPI = 2 * NPAIR + 2;
@@ -1832,7 +1792,6 @@ __global__ void __launch_bounds__((2 * NPAIR + 6) * 32, NACC == 1 ? 2 : 1) tc_ce
   } else {
     // epilogue warps: TMEM lane quarter warp % 4, column c of each tile
     const int quarter = warp & 3, c = quarter * 32 + lane;
-    const uint64_t pol = l2_evict_first();   // R is read once, by the next launch
     const int rend = min(nrow, ne - r0);
     for (int t = 0; t < nt; ++t) {
       const int b = t % NACC;
@@ -1845,21 +1804,7 @@ __global__ void __launch_bounds__((2 * NPAIR + 6) * 32, NACC == 1 ? 2 : 1) tc_ce
       const bool run = __all_sync(0xffffffffu, okacc && !*(volatile int*)abort_flag);
       const int c0 = (t0 + t) * 128, ncv = min(128, P.ncol - c0);
       float* dst = P.R + ((int64_t)e * ne + r0) * P.ldr + c0 + c;
-      for (int cb = 0; cb < nrow; cb += 16) {
-        float acc[16];
-        __syncwarp();
-        if (run) {
-          tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + b * 256 + cb, acc);
-          tmem_wait_ld();
-        }
-        if (!run || c >= ncv) continue;
-#pragma unroll
-        for (int j = 0; j < 16; ++j)
-          if (cb + j < rend) {
-            if (P.r_evict) st_global_hint(dst + (int64_t)(cb + j) * P.ldr, acc[j], pol);
-            else dst[(int64_t)(cb + j) * P.ldr] = acc[j];
-          }
-      }
+      if (run) store_rows(tmem + ((uint32_t)(quarter * 32) << 16) + b * 256, nrow, rend, dst, P.ldr, c < ncv);
       tc_fence_before();
       if (!run) break;
       mbar_arrive(tmeb(b));   // TMEM columns of tile t free for tile t + NACC
@@ -2059,18 +2004,7 @@ __global__ void __launch_bounds__(BFW_THREADS, 1) tc_cell_bf16_whole_kernel(RPar
     const int r0 = h * B.nh;
     const int c = wq * 32 + lane;
     float* dst = P.R + ((int64_t)e * ne + r0) * P.ldr + c0 + c;
-    for (int cb = 0; cb < B.nh; cb += 16) {
-      float acc[16];
-      __syncwarp();
-      if (run) {
-        tmem_ld16(tmem + ((uint32_t)(wq * 32) << 16) + h * 256 + cb, acc);
-        tmem_wait_ld();
-      }
-      if (!run || c >= ncv) continue;
-#pragma unroll
-      for (int j = 0; j < 16; ++j)
-        if (r0 + cb + j < ne) dst[(int64_t)(cb + j) * P.ldr] = acc[j];
-    }
+    if (run) store_rows(tmem + ((uint32_t)(wq * 32) << 16) + h * 256, B.nh, ne - r0, dst, P.ldr, c < ncv);
   }
   tc_fence_before();
   __syncthreads();
@@ -2084,8 +2018,7 @@ cudaError_t tc_cell_bf16_launch(const TcCellData& d, const TcApplyArgs& a, cudaS
   const BfPlan B = bf_plan(d.ne);
   if (B.np * B.nh > d.mt * 128) return cudaErrorInvalidValue;   // parts stay inside the packed rows
   RParams P{reinterpret_cast<const float*>(d.bf), a.dofmap, a.Yin, a.R, a.ld_in, a.ncol, d.ne, d.mt,
-            nk16, 1, nullptr, 0, 0, a.ncol, 0};
-  P.r_evict = (double)a.ncells * d.ne * a.ncol * 4 > 2.0 * kL2Bytes;
+            nk16, 1, nullptr, 0, 0, a.ldr, 0};
   if (a.Z) {   // projector chunks: only the ring kernels take them
     if (!d.nl || !tc_cell_bf16_nl_ok(a.gather)) return cudaErrorInvalidValue;
     P.nlA = d.nl;
@@ -2179,8 +2112,7 @@ cudaError_t tc_cell_f16_launch(const TcCellData& d, const TcApplyArgs& a, const 
   const BfPlan B = bf_plan(d.ne);
   if (B.np * B.nh > d.mt * 128) return cudaErrorInvalidValue;
   RParams P{reinterpret_cast<const float*>(d.f16), a.dofmap, a.Yin, a.R, a.ld_in, a.ncol, d.ne, d.mt,
-            nk16, 1, nullptr, 0, 0, a.ncol, 0, cmax, d.f16_inv};
-  P.r_evict = (double)a.ncells * d.ne * a.ncol * 4 > 2.0 * kL2Bytes;
+            nk16, 1, nullptr, 0, 0, a.ldr, 0, cmax, d.f16_inv};
   static std::once_flag attr;
   std::call_once(attr, [] {
     cudaFuncSetAttribute(tc_cell_bf16_rings_kernel<2, false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -2262,12 +2194,12 @@ template <bool NL>
 __device__ __forceinline__ void assemble_quad(const AssembleParams& P, int64_t j, int c,
                                               float* absout = nullptr) {
   const int nc = min(4, P.ncol - c);
-  const bool v4 = P.vec && nc == 4;
+  const bool v4 = nc == 4;
   float sum[4] = {0.f, 0.f, 0.f, 0.f};
   const int k0 = P.node_ptr[j], k1 = P.node_ptr[j + 1];
   for (int k = k0; k < k1; ++k) {
-    const float* src = P.R + (int64_t)P.node_ent[k] * P.ncol + c;
-    if (v4) {
+    const float* src = P.R + (int64_t)P.node_ent[k] * P.ldr + c;
+    if (P.vec) {   // 16-byte rows: a ragged last quad is read whole
       const float4 r = __ldg(reinterpret_cast<const float4*>(src));
       sum[0] += r.x; sum[1] += r.y; sum[2] += r.z; sum[3] += r.w;
     } else {
@@ -2283,7 +2215,7 @@ __device__ __forceinline__ void assemble_quad(const AssembleParams& P, int64_t j
 #pragma unroll
       for (int t = 0; t < 4; ++t) {
         const float* zr = P.Z + (4 * st + t) * P.ncol + c;
-        if (v4) {
+        if (v4 && P.vz) {
           const float4 z = __ldg(reinterpret_cast<const float4*>(zr));
           nl[0] = fmaf(cq[t], z.x, nl[0]);
           nl[1] = fmaf(cq[t], z.y, nl[1]);
@@ -2433,7 +2365,8 @@ cudaError_t tc_assemble_launch(const AssembleParams& P0, cudaStream_t s) {
   if (tot == 0) return cudaSuccess;
   AssembleParams P = P0;
   auto al16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
-  P.vec = (P.ncol & 3) == 0 && al16(P.R) && (!P.Z || al16(P.Z));
+  P.vec = (P.ldr & 3) == 0 && al16(P.R);
+  P.vz = (P.ncol & 3) == 0 && P.Z && al16(P.Z);
   P.vin = (P.ld_in & 3) == 0 && al16(P.Yin);
   P.vprev = P.Yprev && (P.ld_prev & 3) == 0 && al16(P.Yprev);
   P.vout = (P.ld_out & 3) == 0 && al16(P.Yout);
@@ -2451,7 +2384,8 @@ cudaError_t tc_assemble_cmax_launch(const AssembleParams& P0, uint32_t* cmax, cu
   if (e != cudaSuccess || P0.M <= 0) return e;
   AssembleParams P = P0;
   auto al16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
-  P.vec = (P.ncol & 3) == 0 && al16(P.R) && (!P.Z || al16(P.Z));
+  P.vec = (P.ldr & 3) == 0 && al16(P.R);
+  P.vz = (P.ncol & 3) == 0 && P.Z && al16(P.Z);
   P.vin = (P.ld_in & 3) == 0 && al16(P.Yin);
   P.vprev = P.Yprev && (P.ld_prev & 3) == 0 && al16(P.Yprev);
   P.vout = (P.ld_out & 3) == 0 && al16(P.Yout);
@@ -2580,7 +2514,7 @@ __global__ void __launch_bounds__(GR_THREADS, 1) tc_gram_kernel(GramParams P) {
   const uint32_t tmem = *tmem_slot;
 
   if (warp == 4) {
-    if (lane == 0 && nk > 0) {
+    if (elect_one() && nk > 0) {
       const uint32_t idesc = idesc_tf32(128, 128);
       for (int i = 0; i < nk; ++i) {
         const int s = i % S;
@@ -3001,7 +2935,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1) tc_tall_kernel(TallParams P) {
   const int bne = (ncv + 15) / 16 * 16;
 
   if (warp == 4) {
-    if (lane == 0 && nk > 0) {
+    if (elect_one() && nk > 0) {
       const uint32_t idesc = idesc_tf32(128, bne);
       for (int i = 0; i < nk; ++i) {
         const int s = i % S;
@@ -3262,7 +3196,7 @@ __global__ void __launch_bounds__(TW_THREADS, 1) tc_tall_wide_kernel(TallParams 
   const int bne = (ncv + 15) / 16 * 16;
 
   if (warp == TW_PROD) {
-    if (lane == 0 && nk > 0) {
+    if (elect_one() && nk > 0) {
       const uint32_t idesc = idesc_tf32(128, bne);
       for (int i = 0; i < nk; ++i) {
         const int s = i % S;

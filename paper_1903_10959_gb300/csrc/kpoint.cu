@@ -213,7 +213,8 @@ chfsi_status kapply_mixed(chfsi_ctx* ctx, const float* Yin, int64_t ld_in, float
   const HostMesh& m = ctx->mesh;
   const int ncol = 2 * nvec;
   chfsi_status st;
-  if ((st = kgrow(ctx, ctx->kY, (size_t)m.ncells * m.ne * ncol * 4)) != CHFSI_OK) return st;
+  const int64_t ldr = (ncol + 3) & ~3;   // 16-byte rows of R
+  if ((st = kgrow(ctx, ctx->kY, (size_t)m.ncells * m.ne * ldr * 4)) != CHFSI_OK) return st;
   TcCellData view = ctx->tc;
   view.bf = ctx->kbf;
   TcApplyArgs ra{};
@@ -223,6 +224,7 @@ chfsi_status kapply_mixed(chfsi_ctx* ctx, const float* Yin, int64_t ld_in, float
   ra.Yin = Yin;
   ra.ld_in = ld_in;
   ra.R = (float*)ctx->kY.ptr;
+  ra.ldr = ldr;
   ra.split3 = 1;
   ra.gather = 2;
   ra.kG = ctx->kgbf;
@@ -233,6 +235,7 @@ chfsi_status kapply_mixed(chfsi_ctx* ctx, const float* Yin, int64_t ld_in, float
   ap.M = m.ndofs;
   ap.ncol = ncol;
   ap.R = (const float*)ctx->kY.ptr;
+  ap.ldr = ldr;
   ap.Yin = Yin;
   ap.ld_in = ld_in;
   ap.Yout = Yout;

@@ -93,6 +93,7 @@ size_t estimate_bytes(const chfsi_request& r) {
   b += M * n * es;                                                  // X
   b += std::max(M * n * es, M * B * 16);                            // rotation / binary64 pair
   b += M * B * es + M * B * 8;                                      // filter block, binary64 apply
+  if (mixed) b += 2 * M * ((B + 3) / 4 * 4) * es;                   // padded copies of a ragged block
   b += ncells * ne * ((B + 1) & ~(size_t)1) * 8;                    // dense cell blocks R_e (binary64 applications)
   {                                                                 // digit words of the binary64 products
     size_t words = 0, scales = 0;

@@ -53,7 +53,8 @@ struct TcApplyArgs {
   int ncol;
   const float* Yin;
   int64_t ld_in;
-  float* R;                 // ncells * ne * ncol scratch
+  float* R;                 // dense cell blocks, rows of stride ldr (the ring kernel writes whole 16-byte
+  int64_t ldr;              //   quads when ldr is a multiple of 4: ldr >= ncol rounded up)
   int split3;
   int tile = 64;            // columns per CTA of the cell kernel: 64 or 128
   int gather = 2;           // BF16x3: 2 = decoupled matrix / Y rings, 0 = one shared ring, 1 = rows staged by
@@ -126,7 +127,8 @@ struct AssembleParams {
   const int32_t* node_ent;
   int64_t M;
   int ncol;
-  const float* R;             // dense cell blocks, (cell, local node) rows x ncol
+  const float* R;             // dense cell blocks, (cell, local node) rows of stride ldr (>= ncol rounded up
+  int64_t ldr;                //   to a multiple of 4 when it is one)
   const float* Yin;
   int64_t ld_in;
   float* Yout;
@@ -138,7 +140,7 @@ struct AssembleParams {
   const float* dof_c;         // 4 h-scaled coefficients per entry
   const float* Z;             // projected block, (4 nsite) x ncol
   float alpha, beta, shift;
-  int vec, vin, vprev, vout;  // set by the launcher
+  int vec, vz, vin, vprev, vout;  // set by the launcher
 };
 cudaError_t tc_assemble_launch(const AssembleParams& P, cudaStream_t s);
 // The same update with the column maxima of |Y_out| as a by-product: cmax
