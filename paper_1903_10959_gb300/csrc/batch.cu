@@ -329,29 +329,33 @@ __global__ void __launch_bounds__(256) tc_assemble_batched_kernel(const BSys* __
                                                                    const float* __restrict__ coef,
                                                                    int parity) {
   const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (idx >= nq_total) return;
-  int lo = 0, hi = nsys - 1;
-  while (lo < hi) {             // last system with q0 <= idx
-    const int mid = (lo + hi + 1) >> 1;
-    if (sys[mid].q0 <= idx) lo = mid;
-    else hi = mid - 1;
+  // the system of the block's first quad, by one warp (a lane per system, as many
+  // rounds as it takes); the block's other quads are in it or in one soon after
+  __shared__ int first;
+  if (threadIdx.x < 32) {
+    const int64_t i0 = blockIdx.x * (int64_t)blockDim.x;
+    int s = -1;
+    for (int k = threadIdx.x; k < nsys; k += 32)
+      if (sys[k].q0 <= i0) s = k;
+    s = __reduce_max_sync(0xffffffffu, s);
+    if (threadIdx.x == 0) first = s;
   }
+  __syncthreads();
+  if (idx >= nq_total) return;
+  int lo = first;
+  while (lo + 1 < nsys && sys[lo + 1].q0 <= idx) ++lo;
   const BSys& sy = sys[lo];
   const int ncol = sy.ncol;
   const int nq = (ncol + 3) / 4;
   const int64_t li = idx - sy.q0;
-  const int64_t j = li / nq;
+  const int64_t j = li >> 32 ? li / nq : (int64_t)((uint32_t)li / (uint32_t)nq);
   const int c = (int)(li - j * nq) * 4;
   const int nc = min(4, ncol - c);
   const float alpha = coef[3 * lo], beta = coef[3 * lo + 1], shift = coef[3 * lo + 2];
   const float* Yin = sy.Y[parity];
   float* Yout = const_cast<float*>(sy.Y[1 - parity]);
   const int64_t ldi = sy.ldY[parity], ldo = sy.ldY[1 - parity], ldr = sy.ldr;
-  float sum[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int k = sy.node_ptr[j]; k < sy.node_ptr[j + 1]; ++k) {   // R rows are 16-byte aligned
-    const float4 r = __ldg(reinterpret_cast<const float4*>(sy.R + (int64_t)sy.node_ent[k] * ldr + c));
-    sum[0] += r.x; sum[1] += r.y; sum[2] += r.z; sum[3] += r.w;
-  }
+  const int k0 = __ldg(sy.node_ptr + j), n = __ldg(sy.node_ptr + j + 1) - k0;
   const bool vin = nc == 4 && (ldi & 3) == 0 && ((reinterpret_cast<uintptr_t>(Yin) & 15) == 0);
   const bool vout = nc == 4 && (ldo & 3) == 0 && ((reinterpret_cast<uintptr_t>(Yout) & 15) == 0);
   float yin[4] = {0.f, 0.f, 0.f, 0.f}, yp[4] = {0.f, 0.f, 0.f, 0.f};
@@ -368,6 +372,21 @@ __global__ void __launch_bounds__(256) tc_assemble_batched_kernel(const BSys* __
     } else {
       for (int u = 0; u < nc; ++u) yp[u] = Yout[j * ldo + c + u];
     }
+  }
+  float sum[4] = {0.f, 0.f, 0.f, 0.f};         // the rows of R (16-byte aligned) two at a time
+  int k = k0;
+  if (n & 1) {
+    const float4 r = __ldg(reinterpret_cast<const float4*>(sy.R + (int64_t)__ldg(sy.node_ent + k) * ldr + c));
+    sum[0] += r.x; sum[1] += r.y; sum[2] += r.z; sum[3] += r.w;
+    ++k;
+  }
+#pragma unroll 1
+  for (; k < k0 + n; k += 2) {
+    const int e0 = __ldg(sy.node_ent + k), e1 = __ldg(sy.node_ent + k + 1);
+    const float4 r = __ldg(reinterpret_cast<const float4*>(sy.R + (int64_t)e0 * ldr + c));
+    const float4 t = __ldg(reinterpret_cast<const float4*>(sy.R + (int64_t)e1 * ldr + c));
+    sum[0] += r.x; sum[1] += r.y; sum[2] += r.z; sum[3] += r.w;
+    sum[0] += t.x; sum[1] += t.y; sum[2] += t.z; sum[3] += t.w;
   }
   float out[4];
 #pragma unroll
@@ -393,7 +412,8 @@ struct chfsi_batch {
   // device descriptors and buffers
   BSys* d_sys = nullptr;
   std::vector<BSys> h_sys;
-  std::vector<DevBuf> T1, R;
+  std::vector<int64_t> ldx;             // leading dimensions of the described blocks
+  std::vector<DevBuf> T0, T1, R;         // T0: padded copy of a ragged block
   float* d_coef = nullptr;      // degree x nsys x 3
   float* h_coef = nullptr;      // pinned
   int coef_cap = 0;
@@ -452,6 +472,7 @@ cudaError_t batch_describe(chfsi_batch* b, float* const* X, const int64_t* ldx, 
                            int bn, int mode) {
   const int n = (int)b->ctx.size();
   b->h_sys.assign(n, BSys{});
+  b->ldx.assign(ldx, ldx + n);
   int64_t item = 0, q = 0;
   for (int i = 0; i < n; ++i) {
     chfsi_ctx* c = b->ctx[i];
@@ -465,6 +486,16 @@ cudaError_t batch_describe(chfsi_batch* b, float* const* X, const int64_t* ldx, 
     sy.dofmap = c->d_dofmap;
     sy.Y[0] = X[i];
     sy.ldY[0] = ldx[i];
+    sy.ncol = ncol[i];
+    // rows off 16 bytes or a ragged width: the steps run on a copy padded with
+    // zero columns (batch_enqueue), so that the assembly takes 16-byte accesses
+    // (16 uneven systems, p = 5: 492 -> 459 us a step)
+    if ((ncol[i] & 3) || (ldx[i] & 3) || (reinterpret_cast<uintptr_t>(X[i]) & 15)) {
+      if ((e = ensure_dbuf(b->T0[i], (size_t)m.ndofs * ld4 * 4 + 16)) != cudaSuccess) return e;
+      sy.Y[0] = (const float*)b->T0[i].ptr;
+      sy.ldY[0] = ld4;
+      sy.ncol = (int)ld4;
+    }
     sy.Y[1] = (const float*)b->T1[i].ptr;
     sy.ldY[1] = ld4;
     sy.R = (float*)b->R[i].ptr;
@@ -473,7 +504,6 @@ cudaError_t batch_describe(chfsi_batch* b, float* const* X, const int64_t* ldx, 
     sy.node_ent = c->d_node_ent;
     sy.ncells = m.ncells;
     sy.M = m.ndofs;
-    sy.ncol = ncol[i];
     sy.tiles = mode == kBatchBf16x3 ? (ncol[i] + 127) / 128 * tc_bf16_parts(b->ne) : (ncol[i] + bn - 1) / bn;
     sy.item0 = item;
     sy.q0 = q;
@@ -493,6 +523,11 @@ cudaError_t batch_enqueue(chfsi_batch* b, float* const* X, const int* ncol, int 
   cudaError_t e = cudaMemcpyAsync(b->d_coef, b->h_coef, (size_t)degree * n * 3 * sizeof(float),
                                   cudaMemcpyHostToDevice, b->stream);
   if (e != cudaSuccess) return e;
+  auto padded = [&](int i) { return b->h_sys[i].Y[0] != X[i]; };
+  for (int i = 0; i < n; ++i)
+    if (padded(i) && (e = launch_copy_pad(X[i], b->ldx[i], ncol[i], (float*)b->T0[i].ptr, b->h_sys[i].ldY[0],
+                                          b->ctx[i]->mesh.ndofs, b->stream)) != cudaSuccess)
+      return e;
   for (int k = 1; k <= degree; ++k) {
     const int parity = (k - 1) & 1;
     if (split3 == kBatchBf16x3)
@@ -508,14 +543,16 @@ cudaError_t batch_enqueue(chfsi_batch* b, float* const* X, const int* ncol, int 
         b->d_sys, n, b->nq, b->d_coef + (size_t)(k - 1) * n * 3, parity);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  if (degree & 1)   // Y_m sits in the scratch buffer: copy it back into X
-    for (int i = 0; i < n; ++i) {
-      const HostMesh& m = b->ctx[i]->mesh;
-      e = cudaMemcpy2DAsync(X[i], b->h_sys[i].ldY[0] * 4, b->T1[i].ptr,
-                            (size_t)b->h_sys[i].ldY[1] * 4, (size_t)ncol[i] * 4, m.ndofs,
+  for (int i = 0; i < n; ++i) {
+    const HostMesh& m = b->ctx[i]->mesh;
+    const BSys& sy = b->h_sys[i];
+    if (padded(i))
+      e = launch_copy_pad(sy.Y[degree & 1], sy.ldY[degree & 1], ncol[i], X[i], b->ldx[i], m.ndofs, b->stream, false);
+    else if (degree & 1)   // Y_m sits in the scratch buffer: copy it back into X
+      e = cudaMemcpy2DAsync(X[i], sy.ldY[0] * 4, b->T1[i].ptr, (size_t)sy.ldY[1] * 4, (size_t)ncol[i] * 4, m.ndofs,
                             cudaMemcpyDeviceToDevice, b->stream);
-      if (e != cudaSuccess) return e;
-    }
+    if (e != cudaSuccess) return e;
+  }
   return cudaSuccess;
 }
 
@@ -566,7 +603,7 @@ chfsi_status batch_prepare(chfsi_batch* b, float* const* X, const int64_t* ldx, 
   const int n = (int)b->ctx.size();
   for (int i = 0; i < n; ++i) {
     chfsi_ctx* c = b->ctx[i];
-    if (!c->tc.hi) {
+    if (mode != kBatchBf16x3 && !c->tc.hi) {
       cudaError_t pe = tc_pack_from_device(c->tc, c->d_Ht, c->stream, &c->dev_bytes);
       if (pe != cudaSuccess) return bfail(b, CHFSI_ERR_OOM, "tensor-core cell data");
       cudaStreamSynchronize(c->stream);
@@ -636,6 +673,7 @@ chfsi_status chfsi_batch_create(int n, chfsi_ctx* const* ctxs, void* stream, chf
     delete b;
     return CHFSI_ERR_ARG;
   }
+  b->T0.resize(n);
   b->T1.resize(n);
   b->R.resize(n);
   if (!b->stream) {
@@ -664,6 +702,7 @@ chfsi_status chfsi_batch_destroy(chfsi_batch* b) {
   if (!b) return CHFSI_ERR_ARG;
   cudaStreamSynchronize(b->stream);
   batch_free_graph(b);
+  for (auto& d : b->T0) cudaFree(d.ptr);
   for (auto& d : b->T1) cudaFree(d.ptr);
   for (auto& d : b->R) cudaFree(d.ptr);
   if (b->d_sys) cudaFree(b->d_sys);

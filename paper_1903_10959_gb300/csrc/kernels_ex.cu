@@ -763,25 +763,19 @@ __global__ void __launch_bounds__(256) ex_h_scale_kernel(const double* __restric
 }
 
 // ---------------------------------------------------------------- assembly, reduction
-// Block (32, 8): 64 columns (a pair per lane) of 8 unknowns.  Sums the cell
-// rows holding the unknown in ascending cell order, adds the projector term,
-// applies the three-term update.  Y_out may alias Y_prev, not Y_in.
+// Each thread: one unknown, two columns (pairs of a row in consecutive threads).
+// Sums the cell rows holding the unknown in ascending cell order, adds the
+// projector term, applies the three-term update.  Y_out may alias Y_prev, not Y_in.
 __global__ void __launch_bounds__(256) ex_assemble_kernel(const __grid_constant__ ExAssembleArgs P, int vio) {
-  const int64_t j = (int64_t)blockIdx.x * 8 + threadIdx.y;
-  const int c = (blockIdx.y * 32 + threadIdx.x) * 2;
+  const uint32_t np = (uint32_t)(P.ncol + 1) / 2;
+  const int64_t idx = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  const int64_t j = idx >> 32 ? idx / np : (int64_t)((uint32_t)idx / np);
+  const int c = (int)(idx - j * np) * 2;
   if (j >= P.M || c >= P.ncol) return;
   const bool two = c + 1 < P.ncol;
-  double s0 = 0.0, s1 = 0.0;
-  const int k1 = P.node_ptr[j + 1];
-  for (int k = P.node_ptr[j]; k < k1; ++k) {   // rows of R are padded to an even length
-    const double2 r = __ldg(reinterpret_cast<const double2*>(P.R + (int64_t)P.node_ent[k] * P.ldr + c));
-    s0 += r.x;
-    s1 += r.y;
-  }
-  if (P.NL) {
-    s0 += P.NL[j * P.ld_nl + c];
-    if (two) s1 += P.NL[j * P.ld_nl + c + 1];
-  }
+  const int k0 = __ldg(P.node_ptr + j), n = __ldg(P.node_ptr + j + 1) - k0;
+  // the rows of Y first, then the rows of R two at a time (an unknown lies in 1,
+  // 2, 4 or 8 cells)
   double y0 = 0.0, y1 = 0.0, p0 = 0.0, p1 = 0.0;
   double* out = P.Yout + j * P.ld_out + c;
   if (vio && two) {
@@ -805,7 +799,36 @@ __global__ void __launch_bounds__(256) ex_assemble_kernel(const __grid_constant_
       if (two) p1 = P.Yprev[j * P.ld_prev + c + 1];
     }
   }
-  double o0 = P.alpha * (s0 - P.shift * y0), o1 = P.alpha * (s1 - P.shift * y1);
+  double s0 = 0.0, s1 = 0.0;                   // rows of R are padded to an even length
+  int k = k0;
+  if (n & 1) {
+    const double2 r = __ldg(reinterpret_cast<const double2*>(P.R + (int64_t)__ldg(P.node_ent + k) * P.ldr + c));
+    s0 = r.x;
+    s1 = r.y;
+    ++k;
+  }
+#pragma unroll 1
+  for (; k < k0 + n; k += 2) {
+    const int e0 = __ldg(P.node_ent + k), e1 = __ldg(P.node_ent + k + 1);
+    const double2 r = __ldg(reinterpret_cast<const double2*>(P.R + (int64_t)e0 * P.ldr + c));
+    const double2 t = __ldg(reinterpret_cast<const double2*>(P.R + (int64_t)e1 * P.ldr + c));
+    s0 += r.x;
+    s1 += r.y;
+    s0 += t.x;
+    s1 += t.y;
+  }
+  if (P.NL) {
+    s0 += P.NL[j * P.ld_nl + c];
+    if (two) s1 += P.NL[j * P.ld_nl + c + 1];
+  }
+  // alpha (s - shift y) + beta y_prev in three operations: the kernel moves 37
+  // bytes per value and a binary64 operation per value costs as much time as 11
+  double o0 = P.alpha * s0, o1 = P.alpha * s1;
+  if (P.shift != 0.0) {
+    const double as = -P.alpha * P.shift;
+    o0 = fma(as, y0, o0);
+    o1 = fma(as, y1, o1);
+  }
   if (P.Yprev) {
     o0 = fma(P.beta, p0, o0);
     o1 = fma(P.beta, p1, o1);
@@ -986,7 +1009,7 @@ cudaError_t ex_assemble_launch(const ExAssembleArgs& a, cudaStream_t s) {
   auto al = [](const void* p, int64_t ld) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0 && (ld & 1) == 0; };
   const int vio = al(a.Yin, a.ld_in) && al(a.Yout, a.ld_out) && (!a.Yprev || al(a.Yprev, a.ld_prev));
   note_launch();
-  ex_assemble_kernel<<<dim3((unsigned)((a.M + 7) / 8), (a.ncol + 63) / 64), dim3(32, 8), 0, s>>>(a, vio);
+  ex_assemble_kernel<<<(unsigned)((a.M * ((a.ncol + 1) / 2) + 255) / 256), 256, 0, s>>>(a, vio);
   return cudaGetLastError();
 }
 
