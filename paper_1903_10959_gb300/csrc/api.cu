@@ -703,15 +703,25 @@ chfsi_status tall64_impl(chfsi_ctx* ctx, const double* X, int64_t ldx, int n1, i
 }
 
 // X <- X U (U n x n column-major; trans / upper flags as launch_tallgemm_fp64).
+// In binary64 in place: ex_tall has copied a slice's rows before it writes them.
 chfsi_status rotate_impl(chfsi_ctx* ctx, chfsi_precision prec, void* X, int64_t ldx, int n,
                          const double* U, int upper, int trans) {
   const HostMesh& m = ctx->mesh;
   const size_t es = esize(prec);
   chfsi_status st;
+  if (prec == CHFSI_FP64) {
+    const std::string err = ctx->err;
+    if (grow(ctx, ctx->work, ex_tall_work_bytes(m.ndofs, n, n)) == CHFSI_OK) {
+      ctx->ex_used = true;
+      CK(ex_tall((const double*)X, ldx, U, n, m.ndofs, n, n, (double*)X, ldx, upper, trans, ctx->work.ptr, ctx->stream));
+      return CHFSI_OK;
+    }
+    ctx->err = err;
+  }
   if ((st = grow(ctx, ctx->rot, (size_t)m.ndofs * n * es)) != CHFSI_OK) return st;
   if (prec == CHFSI_FP64) {
-    if ((st = tall64_impl(ctx, (const double*)X, ldx, n, n, U, n, (double*)ctx->rot.ptr, n, upper, trans)) != CHFSI_OK)
-      return st;
+    CK(launch_tallgemm_fp64((const double*)X, ldx, U, n, m.ndofs, n, n, (double*)ctx->rot.ptr, n, upper, trans,
+                            ctx->stream));
   } else {
     if ((st = grow(ctx, ctx->work, tc_tallgemm_work_bytes(n, n))) != CHFSI_OK) return st;
     CK(tc_tallgemm_mixed((const float*)X, ldx, U, n, m.ndofs, n, n, (float*)ctx->rot.ptr, n, upper,
