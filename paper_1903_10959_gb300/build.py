@@ -21,7 +21,7 @@ LIB = os.path.join(HERE, "libchfsi.so")
 CUDA_HOME = os.environ.get("CUDA_HOME", "/usr/local/cuda")
 NVCC = os.path.join(CUDA_HOME, "bin", "nvcc")
 GENCODE = ["-gencode", "arch=compute_103a,code=sm_103a"]
-CUDA_SOURCES = ["kernels_fp64.cu", "kernels_tc.cu", "kernels_mf.cu", "kernels_ex.cu", "cellmat.cu", "api.cu", "batch.cu", "server.cu",
+CUDA_SOURCES = ["kernels_fp64.cu", "kernels_tc.cu", "kernels_mf.cu", "kernels_ex.cu", "kernels_chol.cu", "cellmat.cu", "api.cu", "batch.cu", "server.cu",
                 "density.cu", "scf.cu", "kpoint.cu"]
 CXX_SOURCES = ["mesh.cpp", "partition.cpp"]
 

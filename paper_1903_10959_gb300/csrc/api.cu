@@ -744,44 +744,21 @@ chfsi_status ensure_solver(chfsi_ctx* ctx) {
 chfsi_status cholgs_impl(chfsi_ctx* ctx, void* X, int64_t ldx, int n, chfsi_precision prec) {
   chfsi_status st;
   if (n == 0) return CHFSI_OK;
-  if ((st = ensure_solver(ctx)) != CHFSI_OK) return st;
   if ((st = grow(ctx, ctx->Ssq, (size_t)n * n * 8 + 64)) != CHFSI_OK) return st;
   double* S = (double*)ctx->Ssq.ptr;
   int* dinfo = (int*)((char*)ctx->Ssq.ptr + (size_t)n * n * 8);
   // 1. S = X^T X (lower triangle)
   if ((st = gram_impl(ctx, prec, X, ldx, X, ldx, n, n, S, n, 1)) != CHFSI_OK) return st;
-  // 2. S = L L^T
-  int lw = 0;
-  CS(cusolverDnDpotrf_bufferSize(ctx->sol, CUBLAS_FILL_MODE_LOWER, n, S, n, &lw));
-  size_t dws = 0, hws = 0;
-  CS(cusolverDnXtrtri_bufferSize(ctx->sol, CUBLAS_FILL_MODE_LOWER, CUBLAS_DIAG_NON_UNIT, n,
-                                 CUDA_R_64F, S, n, &dws, &hws));
-  size_t need = std::max<size_t>((size_t)lw * 8, dws) + 256;
-  if ((st = grow(ctx, ctx->work, need)) != CHFSI_OK) return st;
-  CS(cusolverDnDpotrf(ctx->sol, CUBLAS_FILL_MODE_LOWER, n, S, n, (double*)ctx->work.ptr, lw, dinfo));
+  // 2. S = L L^T and L^{-1} (lower triangle; the strict upper triangle zero)
+  if ((st = grow(ctx, ctx->tinv, (size_t)n * n * 8)) != CHFSI_OK) return st;
+  double* Linv = (double*)ctx->tinv.ptr;
+  CK(launch_chol_inverse(S, n, Linv, dinfo, ctx->stream));
   int info = 0;
   CK(cudaMemcpyAsync(&info, dinfo, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
   if (info != 0)
     return fail(ctx, CHFSI_ERR_NOT_SPD, "CholGS: potrf info = " + std::to_string(info));
-  // 3. L^{-1} (lower triangle; the strict upper triangle zero): the
-  // warp-per-column forward substitution of kernels_fp64.cu (L_ii > 0 after
-  // potrf), cuSOLVER's trtri in place beyond its shared-memory limit
-  double* Linv = S;
-  if (trinv_lower_supported(n)) {
-    if ((st = grow(ctx, ctx->tinv, (size_t)n * n * 8)) != CHFSI_OK) return st;
-    Linv = (double*)ctx->tinv.ptr;
-    CK(cudaMemsetAsync(Linv, 0, (size_t)n * n * 8, ctx->stream));
-    CK(launch_trinv_lower_fp64(S, n, n, Linv, n, ctx->stream));
-  } else {
-    std::vector<char> hwork(hws + 16);
-    CS(cusolverDnXtrtri(ctx->sol, CUBLAS_FILL_MODE_LOWER, CUBLAS_DIAG_NON_UNIT, n, CUDA_R_64F, S, n,
-                        ctx->work.ptr, dws, hwork.data(), hws, dinfo));
-    CK(cudaMemcpyAsync(&info, dinfo, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
-    if (info != 0) return fail(ctx, CHFSI_ERR_NOT_SPD, "CholGS: trtri info = " + std::to_string(info));
-  }
-  // 4. X <- X L^{-T}: U(k, j) = Linv(j, k), nonzero for k <= j
+  // 3. X <- X L^{-T}: U(k, j) = Linv(j, k), nonzero for k <= j
   return rotate_impl(ctx, prec, X, ldx, n, Linv, 1, 1);
 }
 
