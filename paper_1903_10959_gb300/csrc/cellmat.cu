@@ -16,8 +16,11 @@
 //                     mass of a uniform mesh), the same in every cell, and goes
 //                     into the 1-D factors and the shared kinetic matrix: one
 //                     addition per entry is left.
-// Both are bound by the binary64 ALU rate (2 FMA per clock and SM).  12^3 cells,
-// p = 6, 108 wells: 0.43 and 2.0 ms (on 16 host threads, with the upload: 185 ms).
+// Both are bound by the binary64 ALU rate (2 FMA per clock and SM; 1.06 ms for the
+// matrices below).  12^3 cells, p = 6, 108 wells: 0.25 and 1.25 ms (0.43 and 2.0
+// with a barrier per well, one z pair per round and the loads of K one by one; on
+// 16 host threads, with the upload: 185).  The digit words take no binary64
+// operation beyond the contractions.
 #include <algorithm>
 #include <mutex>
 
@@ -28,18 +31,17 @@ namespace chfsi {
 
 namespace {
 
-constexpr int PW = 32;       // wells per batch of 1-D factors
 constexpr int PT = 256;
 
 // wells: n x 5 (centre, depth, 1 / (2 w^2)), images as explicit centres; a well
 // whose largest value in the cell is below e^-41.5 (1e-18) of its depth is
 // left out.  Sums in the order of the list.
-__global__ void __launch_bounds__(PT) potential_kernel(CellMatArgs P) {
+__global__ void __launch_bounds__(PT) potential_kernel(CellMatArgs P, int pw) {
   extern __shared__ double sm[];
   const int q = P.q, q2 = q * q, nq = q2 * q;
-  double* g = sm;                                     // PW x 3 x q
-  double* yz = g + PW * 3 * q;                        // q^2: D g_y g_z of one well
-  double* v = yz + q2;                                // q^3
+  double* g = sm;                                     // pw x 3 x q
+  double* yz = g + pw * 3 * q;                        // pw x q^2: D g_y g_z
+  double* v = yz + pw * q2;                           // q^3
   __shared__ int list[PT];
   __shared__ int cnt[PT / 32];
   const int64_t e = blockIdx.x;
@@ -77,8 +79,8 @@ __global__ void __launch_bounds__(PT) potential_kernel(CellMatArgs P) {
     }
     if (in) list[base + __popc(b & ((1u << lane) - 1))] = w0 + tid;
     __syncthreads();
-    for (int l0 = 0; l0 < total; l0 += PW) {
-      const int nl = min(PW, total - l0);
+    for (int l0 = 0; l0 < total; l0 += pw) {
+      const int nl = min(pw, total - l0);
       for (int t = tid; t < nl * 3 * q; t += PT) {
         const int k = t / (3 * q), a = t / q % 3, i = t % q;
         const double* w = P.wells + 5 * (int64_t)list[l0 + k];
@@ -86,14 +88,19 @@ __global__ void __launch_bounds__(PT) potential_kernel(CellMatArgs P) {
         g[t] = exp(-d * d * w[4]);
       }
       __syncthreads();
-      for (int k = 0; k < nl; ++k) {
+      for (int t = tid; t < nl * q2; t += PT) {
+        const int k = t / q2, i = t % q2;
         const double* gk = g + k * 3 * q;
-        const double dep = P.wells[5 * (int64_t)list[l0 + k] + 3];
-        for (int t = tid; t < q2; t += PT) yz[t] = dep * gk[q + t % q] * gk[2 * q + t / q];
-        __syncthreads();
-        for (int t = tid; t < nq; t += PT) v[t] = fma(-yz[t / q], gk[t % q], v[t]);
-        __syncthreads();
+        yz[t] = P.wells[5 * (int64_t)list[l0 + k] + 3] * gk[q + i % q] * gk[2 * q + i / q];
       }
+      __syncthreads();
+      for (int t = tid; t < nq; t += PT) {
+        const int i = t / q, a = t % q;
+        double s = v[t];
+        for (int k = 0; k < nl; ++k) s = fma(-yz[k * q2 + i], g[k * 3 * q + a], s);
+        v[t] = s;
+      }
+      __syncthreads();
     }
   }
   for (int t = tid; t < nq; t += PT) {
@@ -107,100 +114,144 @@ __device__ __forceinline__ int pair_index(int i, int l) {   // unordered pairs, 
   const int a = max(i, l), b = min(i, l);
   return a * (a + 1) / 2 + b;
 }
+// The first index of an unordered pair.
+__device__ __forceinline__ int pair_first(int u) {
+  int i = 0;
+  while ((i + 1) * (i + 2) / 2 <= u) ++i;
+  return i;
+}
+// fixed_of for a term that may exceed the scale (s < 0) in a sum that does not:
+// modulo 2^64.
+__device__ __forceinline__ uint64_t fixed_term(double v, int s) {
+  return s >= 0 ? (uint64_t)fixed_of(v, s) : s > -64 ? (uint64_t)fixed_of(v, 0) << -s : 0;
+}
+// Threads per cell: shared memory admits one block per SM for p >= 7, two for p =
+// 5, 6 (p = 7: 1.35 ms with 512 threads, 1.16 with 1,024; p = 6: 1.53 and 1.89).
+__host__ __device__ constexpr int cell_threads(int n1) { return n1 >= 8 ? 1024 : n1 >= 6 ? 512 : 256; }
+constexpr int ZB = 2;                     // z pairs per round
 
 // WORDS: digit words instead of the binary64 entries: entry (l, k) under the
-// scale of row l at W[(e NE + k) ldw + l].
+// scale of row l at W[(e NE + k) ldw + l], the sum of the kinetic part (twice the
+// precision of binary64) and the potential part in integers.
 template <int N1, bool WORDS>
-__global__ void __launch_bounds__(256) cell_matrix_kernel(CellMatArgs P, int jb, const int16_t* __restrict__ hexp,
+__global__ void __launch_bounds__(cell_threads(N1)) cell_matrix_kernel(CellMatArgs P, int jb, const int16_t* __restrict__ hexp,
                                                           uint64_t* __restrict__ W, int ldw) {
-  constexpr int NU = N1 * (N1 + 1) / 2, NN = N1 * N1, NE = NN * N1;
+  constexpr int NU = N1 * (N1 + 1) / 2, NN = N1 * N1, NE = NN * N1, N4 = NN * NN;
+  constexpr int NT = cell_threads(N1);
   extern __shared__ double sm[];
   const int q = P.q, q2 = q * q, nq = q2 * q;
   double* bb = sm;                        // 3 x q x NU: s_i B_ai B_al s_l per axis
   double* t1 = bb + 3 * q * NU;           // q^2 x NU
-  double* slab = t1 + q2 * NU;            // jb x NU
-  double* t2 = slab + jb * NU;            // q x jb x NU; first w V jac, q^3
+  double* slab = t1 + q2 * NU;            // ZB x jb x NU
+  double* t2 = slab + ZB * jb * NU;       // q x jb x NU; first w V jac, q^3
+  uint16_t* idx = reinterpret_cast<uint16_t*>(t2 + max(q * jb * NU, nq));   // N4: (row, column) -> (jm, il)
   __shared__ bool live[NE];               // nodes that are not eliminated
   const int64_t e = blockIdx.x;
-  for (int t = threadIdx.x; t < 3 * q * NU; t += 256) {
+  for (int t = threadIdx.x; t < 3 * q * NU; t += NT) {
     const int ax = t / (q * NU), a = t / NU % q, u = t % NU;
-    int i = 0;
-    while ((i + 1) * (i + 2) / 2 <= u) ++i;
-    const int l = u - i * (i + 1) / 2;
+    const int i = pair_first(u), l = u - i * (i + 1) / 2;
     bb[t] = P.B[a * N1 + i] * P.B[a * N1 + l] * (P.s1[ax * N1 + i] * P.s1[ax * N1 + l]);
   }
   const double* by = bb + q * NU;
   const double* bz = by + q * NU;
-  for (int t = threadIdx.x; t < nq; t += 256) t2[t] = P.wv[e * nq + t];
-  for (int l = threadIdx.x; l < NE; l += 256) live[l] = P.dofmap[e * NE + l] >= 0;
-  __syncthreads();
-  for (int t = threadIdx.x; t < q2 * NU; t += 256) {      // x: (c b a) -> (c b il)
+  for (int t = threadIdx.x; t < nq; t += NT) t2[t] = P.wv[e * nq + t];
+  int dead = 0;
+  for (int l = threadIdx.x; l < NE; l += NT) {
+    live[l] = P.dofmap[e * NE + l] >= 0;
+    dead |= !live[l];
+  }
+  for (int t = threadIdx.x; t < N4; t += NT) {
+    const int r = t / NN, c = t % NN;
+    idx[t] = (uint16_t)(pair_index(r / N1, c / N1) * NU + pair_index(r % N1, c % N1));
+  }
+  dead = __syncthreads_or(dead);
+  for (int t = threadIdx.x; t < q2 * NU; t += NT) {      // x: (c b a) -> (c b il)
     const int u = t % NU, cb = t / NU;
     double s = 0.0;
     for (int a = 0; a < q; ++a) s = fma(bb[a * NU + u], t2[cb * q + a], s);
     t1[t] = s;
   }
   for (int j0 = 0; j0 < NU; j0 += jb) {                   // y pairs, jb at a time
-    const int nj = min(jb, NU - j0);
+    const int nj = min(jb, NU - j0), nt = nj * NU;
     __syncthreads();
-    for (int t = threadIdx.x; t < q * nj * NU; t += 256) {   // y: (c b il) -> (c jm il)
-      const int u = t % NU, w = t / NU % nj, c = t / (nj * NU);
+    for (int t = threadIdx.x; t < q * nt; t += NT) {     // y: (c b il) -> (c jm il)
+      const int u = t % NU, w = t / NU % nj, c = t / nt;
       double s = 0.0;
       for (int b = 0; b < q; ++b) s = fma(by[b * NU + j0 + w], t1[(c * q + b) * NU + u], s);
       t2[t] = s;
     }
-    for (int k = 0; k < N1; ++k)
-      for (int nk = 0; nk <= k; ++nk) {
-        const int z = k * (k + 1) / 2 + nk;
-        __syncthreads();
-        for (int t = threadIdx.x; t < nj * NU; t += 256) {
-          double s = 0.0;
-          for (int c = 0; c < q; ++c) s = fma(bz[c * NU + z], t2[c * nj * NU + t], s);
-          slab[t] = s;
-        }
-        __syncthreads();
-        // entries (i j k), (l m nk), and for nk < k the transposed block
-        for (int side = 0; side < (nk < k ? 2 : 1); ++side) {
-          const int kr = side ? nk : k, kc = side ? k : nk;
-          for (int t = threadIdx.x; t < NN * NN; t += 256) {
-            const int r = t / NN, c = t % NN;
-            const int jm = pair_index(r / N1, c / N1) - j0;
-            if (jm < 0 || jm >= nj) continue;
-            const int row = r + NN * kr, col = c + NN * kc;
-            const double x = slab[jm * NU + pair_index(r % N1, c % N1)];
-            const bool on = live[row] && live[col];
-            const double kin = P.K[(int64_t)row * NE + col];
-            if (!WORDS) {
-              P.Ht[(e * NE + row) * NE + col] = on ? kin + x : 0.0;
-            } else {   // kin + x exactly, plus the kinetic remainder (the matrix is symmetric: col is the word's row)
-              const double h = kin + x, t = h - kin;
-              const double lo = ((kin - (h - t)) + (x - t)) + P.K[(int64_t)(NE + row) * NE + col];
-              const int ex = hexp[e * NE + col];
-              W[(e * NE + row) * ldw + col] =
-                  on ? fixed_of(h, ex - expo(h)) + fixed_of(lo, ex - expo(lo)) + kZeroWord : kZeroWord;
+    for (int z0 = 0; z0 < NU; z0 += ZB) {                 // z: -> ZB slabs (jm il)
+      const int nz = min(ZB, NU - z0);
+      __syncthreads();
+      for (int t = threadIdx.x; t < nz * nt; t += NT) {
+        const int zz = t / nt, w = t - zz * nt;
+        double s = 0.0;
+        for (int c = 0; c < q; ++c) s = fma(bz[c * NU + z0 + zz], t2[c * nt + w], s);
+        slab[t] = s;
+      }
+      __syncthreads();
+      // pair z = (k, nk): entries (i j k), (l m nk), and for nk < k the
+      // transposed block
+      for (int zz = 0; zz < nz; ++zz) {
+        const int kf = pair_first(z0 + zz), ks = z0 + zz - kf * (kf + 1) / 2;
+        const double* x = slab + zz * nt;
+        for (int side = 0; side < (ks < kf ? 2 : 1); ++side) {
+          const int kr = side ? ks : kf, kc = side ? kf : ks;
+          // U entries per thread at a time: the loads of K come from L2
+          constexpr int U = (N4 + NT - 1) / NT < 5 ? (N4 + NT - 1) / NT : 5;
+          for (int t0 = threadIdx.x; t0 < N4; t0 += NT * U) {
+            int id[U];
+            double k0[U], k1[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              const int t = t0 + NT * u, r = t / NN, c = t % NN;
+              id[u] = t < N4 ? (int)idx[t] - j0 * NU : -1;
+              if (id[u] >= nt) id[u] = -1;
+              if (id[u] >= 0) {
+                const int64_t o = (int64_t)(r + NN * kr) * NE + c + NN * kc;
+                k0[u] = __ldg(P.K + o);
+                if (WORDS) k1[u] = __ldg(P.K + NE * NE + o);
+              }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              if (id[u] < 0) continue;
+              const int t = t0 + NT * u, r = t / NN, c = t % NN;
+              const int row = r + NN * kr, col = c + NN * kc;
+              const bool on = !dead || (live[row] && live[col]);
+              if (!WORDS) {
+                P.Ht[(e * NE + row) * NE + col] = on ? k0[u] + x[id[u]] : 0.0;
+              } else {   // the matrix is symmetric: col is the word's row
+                const double v = x[id[u]];
+                const int ex = hexp[e * NE + col];
+                W[(e * NE + row) * ldw + col] = on ? fixed_term(k0[u], ex - expo(k0[u])) + fixed_term(k1[u], ex - expo(k1[u])) +
+                                                         fixed_term(v, ex - expo(v)) + kZeroWord
+                                                   : kZeroWord;
+              }
             }
           }
         }
       }
+    }
   }
 }
 
 template <int N1, bool WORDS>
 cudaError_t launch_n(const CellMatArgs& P, const int16_t* hexp, uint64_t* W, int ldw, cudaStream_t s) {
-  constexpr int NU = N1 * (N1 + 1) / 2;
+  constexpr int NU = N1 * (N1 + 1) / 2, NN = N1 * N1;
   const int q = P.q;
   auto bytes = [q](int jb) {
-    return sizeof(double) * ((size_t)3 * q * NU + q * q * NU + jb * NU +
-                             std::max((size_t)q * jb * NU, (size_t)q * q * q));
+    return sizeof(double) * ((size_t)3 * q * NU + q * q * NU + ZB * jb * NU + std::max((size_t)q * jb * NU, (size_t)q * q * q)) +
+           sizeof(uint16_t) * NN * NN;
   };
-  int jb = NU;                       // all y pairs at once but for the largest rules (p = 8, q > 10)
+  int jb = NU;                       // all y pairs at once unless they don't fit (p = 8 and the finest rules)
   while (bytes(jb) > 226 * 1024) jb = (jb + 1) / 2;
   static std::once_flag attr;
   std::call_once(attr, [] {
     cudaFuncSetAttribute(cell_matrix_kernel<N1, WORDS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
   });
   note_launch();
-  cell_matrix_kernel<N1, WORDS><<<(unsigned)P.ncells, 256, bytes(jb), s>>>(P, jb, hexp, W, ldw);
+  cell_matrix_kernel<N1, WORDS><<<(unsigned)P.ncells, cell_threads(N1), bytes(jb), s>>>(P, jb, hexp, W, ldw);
   return cudaGetLastError();
 }
 template <bool WORDS>
@@ -221,9 +272,11 @@ cudaError_t launch_any(const CellMatArgs& P, const int16_t* hexp, uint64_t* W, i
 
 cudaError_t launch_cell_matrices(const CellMatArgs& P, cudaStream_t s) {
   const int q = P.q;
-  const size_t smem = sizeof(double) * ((size_t)PW * 3 * q + q * q + q * q * q);
+  // wells per batch: as fit in the 48 KB that need no opt-in (q = 7: 32)
+  const size_t per = sizeof(double) * (3 * q + q * q), base = sizeof(double) * q * q * q;
+  const int pw = (int)std::min<size_t>(32, std::max<size_t>(1, (46 * 1024 - std::min<size_t>(base, 46 * 1024)) / per));
   note_launch();
-  potential_kernel<<<(unsigned)P.ncells, PT, smem, s>>>(P);
+  potential_kernel<<<(unsigned)P.ncells, PT, base + pw * per, s>>>(P, pw);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   return launch_any<false>(P, nullptr, nullptr, 0, s);

@@ -306,11 +306,16 @@ void build_well_images(const HostMesh& m, const Wells& wl, std::vector<double>& 
   for (size_t a = 0; a < wl.depth.size(); ++a)
     for (int sz = -1; sz <= 1; ++sz) for (int sy = -1; sy <= 1; ++sy) for (int sx = -1; sx <= 1; ++sx) {
       if ((!m.per[0] && sx) || (!m.per[1] && sy) || (!m.per[2] && sz)) continue;
-      out.push_back(wl.xyz[3 * a] + sx * m.len[0]);
-      out.push_back(wl.xyz[3 * a + 1] + sy * m.len[1]);
-      out.push_back(wl.xyz[3 * a + 2] + sz * m.len[2]);
-      out.push_back(wl.depth[a]);
-      out.push_back(1.0 / (2.0 * wl.width[a] * wl.width[a]));
+      const double x[3] = {wl.xyz[3 * a] + sx * m.len[0], wl.xyz[3 * a + 1] + sy * m.len[1],
+                           wl.xyz[3 * a + 2] + sz * m.len[2]};
+      const double g = 1.0 / (2.0 * wl.width[a] * wl.width[a]);
+      double r2 = 0.0;
+      for (int ax = 0; ax < 3; ++ax) {
+        const double d = x[ax] < 0.0 ? -x[ax] : std::max(0.0, x[ax] - m.len[ax]);
+        r2 += d * d;
+      }
+      if (r2 * g > 42.0) continue;   // below e^-41.5 of the depth in every cell (potential_kernel)
+      out.insert(out.end(), {x[0], x[1], x[2], wl.depth[a], g});
     }
 }
 
