@@ -267,15 +267,6 @@ struct Chunks {
   }
 };
 
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
 template <int MODE>
 __global__ void __launch_bounds__(EX_THREADS, 1) ex_kernel(const __grid_constant__ ExParams P) {
   constexpr int SH = MODE == EX_CELL ? 45 : 41;   // units of the integer sums

@@ -593,6 +593,7 @@ struct RParams {
   const int64_t* pj_row;
   int pj_npmax;
   int tpc;                  // multi-tile kernel: column tiles per CTA
+  int64_t nitems;           // stream kernel: (cell, column tile, row part) items
 };
 
 template <int BN, bool MULTI>
@@ -1355,9 +1356,6 @@ __host__ __device__ inline BfrPlan bfr_plan(int ne, int npair, int nt = 3, int p
   return r;
 }
 
-// MULTI: grid x runs over the (system, cell, column tile, row part) items of
-// a batch (TcBatchSys: A = the system's packed BF16x3 copy, tiles = column
-// tiles x parts, items of system s from item0), all systems of one degree.
 // NT = 2: the FP16x2 form (P.A the fp16 terms, P.cinv the per-cell inverse
 // scales, P.cmax the column maxima of Yin): three MMAs per chunk.
 // NLC: the projector chunks are compiled in (a separate instantiation, so the
@@ -1370,45 +1368,24 @@ __host__ __device__ inline BfrPlan bfr_plan(int ne, int npair, int nt = 3, int p
 // M^{-1/2}, the same for every cell of the uniform periodic mesh), the rows
 // of Y gathered with each (real, imaginary) column pair swapped and the new
 // imaginary part negated, so R holds T~_e Y_r + G~ Y_i, T~_e Y_i - G~ Y_r.
-template <int NPAIR, bool MULTI, int NT = 3, bool NLC = false, bool PROJ = false, bool KPT = false>
+template <int NPAIR, int NT = 3, bool NLC = false, bool PROJ = false, bool KPT = false>
 __global__ void __launch_bounds__((2 * NPAIR + 2) * 32, 2) tc_cell_bf16_rings_kernel(RParams P) {
-  static_assert(NT == 3 || (NT == 2 && !MULTI), "BF16x3, or single-system FP16x2");
-  static_assert(!NLC || (NT == 3 && !MULTI), "projector chunks: single-system BF16x3");
-  static_assert(!PROJ || (NT == 3 && !MULTI && !NLC), "projection: single-system BF16x3");
-  static_assert(!KPT || (NT == 3 && !MULTI && !NLC && !PROJ), "Bloch term: single-system BF16x3");
+  static_assert(NT == 3 || NT == 2, "BF16x3 or FP16x2");
+  static_assert(!NLC || NT == 3, "projector chunks: BF16x3");
+  static_assert(!PROJ || (NT == 3 && !NLC), "projection: BF16x3");
+  static_assert(!KPT || (NT == 3 && !NLC && !PROJ), "Bloch term: BF16x3");
   constexpr int NTHR = (2 * NPAIR + 2) * 32;
   constexpr int WPROD = 2 * NPAIR, WMMA = 2 * NPAIR + 1;
   constexpr int YT = NT * 128 * BF_KC * 2;   // Y stage bytes
   extern __shared__ __align__(1024) unsigned char smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  int64_t e = P.e_off + blockIdx.y;
+  const int64_t e = P.e_off + blockIdx.y;
   const int ne = P.ne, nk = P.nk;
   const BfrPlan B = bfr_plan(ne, NPAIR, NT, PROJ ? P.pj_npmax : 0);
   const int nrow = PROJ ? P.pj_np[e] : B.nh;   // B-operand rows of this CTA
   if (PROJ && nrow == 0) return;                // a cell owning no projector rows: nothing to do
-  int h = blockIdx.x % B.np;
-  int c0 = (blockIdx.x / B.np) * 128;
-  if (MULTI) {   // item -> (system, cell, tile, part): binary search over the systems' first items
-    const int64_t item = blockIdx.x;
-    int lo = 0, hi = P.nsys - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (P.sys[mid].item0 <= item) lo = mid; else hi = mid - 1;
-    }
-    const TcBatchSys& sy = P.sys[lo];
-    const int64_t li = item - sy.item0;
-    e = li / sy.tiles;
-    const int t = (int)(li % sy.tiles);
-    h = t % B.np;
-    c0 = (t / B.np) * 128;
-    P.A = sy.A;
-    P.dofmap = sy.dofmap;
-    P.Yin = sy.Y[P.parity];
-    P.ld_in = sy.ldY[P.parity];
-    P.R = sy.R;
-    P.ncol = sy.ncol;
-    P.ldr = sy.ldr;
-  }
+  const int h = blockIdx.x % B.np;
+  const int c0 = (blockIdx.x / B.np) * 128;
   const int ncv = min(128, P.ncol - c0);
   const int r0 = h * B.nh;
   const int SM = B.sm, SY = B.sy;
@@ -1606,6 +1583,533 @@ __global__ void __launch_bounds__((2 * NPAIR + 2) * 32, 2) tc_cell_bf16_rings_ke
   tc_fence_before();
   __syncthreads();
   if (warp == WMMA) tmem_dealloc(tmem, B.alloc);
+}
+
+// ----------------------------------------------------------------- BF16x3 cell kernel, one thread block per SM
+// One thread block per SM works through (cell, column tile, row part) items, so
+// that the MMAs of an item follow those of the one before without a gap:
+//  sets of four gather warps, which take the chunks in turn and split them
+//  four warps   store the finished accumulator (two of them, taken in turn)
+//  one          looks up the coming items: pointers, sizes, the rows to gather
+//  one          copies the matrix chunks (bulk copies, as far ahead as the ring goes)
+//  one          issues the MMAs
+// The split Y chunks go to TMEM (A operand), beside the accumulators: with both
+// operands in shared memory a chunk of 176 rows reads 58 KB of it for its six
+// MMAs and writes 29 (684 clocks at 128 B/clk, for 528 of math); with Y in TMEM it
+// reads 34 and writes 17 (396, and up to 128 for the rows on their way).
+// One system: four sets, whose rows are copied ahead to shared memory (kAhead
+// chunks each).  A batch: two sets with the next chunk in registers; the matrices
+// of its systems come from HBM, once per 14 to 22 chunks, and the shared memory is
+// better spent on their ring.
+// The ring kernel (two blocks per SM, one item each) and this one: 16^3 cells, p =
+// 6, 1,100 columns 4.9 and 4.1 ms; 8^3, p = 6, 110 complex columns with the Bloch
+// chunks 279 and 240 us; 16 systems of p = 5 690 and 600 us.  What bounds it is the
+// tensor core (2.9 ms of the 4.1) together with the shared memory it reads from.
+struct StreamPlan {
+  int np, nh, nacc, alloc, sm, sy, total;
+};
+constexpr int kItems = 4;                               // items looked up ahead
+constexpr int kAhead = 3, kYStage = 17 * 128;           // chunks of Y copied ahead; bytes of a warp's stage
+__host__ __device__ constexpr int stream_sets(bool multi) { return multi ? 2 : 4; }
+__host__ __device__ constexpr int stream_threads(bool multi) { return (4 * stream_sets(multi) + 7) * 32; }
+__device__ const __align__(16) float g_zero_row[128] = {};   // the row of an eliminated or padding node
+struct StreamItem {
+  const char* A;            // chunk 0 of the matrix block (its first row)
+  float* R;                 // row 0, column c0 of the result
+  int64_t ldr, e;
+  int nkt, nrow, rend, c0, ncv, nl0, r0;   // chunks (0: nothing to do), rows computed and stored
+  int vec;                  // rows of Y (1) and Z (2) lie on 16-byte boundaries
+};
+// Row parts of at most nh rows; accumulators, Y stages and matrix stages as fit.
+__host__ __device__ inline StreamPlan stream_plan(int ne, bool multi, int nt = 3, int proj_nh = 0) {
+  StreamPlan r;
+  const int ycols = 8 * nt;
+  const int most = (512 - 2 * ycols) / 32 * 16;
+  r.np = proj_nh > 0 ? 1 : (ne + most - 1) / most;
+  r.nh = proj_nh > 0 ? proj_nh : ((ne + r.np - 1) / r.np + 15) / 16 * 16;
+  r.nacc = 2 * r.nh + 2 * ycols <= 512 ? 2 : 1;
+  r.sy = (512 - r.nacc * r.nh) / ycols;
+  if (r.sy > 6) r.sy = 6;
+  r.alloc = 32;
+  while (r.alloc < r.nacc * r.nh + r.sy * ycols) r.alloc *= 2;
+  const int tail = 512 + kItems * (128 + (ne + BF_KC - 1) / BF_KC * BF_KC * 8);   // barriers, items
+  const int mstage = nt * r.nh * 32, ystages = multi ? 0 : 4 * stream_sets(multi) * kAhead * kYStage;
+  r.sm = (224 * 1024 - tail - ystages) / mstage;
+  if (r.sm > 12) r.sm = 12;
+  r.total = r.sm * mstage + ystages + tail;
+  return r;
+}
+
+// MULTI: the items of all systems of a batch (TcBatchSys: A = the system's packed
+// BF16x3 copy, tiles = column tiles x parts, items of system s from item0), all
+// systems of one degree.
+// NT = 2: the FP16x2 form (P.A the fp16 terms, P.cinv the per-cell inverse
+// scales, P.cmax the column maxima of Yin): three MMAs per chunk.
+// NLC: the K loop continues over the cell's projector chunks.  PROJ: the
+// projection Z = C~^T Y instead of the cell products: the streamed operand is
+// the cell's projection block (np[e] rows = its projectors, K = its nodes),
+// the result (128 columns x np[e]) goes to rows pj_row[e] .. of R.
+// KPT: the Bloch term of H~(k): the K loop continues over a second pass of
+// the cell's nodes against one shared block (P.nlA: G~ = M^{-1/2} (k.G_e)
+// M^{-1/2}, the same for every cell of the uniform periodic mesh), the rows
+// of Y gathered with each (real, imaginary) column pair swapped and the new
+// imaginary part negated, so R holds T~_e Y_r + G~ Y_i, T~_e Y_i - G~ Y_r.
+template <bool MULTI, int NT, bool NLC, bool PROJ, bool KPT, bool OWN>
+__global__ void __launch_bounds__(stream_threads(MULTI), 1) tc_cell_bf16_stream_kernel(RParams P) {
+  static_assert(NT == 3 || (NT == 2 && !MULTI), "BF16x3, or single-system FP16x2");
+  static_assert(!NLC || (NT == 3 && !MULTI), "projector chunks: single-system BF16x3");
+  static_assert(!PROJ || (NT == 3 && !MULTI && !NLC), "projection: single-system BF16x3");
+  static_assert(!KPT || (NT == 3 && !MULTI && !NLC && !PROJ), "Bloch term: single-system BF16x3");
+  constexpr int NSET = stream_sets(MULTI), NGATHER = 4 * NSET;
+  constexpr int WITEM = NGATHER + 4, WPROD = WITEM + 1, WMMA = WPROD + 1;
+  constexpr int YCOL = NT * BF_KC / 2;       // TMEM columns of a Y stage
+  extern __shared__ __align__(1024) unsigned char smem[];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int ne = P.ne, nk = P.nk;
+  const StreamPlan B = stream_plan(ne, MULTI, NT, PROJ ? P.pj_npmax : 0);
+  const int SM = B.sm, SY = B.sy;
+  const int mstage = NT * B.nh * 32;       // matrix stage (the launch's largest block)
+  unsigned char* ybase = smem + SM * mstage;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(ybase + (MULTI ? 0 : NGATHER * kAhead * kYStage));
+  StreamItem* items = reinterpret_cast<StreamItem*>(bars + 64);
+  const float** rows = reinterpret_cast<const float**>(reinterpret_cast<unsigned char*>(items) + kItems * 128);
+  // barriers: matrix full (tx) / empty, Y full / empty, accumulator full / empty, item
+  // full / empty; with fewer Y stages than sets (OWN), one per set: its last chunk is
+  // used up, so that at most one phase of the stage's barrier can be outstanding (SY >=
+  // NSET / 2)
+  const uint32_t mbase = smem_u32(smem), bar0 = smem_u32(bars);
+  auto fa = [&](int s) { return bar0 + 8 * s; };
+  auto ea = [&](int s) { return bar0 + 8 * (SM + s); };
+  auto fy = [&](int s) { return bar0 + 8 * (2 * SM + s); };
+  auto ey = [&](int s) { return bar0 + 8 * (2 * SM + SY + s); };
+  auto facc = [&](int s) { return bar0 + 8 * (2 * SM + 2 * SY + s); };
+  auto eacc = [&](int s) { return bar0 + 8 * (2 * SM + 2 * SY + 2 + s); };
+  auto fi = [&](int s) { return bar0 + 8 * (2 * SM + 2 * SY + 4 + s); };
+  auto ei = [&](int s) { return bar0 + 8 * (2 * SM + 2 * SY + 4 + kItems + s); };
+  auto es = [&](int s) { return bar0 + 8 * (2 * SM + 2 * SY + 4 + 2 * kItems + s); };
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 62);
+  int* abort_flag = reinterpret_cast<int*>(bars + 63);
+  if (tid == 0) {
+    for (int s = 0; s < SM; ++s) {
+      mbar_init(fa(s), 1);
+      mbar_init(ea(s), 1);
+    }
+    for (int s = 0; s < SY; ++s) {
+      mbar_init(fy(s), 4);
+      mbar_init(ey(s), 1);
+    }
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(facc(s), 1);
+      mbar_init(eacc(s), 4);
+    }
+    for (int s = 0; s < kItems; ++s) {
+      mbar_init(fi(s), 1);
+      mbar_init(ei(s), NGATHER + 6);
+    }
+    for (int s = 0; s < NSET; ++s) mbar_init(es(s), 1);
+    *abort_flag = 0;
+    fence_mbar_init();
+  }
+  if (warp == WMMA) {
+    tmem_alloc(smem_u32(tmem_slot), B.alloc);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem_y = tmem + B.nacc * B.nh;
+  const int64_t term_bytes = (int64_t)P.mt * 4096;
+  auto give_up = [&](int code) {
+    atomicExch(&g_tc_status, code);
+    *(volatile int*)abort_flag = 1;
+  };
+  int ib = 0, iph = 0;                       // item buffer, its phase
+
+  if (warp == WITEM) {
+    const int ntp = MULTI ? 1 : (P.ncol + 127) / 128 * B.np;
+    for (int64_t item = blockIdx.x; item < P.nitems; item += gridDim.x) {
+      if (!__all_sync(0xffffffffu, mbar_wait(ei(ib), iph ^ 1))) {
+        if (lane == 0) give_up(45);
+        break;
+      }
+      int64_t e;
+      int x;
+      if (MULTI) {   // binary search over the systems' first items
+        int lo = 0, hi = P.nsys - 1;
+        while (lo < hi) {
+          const int mid = (lo + hi + 1) >> 1;
+          if (P.sys[mid].item0 <= item) lo = mid; else hi = mid - 1;
+        }
+        const TcBatchSys& sy = P.sys[lo];
+        const int64_t li = item - sy.item0;
+        e = li / sy.tiles;
+        x = (int)(li - e * sy.tiles);
+        P.A = sy.A;
+        P.dofmap = sy.dofmap;
+        P.Yin = sy.Y[P.parity];
+        P.ld_in = sy.ldY[P.parity];
+        P.R = sy.R;
+        P.ncol = sy.ncol;
+        P.ldr = sy.ldr;
+      } else {
+        e = item >> 31 ? item / ntp : (int64_t)((uint32_t)item / (uint32_t)ntp);
+        x = (int)(item - e * ntp);
+      }
+      const int c0 = x / B.np * 128, r0 = x % B.np * B.nh;
+      const float** rp = rows + ib * nk * BF_KC;
+#pragma unroll 8
+      for (int l = lane; l < nk * BF_KC; l += 32) {
+        const int g = l < ne ? __ldg(P.dofmap + e * ne + l) : -1;
+        rp[l] = g >= 0 ? P.Yin + (int64_t)g * P.ld_in + c0 : g_zero_row;
+      }
+      if (lane == 0) {
+        StreamItem& I = items[ib];
+        I.e = e;
+        I.c0 = c0;
+        I.r0 = r0;
+        I.ncv = min(128, P.ncol - c0);
+        I.nrow = PROJ ? P.pj_np[e] : min(B.nh, P.mt * 128 - r0);
+        I.rend = PROJ ? I.nrow : min(I.nrow, ne - r0);
+        I.nl0 = NLC ? P.nl_off[e] : 0;
+        I.nkt = PROJ && I.nrow == 0 ? 0 : NLC ? nk + P.nl_off[e + 1] - I.nl0 : (KPT ? 2 * nk : nk);
+        I.A = reinterpret_cast<const char*>(P.A) +
+              (PROJ ? P.pj_off[e] * 2 : e * (int64_t)nk * NT * term_bytes + (int64_t)r0 * 32);
+        I.R = P.R + (PROJ ? P.pj_row[e] : e * ne + r0) * P.ldr + c0;
+        I.ldr = P.ldr;
+        I.vec = ((reinterpret_cast<uintptr_t>(P.Yin) & 15) == 0 && P.ld_in % 4 == 0 ? 1 : 0) |
+                (NLC && (reinterpret_cast<uintptr_t>(P.Z) & 15) == 0 && P.ldz % 4 == 0 ? 2 : 0);
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(fi(ib));
+      if (++ib == kItems) ib = 0, iph ^= 1;
+    }
+  } else if (warp == WPROD) {
+    if (lane == 0) {
+      int issued = 0, s = 0, ph = 1;         // stage of the chunk, phase of its release
+      bool ok = true;
+      for (int64_t item = blockIdx.x; ok && item < P.nitems; item += gridDim.x) {
+        if (!mbar_wait(fi(ib), iph)) {
+          give_up(45);
+          break;
+        }
+        const StreamItem I = items[ib];
+        mbar_arrive(ei(ib));
+        if (++ib == kItems) ib = 0, iph ^= 1;
+        const int hrow = I.nrow * 32;        // bytes of one term of a chunk (rows of 32 B)
+        const int64_t tstride = PROJ ? (int64_t)hrow : term_bytes;   // bytes between terms and chunks
+        // chunk i >= nk: of the projector / Bloch block
+        const char* An = NLC || KPT ? reinterpret_cast<const char*>(P.nlA) + ((int64_t)I.nl0 - nk) * NT * term_bytes +
+                                          (int64_t)I.r0 * 32
+                                    : I.A;
+        for (int i = 0; i < I.nkt; ++i) {
+          if (!mbar_wait(ea(s), ph)) {
+            give_up(41);
+            ok = false;
+            break;
+          }
+          const uint32_t dst = mbase + s * mstage;
+          mbar_arrive_expect_tx(fa(s), NT * hrow);
+          const char* src = (!(NLC || KPT) || i < nk ? I.A : An) + (int64_t)i * NT * tstride;
+#pragma unroll
+          for (int p = 0; p < NT; ++p) bulk_g2s(dst + p * hrow, src + p * tstride, hrow, fa(s));
+          ++issued;
+          if (++s == SM) s = 0, ph ^= 1;
+        }
+      }
+      if (*(volatile int*)abort_flag)
+        for (int i = max(0, issued - SM); i < issued; ++i) mbar_wait(fa(i % SM), (i / SM) & 1);
+    }
+  } else if (warp == WMMA) {
+    if (elect_one()) {
+      int sa = 0, pa = 0, sy = 0, py = 0, set = 0;
+      int b = 0, pb = 1;                     // accumulator, phase of its release
+      bool ok = true;
+      for (int64_t item = blockIdx.x; ok && item < P.nitems; item += gridDim.x) {
+        if (!mbar_wait(fi(ib), iph)) {
+          give_up(45);
+          break;
+        }
+        const int nkt = items[ib].nkt, nrow = items[ib].nrow;
+        mbar_arrive(ei(ib));
+        if (++ib == kItems) ib = 0, iph ^= 1;
+        if (nkt == 0) continue;
+        if (!mbar_wait(eacc(b), pb)) {
+          give_up(46);
+          break;
+        }
+        const uint32_t idesc = NT == 3 ? idesc_bf16(128, nrow) : idesc_f16(128, nrow);
+        const uint32_t acc = tmem + b * B.nh;
+        const int hrow = nrow * 32;
+        for (int i = 0; i < nkt; ++i) {
+          if (!mbar_wait(fa(sa), pa) || !mbar_wait(fy(sy), py)) {
+            give_up(42);
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint32_t y = tmem_y + sy * YCOL;
+          const uint32_t hb = mbase + sa * mstage;
+          uint64_t hd[NT];
+#pragma unroll
+          for (int p = 0; p < NT; ++p) hd[p] = umma_desc(hb + p * hrow, 128, 256);
+          if (NT == 3) {
+            mma_f16_ts(acc, y, hd[NT - 1], idesc, i > 0);
+            mma_f16_ts(acc, y + 8, hd[1], idesc, 1);
+            mma_f16_ts(acc, y + 8 * (NT - 1), hd[0], idesc, 1);
+          }
+          mma_f16_ts(acc, y, hd[1], idesc, NT == 3 || i > 0);
+          mma_f16_ts(acc, y + 8, hd[0], idesc, 1);
+          mma_f16_ts(acc, y, hd[0], idesc, 1);
+          umma_commit(ea(sa));
+          umma_commit(ey(sy));
+          if (OWN) {
+            umma_commit(es(set));
+            if (++set == NSET) set = 0;
+          }
+          if (++sa == SM) sa = 0, pa ^= 1;
+          if (++sy == SY) sy = 0, py ^= 1;
+        }
+        umma_commit(facc(b));
+        if (++b == B.nacc) b = 0, pb ^= 1;
+      }
+    }
+  } else if (warp >= NGATHER) {
+    // ---- store the accumulator: TMEM lane quarter = warp % 4, lane = column
+    const int qc = (warp & 3) * 32 + lane;
+    int b = 0, pb = 0;
+    for (int64_t item = blockIdx.x; item < P.nitems; item += gridDim.x) {
+      if (!__all_sync(0xffffffffu, mbar_wait(fi(ib), iph))) {
+        if (lane == 0) give_up(45);
+        break;
+      }
+      const StreamItem I = items[ib];
+      __syncwarp();
+      if (lane == 0) mbar_arrive(ei(ib));
+      if (++ib == kItems) ib = 0, iph ^= 1;
+      if (I.nkt == 0) continue;
+      const bool on = qc < I.ncv;
+      // FP16x2: undo the cell's and the column's scales (exact powers of two)
+      const float back = NT == 2 && on ? P.cinv[I.e] / f16_scale_of(__uint_as_float(P.cmax[I.c0 + qc])) : 1.f;
+      const bool done = mbar_wait(facc(b), pb);
+      if (!__all_sync(0xffffffffu, done && !*(volatile int*)abort_flag)) {
+        if (lane == 0) give_up(44);
+        break;
+      }
+      tc_fence_after();
+      store_rows(tmem + ((uint32_t)((warp & 3) * 32) << 16) + b * B.nh, I.nrow, I.rend, I.R + qc, I.ldr, on, back);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(eacc(b));
+      if (++b == B.nacc) b = 0, pb ^= 1;
+    }
+  } else {
+    // ---- gather + split (the values are those of tc_cell_bf16_kernel): a warp takes
+    // the 16 rows of a chunk at the 32 columns of its TMEM lane quarter.  Columns
+    // past the edge hold anything: their results are not stored.
+    const int set = warp >> 2, qw = (warp & 3) * 32;
+    int64_t item = blockIdx.x;
+    int i = set, nkt = 0, nl0 = 0, c0 = 0, ncv = 0, vec = 0;   // the set's next chunk, from the item's first
+    float scale = 1.f;
+    bool entered = false, ok = true;
+    const float* const* rp = nullptr;
+    // moves on to the item of the set's next chunk; false after the last one, and
+    // if that item has not been looked up yet and `wait` is not set (a warp that
+    // waits for it must not hold chunks back: the items' buffers come free only as
+    // the accumulators of the items before are stored)
+    auto find = [&](bool wait) {
+      while (ok && item < P.nitems) {
+        if (!entered) {
+          if (!wait && !__all_sync(0xffffffffu, mbar_test(fi(ib), iph))) return false;
+          ok = __all_sync(0xffffffffu, mbar_wait(fi(ib), iph));
+          if (!ok) break;
+          const StreamItem& I = items[ib];
+          nkt = I.nkt;
+          nl0 = I.nl0;
+          c0 = I.c0;
+          ncv = I.ncv;
+          vec = I.vec;
+          rp = rows + ib * nk * BF_KC;
+          if (NT == 2) scale = f16_scale_of(__uint_as_float(P.cmax[c0 + min(qw + lane, ncv - 1)]));   // a power of two
+          entered = true;
+        }
+        if (i < nkt) return true;
+        i -= nkt;
+        entered = false;
+        __syncwarp();
+        if (lane == 0) mbar_arrive(ei(ib));
+        if (++ib == kItems) ib = 0, iph ^= 1;
+        item += gridDim.x;
+      }
+      return false;
+    };
+    // test hook (off by default): warp 0 of the first block withholds its first arrival
+    bool withhold = g_tc_withhold != 0 && blockIdx.x == 0 && warp == 0;
+    int s = set % SY, ph = (set / SY & 1) ^ 1;   // stage of the set's chunk, phase of its release
+    int po = 1;                              // phase of the set's last chunk
+    auto split = [&](const float (&v)[BF_KC], float sc, uint32_t (&w)[NT][BF_KC / 2]) {
+#pragma unroll
+      for (int a = 0; a < BF_KC; a += 2) {
+        const float x = NT == 2 || KPT ? v[a] * sc : v[a], y = NT == 2 || KPT ? v[a + 1] * sc : v[a + 1];
+        if (NT == 3) bf16_split3_pair(x, y, w[0][a / 2], w[1][a / 2], w[NT - 1][a / 2]);
+        else f16_split2_pair(x, y, w[0][a / 2], w[1][a / 2]);
+      }
+    };
+    auto put = [&](const uint32_t (&w)[NT][BF_KC / 2]) {
+      ok = __all_sync(0xffffffffu, (!OWN || mbar_wait(es(set), po)) && mbar_wait(ey(s), ph));
+      if (!ok) return;
+      po ^= 1;
+      tc_fence_after();
+#pragma unroll
+      for (int p = 0; p < NT; ++p) tmem_st8(tmem_y + ((uint32_t)qw << 16) + s * YCOL + p * 8, w[p]);
+      tmem_wait_st();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0 && !withhold) mbar_arrive(fy(s));
+      withhold = false;
+      s += NSET;
+      while (s >= SY) s -= SY, ph ^= 1;
+    };
+    if (MULTI) {
+      auto load = [&](float (&v)[BF_KC]) {
+        if (!find(true)) return false;       // one chunk held back at most, two items on (kItems > 3)
+        const float* const* r = rp + i * BF_KC;
+        const int cl = min(qw + lane, ncv - 1);
+#pragma unroll
+        for (int a = 0; a < BF_KC; a += 2) {
+          const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(r + a);
+          v[a] = __ldg(reinterpret_cast<const float*>(t.x) + cl);
+          v[a + 1] = __ldg(reinterpret_cast<const float*>(t.y) + cl);
+        }
+        i += NSET;
+        return true;
+      };
+      auto put_chunk = [&](const float (&v)[BF_KC]) {
+        uint32_t w[NT][BF_KC / 2];
+        split(v, 1.f, w);
+        put(w);
+        return ok;
+      };
+      float va[BF_KC], vb[BF_KC];
+      bool more = load(va);
+      while (more) {
+        more = load(vb);
+        if (!put_chunk(va) || !more) break;
+        more = load(va);
+        if (!put_chunk(vb)) break;
+      }
+    } else {
+      unsigned char* const stage = ybase + warp * (kAhead * kYStage);
+      int issued = 0;
+      // starts the copies of the set's next chunk, if there is one.  Chunks past nk:
+      // the projectors' (rows of Z), or the cell's rows again with (re, im) -> (im, -re)
+      auto issue = [&](bool wait) {
+        if (find(wait)) {
+          const bool nl = NLC && i >= nk, bloch = KPT && i >= nk;
+          unsigned char* const st = stage + issued % kAhead * kYStage;
+          const uint32_t dst = smem_u32(st);
+          const float* const* r = rp + (bloch ? i - nk : i) * BF_KC;
+          auto row = [&](int a) -> const float* {
+            if (!nl) return r[a];
+            const int g = __ldg(P.nl_zrow + (int64_t)(nl0 + i - nk) * BF_KC + a);
+            return g >= 0 ? P.Z + (int64_t)g * P.ldz + c0 : g_zero_row;
+          };
+          if (nl ? vec & 2 : vec & 1) {
+            const int col = (lane & 7) * 4, left = (ncv - qw - col) * 4;
+            if (left > 0) {
+#pragma unroll
+              for (int k = 0; k < 4; ++k) {
+                const int a = k * 4 + (lane >> 3);
+                cp_async16_part(dst + a * 128 + col * 4, row(a) + qw + col, min(left, 16));
+              }
+            }
+          } else if (qw + lane < ncv) {
+#pragma unroll
+            for (int a = 0; a < BF_KC; ++a) cp_async4(dst + a * 128 + lane * 4, row(a) + qw + lane);
+          }
+          if (NT == 2 || KPT) reinterpret_cast<float*>(st + BF_KC * 128)[lane] = NT == 2 ? scale : (bloch ? 1.f : 0.f);
+          ++issued;
+          i += NSET;
+        }
+        cp_async_commit();
+      };
+#pragma unroll 1
+      for (int n = 0; ok; ++n) {
+        while (issued < n + kAhead) {        // as far ahead as items are known, one chunk at least
+          const int before = issued;
+          issue(before == n);
+          if (issued == before) break;
+        }
+        if (issued == n) break;              // all done
+        if (issued == n + kAhead) cp_async_wait<kAhead - 1>();
+        else cp_async_wait<0>();
+        __syncwarp();
+        const float* const st = reinterpret_cast<const float*>(stage + n % kAhead * kYStage);
+        float v[BF_KC], sc = 1.f;
+        int cl = lane;
+        if (NT == 2) sc = st[BF_KC * 32 + lane];
+        if (KPT && st[BF_KC * 32 + lane] != 0.f) {
+          cl ^= 1;
+          if (lane & 1) sc = -1.f;
+        }
+#pragma unroll
+        for (int a = 0; a < BF_KC; ++a) v[a] = st[a * 32 + cl];
+        uint32_t w[NT][BF_KC / 2];
+        split(v, sc, w);
+        __syncwarp();
+        issue(false);                        // into the stage just read
+        put(w);
+      }
+      cp_async_wait<0>();
+    }
+    if (!ok && lane == 0) give_up(43);
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == WMMA) tmem_dealloc(tmem, B.alloc);
+}
+
+// Thread blocks of a launch: one per SM.
+static unsigned stream_grid(int64_t nitems) {
+  static int sms = 0;
+  static std::once_flag once;
+  std::call_once(once, [] {
+    int d = 0;
+    cudaGetDevice(&d);
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, d) != cudaSuccess || sms < 1) sms = 152;
+  });
+  return (unsigned)std::min<int64_t>(nitems, sms);
+}
+template <bool MULTI, int NT, bool NLC, bool PROJ, bool KPT, bool OWN>
+static cudaError_t stream_launch_own(const RParams& P, int smem, cudaStream_t s) {
+  static std::once_flag attr;
+  std::call_once(attr, [] {
+    cudaFuncSetAttribute(tc_cell_bf16_stream_kernel<MULTI, NT, NLC, PROJ, KPT, OWN>,
+                         cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+  });
+  note_launch();
+  tc_cell_bf16_stream_kernel<MULTI, NT, NLC, PROJ, KPT, OWN><<<stream_grid(P.nitems), stream_threads(MULTI), smem, s>>>(P);
+  return cudaGetLastError();
+}
+template <bool MULTI, int NT = 3, bool NLC = false, bool PROJ = false, bool KPT = false>
+static cudaError_t stream_launch(const RParams& P, cudaStream_t s) {
+  if (P.nitems <= 0) return cudaSuccess;
+  const StreamPlan B = stream_plan(P.ne, MULTI, NT, PROJ ? P.pj_npmax : 0);
+  if (B.sy < stream_sets(MULTI)) return stream_launch_own<MULTI, NT, NLC, PROJ, KPT, true>(P, B.total, s);
+  return stream_launch_own<MULTI, NT, NLC, PROJ, KPT, false>(P, B.total, s);
+}
+
+// Items of a launch when the stream kernel takes it, else 0 (the ring kernel).  It
+// needs two items per SM to have anything to overlap (4^3 cells, p = 7, 110
+// columns: 192 items 56 us per step, as rings 45; 5^3, p = 5: 125 items 28 and 26;
+// 7^3, p = 5: 343 items 49 and 50; 10^3, p = 6, 437 columns: 8,000 items 730 and
+// 824), and up to 128 nodes per cell more than one column tile: there three thread
+// blocks of the ring kernel share an SM (11^3, p = 4: 22 columns 53 and 49 us, 437
+// columns 246 and 265).
+static int64_t stream_items(int64_t ncells, int ncol, int ne, int nt = 3, bool proj = false) {
+  const int tiles = (ncol + 127) / 128;
+  const int64_t items = ncells * tiles * (proj ? 1 : stream_plan(ne, false, nt).np);
+  return items >= 2 * (int64_t)stream_grid(INT64_MAX) && (ne > 128 || tiles > 1) ? items : 0;
 }
 
 // ----------------------------------------------------------------- BF16x3 cell kernel, several column tiles per CTA
@@ -2030,9 +2534,10 @@ cudaError_t tc_cell_bf16_launch(const TcCellData& d, const TcApplyArgs& a, cudaS
   if (a.kG) {   // the Bloch block: the ring kernel with two-column pairs
     if (a.Z || (a.ncol & 1) || (a.ld_in & 1)) return cudaErrorInvalidValue;
     P.nlA = a.kG;
+    if ((P.nitems = stream_items(a.ncells, a.ncol, d.ne)) > 0) return stream_launch<false, 3, false, false, true>(P, s);
     static std::once_flag attrk;
     std::call_once(attrk, [] {
-      cudaFuncSetAttribute(tc_cell_bf16_rings_kernel<2, false, 3, false, false, true>,
+      cudaFuncSetAttribute(tc_cell_bf16_rings_kernel<2, 3, false, false, true>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     });
     const BfrPlan BK = bfr_plan(d.ne, 2);
@@ -2040,21 +2545,22 @@ cudaError_t tc_cell_bf16_launch(const TcCellData& d, const TcApplyArgs& a, cudaS
       P.e_off = e0;
       dim3 grid((unsigned)(((a.ncol + 127) / 128) * B.np), (unsigned)std::min<int64_t>(65535, a.ncells - e0));
       note_launch();
-      tc_cell_bf16_rings_kernel<2, false, 3, false, false, true><<<grid, 6 * 32, BK.total, s>>>(P);
+      tc_cell_bf16_rings_kernel<2, 3, false, false, true><<<grid, 6 * 32, BK.total, s>>>(P);
     }
     return cudaGetLastError();
   }
+  if (a.gather == 2 && (P.nitems = stream_items(a.ncells, a.ncol, d.ne)) > 0)
+    return P.nlA ? stream_launch<false, 3, true>(P, s) : stream_launch<false>(P, s);
   static std::once_flag attr;
   std::call_once(attr, [] {
     cudaFuncSetAttribute(tc_cell_bf16_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     cudaFuncSetAttribute(tc_cell_bf16_async_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    cudaFuncSetAttribute(tc_cell_bf16_rings_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    cudaFuncSetAttribute(tc_cell_bf16_rings_kernel<4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    cudaFuncSetAttribute(tc_cell_bf16_rings_kernel<2, false, 3, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaFuncSetAttribute(tc_cell_bf16_rings_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    cudaFuncSetAttribute(tc_cell_bf16_rings_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    cudaFuncSetAttribute(tc_cell_bf16_rings_kernel<2, 3, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          200 * 1024);
-    cudaFuncSetAttribute(tc_cell_bf16_rings_kernel<4, false, 3, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaFuncSetAttribute(tc_cell_bf16_rings_kernel<4, 3, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          200 * 1024);
-    cudaFuncSetAttribute(tc_cell_bf16_rings_kernel<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     cudaFuncSetAttribute(tc_cell_bf16_whole_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     cudaFuncSetAttribute(tc_cell_bf16_tiles_kernel<2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     cudaFuncSetAttribute(tc_cell_bf16_tiles_kernel<4, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
@@ -2087,17 +2593,17 @@ cudaError_t tc_cell_bf16_launch(const TcCellData& d, const TcApplyArgs& a, cudaS
     if (async)
       tc_cell_bf16_async_kernel<<<grid, BFA_THREADS, BA.total, s>>>(P);
     else if (a.gather == 2 && P.nlA)
-      tc_cell_bf16_rings_kernel<2, false, 3, true><<<grid, 6 * 32, BR.total, s>>>(P);
+      tc_cell_bf16_rings_kernel<2, 3, true><<<grid, 6 * 32, BR.total, s>>>(P);
     else if (a.gather == 3 && P.nlA)
-      tc_cell_bf16_rings_kernel<4, false, 3, true><<<grid, 10 * 32, BR4.total, s>>>(P);
+      tc_cell_bf16_rings_kernel<4, 3, true><<<grid, 10 * 32, BR4.total, s>>>(P);
     else if (a.gather == 2)
-      tc_cell_bf16_rings_kernel<2, false><<<grid, 6 * 32, BR.total, s>>>(P);
+      tc_cell_bf16_rings_kernel<2><<<grid, 6 * 32, BR.total, s>>>(P);
     else if (a.gather == 3)
-      tc_cell_bf16_rings_kernel<4, false><<<grid, 10 * 32, BR4.total, s>>>(P);
+      tc_cell_bf16_rings_kernel<4><<<grid, 10 * 32, BR4.total, s>>>(P);
     else if (a.gather == 4 && bfw_supported(d.ne))
       tc_cell_bf16_whole_kernel<<<dim3((unsigned)((a.ncol + 127) / 128), grid.y), BFW_THREADS, BW.total, s>>>(P);
     else if (a.gather == 4)
-      tc_cell_bf16_rings_kernel<2, false><<<grid, 6 * 32, BR.total, s>>>(P);
+      tc_cell_bf16_rings_kernel<2><<<grid, 6 * 32, BR.total, s>>>(P);
     else
       tc_cell_bf16_kernel<<<grid, CELL_THREADS, B.total, s>>>(P);
   }
@@ -2113,9 +2619,10 @@ cudaError_t tc_cell_f16_launch(const TcCellData& d, const TcApplyArgs& a, const 
   if (B.np * B.nh > d.mt * 128) return cudaErrorInvalidValue;
   RParams P{reinterpret_cast<const float*>(d.f16), a.dofmap, a.Yin, a.R, a.ld_in, a.ncol, d.ne, d.mt,
             nk16, 1, nullptr, 0, 0, a.ldr, 0, cmax, d.f16_inv};
+  if ((P.nitems = stream_items(a.ncells, a.ncol, d.ne, 2)) > 0) return stream_launch<false, 2>(P, s);
   static std::once_flag attr;
   std::call_once(attr, [] {
-    cudaFuncSetAttribute(tc_cell_bf16_rings_kernel<2, false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaFuncSetAttribute(tc_cell_bf16_rings_kernel<2, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          200 * 1024);
   });
   const BfrPlan BR = bfr_plan(d.ne, 2, 2);
@@ -2123,7 +2630,7 @@ cudaError_t tc_cell_f16_launch(const TcCellData& d, const TcApplyArgs& a, const 
     P.e_off = e0;
     dim3 grid((unsigned)(((a.ncol + 127) / 128) * B.np), (unsigned)std::min<int64_t>(65535, a.ncells - e0));
     note_launch();
-    tc_cell_bf16_rings_kernel<2, false, 2><<<grid, 6 * 32, BR.total, s>>>(P);
+    tc_cell_bf16_rings_kernel<2, 2><<<grid, 6 * 32, BR.total, s>>>(P);
   }
   return cudaGetLastError();
 }
@@ -2139,19 +2646,24 @@ cudaError_t tc_nl_project_cells(const TcCellData& d, const int32_t* dofmap, int6
   P.pj_off = d.pj_off;
   P.pj_row = d.pj_row;
   P.pj_npmax = d.pj_npmax;
-  static std::once_flag attr;
-  std::call_once(attr, [] {
-    cudaFuncSetAttribute(tc_cell_bf16_rings_kernel<2, false, 3, false, true>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-  });
-  const BfrPlan BR = bfr_plan(d.ne, 2, 3, d.pj_npmax);
-  for (int64_t e0 = 0; e0 < ncells; e0 += 65535) {
-    P.e_off = e0;
-    dim3 grid((unsigned)((ncol + 127) / 128), (unsigned)std::min<int64_t>(65535, ncells - e0));
-    note_launch();
-    tc_cell_bf16_rings_kernel<2, false, 3, false, true><<<grid, 6 * 32, BR.total, s>>>(P);
+  cudaError_t e = cudaSuccess;
+  if ((P.nitems = stream_items(ncells, ncol, d.ne, 3, true)) > 0) {
+    e = stream_launch<false, 3, false, true>(P, s);
+  } else {
+    static std::once_flag attr;
+    std::call_once(attr, [] {
+      cudaFuncSetAttribute(tc_cell_bf16_rings_kernel<2, 3, false, true>,
+                           cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    });
+    const BfrPlan BR = bfr_plan(d.ne, 2, 3, d.pj_npmax);
+    for (int64_t e0 = 0; e0 < ncells; e0 += 65535) {
+      P.e_off = e0;
+      dim3 grid((unsigned)((ncol + 127) / 128), (unsigned)std::min<int64_t>(65535, ncells - e0));
+      note_launch();
+      tc_cell_bf16_rings_kernel<2, 3, false, true><<<grid, 6 * 32, BR.total, s>>>(P);
+    }
+    e = cudaGetLastError();
   }
-  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const int64_t tot = (int64_t)4 * nsite * ncol;
   note_launch();
@@ -2160,25 +2672,16 @@ cudaError_t tc_nl_project_cells(const TcCellData& d, const int32_t* dofmap, int6
   return cudaGetLastError();
 }
 
-int tc_bf16_parts(int ne) { return bf_plan(ne).np; }
+int tc_bf16_parts(int ne) { return stream_plan(ne, true).np; }
 
 cudaError_t tc_cell_bf16_multi_launch(const TcBatchSys* d_sys, int nsys, int64_t nitems, int ne, int mt,
                                       int parity, cudaStream_t s) {
   if (nitems == 0 || nsys == 0) return cudaSuccess;
   if (nitems > 0x7fffffff) return cudaErrorInvalidValue;
   const int nk16 = (ne + BF_KC - 1) / BF_KC;
-  const BfPlan B0 = bf_plan(ne);
-  if (B0.np * B0.nh > mt * 128) return cudaErrorInvalidValue;
   RParams P{nullptr, nullptr, nullptr, nullptr, 0, 0, ne, mt, nk16, 1, d_sys, nsys, parity, 0, 0};
-  static std::once_flag attr;
-  std::call_once(attr, [] {
-    cudaFuncSetAttribute(tc_cell_bf16_rings_kernel<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         200 * 1024);
-  });
-  const BfrPlan BR = bfr_plan(ne, 2);
-  note_launch();
-  tc_cell_bf16_rings_kernel<2, true><<<(unsigned)nitems, 6 * 32, BR.total, s>>>(P);
-  return cudaGetLastError();
+  P.nitems = nitems;
+  return stream_launch<true>(P, s);
 }
 
 // Each thread: one unknown j, 4 consecutive columns.  Sums the cell rows

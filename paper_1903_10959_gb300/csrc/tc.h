@@ -57,7 +57,8 @@ struct TcApplyArgs {
   int64_t ldr;              //   quads when ldr is a multiple of 4: ldr >= ncol rounded up)
   int split3;
   int tile = 64;            // columns per CTA of the cell kernel: 64 or 128
-  int gather = 2;           // BF16x3: 2 = decoupled matrix / Y rings, 0 = one shared ring, 1 = rows staged by
+  int gather = 2;           // BF16x3: 2 = decoupled matrix / Y rings (with two items per SM and more the kernel
+                            // of one block per SM), 0 = one shared ring, 1 = rows staged by
                             // bulk async copies (when aligned), 3 = rings with four gather warp pairs
   // BF16x3 ring kernels: when set, each cell's K loop continues over its
   // projector chunks (TcCellData::nl) with the rows of Z as the gathered
