@@ -299,15 +299,15 @@ def run_reference(args):
 # x 2 flops x 2.07 GHz = 1.259 TFLOP/s (the nominal 1.25).
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
 # MMA passes the cell kernel issues per algorithmic multiply-add, by precision.
-MMA_PASSES = {"bf16x3": 6, "f16x2": 3, "mixed": 3, "tf32": 1}
+MMA_PASSES = {"bf16x3": 6, "f16x2": 3, "mixed": 3, "tf32": 1, "fp64": 35}
 # Cell-matrix bytes per element each precision's cell kernel reads.
 CELL_MATRIX_BYTES = {"bf16x3": 6, "f16x2": 4, "mixed": 8, "tf32": 4, "fp64": 8}
-CELL_KERNEL = {"bf16x3": "tc_cell_bf16_kernel", "f16x2": "tc_cell_bf16_rings_kernel<2, 0, 2>",
+CELL_KERNEL = {"bf16x3": "tc_cell_bf16_kernel", "f16x2": "tc_cell_bf16_stream_kernel<0, 2>",
                "mixed": "tc_cell_r_kernel",
-               "tf32": "tc_cell_r_kernel", "fp64": "cell_fp64_kernel"}
-# The BF16x3 cell kernel each gather mode launches.
+               "tf32": "tc_cell_r_kernel", "fp64": "ex_kernel<0>"}
+# The BF16x3 cell kernel each gather mode launches (rings: for two items per SM and more).
 BF16_KERNEL = {"registers": "tc_cell_bf16_kernel", "async": "tc_cell_bf16_async_kernel",
-               "rings": "tc_cell_bf16_rings_kernel", "rings4": "tc_cell_bf16_rings_kernel",
+               "rings": "tc_cell_bf16_stream_kernel", "rings4": "tc_cell_bf16_rings_kernel",
                "whole": "tc_cell_bf16_whole_kernel"}
 
 
@@ -387,6 +387,14 @@ def rooflines(prec, s, n, M, peaks, col_steps, steps_blocks, nblocks, cell_ms, c
                                              "(14 n1^4 + 3 n1^3 + 4 (q n1^3 + q^2 n1^2 + q^3 n1) + q^3 "
                                              "+ n1^3 per cell and vector) / event time"})
             roof["frac"] = roof["achieved"] / peak
+        else:
+            # exact products of 8-bit digits: 35 fp16 MMAs per multiply-add
+            mma, mma_note = dtype_peak("f16x2", peaks)
+            roof.update({"bound": "tensor", "peak": mma, "frac": achieved / mma,
+                         "peak_note": mma_note + "; achieved = algorithmic flops (N_c 2 n_e^2 per vector) / event time",
+                         "executed_mma": {"passes_per_flop": MMA_PASSES[prec], "tflops": MMA_PASSES[prec] * achieved,
+                                          "frac_of_peak": MMA_PASSES[prec] * achieved / mma,
+                                          "note": "MMA work the digit products issue (not the method's work)"}})
         return roof, None, None
     cell_bytes = (steps_blocks * nblocks * ncells * ne * ne * s_h
                   + col_steps * M * sx + col_steps * ncells * ne * sx)
@@ -633,7 +641,7 @@ def run_ours(args):
     peaks = load_peaks()
     cell_ms, asm_ms, cell_n, asm_n, nl_ms, nl_n = [float(v) for v in kt]
     roof, asm_roof, step_roof = rooflines(prec, s, n, M, peaks, col_steps, steps_blocks, nblocks,
-                                          cell_ms, cell_n, asm_ms, asm_n, ctx.fp64_operator,
+                                          cell_ms, cell_n, asm_ms, asm_n, args.fp64_op,
                                           gather=args.gather)
     alg_flops = col_steps * ncells * 2 * ne * ne
     phase_timed = phase.copy()
@@ -947,7 +955,7 @@ def run_kpoint(args):
                    "roofline": {"bound": "tensor", "achieved": mflops / t_mixed / 1e12, "peak": bpeak,
                                 "unit": "TFLOP/s", "frac": mflops / t_mixed / 1e12 / bpeak,
                                 "traffic": None,
-                                "kernel": "tc_cell_bf16_rings_kernel (Bloch pairs) + tc_assemble_kernel",
+                                "kernel": "tc_cell_bf16_stream_kernel (Bloch pairs) + tc_assemble_kernel",
                                 "flops_per_apply": mflops,
                                 "peak_note": bnote + "; achieved = algorithmic N_c 8 n_e^2 flops per complex "
                                                      "band (one complex n_e x n_e block per cell) / event time "
@@ -1040,7 +1048,7 @@ def run_batch(args):
         "speedup_vs_sequential": t_seq / t_batch,
         "roofline": {"bound": "tensor", "achieved": achieved, "peak": bf16_peak, "unit": "TFLOP/s",
                      "frac": achieved / bf16_peak, "traffic": None,
-                     "kernel": "tc_cell_bf16_rings_kernel<2, true> (multi-system) + tc_assemble_batched_kernel",
+                     "kernel": "tc_cell_bf16_stream_kernel<1> (multi-system) + tc_assemble_batched_kernel",
                      "peak_note": bf16_note + "; algorithmic flops N_c 2 n_e^2 per vector over the whole "
                                   "filter (cell + assembly launches)",
                      "executed_mma": {"passes_per_flop": 6, "frac_of_peak": 6 * achieved / bf16_peak}},

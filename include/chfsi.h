@@ -134,7 +134,7 @@ chfsi_status chfsi_set_projectors(chfsi_ctx* ctx, int n, const double* xyz, cons
 
 /* Build the cell matrices H~_e = D_e^{-1/2} (1/2 K_e + V_e) D_e^{-1/2}
  * (Eq. discreteHam scaled as in Eq. hep; D_e = global mass at the cell's
- * nodes) in binary64 on the host, and upload them together with the
+ * nodes) in binary64 on the device, together with the
  * precision-specific device copies and the projector data. */
 chfsi_status chfsi_build(chfsi_ctx* ctx);
 
