@@ -310,7 +310,7 @@ __global__ void tc_pack_nl_kernel(const int64_t* __restrict__ pos, const double*
 cudaError_t tc_pack_nl(TcCellData& d, const int32_t* chunk_off, int64_t ncells, const int32_t* zrow,
                        const int64_t* nz_pos, const double* nz_val, int64_t nnz, cudaStream_t s,
                        int64_t* dev_bytes) {
-  const int64_t nchunk = chunk_off[ncells];
+  const int64_t nchunk = d.nl_chunks = chunk_off[ncells];
   const int64_t per_chunk = (int64_t)d.mt * 2048;
   const size_t bytes = (size_t)nchunk * 3 * per_chunk * sizeof(uint16_t);
   int64_t* dpos = nullptr;
@@ -1606,7 +1606,7 @@ __global__ void __launch_bounds__((2 * NPAIR + 2) * 32, 2) tc_cell_bf16_rings_ke
 // chunks 279 and 240 us; 16 systems of p = 5 690 and 600 us.  What bounds it is the
 // tensor core (2.9 ms of the 4.1) together with the shared memory it reads from.
 struct StreamPlan {
-  int np, nh, nacc, alloc, sm, sy, total;
+  int np, nh, alloc, sm, sy, total;
 };
 constexpr int kItems = 4;                               // items looked up ahead
 constexpr int kAhead = 3, kYStage = 17 * 128;           // chunks of Y copied ahead; bytes of a warp's stage
@@ -1617,21 +1617,20 @@ struct StreamItem {
   const char* A;            // chunk 0 of the matrix block (its first row)
   float* R;                 // row 0, column c0 of the result
   int64_t ldr, e;
-  int nkt, nrow, rend, c0, ncv, nl0, r0;   // chunks (0: nothing to do), rows computed and stored
+  int nkt, nrow, rend, c0, ncv, nl0, r0;   // chunks, rows computed and stored
   int vec;                  // rows of Y (1) and Z (2) lie on 16-byte boundaries
 };
 // Row parts of at most nh rows; accumulators, Y stages and matrix stages as fit.
-__host__ __device__ inline StreamPlan stream_plan(int ne, bool multi, int nt = 3, int proj_nh = 0) {
+__host__ __device__ inline StreamPlan stream_plan(int ne, bool multi, int nt = 3) {
   StreamPlan r;
   const int ycols = 8 * nt;
   const int most = (512 - 2 * ycols) / 32 * 16;
-  r.np = proj_nh > 0 ? 1 : (ne + most - 1) / most;
-  r.nh = proj_nh > 0 ? proj_nh : ((ne + r.np - 1) / r.np + 15) / 16 * 16;
-  r.nacc = 2 * r.nh + 2 * ycols <= 512 ? 2 : 1;
-  r.sy = (512 - r.nacc * r.nh) / ycols;
+  r.np = (ne + most - 1) / most;
+  r.nh = ((ne + r.np - 1) / r.np + 15) / 16 * 16;
+  r.sy = (512 - 2 * r.nh) / ycols;
   if (r.sy > 6) r.sy = 6;
   r.alloc = 32;
-  while (r.alloc < r.nacc * r.nh + r.sy * ycols) r.alloc *= 2;
+  while (r.alloc < 2 * r.nh + r.sy * ycols) r.alloc *= 2;
   const int tail = 512 + kItems * (128 + (ne + BF_KC - 1) / BF_KC * BF_KC * 8);   // barriers, items
   const int mstage = nt * r.nh * 32, ystages = multi ? 0 : 4 * stream_sets(multi) * kAhead * kYStage;
   r.sm = (224 * 1024 - tail - ystages) / mstage;
@@ -1645,28 +1644,24 @@ __host__ __device__ inline StreamPlan stream_plan(int ne, bool multi, int nt = 3
 // systems of one degree.
 // NT = 2: the FP16x2 form (P.A the fp16 terms, P.cinv the per-cell inverse
 // scales, P.cmax the column maxima of Yin): three MMAs per chunk.
-// NLC: the K loop continues over the cell's projector chunks.  PROJ: the
-// projection Z = C~^T Y instead of the cell products: the streamed operand is
-// the cell's projection block (np[e] rows = its projectors, K = its nodes),
-// the result (128 columns x np[e]) goes to rows pj_row[e] .. of R.
+// NLC: the K loop continues over the cell's projector chunks.
 // KPT: the Bloch term of H~(k): the K loop continues over a second pass of
 // the cell's nodes against one shared block (P.nlA: G~ = M^{-1/2} (k.G_e)
 // M^{-1/2}, the same for every cell of the uniform periodic mesh), the rows
 // of Y gathered with each (real, imaginary) column pair swapped and the new
 // imaginary part negated, so R holds T~_e Y_r + G~ Y_i, T~_e Y_i - G~ Y_r.
-template <bool MULTI, int NT, bool NLC, bool PROJ, bool KPT, bool OWN>
+template <bool MULTI, int NT, bool NLC, bool KPT, bool OWN>
 __global__ void __launch_bounds__(stream_threads(MULTI), 1) tc_cell_bf16_stream_kernel(RParams P) {
   static_assert(NT == 3 || (NT == 2 && !MULTI), "BF16x3, or single-system FP16x2");
   static_assert(!NLC || (NT == 3 && !MULTI), "projector chunks: single-system BF16x3");
-  static_assert(!PROJ || (NT == 3 && !MULTI && !NLC), "projection: single-system BF16x3");
-  static_assert(!KPT || (NT == 3 && !MULTI && !NLC && !PROJ), "Bloch term: single-system BF16x3");
+  static_assert(!KPT || (NT == 3 && !MULTI && !NLC), "Bloch term: single-system BF16x3");
   constexpr int NSET = stream_sets(MULTI), NGATHER = 4 * NSET;
   constexpr int WITEM = NGATHER + 4, WPROD = WITEM + 1, WMMA = WPROD + 1;
   constexpr int YCOL = NT * BF_KC / 2;       // TMEM columns of a Y stage
   extern __shared__ __align__(1024) unsigned char smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int ne = P.ne, nk = P.nk;
-  const StreamPlan B = stream_plan(ne, MULTI, NT, PROJ ? P.pj_npmax : 0);
+  const StreamPlan B = stream_plan(ne, MULTI, NT);
   const int SM = B.sm, SY = B.sy;
   const int mstage = NT * B.nh * 32;       // matrix stage (the launch's largest block)
   unsigned char* ybase = smem + SM * mstage;
@@ -1718,7 +1713,7 @@ __global__ void __launch_bounds__(stream_threads(MULTI), 1) tc_cell_bf16_stream_
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  const uint32_t tmem_y = tmem + B.nacc * B.nh;
+  const uint32_t tmem_y = tmem + 2 * B.nh;
   const int64_t term_bytes = (int64_t)P.mt * 4096;
   auto give_up = [&](int code) {
     atomicExch(&g_tc_status, code);
@@ -1769,13 +1764,12 @@ __global__ void __launch_bounds__(stream_threads(MULTI), 1) tc_cell_bf16_stream_
         I.c0 = c0;
         I.r0 = r0;
         I.ncv = min(128, P.ncol - c0);
-        I.nrow = PROJ ? P.pj_np[e] : min(B.nh, P.mt * 128 - r0);
-        I.rend = PROJ ? I.nrow : min(I.nrow, ne - r0);
+        I.nrow = min(B.nh, P.mt * 128 - r0);
+        I.rend = min(I.nrow, ne - r0);
         I.nl0 = NLC ? P.nl_off[e] : 0;
-        I.nkt = PROJ && I.nrow == 0 ? 0 : NLC ? nk + P.nl_off[e + 1] - I.nl0 : (KPT ? 2 * nk : nk);
-        I.A = reinterpret_cast<const char*>(P.A) +
-              (PROJ ? P.pj_off[e] * 2 : e * (int64_t)nk * NT * term_bytes + (int64_t)r0 * 32);
-        I.R = P.R + (PROJ ? P.pj_row[e] : e * ne + r0) * P.ldr + c0;
+        I.nkt = NLC ? nk + P.nl_off[e + 1] - I.nl0 : (KPT ? 2 * nk : nk);
+        I.A = reinterpret_cast<const char*>(P.A) + e * nk * NT * term_bytes + (int64_t)r0 * 32;
+        I.R = P.R + (e * ne + r0) * P.ldr + c0;
         I.ldr = P.ldr;
         I.vec = ((reinterpret_cast<uintptr_t>(P.Yin) & 15) == 0 && P.ld_in % 4 == 0 ? 1 : 0) |
                 (NLC && (reinterpret_cast<uintptr_t>(P.Z) & 15) == 0 && P.ldz % 4 == 0 ? 2 : 0);
@@ -1797,7 +1791,6 @@ __global__ void __launch_bounds__(stream_threads(MULTI), 1) tc_cell_bf16_stream_
         mbar_arrive(ei(ib));
         if (++ib == kItems) ib = 0, iph ^= 1;
         const int hrow = I.nrow * 32;        // bytes of one term of a chunk (rows of 32 B)
-        const int64_t tstride = PROJ ? (int64_t)hrow : term_bytes;   // bytes between terms and chunks
         // chunk i >= nk: of the projector / Bloch block
         const char* An = NLC || KPT ? reinterpret_cast<const char*>(P.nlA) + ((int64_t)I.nl0 - nk) * NT * term_bytes +
                                           (int64_t)I.r0 * 32
@@ -1810,9 +1803,9 @@ __global__ void __launch_bounds__(stream_threads(MULTI), 1) tc_cell_bf16_stream_
           }
           const uint32_t dst = mbase + s * mstage;
           mbar_arrive_expect_tx(fa(s), NT * hrow);
-          const char* src = (!(NLC || KPT) || i < nk ? I.A : An) + (int64_t)i * NT * tstride;
+          const char* src = (!(NLC || KPT) || i < nk ? I.A : An) + (int64_t)i * NT * term_bytes;
 #pragma unroll
-          for (int p = 0; p < NT; ++p) bulk_g2s(dst + p * hrow, src + p * tstride, hrow, fa(s));
+          for (int p = 0; p < NT; ++p) bulk_g2s(dst + p * hrow, src + p * term_bytes, hrow, fa(s));
           ++issued;
           if (++s == SM) s = 0, ph ^= 1;
         }
@@ -1833,7 +1826,6 @@ __global__ void __launch_bounds__(stream_threads(MULTI), 1) tc_cell_bf16_stream_
         const int nkt = items[ib].nkt, nrow = items[ib].nrow;
         mbar_arrive(ei(ib));
         if (++ib == kItems) ib = 0, iph ^= 1;
-        if (nkt == 0) continue;
         if (!mbar_wait(eacc(b), pb)) {
           give_up(46);
           break;
@@ -1871,7 +1863,7 @@ __global__ void __launch_bounds__(stream_threads(MULTI), 1) tc_cell_bf16_stream_
           if (++sy == SY) sy = 0, py ^= 1;
         }
         umma_commit(facc(b));
-        if (++b == B.nacc) b = 0, pb ^= 1;
+        if (++b == 2) b = 0, pb ^= 1;
       }
     }
   } else if (warp >= NGATHER) {
@@ -1887,7 +1879,6 @@ __global__ void __launch_bounds__(stream_threads(MULTI), 1) tc_cell_bf16_stream_
       __syncwarp();
       if (lane == 0) mbar_arrive(ei(ib));
       if (++ib == kItems) ib = 0, iph ^= 1;
-      if (I.nkt == 0) continue;
       const bool on = qc < I.ncv;
       // FP16x2: undo the cell's and the column's scales (exact powers of two)
       const float back = NT == 2 && on ? P.cinv[I.e] / f16_scale_of(__uint_as_float(P.cmax[I.c0 + qc])) : 1.f;
@@ -1901,7 +1892,7 @@ __global__ void __launch_bounds__(stream_threads(MULTI), 1) tc_cell_bf16_stream_
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(eacc(b));
-      if (++b == B.nacc) b = 0, pb ^= 1;
+      if (++b == 2) b = 0, pb ^= 1;
     }
   } else {
     // ---- gather + split (the values are those of tc_cell_bf16_kernel): a warp takes
@@ -2080,23 +2071,23 @@ static unsigned stream_grid(int64_t nitems) {
   });
   return (unsigned)std::min<int64_t>(nitems, sms);
 }
-template <bool MULTI, int NT, bool NLC, bool PROJ, bool KPT, bool OWN>
+template <bool MULTI, int NT, bool NLC, bool KPT, bool OWN>
 static cudaError_t stream_launch_own(const RParams& P, int smem, cudaStream_t s) {
   static std::once_flag attr;
   std::call_once(attr, [] {
-    cudaFuncSetAttribute(tc_cell_bf16_stream_kernel<MULTI, NT, NLC, PROJ, KPT, OWN>,
+    cudaFuncSetAttribute(tc_cell_bf16_stream_kernel<MULTI, NT, NLC, KPT, OWN>,
                          cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
   });
   note_launch();
-  tc_cell_bf16_stream_kernel<MULTI, NT, NLC, PROJ, KPT, OWN><<<stream_grid(P.nitems), stream_threads(MULTI), smem, s>>>(P);
+  tc_cell_bf16_stream_kernel<MULTI, NT, NLC, KPT, OWN><<<stream_grid(P.nitems), stream_threads(MULTI), smem, s>>>(P);
   return cudaGetLastError();
 }
-template <bool MULTI, int NT = 3, bool NLC = false, bool PROJ = false, bool KPT = false>
+template <bool MULTI, int NT = 3, bool NLC = false, bool KPT = false>
 static cudaError_t stream_launch(const RParams& P, cudaStream_t s) {
   if (P.nitems <= 0) return cudaSuccess;
-  const StreamPlan B = stream_plan(P.ne, MULTI, NT, PROJ ? P.pj_npmax : 0);
-  if (B.sy < stream_sets(MULTI)) return stream_launch_own<MULTI, NT, NLC, PROJ, KPT, true>(P, B.total, s);
-  return stream_launch_own<MULTI, NT, NLC, PROJ, KPT, false>(P, B.total, s);
+  const StreamPlan B = stream_plan(P.ne, MULTI, NT);
+  if (B.sy < stream_sets(MULTI)) return stream_launch_own<MULTI, NT, NLC, KPT, true>(P, B.total, s);
+  return stream_launch_own<MULTI, NT, NLC, KPT, false>(P, B.total, s);
 }
 
 // Items of a launch when the stream kernel takes it, else 0 (the ring kernel).  It
@@ -2105,10 +2096,14 @@ static cudaError_t stream_launch(const RParams& P, cudaStream_t s) {
 // 7^3, p = 5: 343 items 49 and 50; 10^3, p = 6, 437 columns: 8,000 items 730 and
 // 824), and up to 128 nodes per cell more than one column tile: there three thread
 // blocks of the ring kernel share an SM (11^3, p = 4: 22 columns 53 and 49 us, 437
-// columns 246 and 265).
-static int64_t stream_items(int64_t ncells, int ncol, int ne, int nt = 3, bool proj = false) {
+// columns 246 and 265).  With projector chunks (filter steps): 9^3, p = 6, 308
+// columns 520 and 587 us, but 12^3, p = 7, 1,100 columns 6.48 and 6.40 ms, and where
+// the projectors take more chunks than the nodes (6^3, p = 6) 87 and 83 ms, because
+// the rows of Z are looked up one chunk at a time.
+static int64_t stream_items(int64_t ncells, int ncol, int ne, int nt = 3, int64_t nl_chunks = 0) {
   const int tiles = (ncol + 127) / 128;
-  const int64_t items = ncells * tiles * (proj ? 1 : stream_plan(ne, false, nt).np);
+  const int64_t items = ncells * tiles * stream_plan(ne, false, nt).np;
+  if (nl_chunks > 0 && (ne > 343 || nl_chunks > ncells * ((ne + BF_KC - 1) / BF_KC))) return 0;
   return items >= 2 * (int64_t)stream_grid(INT64_MAX) && (ne > 128 || tiles > 1) ? items : 0;
 }
 
@@ -2534,7 +2529,7 @@ cudaError_t tc_cell_bf16_launch(const TcCellData& d, const TcApplyArgs& a, cudaS
   if (a.kG) {   // the Bloch block: the ring kernel with two-column pairs
     if (a.Z || (a.ncol & 1) || (a.ld_in & 1)) return cudaErrorInvalidValue;
     P.nlA = a.kG;
-    if ((P.nitems = stream_items(a.ncells, a.ncol, d.ne)) > 0) return stream_launch<false, 3, false, false, true>(P, s);
+    if ((P.nitems = stream_items(a.ncells, a.ncol, d.ne)) > 0) return stream_launch<false, 3, false, true>(P, s);
     static std::once_flag attrk;
     std::call_once(attrk, [] {
       cudaFuncSetAttribute(tc_cell_bf16_rings_kernel<2, 3, false, false, true>,
@@ -2549,7 +2544,7 @@ cudaError_t tc_cell_bf16_launch(const TcCellData& d, const TcApplyArgs& a, cudaS
     }
     return cudaGetLastError();
   }
-  if (a.gather == 2 && (P.nitems = stream_items(a.ncells, a.ncol, d.ne)) > 0)
+  if (a.gather == 2 && (P.nitems = stream_items(a.ncells, a.ncol, d.ne, 3, P.nlA ? d.nl_chunks : 0)) > 0)
     return P.nlA ? stream_launch<false, 3, true>(P, s) : stream_launch<false>(P, s);
   static std::once_flag attr;
   std::call_once(attr, [] {
@@ -2646,24 +2641,19 @@ cudaError_t tc_nl_project_cells(const TcCellData& d, const int32_t* dofmap, int6
   P.pj_off = d.pj_off;
   P.pj_row = d.pj_row;
   P.pj_npmax = d.pj_npmax;
-  cudaError_t e = cudaSuccess;
-  if ((P.nitems = stream_items(ncells, ncol, d.ne, 3, true)) > 0) {
-    e = stream_launch<false, 3, false, true>(P, s);
-  } else {
-    static std::once_flag attr;
-    std::call_once(attr, [] {
-      cudaFuncSetAttribute(tc_cell_bf16_rings_kernel<2, 3, false, true>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    });
-    const BfrPlan BR = bfr_plan(d.ne, 2, 3, d.pj_npmax);
-    for (int64_t e0 = 0; e0 < ncells; e0 += 65535) {
-      P.e_off = e0;
-      dim3 grid((unsigned)((ncol + 127) / 128), (unsigned)std::min<int64_t>(65535, ncells - e0));
-      note_launch();
-      tc_cell_bf16_rings_kernel<2, 3, false, true><<<grid, 6 * 32, BR.total, s>>>(P);
-    }
-    e = cudaGetLastError();
+  static std::once_flag attr;
+  std::call_once(attr, [] {
+    cudaFuncSetAttribute(tc_cell_bf16_rings_kernel<2, 3, false, true>,
+                         cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  });
+  const BfrPlan BR = bfr_plan(d.ne, 2, 3, d.pj_npmax);
+  for (int64_t e0 = 0; e0 < ncells; e0 += 65535) {
+    P.e_off = e0;
+    dim3 grid((unsigned)((ncol + 127) / 128), (unsigned)std::min<int64_t>(65535, ncells - e0));
+    note_launch();
+    tc_cell_bf16_rings_kernel<2, 3, false, true><<<grid, 6 * 32, BR.total, s>>>(P);
   }
+  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const int64_t tot = (int64_t)4 * nsite * ncol;
   note_launch();

@@ -30,6 +30,7 @@ struct TcCellData {
   int32_t* nl_off = nullptr;       // ncells + 1 chunk offsets
   int32_t* nl_zrow = nullptr;      // 16 rows of Z per chunk (-1: padding)
   size_t nl_bytes = 0;
+  int64_t nl_chunks = 0;           // all cells together
   // the projection Z = C~^T Y as per-cell BF16x3 blocks (NlCells::np / poff /
   // prow) and the per-site reduction lists; packed with the chunks above
   uint16_t* pj = nullptr;

@@ -10,7 +10,7 @@ import numpy as np
 import pytest
 import torch
 
-from paper_1903_10959_gb300 import Context, workloads as W
+from paper_1903_10959_gb300 import ChfsiError, Context
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
@@ -80,5 +80,26 @@ def test_bloch_chunks(p, cells):
             z = torch.empty_like(x)
             ctx.apply_kpoint_mixed(x, z)
             assert torch.equal(Y[:, c:c + 50], z)
+    finally:
+        ctx.destroy()
+
+
+def test_bounded_waits():
+    """A withheld arrival runs the waits of one block out: an error, and the context
+    goes on (ERR_TIMEOUT; the hook is off by default)."""
+    ctx = _ctx(5, 7)
+    try:
+        X = _block(ctx, 40)
+        Y, Z = torch.empty_like(X), torch.empty_like(X)
+        ctx.apply(X, Y, prec="bf16x3")
+        ctx.debug_withhold_arrival(True)
+        try:
+            with pytest.raises(ChfsiError) as ei:
+                ctx.apply(X, Z, prec="bf16x3")
+            assert ei.value.status == 7
+        finally:
+            ctx.debug_withhold_arrival(False)
+        ctx.apply(X, Z, prec="bf16x3")
+        assert torch.equal(Y, Z)
     finally:
         ctx.destroy()
