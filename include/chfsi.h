@@ -170,7 +170,9 @@ chfsi_status chfsi_set_gemm_kernels(chfsi_ctx* ctx, int tall, int gram);
 /* Variant of the BF16x3 cell kernel (results are bit-identical): 2 (default)
  * = warps gather the cell's rows of Y into registers and split them, with the
  * cell-matrix chunks and the split Y chunks in separate shared-memory rings
- * (the matrix copies run up to five chunks ahead at p = 6); 0 = one ring
+ * (the matrix copies run up to five chunks ahead at p = 6), or, in launches of
+ * two (cell, column tile, row part) items per SM and more, one thread block per
+ * SM over the items with the split Y chunks in tensor memory; 0 = one ring
  * shared by both operands; 1 = the rows staged by bulk async copies several
  * chunks ahead and split from shared memory (used when the block is 16-byte
  * aligned with a leading dimension and a column count that are multiples of
