@@ -182,6 +182,7 @@ void free_device_data(chfsi_ctx* ctx, bool keep = false) {
   }
   tc_build(ctx->tc, m.ncells, m.ne, &ctx->dev_bytes);   // the other packed copies
   ctx->ex_ready = false;
+  ctx->ex_capture = 0;
   ctx->ex_off = false;
   ctx->kpack_valid = false;   // the mixed Bloch packs hold the old cell matrices
   release(ctx, ctx->d_site_ptr, ctx->hproj.site_ptr.size() * 8);
@@ -271,6 +272,17 @@ bool stays_matrix_free(const chfsi_ctx* ctx, int ncol) {
                                 ex_cell_tiles(ctx->mesh.ncells, ctx->mesh.ne, ncol) > kFewTiles));
 }
 
+// The stream capture that s takes part in (0: none).
+uint64_t capture_id(cudaStream_t s) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  unsigned long long id = 0;
+  if (cudaStreamGetCaptureInfo(s, &cs, &id) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return cs == cudaStreamCaptureStatusActive ? (uint64_t)id + 1 : 0;
+}
+
 // Whether a binary64 step of ncol columns takes the digit-slice cell products
 // (kernels_ex.cu): the cell matrices are resident, the block is not one for the
 // matrix-free kernel, and the words of the matrices, of the block and its dense
@@ -286,15 +298,21 @@ bool ensure_ex(chfsi_ctx* ctx, int ncol, int64_t* ldr) {
       if (dalloc(ctx, (void**)&d.words, d.word_bytes) != cudaSuccess) d.words = nullptr;
       if (d.words && dalloc(ctx, (void**)&d.hsum, d.exp_bytes) != cudaSuccess) d.hsum = nullptr;
     }
-    if (!d.hsum || ex_pack_cells(d, ctx->cellmat, m.ne, ctx->stream) != cudaSuccess) {
-      cudaGetLastError();
-      release(ctx, d.words, d.word_bytes);
-      release(ctx, d.hsum, d.exp_bytes);
-      d = ExCellData();
-      ctx->ex_off = true;
-      return false;
+    // in a stream capture the packing is only recorded, once per capture: calls
+    // outside the graph still have to pack
+    const uint64_t capture = capture_id(ctx->stream);
+    if (!capture || capture != ctx->ex_capture) {
+      if (!d.hsum || ex_pack_cells(d, ctx->cellmat, m.ne, ctx->stream) != cudaSuccess) {
+        cudaGetLastError();
+        release(ctx, d.words, d.word_bytes);
+        release(ctx, d.hsum, d.exp_bytes);
+        d = ExCellData();
+        ctx->ex_off = true;
+        return false;
+      }
+      ctx->ex_capture = capture;
+      ctx->ex_ready = !capture;
     }
-    ctx->ex_ready = true;
   }
   const std::string err = ctx->err;
   // the partial sums of the narrow blocks that follow on the matrix-free kernel

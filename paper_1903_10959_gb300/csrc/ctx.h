@@ -45,6 +45,7 @@ struct chfsi_ctx {
   // the next build); ex_used: a digit-slice kernel ran since the last status read
   chfsi::ExCellData ex;
   bool ex_ready = false, ex_off = false, ex_used = false;
+  uint64_t ex_capture = 0;         // stream capture in which the packing was recorded
   int32_t* d_dofmap = nullptr;
   uint8_t* d_modes = nullptr;
   int32_t* d_cells = nullptr;
