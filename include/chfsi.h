@@ -230,7 +230,12 @@ chfsi_status chfsi_fill_uniform(chfsi_ctx* ctx, void* X, int64_t ldx, int64_t ro
  * library-owned device copy: three bf16 terms, 6 B per entry, for
  * CHFSI_MIXED_BF16X3; the TF32 hi / lo pair, 8 B per entry, for the TF32
  * forms) and returns CHFSI_ERR_OOM when that copy does not fit.  The same
- * holds for every entry point below that takes a mixed precision. */
+ * holds for every entry point below that takes a mixed precision.  In
+ * CHFSI_FP64 the call is asynchronous on the context's stream: when a bounded
+ * device wait gives up in it, a later call on this context returns
+ * CHFSI_ERR_TIMEOUT, at the latest the first one after the caller has
+ * synchronised the stream (chfsi_last_timings synchronises and asks for
+ * nothing else). */
 chfsi_status chfsi_apply(chfsi_ctx* ctx, const void* X, int64_t ldx, void* Y, int64_t ldy,
                          int ncol, chfsi_precision prec);
 
@@ -263,7 +268,8 @@ chfsi_status chfsi_apply_noalloc(chfsi_ctx* ctx, const double* X, int64_t ldx, d
  * gather warp of the first thread block withholds its arrival on the first
  * K-chunk's barrier, so the MMA warp's bounded wait (2 s) runs out; the
  * kernel unwinds (waits for its own copies in flight, frees its TMEM) and the
- * call returns CHFSI_ERR_TIMEOUT without latching the context.  on = 0
+ * call returns CHFSI_ERR_TIMEOUT without latching the context.  The same holds
+ * for the binary64 digit-slice launches of this context alone.  on = 0
  * restores normal operation; the next call gives the normal result.  For
  * tests of the error path only.  Synchronises the stream. */
 chfsi_status chfsi_debug_withhold_arrival(chfsi_ctx* ctx, int on);

@@ -81,6 +81,15 @@ chfsi_status fail(chfsi_ctx* c, chfsi_status st, const std::string& msg) {
   do {                                                                                    \
     if (!ctx) return CHFSI_ERR_ARG;                                                       \
     if (ctx->latched != CHFSI_OK) return ctx->latched;                                    \
+    chfsi_status late_ = late_timeout(ctx);                                               \
+    if (late_ != CHFSI_OK) return late_;                                                  \
+  } while (0)
+// Waits for the context's stream, and reports a wait that gave up in what ran.
+#define SYNC_CTX()                                                                        \
+  do {                                                                                    \
+    CK(cudaStreamSynchronize(ctx->stream));                                               \
+    chfsi_status late_ = late_timeout(ctx);                                               \
+    if (late_ != CHFSI_OK) return late_;                                                  \
   } while (0)
 
 cudaError_t dalloc(chfsi_ctx* ctx, void** p, size_t bytes) {
@@ -360,7 +369,7 @@ chfsi_status apply_step(chfsi_ctx* ctx, chfsi_precision prec, const void* Yin, i
         KTimer kt(ctx, 0);
         CK(ex_cell_launch(ctx->ex, ExCellArgs{ctx->d_dofmap, m.ncells, m.ne, ncol, (const double*)Yin, ld_in,
                                               (double*)ctx->Rb.ptr, ldr, ctx->exb.ptr},
-                          ctx->stream));
+                          ctx->watch, ctx->stream));
       }
       KTimer kt(ctx, 1);
       CK(ex_assemble_launch(ExAssembleArgs{ctx->d_node_ptr, ctx->d_node_ent, m.ndofs, ncol,
@@ -511,13 +520,13 @@ chfsi_status check_x(chfsi_ctx* ctx, const void* X, int64_t ldx, int ncol, chfsi
 
 // Device-side bounded waits report through a status word; map it to an error.
 chfsi_status check_device_status(chfsi_ctx* ctx, chfsi_precision prec) {
-  int v = is_mixed(prec) ? tc_read_status(ctx->stream) : 0;
-  if (!v && ctx->ex_used) {
-    v = ex_read_status(ctx->stream);
-    ctx->ex_used = false;
-  }
+  const int v = is_mixed(prec) ? tc_read_status(ctx->stream) : 0;
   if (v) return fail(ctx, CHFSI_ERR_TIMEOUT, "device wait timed out (site " + std::to_string(v) + ")");
-  return CHFSI_OK;
+  if (ctx->ex_used) {
+    ctx->ex_used = false;
+    CK(cudaStreamSynchronize(ctx->stream));
+  }
+  return late_timeout(ctx);
 }
 
 void tic(chfsi_ctx* ctx) { cudaEventRecord(ctx->ev[0], ctx->stream); }
@@ -688,7 +697,7 @@ chfsi_status gram_impl(chfsi_ctx* ctx, chfsi_precision prec, const void* A, int6
     if ((st = grow(ctx, ctx->part, want)) == CHFSI_OK) {
       ctx->ex_used = true;
       CK(ex_gram((const double*)A, lda, (const double*)Bm, ldb, m.ndofs, n1, n2, C, ldc, lower, ctx->part.ptr,
-                 ctx->part.bytes, ctx->stream));
+                 ctx->part.bytes, ctx->watch, ctx->stream));
       return CHFSI_OK;
     }
     want = (size_t)8 * 8 * n1 * n2;
@@ -712,7 +721,7 @@ chfsi_status tall64_impl(chfsi_ctx* ctx, const double* X, int64_t ldx, int n1, i
   const std::string err = ctx->err;
   if (grow(ctx, ctx->work, ex_tall_work_bytes(m.ndofs, n1, n2)) == CHFSI_OK) {
     ctx->ex_used = true;
-    CK(ex_tall(X, ldx, U, ldu, m.ndofs, n1, n2, C, ldc, upper, trans, ctx->work.ptr, ctx->stream));
+    CK(ex_tall(X, ldx, U, ldu, m.ndofs, n1, n2, C, ldc, upper, trans, ctx->work.ptr, ctx->watch, ctx->stream));
     return CHFSI_OK;
   }
   ctx->err = err;
@@ -731,7 +740,8 @@ chfsi_status rotate_impl(chfsi_ctx* ctx, chfsi_precision prec, void* X, int64_t 
     const std::string err = ctx->err;
     if (grow(ctx, ctx->work, ex_tall_work_bytes(m.ndofs, n, n)) == CHFSI_OK) {
       ctx->ex_used = true;
-      CK(ex_tall((const double*)X, ldx, U, n, m.ndofs, n, n, (double*)X, ldx, upper, trans, ctx->work.ptr, ctx->stream));
+      CK(ex_tall((const double*)X, ldx, U, n, m.ndofs, n, n, (double*)X, ldx, upper, trans, ctx->work.ptr, ctx->watch,
+                 ctx->stream));
       return CHFSI_OK;
     }
     ctx->err = err;
@@ -773,7 +783,7 @@ chfsi_status cholgs_impl(chfsi_ctx* ctx, void* X, int64_t ldx, int n, chfsi_prec
   CK(launch_chol_inverse(S, n, Linv, dinfo, ctx->stream));
   int info = 0;
   CK(cudaMemcpyAsync(&info, dinfo, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-  CK(cudaStreamSynchronize(ctx->stream));
+  SYNC_CTX();
   if (info != 0)
     return fail(ctx, CHFSI_ERR_NOT_SPD, "CholGS: potrf info = " + std::to_string(info));
   // 3. X <- X L^{-T}: U(k, j) = Linv(j, k), nonzero for k <= j
@@ -841,7 +851,7 @@ chfsi_status rr_impl(chfsi_ctx* ctx, void* X, int64_t ldx, int n, chfsi_precisio
   CK(cudaMemcpyAsync(&info, dinfo, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
   if (evals_host)
     CK(cudaMemcpyAsync(evals_host, W, (size_t)n * 8, cudaMemcpyDeviceToHost, ctx->stream));
-  CK(cudaStreamSynchronize(ctx->stream));
+  SYNC_CTX();
   if (info != 0) return fail(ctx, CHFSI_ERR_EIG, "RR: syevd info = " + std::to_string(info));
   // 3. X <- X Q
   return rotate_impl(ctx, prec, X, ldx, n, Hh, 0, 0);
@@ -982,6 +992,14 @@ cudaError_t noalloc_scratch(chfsi_ctx* ctx, void** out) {
 
 // ===================================================================== C ABI
 namespace chfsi {
+chfsi_status late_timeout(chfsi_ctx* ctx) {
+  volatile int* w = ctx->h_status;
+  const int v = *w;
+  if (!v) return CHFSI_OK;
+  *w = 0;
+  return fail(ctx, CHFSI_ERR_TIMEOUT, "device wait timed out (site " + std::to_string(v) + ")");
+}
+
 // Rayleigh-Ritz for the library's own drivers (batched solve): fp64_apply
 // applies H~ with binary64 cell products to a binary32 block.
 chfsi_status rayleigh_ritz_internal(chfsi_ctx* ctx, void* X, int64_t ldx, int n, chfsi_precision prec,
@@ -1025,10 +1043,13 @@ chfsi_status chfsi_create(const chfsi_mesh_desc* desc, void* stream, chfsi_ctx**
       (e = upload(ctx, &ctx->d_msq, minv_sqrt(m))) != cudaSuccess ||
       (e = cudaEventCreate(&ctx->ev[0])) != cudaSuccess ||
       (e = cudaEventCreate(&ctx->ev[1])) != cudaSuccess ||
+      (e = cudaHostAlloc((void**)&ctx->h_status, sizeof(int), cudaHostAllocMapped)) != cudaSuccess ||
+      (e = cudaHostGetDevicePointer((void**)&ctx->watch.status, ctx->h_status, 0)) != cudaSuccess ||
       (e = cudaStreamSynchronize(ctx->stream)) != cudaSuccess) {
     chfsi_destroy(ctx);
     return e == cudaErrorMemoryAllocation ? CHFSI_ERR_OOM : CHFSI_ERR_CUDA;
   }
+  *(volatile int*)ctx->h_status = 0;
   *out = ctx;
   return CHFSI_OK;
 }
@@ -1047,6 +1068,7 @@ chfsi_status chfsi_destroy(chfsi_ctx* ctx) {
   release(ctx, ctx->d_msq, m.mass.size() * 8);
   release(ctx, ctx->d_K, ((size_t)2 * m.ne * m.ne + 3 * m.n1 + 2 * m.q + (size_t)m.q * m.n1) * 8);
   dfree(ctx, ctx->wellb.ptr, ctx->wellb.bytes);
+  if (ctx->h_status) cudaFreeHost(ctx->h_status);
   if (ctx->d_kfac) cudaFree(ctx->d_kfac);
   ctx->d_kfac = nullptr;
   for (void* q : {(void*)ctx->d_kA, (void*)ctx->d_kG, (void*)ctx->kbf, (void*)ctx->kgbf})
@@ -1093,7 +1115,7 @@ chfsi_status chfsi_kernel_timings(chfsi_ctx* ctx, double* out6) {
   double* out4 = out6;
   CHECK_CTX();
   if (!out4) return CHFSI_ERR_ARG;
-  CK(cudaStreamSynchronize(ctx->stream));
+  SYNC_CTX();
   for (auto& r : ctx->krec) {
     float ms = 0.f;
     cudaEventElapsedTime(&ms, r.a, r.b);
@@ -1167,7 +1189,7 @@ chfsi_status chfsi_set_projectors(chfsi_ctx* ctx, int n, const double* xyz, cons
 
 chfsi_status chfsi_build(chfsi_ctx* ctx) {
   CHECK_CTX();
-  CK(cudaStreamSynchronize(ctx->stream));
+  SYNC_CTX();
   free_device_data(ctx, true);
   const HostMesh& m = ctx->mesh;
   const int nq = m.q * m.q * m.q;
@@ -1388,7 +1410,7 @@ chfsi_status chfsi_apply(chfsi_ctx* ctx, const void* X, int64_t ldx, void* Y, in
   if (ncol > 0 && (!Y || ldy < ncol)) return fail(ctx, CHFSI_ERR_ARG, "bad Y / ldy");
   st = apply_blocks(ctx, prec, X, ldx, Y, ldy, ncol);
   // a binary64 application stays asynchronous: a wait that gave up in it is
-  // reported by the next call that synchronises
+  // reported by a later call on the context (late_timeout)
   if (st == CHFSI_OK && is_mixed(prec)) st = check_device_status(ctx, prec);
   return st;
 }
@@ -1454,7 +1476,9 @@ chfsi_status chfsi_apply_noalloc(chfsi_ctx* ctx, const double* X, int64_t ldx, d
 }
 
 chfsi_status chfsi_debug_withhold_arrival(chfsi_ctx* ctx, int on) {
-  CHECK_CTX();
+  if (!ctx) return CHFSI_ERR_ARG;
+  if (ctx->latched != CHFSI_OK) return ctx->latched;
+  ctx->watch.withhold = on != 0;
   CK(tc_set_withhold(on, ctx->stream));
   return CHFSI_OK;
 }
@@ -1535,7 +1559,7 @@ chfsi_status chfsi_rayleigh_ritz_split(chfsi_ctx* ctx, const void* X, int64_t ld
   int info = 0;
   CK(cudaMemcpyAsync(&info, dinfo, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaMemcpyAsync(evals_fr_host, W, (size_t)n_fr * 8, cudaMemcpyDeviceToHost, ctx->stream));
-  CK(cudaStreamSynchronize(ctx->stream));
+  SYNC_CTX();
   if (info != 0 || meig != n_fr)
     return fail(ctx, CHFSI_ERR_EIG, "split RR: syevdx info = " + std::to_string(info) +
                                         ", eigenpairs " + std::to_string(meig));
@@ -1586,7 +1610,7 @@ chfsi_status chfsi_density(chfsi_ctx* ctx, const void* X, int64_t ldx, int n, co
   a.is_double = prec == CHFSI_FP64;
   a.rho = rho;
   CK(launch_density(a, ctx->stream));
-  CK(cudaStreamSynchronize(ctx->stream));   // the host table must outlive its copy
+  SYNC_CTX();   // the host table must outlive its copy
   return CHFSI_OK;
 }
 
@@ -1830,14 +1854,14 @@ chfsi_status chfsi_unscale(chfsi_ctx* ctx, void* X, int64_t ldx, int ncol, chfsi
   for (int64_t j = 0; j < m.ndofs; ++j) s[j] = 1.0 / std::sqrt(m.mass[j]);
   CK(cudaMemcpyAsync(ctx->vec.ptr, s.data(), s.size() * 8, cudaMemcpyHostToDevice, ctx->stream));
   CK(launch_scale_rows(X, ldx, m.ndofs, ncol, (const double*)ctx->vec.ptr, prec == CHFSI_FP64, ctx->stream));
-  CK(cudaStreamSynchronize(ctx->stream));
+  SYNC_CTX();
   return CHFSI_OK;
 }
 
 chfsi_status chfsi_last_timings(chfsi_ctx* ctx, double* out4) {
   CHECK_CTX();
   if (!out4) return CHFSI_ERR_ARG;
-  CK(cudaStreamSynchronize(ctx->stream));
+  SYNC_CTX();
   for (int i = 0; i < 4; ++i) out4[i] = ctx->times[i];
   return CHFSI_OK;
 }

@@ -42,10 +42,12 @@ struct chfsi_ctx {
   chfsi::TcCellData tc;                   // tensor-core copies (mixed precisions)
   // digit slices of the binary64 cell matrices (packed on first binary64 use;
   // ex_off: they did not fit, the binary64 operator stays on the ALUs until
-  // the next build); ex_used: a digit-slice kernel ran since the last status read
+  // the next build); ex_used: a digit-slice kernel ran since the last status check
   chfsi::ExCellData ex;
   bool ex_ready = false, ex_off = false, ex_used = false;
   uint64_t ex_capture = 0;         // stream capture in which the packing was recorded
+  chfsi::ExWatch watch{};          // where their bounded waits report: the device's view of
+  int* h_status = nullptr;         //   this word (pinned host memory)
   int32_t* d_dofmap = nullptr;
   uint8_t* d_modes = nullptr;
   int32_t* d_cells = nullptr;
@@ -109,4 +111,7 @@ struct chfsi_ctx {
 namespace chfsi {
 chfsi_status rayleigh_ritz_internal(chfsi_ctx* ctx, void* X, int64_t ldx, int n, chfsi_precision prec,
                                     double* evals_host, bool fp64_apply);
+// CHFSI_ERR_TIMEOUT (once) when a bounded wait of the context's digit-slice kernels
+// gave up in work that has run by now; does not synchronise.
+chfsi_status late_timeout(chfsi_ctx* ctx);
 }  // namespace chfsi

@@ -9,6 +9,16 @@
 
 namespace chfsi {
 
+// Where a launch reports a bounded wait that gave up: a word of the context's own
+// (contexts run side by side on their streams, and one must not read or clear
+// another's) in host memory that the device can write, so that the host reads it
+// after any synchronisation without a copy.  withhold: test hook, one arrival of
+// the launch's first thread block is left out.
+struct ExWatch {
+  int* status;
+  int withhold;
+};
+
 // The binary64 cell matrices as digit words.
 struct ExCellData {
   uint64_t* words = nullptr;   // per cell, K-major: word of (row l, column k) at [(e ne + k) rp + l]
@@ -36,7 +46,7 @@ struct ExCellArgs {
   void* work;
 };
 size_t ex_cell_work_bytes(int64_t ncells, int ne, int ncol);
-cudaError_t ex_cell_launch(const ExCellData& d, const ExCellArgs& a, cudaStream_t s);
+cudaError_t ex_cell_launch(const ExCellData& d, const ExCellArgs& a, const ExWatch& w, cudaStream_t s);
 
 // Y_out = alpha (sum of the cell rows + NL - shift Y_in) + beta Y_prev per unknown.
 struct ExAssembleArgs {
@@ -62,14 +72,12 @@ cudaError_t ex_assemble_launch(const ExAssembleArgs& a, cudaStream_t s);
 // work: ex_gram_work_bytes of scratch.
 size_t ex_gram_work_bytes(int64_t M, int n1, int n2, int lower);
 cudaError_t ex_gram(const double* A, int64_t lda, const double* B, int64_t ldb, int64_t M, int n1, int n2,
-                    double* C, int64_t ldc, int lower, void* work, size_t work_bytes, cudaStream_t s);
+                    double* C, int64_t ldc, int lower, void* work, size_t work_bytes, const ExWatch& w,
+                    cudaStream_t s);
 
 // C (M x n2) = A (M x n1) U (contract of launch_tallgemm_fp64).
 size_t ex_tall_work_bytes(int64_t M, int n1, int n2);
 cudaError_t ex_tall(const double* A, int64_t lda, const double* U, int64_t ldu, int64_t M, int n1, int n2,
-                    double* C, int64_t ldc, int upper, int trans, void* work, cudaStream_t s);
-
-// Read and clear the status word of the bounded waits (0: no timeout).
-int ex_read_status(cudaStream_t s);
+                    double* C, int64_t ldc, int upper, int trans, void* work, const ExWatch& w, cudaStream_t s);
 
 }  // namespace chfsi

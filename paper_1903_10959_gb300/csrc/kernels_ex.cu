@@ -58,8 +58,6 @@ using namespace ptx;
 
 namespace {
 
-__device__ int g_ex_status = 0;   // nonzero after a bounded wait gave up
-
 constexpr int NA = 7, NB = 8;               // digits of the M and the N operand
 constexpr int NG = 8;                       // accumulator groups
 constexpr int KC = 16;                      // K per chunk (one MMA step)
@@ -109,6 +107,7 @@ struct ExParams {
   int upper;
   double* C;                // R / partial / C
   int64_t ldc;
+  ExWatch watch;
 };
 
 __device__ __forceinline__ int elem_off(int r, int k) {   // 16-bit elements, K-major core matrices
@@ -312,7 +311,10 @@ __global__ void __launch_bounds__(EX_THREADS, 1) ex_kernel(const __grid_constant
   const int seg = MODE == EX_CELL && *P.hsum <= (1 << 24) - (1 << 18) ? 1 << 20 : SEG;   // chunks per segment
   // A role whose wait gives up records it and leaves; the waits of the roles
   // that depend on it then run out in turn, so that every warp reaches the end.
-  auto give_up = [&](int site) { atomicExch(&g_ex_status, site); };
+  auto give_up = [&](int site) {
+    *(volatile int*)P.watch.status = site;
+    __threadfence_system();
+  };
 
   if (warp < 8) {
     // ---- drain: lane quarter warp % 4, N columns HN (warp / 4) ..
@@ -415,7 +417,7 @@ __global__ void __launch_bounds__(EX_THREADS, 1) ex_kernel(const __grid_constant
     };
 #pragma unroll
     for (int d = 0; d < A_DEP; ++d) issue();
-    bool ok = true;
+    bool ok = true, withhold = P.watch.withhold && blockIdx.x == 0 && warp == 8;
     int ph = 1;
     for (int n = 0; n < issued; ++n) {
       cp_async_wait<A_DEP - 1>();
@@ -434,7 +436,8 @@ __global__ void __launch_bounds__(EX_THREADS, 1) ex_kernel(const __grid_constant
       tmem_wait_st();
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(fa(set));
+      if (lane == 0 && !withhold) mbar_arrive(fa(set));
+      withhold = false;
       ph ^= 1;
     }
     cp_async_wait<0>();
@@ -964,7 +967,7 @@ size_t ex_cell_work_bytes(int64_t ncells, int ne, int ncol) {
   return align256(c * ncol * sizeof(int16_t)) + c * padk(ne) * pad2(ncol) * sizeof(uint64_t);
 }
 
-cudaError_t ex_cell_launch(const ExCellData& d, const ExCellArgs& a, cudaStream_t s) {
+cudaError_t ex_cell_launch(const ExCellData& d, const ExCellArgs& a, const ExWatch& w, cudaStream_t s) {
   if (a.ncells <= 0 || a.ncol <= 0) return cudaSuccess;
   const int64_t slice = cell_slice(a.ncells, a.ne, a.ncol);
   int16_t* cexp = (int16_t*)a.work;
@@ -990,6 +993,7 @@ cudaError_t ex_cell_launch(const ExCellData& d, const ExCellArgs& a, cudaStream_
     P.C = a.R;
     P.ldc = a.ldr;
     P.nitems = ex_cell_tiles(n, a.ne, a.ncol);
+    P.watch = w;
     if ((e = launch<EX_CELL>(P, s)) != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -1014,7 +1018,8 @@ size_t ex_gram_work_bytes(int64_t M, int n1, int n2, int lower) {
 }
 
 cudaError_t ex_gram(const double* A, int64_t lda, const double* B, int64_t ldb, int64_t M, int n1, int n2,
-                    double* C, int64_t ldc, int lower, void* work, size_t work_bytes, cudaStream_t s) {
+                    double* C, int64_t ldc, int lower, void* work, size_t work_bytes, const ExWatch& w,
+                    cudaStream_t s) {
   if (n1 <= 0 || n2 <= 0) return cudaSuccess;
   const bool same = B == A && ldb == lda && n2 <= n1;
   const GramPlan g = gram_plan(M, n1, n2, lower, same);
@@ -1054,6 +1059,7 @@ cudaError_t ex_gram(const double* A, int64_t lda, const double* B, int64_t ldb, 
     P.ntile = gram_tiles(n1, n2, lower);
     P.C = partial;
     P.nitems = P.ntile * ((rows + g.rps - 1) / g.rps);
+    P.watch = w;
     if ((e = launch<EX_GRAM>(P, s)) != cudaSuccess) return e;
   }
   const int64_t tot = (int64_t)n1 * n2;
@@ -1068,7 +1074,7 @@ size_t ex_tall_work_bytes(int64_t M, int n1, int n2) {
 }
 
 cudaError_t ex_tall(const double* A, int64_t lda, const double* U, int64_t ldu, int64_t M, int n1, int n2,
-                    double* C, int64_t ldc, int upper, int trans, void* work, cudaStream_t s) {
+                    double* C, int64_t ldc, int upper, int trans, void* work, const ExWatch& w, cudaStream_t s) {
   if (M <= 0 || n1 <= 0 || n2 <= 0) return cudaSuccess;
   int* rexp = (int*)work;
   int* ecol = (int*)((char*)work + align256((size_t)M * 4));
@@ -1108,21 +1114,10 @@ cudaError_t ex_tall(const double* A, int64_t lda, const double* U, int64_t ldu, 
     P.C = C;
     P.ldc = ldc;
     P.nitems = (rows + BM - 1) / BM * ((n2 + BN - 1) / BN);
+    P.watch = w;
     if ((e = launch<EX_TALL>(P, s)) != cudaSuccess) return e;
   }
   return cudaSuccess;
-}
-
-int ex_read_status(cudaStream_t s) {
-  int v = 0;
-  cudaMemcpyFromSymbolAsync(&v, g_ex_status, sizeof(int), 0, cudaMemcpyDeviceToHost, s);
-  cudaStreamSynchronize(s);
-  if (v) {
-    int z = 0;
-    cudaMemcpyToSymbolAsync(g_ex_status, &z, sizeof(int), 0, cudaMemcpyHostToDevice, s);
-    cudaStreamSynchronize(s);
-  }
-  return v;
 }
 
 }  // namespace chfsi

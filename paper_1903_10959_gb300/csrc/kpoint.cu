@@ -122,6 +122,7 @@ unsigned kblk(int64_t n) { return (unsigned)((n + 255) / 256); }
 chfsi_status kcheck(chfsi_ctx* ctx) {
   if (!ctx) return CHFSI_ERR_ARG;
   if (ctx->latched != CHFSI_OK) return ctx->latched;
+  if (chfsi_status late = late_timeout(ctx); late != CHFSI_OK) return late;
   if (!ctx->kset) return kfail(ctx, CHFSI_ERR_STATE, "chfsi_set_kpoint has not been called");
   if (!ctx->built || !ctx->d_wv) return kfail(ctx, CHFSI_ERR_STATE, "the context has no potential (chfsi_build)");
   if (ctx->hproj.nsite > 0) return kfail(ctx, CHFSI_ERR_ARG, "projector Bloch phases are not modelled");
@@ -388,6 +389,7 @@ extern "C" {
 chfsi_status chfsi_set_kpoint(chfsi_ctx* ctx, const double* k) {
   if (!ctx || !k) return CHFSI_ERR_ARG;
   if (ctx->latched != CHFSI_OK) return ctx->latched;
+  if (chfsi_status late = late_timeout(ctx); late != CHFSI_OK) return late;
   const HostMesh& m = ctx->mesh;
   if (!m.per[0] || !m.per[1] || !m.per[2]) return kfail(ctx, CHFSI_ERR_ARG, "Bloch states need a periodic box");
   if (!mf_supported(m.p, m.q)) return kfail(ctx, CHFSI_ERR_ARG, "k-points need 2 <= p <= 8 and q = p + 2");

@@ -463,6 +463,7 @@ extern "C" {
 chfsi_status chfsi_set_potential_qp_device(chfsi_ctx* ctx, const double* v) {
   if (!ctx) return CHFSI_ERR_ARG;
   if (ctx->latched != CHFSI_OK) return ctx->latched;
+  if (chfsi_status late = late_timeout(ctx); late != CHFSI_OK) return late;
   const HostMesh& m = ctx->mesh;
   if (!v) return sfail(ctx, CHFSI_ERR_ARG, "potential values: null pointer");
   if (!mf_supported(m.p, m.q))
@@ -523,6 +524,7 @@ chfsi_status chfsi_poisson(chfsi_ctx* ctx, const double* f, double* phi, double 
                            int* iters, double* rel_residual) {
   if (!ctx) return CHFSI_ERR_ARG;
   if (ctx->latched != CHFSI_OK) return ctx->latched;
+  if (chfsi_status late = late_timeout(ctx); late != CHFSI_OK) return late;
   const HostMesh& m = ctx->mesh;
   if (!f || !phi || !(tol > 0.0) || max_iter < 1) return sfail(ctx, CHFSI_ERR_ARG, "bad Poisson arguments");
   if (!m.per[0] || !m.per[1] || !m.per[2]) return sfail(ctx, CHFSI_ERR_ARG, "the Poisson solve is for periodic meshes");
@@ -535,6 +537,7 @@ chfsi_status chfsi_scf(chfsi_ctx* ctx, const chfsi_scf_params* prm, double* X, i
                        double* res_hist, int* iters_out) {
   if (!ctx || !prm) return CHFSI_ERR_ARG;
   if (ctx->latched != CHFSI_OK) return ctx->latched;
+  if (chfsi_status late = late_timeout(ctx); late != CHFSI_OK) return late;
   const chfsi_scf_params& P = *prm;
   const HostMesh& m = ctx->mesh;
   const int n = P.n_states;
