@@ -94,8 +94,8 @@ struct ExParams {
   const int* hsum;          // bound of the FP32 sums over a whole cell row (ex_h_scale_kernel)
   const int16_t* cexp;      // per (cell of this launch, column)
   int ne, ncol;
-  // GRAM: rows of this launch; splits z0 .. of rps rows
-  int64_t M, rps, z0;
+  // GRAM: rows of this launch, in splits of rps rows
+  int64_t M, rps;
   int n1, n2;
   const int* aexp;          // column scales
   const int* bexp;
@@ -360,7 +360,7 @@ __global__ void __launch_bounds__(EX_THREADS, 1) ex_kernel(const __grid_constant
         } else if (MODE == EX_GRAM) {
           if (j0 + lane < I.nv) en = P.bexp[I.n0 + j0 + lane];
           if (m < I.mv) em = P.aexp[I.m0 + m];
-          out = P.C + (P.z0 + I.row) * (int64_t)P.n1 * P.n2 + (int64_t)(I.n0 + j0) * P.n1 + I.m0 + m;
+          out = P.C + I.row * (int64_t)P.n1 * P.n2 + (int64_t)(I.n0 + j0) * P.n1 + I.m0 + m;
           so = P.n1;
         } else {
           if (j0 + lane < I.nv) en = P.uexp[I.n0 + j0 + lane];
@@ -835,14 +835,14 @@ __global__ void __launch_bounds__(256) ex_assemble_kernel(const __grid_constant_
   }
 }
 
-// C = sum of the row splits, in ascending order.
+// C = (C with add, else 0) + the row splits, in ascending order.
 __global__ void ex_reduce_kernel(const double* __restrict__ partial, int nsplit, int n1, int n2,
-                                 double* __restrict__ C, int64_t ldc, int lower) {
+                                 double* __restrict__ C, int64_t ldc, int lower, int add) {
   const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (idx >= (int64_t)n1 * n2) return;
   const int i = (int)(idx % n1), j = (int)(idx / n1);
   if (lower && i / BM < j / BN * BN / BM) return;    // tile not computed
-  double s = 0.0;
+  double s = add ? C[i + (int64_t)j * ldc] : 0.0;
   for (int z = 0; z < nsplit; ++z) s += partial[(int64_t)z * n1 * n2 + idx];
   C[i + (int64_t)j * ldc] = s;
 }
@@ -897,7 +897,7 @@ int gram_tiles(int n1, int n2, int lower) {
 // Plan of a Gram product: rows in `slices` launches of `srows` rows, each in
 // `nsplit` splits of `rps` rows (the last launch may have fewer).
 struct GramPlan {
-  int64_t srows, slices, rps, nsplit, total;
+  int64_t srows, slices, rps, nsplit;
 };
 GramPlan gram_plan(int64_t M, int n1, int n2, int lower, bool same) {
   GramPlan g;
@@ -906,8 +906,10 @@ GramPlan gram_plan(int64_t M, int n1, int n2, int lower, bool same) {
   g.slices = (M + g.srows - 1) / g.srows;
   g.srows = ((M + g.slices - 1) / g.slices + KC - 1) / KC * KC;      // even slices
   g.slices = (M + g.srows - 1) / g.srows;
-  // splits of a slice: the count whose last wave of tiles is fullest, with the
-  // partial sums of all slices within 64 MB or eight n1 x n2 blocks each
+  // splits of a slice: the count whose last wave of tiles is fullest, up to eight
+  // or as many as write 64 MB of partial sums over all slices (each is written and
+  // read again).  The sums of one slice are added to C before the next one's: kept
+  // for all of them they would take 25 GB at 2.7 million rows and 3,000 columns.
   const int64_t tiles = std::max(1, gram_tiles(n1, n2, lower));
   const int64_t cap = std::max<int64_t>(8, ((int64_t)64 << 20) / ((int64_t)n1 * n2 * 8) / g.slices);
   const int nsm = sm_count();
@@ -922,8 +924,6 @@ GramPlan gram_plan(int64_t M, int n1, int n2, int lower, bool same) {
   }
   g.rps = ((g.srows + best - 1) / best + KC - 1) / KC * KC;
   g.nsplit = (g.srows + g.rps - 1) / g.rps;
-  const int64_t last = M - (g.slices - 1) * g.srows;
-  g.total = (g.slices - 1) * g.nsplit + (last + g.rps - 1) / g.rps;
   return g;
 }
 
@@ -1009,7 +1009,7 @@ cudaError_t ex_assemble_launch(const ExAssembleArgs& a, cudaStream_t s) {
 }
 
 static size_t gram_bytes(const GramPlan& g, int n1, int n2, bool same) {
-  return align256((size_t)(n1 + n2) * sizeof(int)) + align256((size_t)g.total * n1 * n2 * sizeof(double)) +
+  return align256((size_t)(n1 + n2) * sizeof(int)) + align256((size_t)g.nsplit * n1 * n2 * sizeof(double)) +
          (size_t)g.srows * (same ? pad2(n1) : pad2(n1) + pad2(n2)) * sizeof(uint64_t);
 }
 size_t ex_gram_work_bytes(int64_t M, int n1, int n2, int lower) {
@@ -1027,7 +1027,7 @@ cudaError_t ex_gram(const double* A, int64_t lda, const double* B, int64_t ldb, 
   int* aexp = (int*)work;
   int* bexp = same ? aexp : aexp + n1;
   double* partial = (double*)((char*)work + align256((size_t)(n1 + n2) * sizeof(int)));
-  uint64_t* WA = (uint64_t*)((char*)partial + align256((size_t)g.total * n1 * n2 * sizeof(double)));
+  uint64_t* WA = (uint64_t*)((char*)partial + align256((size_t)g.nsplit * n1 * n2 * sizeof(double)));
   uint64_t* WB = same ? WA : WA + (size_t)g.srows * pad2(n1);
   cudaError_t e = col_scale(A, lda, M, n1, 0, aexp, s);
   if (e != cudaSuccess) return e;
@@ -1050,7 +1050,6 @@ cudaError_t ex_gram(const double* A, int64_t lda, const double* B, int64_t ldb, 
     P.sb = pad2(same ? n1 : n2);
     P.M = rows;
     P.rps = g.rps;
-    P.z0 = i * g.nsplit;
     P.n1 = n1;
     P.n2 = n2;
     P.aexp = aexp;
@@ -1058,14 +1057,15 @@ cudaError_t ex_gram(const double* A, int64_t lda, const double* B, int64_t ldb, 
     P.lower = lower;
     P.ntile = gram_tiles(n1, n2, lower);
     P.C = partial;
-    P.nitems = P.ntile * ((rows + g.rps - 1) / g.rps);
+    const int64_t nsplit = (rows + g.rps - 1) / g.rps, tot = (int64_t)n1 * n2;
+    P.nitems = P.ntile * nsplit;
     P.watch = w;
     if ((e = launch<EX_GRAM>(P, s)) != cudaSuccess) return e;
+    note_launch();
+    ex_reduce_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(partial, (int)nsplit, n1, n2, C, ldc, lower, i > 0);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  const int64_t tot = (int64_t)n1 * n2;
-  note_launch();
-  ex_reduce_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(partial, (int)g.total, n1, n2, C, ldc, lower);
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 
 size_t ex_tall_work_bytes(int64_t M, int n1, int n2) {

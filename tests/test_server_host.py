@@ -71,3 +71,14 @@ def test_serving_requests_shape():
         assert 8 <= s.n_want <= max(8, s.ndofs // 8)
     t = W.poisson_arrivals(5, 4000, rate=2.0)
     assert np.all(np.diff(t) > 0) and abs(len(t) / t[-1] - 2.0) < 0.15
+
+
+def test_estimate_of_a_large_binary64_request(lib):
+    """The scratch of the overlap's partial sums does not grow with the unknowns:
+    20^3 cells, p = 7, 3,000 states hold the cell matrices and their digit words,
+    the block and a second one at most, the dense cell blocks of 200 columns, and
+    under 8 GB besides."""
+    cells, ne, M, n = 20 ** 3, 512, 140 ** 3, 3000
+    held = 2 * cells * ne * ne * 8 + 2 * M * n * 8 + cells * ne * 200 * 8 + 3 * M * 200 * 8
+    est = Server.estimate(((20,) * 3, (40.0,) * 3, 7, True), n, prec="fp64")
+    assert held <= est + 2 * M * 200 * 8 and est <= held + (8 << 30)
