@@ -198,11 +198,32 @@ chfsi_status chfsi_set_cell_gather(chfsi_ctx* ctx, int mode);
  * blocks of up to 12 columns (15 for p >= 7) of meshes that fill the GPU and
  * when there are no cell matrices (chfsi_set_potential_qp_device), else the
  * cell matrices.  The matrix-free form needs 2 <= p <= 8 and quad_points =
- * p + 2 (CHFSI_ERR_ARG otherwise).  Both give the same operator to rounding.
- * chfsi_fp64_operator returns 1 when the matrix-free form is selected or, by
- * default, available, else 0. */
+ * p + 2 (CHFSI_ERR_ARG otherwise).  Both give the same operator to rounding;
+ * with -1 the rounding of a column so depends on the width of the block it is
+ * in (the last block of a call may be a narrow one).  chfsi_fp64_operator
+ * returns 1 when the matrix-free form is selected or, by default, available,
+ * else 0: with -1 it does not name the one that a block of a given width takes. */
 chfsi_status chfsi_set_fp64_operator(chfsi_ctx* ctx, int op);
 int          chfsi_fp64_operator(const chfsi_ctx* ctx);
+
+/* Arithmetic of the binary64 products C = A B with the stored cell matrices, of
+ * the overlaps X^T Y and of the rotations X U (CholGS, Rayleigh-Ritz):
+ * 0 (default) = exact products of 8-bit digit slices on the tensor cores.  The
+ * entries of a vector of the contraction (the values of a column of the block at
+ * a cell's nodes and a row of that cell's matrix; two columns; a row of X, each
+ * entry relative to the largest of its column, and a column of U) share one
+ * power-of-two scale, set by the largest: one operand enters as a 54-bit, the
+ * other as a 62-bit fixed-point number, and their products are exact up to the
+ * rounding of sums of 960 terms.  The error of K terms is normwise, |dC_ij| <=
+ * K 2^-53 max_k |A_ik| max_k |B_kj| beyond the rounding of the sums: norms,
+ * eigenvalues and residuals are as accurate as with 1 or more so, but an entry
+ * 2^k below the largest of its vector keeps about 54 - k significant bits, and
+ * none beyond.
+ * 1 = binary64 FMAs on the ALUs, each operand with its own 53 bits, |dC_ij| <=
+ * K 2^-53 sum_k |A_ik| |B_kj|: for results whose small entries count, at 5 to 25
+ * times the time.  0 falls back to 1 when its scratch does not fit in memory.
+ * CHFSI_ERR_ARG for other values. */
+chfsi_status chfsi_set_fp64_products(chfsi_ctx* ctx, int mode);
 
 /* Autotuner of the filter's blocking: times a degree-2 filter on a scratch
  * copy of X (M x n, device; X itself is not modified) for every candidate
@@ -283,7 +304,8 @@ chfsi_status chfsi_filter(chfsi_ctx* ctx, void* X, int64_t ldx, int ncol, int de
 
 /* CholGS (Algorithm CholGS): S = X^T X, S = L L^T, X <- X L^{-T}, in place on
  * X (M x n).  Returns CHFSI_ERR_NOT_SPD and leaves X unchanged when the
- * Cholesky factorisation fails (cuSOLVER potrf + trtri, binary64). */
+ * Cholesky factorisation (binary64, the library's own) meets a pivot that is
+ * not positive. */
 chfsi_status chfsi_cholgs(chfsi_ctx* ctx, void* X, int64_t ldx, int n, chfsi_precision prec);
 
 /* Rayleigh-Ritz (Sec. 3.5): H^ = X^T H~ X, H^ Q = Q D (ascending, binary64

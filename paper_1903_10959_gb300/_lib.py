@@ -153,6 +153,7 @@ _SIGS = {
     "chfsi_scf": (C.c_int, [_vp, C.POINTER(ScfParams), _vp, _i64, _dp, _dp, _dp, _dp, _dp,
                             C.POINTER(C.c_int)]),
     "chfsi_set_fp64_operator": (C.c_int, [_vp, C.c_int]),
+    "chfsi_set_fp64_products": (C.c_int, [_vp, C.c_int]),
     "chfsi_set_cell_gather": (C.c_int, [_vp, C.c_int]),
     "chfsi_fp64_operator": (C.c_int, [_vp]),
     "chfsi_debug_withhold_arrival": (C.c_int, [_vp, C.c_int]),
@@ -447,8 +448,17 @@ class Context:
         code = {"default": -1, "cells": 0, "matrix-free": 1}[op]
         self._check(self._lib.chfsi_set_fp64_operator(self._h, code))
 
+    def set_fp64_products(self, mode):
+        """Binary64 products: "digits" (exact digit slices on the tensor cores, a
+        normwise error bound) or "alu" (FMAs, a componentwise one)
+        (chfsi_set_fp64_products)."""
+        self._check(self._lib.chfsi_set_fp64_products(self._h, {"digits": 0, "alu": 1}[mode]))
+
     @property
     def fp64_operator(self):
+        """"matrix-free" when that form is selected or, by default, available, else
+        "cells"; by default wide blocks take the stored cell matrices all the same
+        (chfsi_set_fp64_operator)."""
         return ("cells", "matrix-free")[self._lib.chfsi_fp64_operator(self._h)]
 
     def debug_withhold_arrival(self, on):

@@ -298,7 +298,7 @@ uint64_t capture_id(cudaStream_t s) {
 // cell blocks fit in memory.  Otherwise the colour-ordered ALU kernels run.
 bool ensure_ex(chfsi_ctx* ctx, int ncol, int64_t* ldr) {
   const HostMesh& m = ctx->mesh;
-  if (!ctx->d_Ht || ctx->ex_off || stays_matrix_free(ctx, ncol)) return false;
+  if (!ctx->d_Ht || ctx->fp64_alu || ctx->ex_off || stays_matrix_free(ctx, ncol)) return false;
   *ldr = (ncol + 1) & ~1;
   if (!ctx->ex_ready) {
     ExCellData& d = ctx->ex;
@@ -694,7 +694,7 @@ chfsi_status gram_impl(chfsi_ctx* ctx, chfsi_precision prec, const void* A, int6
   chfsi_status st;
   if (prec == CHFSI_FP64) {
     size_t want = ex_gram_work_bytes(m.ndofs, n1, n2, lower);
-    if ((st = grow(ctx, ctx->part, want)) == CHFSI_OK) {
+    if (!ctx->fp64_alu && (st = grow(ctx, ctx->part, want)) == CHFSI_OK) {
       ctx->ex_used = true;
       CK(ex_gram((const double*)A, lda, (const double*)Bm, ldb, m.ndofs, n1, n2, C, ldc, lower, ctx->part.ptr,
                  ctx->part.bytes, ctx->watch, ctx->stream));
@@ -719,7 +719,7 @@ chfsi_status tall64_impl(chfsi_ctx* ctx, const double* X, int64_t ldx, int n1, i
                          double* C, int64_t ldc, int upper, int trans) {
   const HostMesh& m = ctx->mesh;
   const std::string err = ctx->err;
-  if (grow(ctx, ctx->work, ex_tall_work_bytes(m.ndofs, n1, n2)) == CHFSI_OK) {
+  if (!ctx->fp64_alu && grow(ctx, ctx->work, ex_tall_work_bytes(m.ndofs, n1, n2)) == CHFSI_OK) {
     ctx->ex_used = true;
     CK(ex_tall(X, ldx, U, ldu, m.ndofs, n1, n2, C, ldc, upper, trans, ctx->work.ptr, ctx->watch, ctx->stream));
     return CHFSI_OK;
@@ -736,7 +736,7 @@ chfsi_status rotate_impl(chfsi_ctx* ctx, chfsi_precision prec, void* X, int64_t 
   const HostMesh& m = ctx->mesh;
   const size_t es = esize(prec);
   chfsi_status st;
-  if (prec == CHFSI_FP64) {
+  if (prec == CHFSI_FP64 && !ctx->fp64_alu) {
     const std::string err = ctx->err;
     if (grow(ctx, ctx->work, ex_tall_work_bytes(m.ndofs, n, n)) == CHFSI_OK) {
       ctx->ex_used = true;
@@ -1323,6 +1323,13 @@ chfsi_status chfsi_set_fp64_operator(chfsi_ctx* ctx, int op) {
   if (op == 1 && !mf_supported(ctx->mesh.p, ctx->mesh.q))
     return fail(ctx, CHFSI_ERR_ARG, "the matrix-free apply needs 2 <= p <= 8 and p + 2 Gauss points");
   ctx->fp64_op = op;
+  return CHFSI_OK;
+}
+
+chfsi_status chfsi_set_fp64_products(chfsi_ctx* ctx, int mode) {
+  CHECK_CTX();
+  if (mode < 0 || mode > 1) return fail(ctx, CHFSI_ERR_ARG, "products: 0 digit slices, 1 ALUs");
+  ctx->fp64_alu = mode == 1;
   return CHFSI_OK;
 }
 

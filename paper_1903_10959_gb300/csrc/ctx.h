@@ -39,6 +39,7 @@ struct chfsi_ctx {
   std::vector<double> wellh;       // host side of the upload
   std::vector<double> fac;
   int fp64_op = -1;                // binary64 cell operator: 0 cell matrices, 1 matrix-free, -1 auto
+  bool fp64_alu = false;           // binary64 products on the ALUs instead of as digit slices
   chfsi::TcCellData tc;                   // tensor-core copies (mixed precisions)
   // digit slices of the binary64 cell matrices (packed on first binary64 use;
   // ex_off: they did not fit, the binary64 operator stays on the ALUs until

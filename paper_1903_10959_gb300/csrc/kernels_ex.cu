@@ -24,6 +24,11 @@
 // times the low eigenvalues), so their sums keep four more bits, 2^(45 - 8 g):
 // the scale of a row of the cell matrix is raised where its first digits would
 // add up to more than 2^11.
+// The error is normwise: an entry 2^k below the largest of its vector enters with
+// 54 - k (M) or 62 - k (N) bits, so K terms are off by K 2^-53 max|a| max|b| at most
+// besides the rounding of the sums, where binary64 FMAs are off by K 2^-53 sum |a||b|:
+// less in the norm, more in an entry that only small values make up
+// (chfsi_set_fp64_products chooses).
 //
 //  ex_kernel<CELL>  R_e = H~_e Y_e for every cell (M: columns of Y, N: rows of
 //                   the cell matrix)
