@@ -295,6 +295,11 @@ chfsi_status chfsi_apply_noalloc(chfsi_ctx* ctx, const double* X, int64_t ldx, d
  * tests of the error path only.  Synchronises the stream. */
 chfsi_status chfsi_debug_withhold_arrival(chfsi_ctx* ctx, int on);
 
+/* Test hook of the out-of-memory paths (no counterpart in the paper; off by
+ * default): while bytes > 0, device allocations of this context that would bring
+ * chfsi_device_bytes above it fail as they do on a full card.  Host only. */
+chfsi_status chfsi_debug_memory_limit(chfsi_ctx* ctx, int64_t bytes);
+
 /* Degree-m Chebyshev filter (Eq. chebFilter) in the scaled form of Zhou &
  * Saad, in place on X (M x ncol): X <- T_m((H~ - c)/e) X / T_m((a0 - c)/e),
  * c = (a + b)/2, e = (b - a)/2; [a, b] is the damped interval, a0 < a the

@@ -157,6 +157,7 @@ _SIGS = {
     "chfsi_set_cell_gather": (C.c_int, [_vp, C.c_int]),
     "chfsi_fp64_operator": (C.c_int, [_vp]),
     "chfsi_debug_withhold_arrival": (C.c_int, [_vp, C.c_int]),
+    "chfsi_debug_memory_limit": (C.c_int, [_vp, _i64]),
     "chfsi_partition_sizes": (C.c_int, [C.POINTER(MeshDesc), C.c_int, C.c_int,
                                         C.POINTER(PartitionInfo)]),
     "chfsi_partition_fill": (C.c_int, [C.POINTER(MeshDesc), C.c_int, C.c_int, _vp, _vp, _vp, _vp,
@@ -464,6 +465,10 @@ class Context:
     def debug_withhold_arrival(self, on):
         """Test hook of the bounded device waits (chfsi_debug_withhold_arrival)."""
         self._check(self._lib.chfsi_debug_withhold_arrival(self._h, int(bool(on))))
+
+    def debug_memory_limit(self, nbytes):
+        """Test hook of the out-of-memory paths (chfsi_debug_memory_limit); 0 lifts it."""
+        self._check(self._lib.chfsi_debug_memory_limit(self._h, int(nbytes)))
 
     def filter(self, X, degree, a, b, a0, prec="fp64"):
         pr = _prec(prec)

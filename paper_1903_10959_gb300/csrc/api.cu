@@ -93,8 +93,10 @@ chfsi_status fail(chfsi_ctx* c, chfsi_status st, const std::string& msg) {
   } while (0)
 
 cudaError_t dalloc(chfsi_ctx* ctx, void** p, size_t bytes) {
-  cudaError_t e = cudaMalloc(p, std::max<size_t>(bytes, 16));
-  if (e == cudaSuccess) ctx->dev_bytes += (int64_t)std::max<size_t>(bytes, 16);
+  const int64_t b = (int64_t)std::max<size_t>(bytes, 16);
+  if (ctx->mem_limit > 0 && ctx->dev_bytes + b > ctx->mem_limit) return cudaErrorMemoryAllocation;
+  cudaError_t e = cudaMalloc(p, (size_t)b);
+  if (e == cudaSuccess) ctx->dev_bytes += b;
   return e;
 }
 void dfree(chfsi_ctx* ctx, void* p, size_t bytes) {
@@ -117,21 +119,27 @@ void release(chfsi_ctx* ctx, T*& p, size_t bytes) {
   p = nullptr;
 }
 
-chfsi_status grow(chfsi_ctx* ctx, DevBuf& b, size_t bytes) {
-  if (b.bytes >= bytes) return CHFSI_OK;
+// Scratch of at least `bytes`, for a form that another one can stand in for: false
+// when it does not fit.
+bool grow_optional(chfsi_ctx* ctx, DevBuf& b, size_t bytes) {
+  if (b.bytes >= bytes) return true;
   if (b.ptr) {
     cudaStreamSynchronize(ctx->stream);
     dfree(ctx, b.ptr, b.bytes);
     b.ptr = nullptr;
     b.bytes = 0;
   }
-  cudaError_t e = dalloc(ctx, &b.ptr, bytes);
-  if (e != cudaSuccess) {
+  if (dalloc(ctx, &b.ptr, bytes) != cudaSuccess) {
     cudaGetLastError();
-    return fail(ctx, CHFSI_ERR_OOM, "device allocation of " + std::to_string(bytes) + " bytes failed");
+    b.ptr = nullptr;
+    return false;
   }
   b.bytes = bytes;
-  return CHFSI_OK;
+  return true;
+}
+chfsi_status grow(chfsi_ctx* ctx, DevBuf& b, size_t bytes) {
+  if (grow_optional(ctx, b, bytes)) return CHFSI_OK;
+  return fail(ctx, CHFSI_ERR_OOM, "device allocation of " + std::to_string(bytes) + " bytes failed");
 }
 
 bool is_mixed(chfsi_precision p) {
@@ -694,7 +702,7 @@ chfsi_status gram_impl(chfsi_ctx* ctx, chfsi_precision prec, const void* A, int6
   chfsi_status st;
   if (prec == CHFSI_FP64) {
     size_t want = ex_gram_work_bytes(m.ndofs, n1, n2, lower);
-    if (!ctx->fp64_alu && (st = grow(ctx, ctx->part, want)) == CHFSI_OK) {
+    if (!ctx->fp64_alu && grow_optional(ctx, ctx->part, want)) {
       ctx->ex_used = true;
       CK(ex_gram((const double*)A, lda, (const double*)Bm, ldb, m.ndofs, n1, n2, C, ldc, lower, ctx->part.ptr,
                  ctx->part.bytes, ctx->watch, ctx->stream));
@@ -718,13 +726,11 @@ chfsi_status gram_impl(chfsi_ctx* ctx, chfsi_precision prec, const void* A, int6
 chfsi_status tall64_impl(chfsi_ctx* ctx, const double* X, int64_t ldx, int n1, int n2, const double* U, int64_t ldu,
                          double* C, int64_t ldc, int upper, int trans) {
   const HostMesh& m = ctx->mesh;
-  const std::string err = ctx->err;
-  if (!ctx->fp64_alu && grow(ctx, ctx->work, ex_tall_work_bytes(m.ndofs, n1, n2)) == CHFSI_OK) {
+  if (!ctx->fp64_alu && grow_optional(ctx, ctx->work, ex_tall_work_bytes(m.ndofs, n1, n2))) {
     ctx->ex_used = true;
     CK(ex_tall(X, ldx, U, ldu, m.ndofs, n1, n2, C, ldc, upper, trans, ctx->work.ptr, ctx->watch, ctx->stream));
     return CHFSI_OK;
   }
-  ctx->err = err;
   CK(launch_tallgemm_fp64(X, ldx, U, ldu, m.ndofs, n1, n2, C, ldc, upper, trans, ctx->stream));
   return CHFSI_OK;
 }
@@ -736,15 +742,11 @@ chfsi_status rotate_impl(chfsi_ctx* ctx, chfsi_precision prec, void* X, int64_t 
   const HostMesh& m = ctx->mesh;
   const size_t es = esize(prec);
   chfsi_status st;
-  if (prec == CHFSI_FP64 && !ctx->fp64_alu) {
-    const std::string err = ctx->err;
-    if (grow(ctx, ctx->work, ex_tall_work_bytes(m.ndofs, n, n)) == CHFSI_OK) {
-      ctx->ex_used = true;
-      CK(ex_tall((const double*)X, ldx, U, n, m.ndofs, n, n, (double*)X, ldx, upper, trans, ctx->work.ptr, ctx->watch,
-                 ctx->stream));
-      return CHFSI_OK;
-    }
-    ctx->err = err;
+  if (prec == CHFSI_FP64 && !ctx->fp64_alu && grow_optional(ctx, ctx->work, ex_tall_work_bytes(m.ndofs, n, n))) {
+    ctx->ex_used = true;
+    CK(ex_tall((const double*)X, ldx, U, n, m.ndofs, n, n, (double*)X, ldx, upper, trans, ctx->work.ptr, ctx->watch,
+               ctx->stream));
+    return CHFSI_OK;
   }
   if ((st = grow(ctx, ctx->rot, (size_t)m.ndofs * n * es)) != CHFSI_OK) return st;
   if (prec == CHFSI_FP64) {
@@ -1487,6 +1489,12 @@ chfsi_status chfsi_debug_withhold_arrival(chfsi_ctx* ctx, int on) {
   if (ctx->latched != CHFSI_OK) return ctx->latched;
   ctx->watch.withhold = on != 0;
   CK(tc_set_withhold(on, ctx->stream));
+  return CHFSI_OK;
+}
+
+chfsi_status chfsi_debug_memory_limit(chfsi_ctx* ctx, int64_t bytes) {
+  if (!ctx || bytes < 0) return CHFSI_ERR_ARG;
+  ctx->mem_limit = bytes;
   return CHFSI_OK;
 }
 

@@ -27,6 +27,7 @@ struct chfsi_ctx {
   int cell_tile = 64;              // columns per CTA of the tensor-core cell kernel
   int cell_gather = 2;             // BF16x3 cell kernel: 2 decoupled rings (default), 0 one ring, 1 async gather, 3 rings with 4 gather pairs
   int64_t dev_bytes = 0;
+  int64_t mem_limit = 0;           // test hook: dev_bytes that allocations may not exceed (0: none)
   // resident device data
   double* d_Ht = nullptr;          // binary64 cell matrices
   double* d_wv = nullptr;          // matrix-free apply: w jac V at the Gauss points per cell
