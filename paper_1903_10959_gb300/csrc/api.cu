@@ -92,12 +92,19 @@ chfsi_status fail(chfsi_ctx* c, chfsi_status st, const std::string& msg) {
     if (late_ != CHFSI_OK) return late_;                                                  \
   } while (0)
 
-cudaError_t dalloc(chfsi_ctx* ctx, void** p, size_t bytes) {
+// Device memory for a form that another one can stand in for.
+cudaError_t dalloc_optional(chfsi_ctx* ctx, void** p, size_t bytes) {
   const int64_t b = (int64_t)std::max<size_t>(bytes, 16);
-  if (ctx->mem_limit > 0 && ctx->dev_bytes + b > ctx->mem_limit) return cudaErrorMemoryAllocation;
-  cudaError_t e = cudaMalloc(p, (size_t)b);
+  cudaError_t e = cudaErrorMemoryAllocation;
+  if (ctx->mem_limit <= 0 || ctx->dev_bytes + b <= ctx->mem_limit) e = cudaMalloc(p, (size_t)b);
   if (e == cudaSuccess) ctx->dev_bytes += b;
+  else *p = nullptr;
   return e;
+}
+// Device memory that the call cannot do without: what only makes products faster
+// gives way to it.
+cudaError_t dalloc(chfsi_ctx* ctx, void** p, size_t bytes) {
+  return with_room(ctx, [&] { return dalloc_optional(ctx, p, bytes); });
 }
 void dfree(chfsi_ctx* ctx, void* p, size_t bytes) {
   if (p) {
@@ -119,26 +126,30 @@ void release(chfsi_ctx* ctx, T*& p, size_t bytes) {
   p = nullptr;
 }
 
-// Scratch of at least `bytes`, for a form that another one can stand in for: false
-// when it does not fit.
-bool grow_optional(chfsi_ctx* ctx, DevBuf& b, size_t bytes) {
+void drop(chfsi_ctx* ctx, DevBuf& b) {
+  dfree(ctx, b.ptr, b.bytes);
+  b.ptr = nullptr;
+  b.bytes = 0;
+}
+bool grow_by(chfsi_ctx* ctx, DevBuf& b, size_t bytes, cudaError_t (*alloc)(chfsi_ctx*, void**, size_t)) {
   if (b.bytes >= bytes) return true;
   if (b.ptr) {
     cudaStreamSynchronize(ctx->stream);
-    dfree(ctx, b.ptr, b.bytes);
-    b.ptr = nullptr;
-    b.bytes = 0;
+    drop(ctx, b);
   }
-  if (dalloc(ctx, &b.ptr, bytes) != cudaSuccess) {
+  if (alloc(ctx, &b.ptr, bytes) != cudaSuccess) {
     cudaGetLastError();
-    b.ptr = nullptr;
     return false;
   }
   b.bytes = bytes;
   return true;
 }
+// Scratch of at least `bytes`, for a form that another one can stand in for: false
+// when it does not fit.
+bool grow_optional(chfsi_ctx* ctx, DevBuf& b, size_t bytes) { return grow_by(ctx, b, bytes, dalloc_optional); }
+// Scratch that the call cannot do without.
 chfsi_status grow(chfsi_ctx* ctx, DevBuf& b, size_t bytes) {
-  if (grow_optional(ctx, b, bytes)) return CHFSI_OK;
+  if (grow_by(ctx, b, bytes, dalloc)) return CHFSI_OK;
   return fail(ctx, CHFSI_ERR_OOM, "device allocation of " + std::to_string(bytes) + " bytes failed");
 }
 
@@ -158,11 +169,10 @@ constexpr bool kMatrixFreeDefault = true;
 void release_scratch(chfsi_ctx* ctx) {
   cudaStreamSynchronize(ctx->stream);
   for (DevBuf* b : {&ctx->T1, &ctx->T2, &ctx->Wb, &ctx->NLb, &ctx->Zb, &ctx->Rb, &ctx->rot, &ctx->cmaxb, &ctx->pjb, &ctx->tinv,
-                    &ctx->exb}) {
-    dfree(ctx, b->ptr, b->bytes);
-    b->ptr = nullptr;
-    b->bytes = 0;
-  }
+                    &ctx->exb})
+    drop(ctx, *b);
+  ctx->ex_off = false;
+  ctx->ex_too_wide = INT_MAX;
 }
 
 bool valid_prec(chfsi_precision p) { return p == CHFSI_FP64 || is_mixed(p); }
@@ -201,6 +211,7 @@ void free_device_data(chfsi_ctx* ctx, bool keep = false) {
   ctx->ex_ready = false;
   ctx->ex_capture = 0;
   ctx->ex_off = false;
+  ctx->ex_too_wide = INT_MAX;
   ctx->kpack_valid = false;   // the mixed Bloch packs hold the old cell matrices
   release(ctx, ctx->d_site_ptr, ctx->hproj.site_ptr.size() * 8);
   release(ctx, ctx->d_site_dof, ctx->hproj.site_dof.size() * 4);
@@ -227,7 +238,7 @@ chfsi_status ensure_tc_data(chfsi_ctx* ctx, chfsi_precision prec) {
   const bool bf16 = prec == CHFSI_MIXED_BF16X3;
   const bool f16 = prec == CHFSI_MIXED_F16X2;
   if (f16 && !ctx->tc.f16) {
-    cudaError_t pe = tc_pack_f16_from_device(ctx->tc, ctx->d_Ht, ctx->stream, &ctx->dev_bytes);
+    cudaError_t pe = with_room(ctx, [&] { return tc_pack_f16_from_device(ctx->tc, ctx->d_Ht, ctx->stream, &ctx->dev_bytes); });
     if (pe != cudaSuccess) {
       cudaGetLastError();
       return fail(ctx, pe == cudaErrorMemoryAllocation ? CHFSI_ERR_OOM : CHFSI_ERR_CUDA,
@@ -235,7 +246,7 @@ chfsi_status ensure_tc_data(chfsi_ctx* ctx, chfsi_precision prec) {
     }
   }
   if (bf16 && !ctx->tc.bf_ready) {
-    cudaError_t pe = tc_pack_bf16_from_device(ctx->tc, ctx->d_Ht, ctx->stream, &ctx->dev_bytes);
+    cudaError_t pe = with_room(ctx, [&] { return tc_pack_bf16_from_device(ctx->tc, ctx->d_Ht, ctx->stream, &ctx->dev_bytes); });
     if (pe != cudaSuccess) {
       cudaGetLastError();
       return fail(ctx, pe == cudaErrorMemoryAllocation ? CHFSI_ERR_OOM : CHFSI_ERR_CUDA,
@@ -243,7 +254,7 @@ chfsi_status ensure_tc_data(chfsi_ctx* ctx, chfsi_precision prec) {
     }
   }
   if (!bf16 && !f16 && !ctx->tc.hi) {
-    cudaError_t pe = tc_pack_from_device(ctx->tc, ctx->d_Ht, ctx->stream, &ctx->dev_bytes);
+    cudaError_t pe = with_room(ctx, [&] { return tc_pack_from_device(ctx->tc, ctx->d_Ht, ctx->stream, &ctx->dev_bytes); });
     if (pe != cudaSuccess) {
       cudaGetLastError();
       return fail(ctx, pe == cudaErrorMemoryAllocation ? CHFSI_ERR_OOM : CHFSI_ERR_CUDA,
@@ -258,12 +269,16 @@ chfsi_status ensure_tc_data(chfsi_ctx* ctx, chfsi_precision prec) {
   if (nl_in_cells && !ctx->tc.nl) {
     NlCells nc;
     build_nl_cells(m, ctx->hproj, nc);
-    cudaError_t pe = tc_pack_nl(ctx->tc, nc.chunk_off.data(), m.ncells, nc.zrow.data(), nc.nz_pos.data(),
-                                nc.nz_val.data(), (int64_t)nc.nz_val.size(), ctx->stream, &ctx->dev_bytes);
+    cudaError_t pe = with_room(ctx, [&] {
+      return tc_pack_nl(ctx->tc, nc.chunk_off.data(), m.ncells, nc.zrow.data(), nc.nz_pos.data(), nc.nz_val.data(),
+                        (int64_t)nc.nz_val.size(), ctx->stream, &ctx->dev_bytes);
+    });
     if (pe == cudaSuccess)
-      pe = tc_pack_proj(ctx->tc, m.ncells, ctx->hproj.nsite, nc.np.data(), nc.poff.data(), nc.prow.data(),
-                        nc.red_ptr.data(), nc.red_row.data(), nc.pz_pos.data(), nc.pz_val.data(),
-                        (int64_t)nc.pz_val.size(), ctx->stream, &ctx->dev_bytes);
+      pe = with_room(ctx, [&] {
+        return tc_pack_proj(ctx->tc, m.ncells, ctx->hproj.nsite, nc.np.data(), nc.poff.data(), nc.prow.data(),
+                            nc.red_ptr.data(), nc.red_row.data(), nc.pz_pos.data(), nc.pz_val.data(),
+                            (int64_t)nc.pz_val.size(), ctx->stream, &ctx->dev_bytes);
+      });
     if (pe == cudaErrorNotSupported) {
       cudaGetLastError();   // too many sites on one cell's rows: the projection stays by site
     } else if (pe != cudaSuccess) {
@@ -304,16 +319,19 @@ uint64_t capture_id(cudaStream_t s) {
 // (kernels_ex.cu): the cell matrices are resident, the block is not one for the
 // matrix-free kernel, and the words of the matrices, of the block and its dense
 // cell blocks fit in memory.  Otherwise the colour-ordered ALU kernels run.
+// It takes its memory after the call's other buffers; a width whose scratch does not
+// fit stays on the ALUs until the next build or chfsi_autotune, and so does every
+// width once the words had to give way to another buffer.
 bool ensure_ex(chfsi_ctx* ctx, int ncol, int64_t* ldr) {
   const HostMesh& m = ctx->mesh;
-  if (!ctx->d_Ht || ctx->fp64_alu || ctx->ex_off || stays_matrix_free(ctx, ncol)) return false;
+  if (!ctx->d_Ht || ctx->fp64_alu || ctx->ex_off || ncol >= ctx->ex_too_wide || stays_matrix_free(ctx, ncol)) return false;
   *ldr = (ncol + 1) & ~1;
   if (!ctx->ex_ready) {
     ExCellData& d = ctx->ex;
     if (!d.hsum) {
       ex_cell_bytes(m.ncells, m.ne, &d.word_bytes, &d.exp_bytes);
-      if (dalloc(ctx, (void**)&d.words, d.word_bytes) != cudaSuccess) d.words = nullptr;
-      if (d.words && dalloc(ctx, (void**)&d.hsum, d.exp_bytes) != cudaSuccess) d.hsum = nullptr;
+      if (dalloc_optional(ctx, (void**)&d.words, d.word_bytes) == cudaSuccess)
+        dalloc_optional(ctx, (void**)&d.hsum, d.exp_bytes);
     }
     // in a stream capture the packing is only recorded, once per capture: calls
     // outside the graph still have to pack
@@ -331,15 +349,16 @@ bool ensure_ex(chfsi_ctx* ctx, int ncol, int64_t* ldr) {
       ctx->ex_ready = !capture;
     }
   }
-  const std::string err = ctx->err;
   // the partial sums of the narrow blocks that follow on the matrix-free kernel
   // are allocated with the first block of any width, as one call always did
   const int nw = std::min(ncol, narrow_columns(ctx));
-  if ((stays_matrix_free(ctx, nw) && grow(ctx, ctx->Wb, (size_t)m.ndofs * nw * sizeof(double)) != CHFSI_OK) ||
-      grow(ctx, ctx->exb, ex_cell_work_bytes(m.ncells, m.ne, ncol)) != CHFSI_OK ||
-      grow(ctx, ctx->Rb, (size_t)m.ncells * m.ne * *ldr * sizeof(double)) != CHFSI_OK) {
-    ctx->err = err;   // no room: the ALU kernels until the next build
-    ctx->ex_off = true;
+  if ((stays_matrix_free(ctx, nw) && !grow_optional(ctx, ctx->Wb, (size_t)m.ndofs * nw * sizeof(double))) ||
+      !grow_optional(ctx, ctx->exb, ex_cell_work_bytes(m.ncells, m.ne, ncol)) ||
+      !grow_optional(ctx, ctx->Rb, (size_t)m.ncells * m.ne * *ldr * sizeof(double))) {
+    ctx->ex_too_wide = ncol;
+    cudaStreamSynchronize(ctx->stream);
+    drop(ctx, ctx->exb);
+    drop(ctx, ctx->Rb);
     return false;
   }
   return true;
@@ -355,14 +374,14 @@ chfsi_status apply_step(chfsi_ctx* ctx, chfsi_precision prec, const void* Yin, i
   const int B = std::max(ncol, 1);
   const size_t es = esize(prec);
   chfsi_status st;
-  int64_t ldr = 0;
-  const bool ex = prec == CHFSI_FP64 && ncol > 0 && ensure_ex(ctx, ncol, &ldr);
-  if (prec == CHFSI_FP64 && !ex && (st = grow(ctx, ctx->Wb, (size_t)m.ndofs * B * es)) != CHFSI_OK) return st;
   const bool nl = ctx->hproj.nsite > 0;
   if (nl) {
     if (prec == CHFSI_FP64 && (st = grow(ctx, ctx->NLb, (size_t)m.ndofs * B * es)) != CHFSI_OK) return st;
     if ((st = grow(ctx, ctx->Zb, (size_t)4 * ctx->hproj.nsite * B * es)) != CHFSI_OK) return st;
   }
+  int64_t ldr = 0;
+  const bool ex = prec == CHFSI_FP64 && ncol > 0 && ensure_ex(ctx, ncol, &ldr);
+  if (prec == CHFSI_FP64 && !ex && (st = grow(ctx, ctx->Wb, (size_t)m.ndofs * B * es)) != CHFSI_OK) return st;
   const int ncolour = (int)m.colour_offsets.size() - 1;
   if (prec == CHFSI_FP64) {
     if (nl) {
@@ -446,8 +465,15 @@ chfsi_status apply_step(chfsi_ctx* ctx, chfsi_precision prec, const void* Yin, i
                        (const float*)Yin, ld_in, ncol, (float*)ctx->Zb.ptr, ctx->stream));
     }
   }
+  if (f16 && !cmax_in) {   // column maxima of the input block (the scales of its fp16 split)
+    if ((st = grow(ctx, ctx->cmaxb, (size_t)3 * ncol * sizeof(uint32_t))) != CHFSI_OK) return st;
+    uint32_t* cm = (uint32_t*)ctx->cmaxb.ptr + 2 * (size_t)ncol;
+    CK(tc_colmax_launch((const float*)Yin, ld_in, m.ndofs, ncol, cm, ctx->stream));
+    cmax_in = cm;
+  }
   // owner-computes: dense cell blocks R_e (one launch over all cells), then the
-  // fixed-order assembly fused with the Chebyshev update
+  // fixed-order assembly fused with the Chebyshev update.  R is the last buffer
+  // of the step to grow: it gives way to the others.
   const int64_t ldr4 = (ncol + 3) & ~3;   // 16-byte rows of R
   if ((st = grow(ctx, ctx->Rb, (size_t)m.ncells * m.ne * ldr4 * sizeof(float))) != CHFSI_OK) return st;
   TcApplyArgs ra{};
@@ -464,12 +490,6 @@ chfsi_status apply_step(chfsi_ctx* ctx, chfsi_precision prec, const void* Yin, i
   if (nl_in_cells) {
     ra.Z = (const float*)ctx->Zb.ptr;
     ra.ldz = ncol;
-  }
-  if (f16 && !cmax_in) {   // column maxima of the input block (the scales of its fp16 split)
-    if ((st = grow(ctx, ctx->cmaxb, (size_t)3 * ncol * sizeof(uint32_t))) != CHFSI_OK) return st;
-    uint32_t* cm = (uint32_t*)ctx->cmaxb.ptr + 2 * (size_t)ncol;
-    CK(tc_colmax_launch((const float*)Yin, ld_in, m.ndofs, ncol, cm, ctx->stream));
-    cmax_in = cm;
   }
   {
     KTimer kt(ctx, 0);
@@ -872,7 +892,6 @@ chfsi_status residual_impl(chfsi_ctx* ctx, const void* X, int64_t ldx, int n, ch
   // binary64 copies of the block and of H~ x (residual check always in binary64)
   if ((st = grow(ctx, ctx->rot, (size_t)m.ndofs * B * 8 * 2)) != CHFSI_OK) return st;
   if ((st = grow(ctx, ctx->lam, (size_t)n * 8 * 4 + 64)) != CHFSI_OK) return st;
-  if ((st = grow(ctx, ctx->part, (size_t)3 * n * 8 * 512)) != CHFSI_OK) return st;
   double* X64 = (double*)ctx->rot.ptr;
   double* Y64 = X64 + (size_t)m.ndofs * B;
   double* dl = (double*)ctx->lam.ptr;
@@ -885,6 +904,7 @@ chfsi_status residual_impl(chfsi_ctx* ctx, const void* X, int64_t ldx, int n, ch
                         prec == CHFSI_FP64, 1, ctx->stream));
     if ((st = apply_step(ctx, CHFSI_FP64, X64, nb, Y64, nb, nullptr, 0, nb, 1.0, 0.0, 0.0)) != CHFSI_OK)
       return st;
+    if ((st = grow(ctx, ctx->part, (size_t)3 * n * 8 * 512)) != CHFSI_OK) return st;
     std::vector<double> h(3 * (size_t)nb);
     if (rayleigh) {
       CK(launch_resid_norms(Y64, nb, X64, nb, m.ndofs, nb, nullptr, nullptr, out,
@@ -994,6 +1014,27 @@ cudaError_t noalloc_scratch(chfsi_ctx* ctx, void** out) {
 
 // ===================================================================== C ABI
 namespace chfsi {
+bool give_way(chfsi_ctx* ctx) {
+  const int64_t before = ctx->dev_bytes;
+  cudaStreamSynchronize(ctx->stream);
+  if (ctx->ex.words || ctx->exb.ptr) {
+    release(ctx, ctx->ex.words, ctx->ex.word_bytes);
+    release(ctx, ctx->ex.hsum, ctx->ex.exp_bytes);
+    ctx->ex = ExCellData();
+    ctx->ex_ready = false;
+    ctx->ex_off = true;
+    drop(ctx, ctx->exb);
+  }
+  for (DevBuf* b : {&ctx->Rb, &ctx->part, &ctx->work, &ctx->wellb}) drop(ctx, *b);
+  if (ctx->tc.bf && !ctx->tc.bf_ready) {
+    cudaFree(ctx->tc.bf);
+    ctx->dev_bytes -= (int64_t)ctx->tc.bf_bytes;
+    ctx->tc.bf = nullptr;
+    ctx->tc.bf_bytes = 0;
+  }
+  return ctx->dev_bytes < before;
+}
+
 chfsi_status late_timeout(chfsi_ctx* ctx) {
   volatile int* w = ctx->h_status;
   const int v = *w;
@@ -1652,10 +1693,11 @@ chfsi_status chfsi_bounds(chfsi_ctx* ctx, int lanczos_steps, uint64_t seed, doub
   double* dot = (double*)ctx->lam.ptr;
   if ((st = grow(ctx, ctx->lam, 64)) != CHFSI_OK) return st;
   dot = (double*)ctx->lam.ptr;
-  if ((st = grow(ctx, ctx->part, (size_t)8 * 1024)) != CHFSI_OK) return st;
   CK(launch_fill_uniform(v, 1, M, 1, stream_key(seed, 7), 1, ctx->stream));
   CK(cudaMemsetAsync(vp, 0, M * 8, ctx->stream));
   auto dotp = [&](const double* x, const double* y, double* r) -> chfsi_status {
+    const chfsi_status gs = grow(ctx, ctx->part, (size_t)8 * 1024);
+    if (gs != CHFSI_OK) return gs;
     CK(launch_gram_fp64(x, 1, y, 1, M, 1, 1, dot, 1, 0, (double*)ctx->part.ptr, ctx->part.bytes,
                         ctx->stream));
     CK(cudaMemcpyAsync(r, dot, 8, cudaMemcpyDeviceToHost, ctx->stream));

@@ -604,12 +604,12 @@ chfsi_status batch_prepare(chfsi_batch* b, float* const* X, const int64_t* ldx, 
   for (int i = 0; i < n; ++i) {
     chfsi_ctx* c = b->ctx[i];
     if (mode != kBatchBf16x3 && !c->tc.hi) {
-      cudaError_t pe = tc_pack_from_device(c->tc, c->d_Ht, c->stream, &c->dev_bytes);
+      cudaError_t pe = with_room(c, [&] { return tc_pack_from_device(c->tc, c->d_Ht, c->stream, &c->dev_bytes); });
       if (pe != cudaSuccess) return bfail(b, CHFSI_ERR_OOM, "tensor-core cell data");
       cudaStreamSynchronize(c->stream);
     }
     if (mode == kBatchBf16x3 && !c->tc.bf_ready) {
-      cudaError_t pe = tc_pack_bf16_from_device(c->tc, c->d_Ht, c->stream, &c->dev_bytes);
+      cudaError_t pe = with_room(c, [&] { return tc_pack_bf16_from_device(c->tc, c->d_Ht, c->stream, &c->dev_bytes); });
       if (pe != cudaSuccess) return bfail(b, CHFSI_ERR_OOM, "BF16x3 cell data");
       cudaStreamSynchronize(c->stream);
     }

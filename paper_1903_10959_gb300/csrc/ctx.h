@@ -1,6 +1,7 @@
 // Private definition of the library context (shared by api.cu and batch.cu).
 #pragma once
 
+#include <climits>
 #include <string>
 #include <vector>
 
@@ -43,10 +44,12 @@ struct chfsi_ctx {
   bool fp64_alu = false;           // binary64 products on the ALUs instead of as digit slices
   chfsi::TcCellData tc;                   // tensor-core copies (mixed precisions)
   // digit slices of the binary64 cell matrices (packed on first binary64 use;
-  // ex_off: they did not fit, the binary64 operator stays on the ALUs until
-  // the next build); ex_used: a digit-slice kernel ran since the last status check
+  // ex_off: they did not fit, or had to give way, and the binary64 operator stays
+  // on the ALUs until the next build or chfsi_autotune; ex_too_wide: the same for
+  // blocks of this width on); ex_used: a digit-slice kernel ran since the last status check
   chfsi::ExCellData ex;
   bool ex_ready = false, ex_off = false, ex_used = false;
+  int ex_too_wide = INT_MAX;
   uint64_t ex_capture = 0;         // stream capture in which the packing was recorded
   chfsi::ExWatch watch{};          // where their bounded waits report: the device's view of
   int* h_status = nullptr;         //   this word (pinned host memory)
@@ -116,4 +119,19 @@ chfsi_status rayleigh_ritz_internal(chfsi_ctx* ctx, void* X, int64_t ldx, int n,
 // CHFSI_ERR_TIMEOUT (once) when a bounded wait of the context's digit-slice kernels
 // gave up in work that has run by now; does not synchronise.
 chfsi_status late_timeout(chfsi_ctx* ctx);
+// Frees the buffers of the context that only make products faster and hold nothing
+// that a call in progress still reads: the digit words of the cell matrices with
+// their scratch, the dense cell blocks of the last application, the partial sums
+// and work of the last product (a call grows these right before the launch that
+// uses them), what the last build uploaded, and BF16x3 terms that await a
+// rebuild's matrices.  False when there were none.
+bool give_way(chfsi_ctx* ctx);
+// An allocation that the call cannot do without: once more after give_way.
+template <class F>
+cudaError_t with_room(chfsi_ctx* ctx, F alloc) {
+  cudaError_t e = alloc();
+  if (e != cudaErrorMemoryAllocation || !give_way(ctx)) return e;
+  cudaGetLastError();
+  return alloc();
+}
 }  // namespace chfsi

@@ -63,7 +63,7 @@ chfsi_status kgrow(chfsi_ctx* ctx, DevBuf& b, size_t bytes) {
   }
   b.ptr = nullptr;
   b.bytes = 0;
-  if (cudaMalloc(&b.ptr, bytes) != cudaSuccess) {
+  if (with_room(ctx, [&] { return cudaMalloc(&b.ptr, bytes); }) != cudaSuccess) {
     cudaGetLastError();
     return kfail(ctx, CHFSI_ERR_OOM, "k-point buffers: device allocation of " + std::to_string(bytes) + " bytes");
   }
@@ -198,7 +198,9 @@ chfsi_status kpack_mixed(chfsi_ctx* ctx) {
     return kfail(ctx, CHFSI_ERR_ARG, "mixed k-points need every cell to share the M^{-1/2} pattern");
   if (!ctx->d_Ht) return kfail(ctx, CHFSI_ERR_STATE, "no cell matrices (device-side potential)");
   const bool fresh_a = !ctx->kbf, fresh_g = !ctx->kgbf;
-  KK(tc_pack_bf16_matrices(ctx->d_Ht, ctx->d_kA, m.ncells, m.ne, &ctx->kbf, &ctx->kbf_bytes, ctx->stream));
+  KK(with_room(ctx, [&] {
+    return tc_pack_bf16_matrices(ctx->d_Ht, ctx->d_kA, m.ncells, m.ne, &ctx->kbf, &ctx->kbf_bytes, ctx->stream);
+  }));
   KK(tc_pack_bf16_matrices(ctx->d_kG, nullptr, 1, m.ne, &ctx->kgbf, &ctx->kgbf_bytes, ctx->stream));
   if (fresh_a) ctx->dev_bytes += (int64_t)ctx->kbf_bytes;
   if (fresh_g) ctx->dev_bytes += (int64_t)ctx->kgbf_bytes;
@@ -410,7 +412,7 @@ chfsi_status chfsi_set_kpoint(chfsi_ctx* ctx, const double* k) {
       for (int d = 0; d < 3; ++d) C[d * nn + i * n1 + l] = k[d] * s;
     }
   if (!ctx->d_kfac) {
-    if (cudaMalloc(&ctx->d_kfac, fac.size() * 8) != cudaSuccess) {
+    if (with_room(ctx, [&] { return cudaMalloc(&ctx->d_kfac, fac.size() * 8); }) != cudaSuccess) {
       cudaGetLastError();
       ctx->d_kfac = nullptr;
       return kfail(ctx, CHFSI_ERR_OOM, "k-point factors");
@@ -455,7 +457,7 @@ chfsi_status chfsi_set_kpoint(chfsi_ctx* ctx, const double* k) {
         }
     for (double** dp : {&ctx->d_kA, &ctx->d_kG})
       if (!*dp) {
-        if (cudaMalloc(dp, (size_t)ne * ne * 8) != cudaSuccess) {
+        if (with_room(ctx, [&] { return cudaMalloc(dp, (size_t)ne * ne * 8); }) != cudaSuccess) {
           cudaGetLastError();
           *dp = nullptr;
           return kfail(ctx, CHFSI_ERR_OOM, "k-point blocks");

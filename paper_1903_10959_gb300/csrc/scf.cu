@@ -195,7 +195,7 @@ chfsi_status scf_grow(chfsi_ctx* ctx, DevBuf& b, size_t bytes) {
   }
   b.ptr = nullptr;
   b.bytes = 0;
-  if (cudaMalloc(&b.ptr, bytes) != cudaSuccess) {
+  if (with_room(ctx, [&] { return cudaMalloc(&b.ptr, bytes); }) != cudaSuccess) {
     cudaGetLastError();
     return sfail(ctx, CHFSI_ERR_OOM, "SCF buffers: device allocation of " + std::to_string(bytes) + " bytes");
   }
@@ -499,7 +499,7 @@ chfsi_status chfsi_set_potential_qp_device(chfsi_ctx* ctx, const double* v) {
       ctx->d_wv = nullptr;
     }
     ctx->nwv = n;
-    if (cudaMalloc(&ctx->d_wv, (size_t)n * 8) != cudaSuccess) {
+    if (with_room(ctx, [&] { return cudaMalloc(&ctx->d_wv, (size_t)n * 8); }) != cudaSuccess) {
       cudaGetLastError();
       ctx->d_wv = nullptr;
       ctx->nwv = 0;

@@ -32,3 +32,97 @@ def test_cholgs_without_digit_scratch():
         assert rel_fro(X.cpu().numpy(), ref) <= 1e-12
     finally:
         ctx.destroy()
+
+
+def work_through(ctx, X0, prec):
+    """The calls of a solve, and what they leave."""
+    X = X0.clone()
+    out = []
+    if prec == "fp64":
+        b = ctx.bounds(20)
+        ctx.filter(X, 4, 8.0, 1.05 * b, -4.0)
+        ctx.cholgs(X)
+        d = ctx.rayleigh_ritz(X)
+        out.append(torch.tensor(d))
+    else:
+        d, _ = ctx.solve(X, 2, 6, 1.05 * ctx.bounds(20), prec=prec)
+        out.append(torch.tensor(d))
+    r, _ = ctx.residuals(X, d, prec=prec)
+    out.append(torch.tensor(r))
+    X64 = X.double()
+    Y = torch.empty_like(X64)
+    ctx.apply(X64, Y)
+    ctx.last_timings()
+    out.append((X64.T @ Y).diagonal().cpu())
+    return out
+
+
+@pytest.mark.parametrize("prec", ["fp64", "bf16x3"])
+@pytest.mark.parametrize("sites", [0, 3])
+def test_solve_in_the_memory_of_the_plain_forms(prec, sites):
+    """At the bytes that the ALU forms need, at twice those, and between: the same
+    calls run, with the same values (1e-10 of the largest; 1e-4 for the filter of a
+    block in BF16x3, whose subspace differs in rounding)."""
+    s = W.small_periodic(seed=360, ncell=5, p=4, L=10.0, n_wells=4, n_want=40)
+    if sites:
+        s.nl_centres = s.centres[:sites].copy()
+        s.nl_h = 0.5 + np.arange(4 * sites).reshape(sites, 4) / 8.0
+    dt = torch.float64 if prec == "fp64" else torch.float32
+
+    def context():
+        c = gpu_context(s)
+        c.set_blocking(44, 1)
+        return c, torch.tensor(W.start_block(3, c.ndofs, 44), dtype=dt, device=DEV)
+
+    ctx, X0 = context()
+    ctx.set_fp64_products("alu")
+    ref = work_through(ctx, X0, prec)
+    need = ctx.device_bytes()
+    ctx.destroy()
+    tol = 1e-10 if prec == "fp64" else 1e-4
+    for part in (1.0, 1.02, 1.1, 1.3, 1.6, 2.0, 3.0):
+        ctx, X0 = context()
+        try:
+            ctx.debug_memory_limit(int(part * need) + 256)
+            got = work_through(ctx, X0, prec)
+            assert ctx.device_bytes() <= int(part * need) + 256
+            assert ctx.last_error() == ""
+            for a, b in zip(got, ref):
+                assert float((a - b).abs().max()) <= tol * max(1.0, float(b.abs().max()))
+        finally:
+            ctx.destroy()
+
+
+def test_one_wide_block_does_not_turn_the_digit_products_off():
+    """A block too wide for its scratch runs on the ALUs; a narrower one that fits
+    takes the digit slices, and so do all widths once there is room."""
+    s = W.small_periodic(seed=361, ncell=4, p=4, L=8.0, n_wells=4, n_want=10)
+    ctx, free = gpu_context(s), gpu_context(s)
+    try:
+        X = torch.tensor(W.start_block(3, ctx.ndofs, 160), device=DEV)
+        Y, A, D = torch.empty_like(X), torch.empty_like(X), torch.empty_like(X)
+        free.apply(X[:, :40], D[:, :40])
+        need = free.device_bytes()
+        free.apply(X, D)
+        free.last_timings()
+        limit = (need + free.device_bytes()) // 2
+        free.set_fp64_products("alu")
+        free.apply(X, A)
+        free.last_timings()
+        ctx.set_blocking(160, 1)
+        ctx.debug_memory_limit(limit)
+        ctx.apply(X, Y)
+        ctx.last_timings()
+        assert torch.equal(Y, A)                       # the ALU form took over
+        ctx.apply(X[:, :40], Y[:, :40])
+        ctx.last_timings()
+        assert torch.equal(Y[:, :40], D[:, :40])       # digit slices, the same bits
+        ctx.debug_memory_limit(0)
+        ctx.autotune(X, prec="fp64")                                # lets go of the scratch and starts over
+        ctx.set_blocking(160, 1)
+        ctx.apply(X, Y)
+        ctx.last_timings()
+        assert torch.equal(Y, D)
+    finally:
+        ctx.destroy()
+        free.destroy()
