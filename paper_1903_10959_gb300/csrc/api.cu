@@ -474,8 +474,14 @@ chfsi_status apply_step(chfsi_ctx* ctx, chfsi_precision prec, const void* Yin, i
   // owner-computes: dense cell blocks R_e (one launch over all cells), then the
   // fixed-order assembly fused with the Chebyshev update.  R is the last buffer
   // of the step to grow: it gives way to the others.
-  const int64_t ldr4 = (ncol + 3) & ~3;   // 16-byte rows of R
-  if ((st = grow(ctx, ctx->Rb, (size_t)m.ncells * m.ne * ldr4 * sizeof(float))) != CHFSI_OK) return st;
+  int64_t ldr4 = (ncol + 3) & ~3;         // 16-byte rows of R, or as wide as fits
+  const std::string err = ctx->err;
+  if ((st = grow(ctx, ctx->Rb, (size_t)m.ncells * m.ne * ldr4 * sizeof(float))) != CHFSI_OK) {
+    if (ldr4 == ncol) return st;
+    ldr4 = ncol;
+    if ((st = grow(ctx, ctx->Rb, (size_t)m.ncells * m.ne * ldr4 * sizeof(float))) != CHFSI_OK) return st;
+    ctx->err = err;
+  }
   TcApplyArgs ra{};
   ra.dofmap = ctx->d_dofmap;
   ra.ncells = m.ncells;
@@ -593,23 +599,35 @@ chfsi_status filter_range(chfsi_ctx* ctx, void* X, int64_t ldx, int ncol, int de
     int ncs = nb;   // columns of the steps
     bool pad = is_mixed(prec) && prec != CHFSI_MIXED_F16X2 && degree >= kPadDegree &&
                ((nb & 3) || (ldx & 3) || (reinterpret_cast<uintptr_t>(Xb) & 15));
+    const std::string err = ctx->err;
     if (pad) {
-      const std::string err = ctx->err;
       const int n4 = (nb + 3) & ~3;
-      if (grow(ctx, ctx->T2, (size_t)m.ndofs * n4 * es) == CHFSI_OK &&
-          grow(ctx, ctx->T1, (size_t)m.ndofs * n4 * es) == CHFSI_OK) {
+      if (grow_optional(ctx, ctx->T2, (size_t)m.ndofs * n4 * es) &&
+          grow_optional(ctx, ctx->T1, (size_t)m.ndofs * n4 * es)) {
         ncs = n4;
         bufs[0] = ctx->T2.ptr;
         bufs[1] = ctx->T1.ptr;
         lds[0] = lds[1] = n4;
         CK(launch_copy_pad((const float*)Xb, ldx, nb, (float*)ctx->T2.ptr, n4, m.ndofs, ctx->stream));
       } else {
-        ctx->err = err;
         pad = false;
-        if ((st = grow(ctx, ctx->T1, (size_t)m.ndofs * nb * es)) != CHFSI_OK) return st;
-        bufs[1] = ctx->T1.ptr;
       }
     }
+    // without room for the copies: the steps run on the block itself
+    auto in_place = [&] {
+      pad = false;
+      cudaStreamSynchronize(ctx->stream);
+      drop(ctx, ctx->T2);
+      drop(ctx, ctx->T1);   // it may have the padded width
+      const chfsi_status gs = grow(ctx, ctx->T1, (size_t)m.ndofs * nb * es);
+      ncs = nb;
+      bufs[0] = Xb;
+      bufs[1] = ctx->T1.ptr;
+      lds[0] = ldx;
+      lds[1] = nb;
+      return gs;
+    };
+    if (!ctx->T1.ptr && (st = in_place()) != CHFSI_OK) return st;
     int cur = 0;  // buffer holding Y_k
     double sig = s1;
     // FP16x2: each step's assembly leaves the column maxima of its output, the
@@ -632,8 +650,17 @@ chfsi_status filter_range(chfsi_ctx* ctx, void* X, int64_t ldx, int ncol, int de
         sig = sn;
       }
       const int nxt = 1 - cur;  // holds Y_{k-2} (or is free at k = 1)
-      st = apply_step(ctx, prec, bufs[cur], lds[cur], bufs[nxt], lds[nxt], bufs[nxt], lds[nxt], ncs,
-                      alpha, beta, c, k == 1 ? nullptr : cm[cur], k == degree ? nullptr : cm[nxt]);
+      auto step = [&] {
+        return apply_step(ctx, prec, bufs[cur], lds[cur], bufs[nxt], lds[nxt], bufs[nxt], lds[nxt], ncs,
+                          alpha, beta, c, k == 1 ? nullptr : cm[cur], k == degree ? nullptr : cm[nxt]);
+      };
+      ctx->pad_steps = pad;
+      st = step();
+      ctx->pad_steps = false;
+      if (st == CHFSI_ERR_OOM && pad && k == 1) {   // the other buffers grow in the first step; X is as it came
+        ctx->err = err;
+        if ((st = in_place()) == CHFSI_OK) st = step();
+      }
       if (st != CHFSI_OK) return st;
       cur = nxt;
     }
@@ -1016,7 +1043,7 @@ cudaError_t noalloc_scratch(chfsi_ctx* ctx, void** out) {
 namespace chfsi {
 bool give_way(chfsi_ctx* ctx) {
   const int64_t before = ctx->dev_bytes;
-  cudaStreamSynchronize(ctx->stream);
+  cudaDeviceSynchronize();   // the context's stream, and those of the filter lanes
   if (ctx->ex.words || ctx->exb.ptr) {
     release(ctx, ctx->ex.words, ctx->ex.word_bytes);
     release(ctx, ctx->ex.hsum, ctx->ex.exp_bytes);
@@ -1026,6 +1053,8 @@ bool give_way(chfsi_ctx* ctx) {
     drop(ctx, ctx->exb);
   }
   for (DevBuf* b : {&ctx->Rb, &ctx->part, &ctx->work, &ctx->wellb}) drop(ctx, *b);
+  if (!ctx->pad_steps) drop(ctx, ctx->T2);
+  for (DevBuf& b : ctx->laneT2) drop(ctx, b);
   if (ctx->tc.bf && !ctx->tc.bf_ready) {
     cudaFree(ctx->tc.bf);
     ctx->dev_bytes -= (int64_t)ctx->tc.bf_bytes;

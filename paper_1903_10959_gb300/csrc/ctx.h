@@ -69,6 +69,7 @@ struct chfsi_ctx {
   float* d_dof_c32 = nullptr;
   // grown scratch
   chfsi::DevBuf T1, T2, Wb, NLb, Zb, rot, Ssq, work, part, vec, lam, Rb;
+  bool pad_steps = false;          // a filter step on padded copies is under way (T2 in use)
   chfsi::DevBuf exb;               // digit slices: the block's words and scales
   chfsi::DevBuf pol;               // binary64 staging block of the polish
   chfsi::DevBuf scfb, scfq, scfr, scfw;   // Poisson / SCF work arrays (scf.cu)
@@ -121,7 +122,8 @@ chfsi_status rayleigh_ritz_internal(chfsi_ctx* ctx, void* X, int64_t ldx, int n,
 chfsi_status late_timeout(chfsi_ctx* ctx);
 // Frees the buffers of the context that only make products faster and hold nothing
 // that a call in progress still reads: the digit words of the cell matrices with
-// their scratch, the dense cell blocks of the last application, the partial sums
+// their scratch, the dense cell blocks of the last application, the padded copies
+// of ragged blocks, the partial sums
 // and work of the last product (a call grows these right before the launch that
 // uses them), what the last build uploaded, and BF16x3 terms that await a
 // rebuild's matrices.  False when there were none.

@@ -126,3 +126,38 @@ def test_one_wide_block_does_not_turn_the_digit_products_off():
     finally:
         ctx.destroy()
         free.destroy()
+
+
+@pytest.mark.parametrize("prec", ["bf16x3", "mixed", "tf32"])
+@pytest.mark.parametrize("lanes,n", [(1, 77), (1, 1), (2, 259)])
+def test_ragged_filter_without_its_copies(prec, lanes, n):
+    """A ragged block filtered in the memory of the steps on the block itself (a
+    scratch block and the dense cell blocks, rows as wide as the block), and with
+    room for one of the padded copies but not for all: the same bits."""
+    s = W.small_periodic(seed=362, ncell=4, p=4, L=8.0, n_wells=4, n_want=10)
+    rows = 64 * 125
+
+    def context():
+        c = gpu_context(s, block=300)
+        c.set_filter_lanes(lanes)
+        x = torch.zeros((c.ndofs, 4), dtype=torch.float32, device=DEV)
+        c.apply(x, torch.empty_like(x), prec=prec)                 # packs the cell data
+        return c, c.device_bytes() - rows * 4 * 4                  # without its dense cell blocks
+
+    ctx, base = context()
+    X0 = torch.tensor(W.start_block(3, ctx.ndofs, n), dtype=torch.float32, device=DEV)
+    ref = X0.clone()
+    ctx.filter(ref, 9, 3.0, 120.0, -2.0, prec=prec)
+    need = base + ctx.ndofs * n * 4 + rows * n * 4 + 4096
+    pad = ctx.ndofs * (n + 3) * 4
+    ctx.destroy()
+    for limit in (need, need + pad // 2, need + pad, need + rows * 3 * 4 + pad):
+        ctx, _ = context()
+        try:
+            X = X0.clone()
+            ctx.debug_memory_limit(limit)
+            ctx.filter(X, 9, 3.0, 120.0, -2.0, prec=prec)
+            assert ctx.device_bytes() <= limit and ctx.last_error() == ""
+            assert torch.equal(X, ref)
+        finally:
+            ctx.destroy()
