@@ -474,28 +474,32 @@ cudaError_t batch_describe(chfsi_batch* b, float* const* X, const int64_t* ldx, 
   b->h_sys.assign(n, BSys{});
   b->ldx.assign(ldx, ldx + n);
   int64_t item = 0, q = 0;
+  // what a system needs: the padded copies of earlier calls and what the member
+  // contexts can do without make room for it
+  auto need = [&](DevBuf& d, size_t bytes) {
+    cudaError_t e = ensure_dbuf(d, bytes);
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();
+    for (auto& t : b->T0) {
+      cudaFree(t.ptr);
+      t = DevBuf{};
+    }
+    for (chfsi_ctx* c : b->ctx) give_way(c);
+    return ensure_dbuf(d, bytes);
+  };
   for (int i = 0; i < n; ++i) {
     chfsi_ctx* c = b->ctx[i];
     const HostMesh& m = c->mesh;
     cudaError_t e;
     const int64_t ld4 = (ncol[i] + 3) / 4 * 4;   // 16-byte rows for the scratch and R
-    if ((e = ensure_dbuf(b->T1[i], (size_t)m.ndofs * ld4 * 4 + 16)) != cudaSuccess) return e;
-    if ((e = ensure_dbuf(b->R[i], (size_t)m.ncells * m.ne * ld4 * 4 + 16)) != cudaSuccess) return e;
+    if ((e = need(b->T1[i], (size_t)m.ndofs * ld4 * 4 + 16)) != cudaSuccess) return e;
+    if ((e = need(b->R[i], (size_t)m.ncells * m.ne * ld4 * 4 + 16)) != cudaSuccess) return e;
     BSys& sy = b->h_sys[i];
     sy.A = mode == kBatchBf16x3 ? reinterpret_cast<const float*>(c->tc.bf) : c->tc.hi;
     sy.dofmap = c->d_dofmap;
     sy.Y[0] = X[i];
     sy.ldY[0] = ldx[i];
     sy.ncol = ncol[i];
-    // rows off 16 bytes or a ragged width: the steps run on a copy padded with
-    // zero columns (batch_enqueue), so that the assembly takes 16-byte accesses
-    // (16 uneven systems, p = 5: 492 -> 459 us a step)
-    if ((ncol[i] & 3) || (ldx[i] & 3) || (reinterpret_cast<uintptr_t>(X[i]) & 15)) {
-      if ((e = ensure_dbuf(b->T0[i], (size_t)m.ndofs * ld4 * 4 + 16)) != cudaSuccess) return e;
-      sy.Y[0] = (const float*)b->T0[i].ptr;
-      sy.ldY[0] = ld4;
-      sy.ncol = (int)ld4;
-    }
     sy.Y[1] = (const float*)b->T1[i].ptr;
     sy.ldY[1] = ld4;
     sy.R = (float*)b->R[i].ptr;
@@ -512,6 +516,25 @@ cudaError_t batch_describe(chfsi_batch* b, float* const* X, const int64_t* ldx, 
   }
   b->nitems = item;
   b->nq = q;
+  // rows off 16 bytes or a ragged width: the steps run on a copy padded with
+  // zero columns (batch_enqueue), so that the assembly takes 16-byte accesses
+  // (16 uneven systems, p = 5: 492 -> 459 us a step).  A copy for which there is no
+  // room next to what every system needs is left out.
+  for (int i = 0; i < n; ++i) {
+    if (!(ncol[i] & 3) && !(ldx[i] & 3) && !(reinterpret_cast<uintptr_t>(X[i]) & 15)) continue;
+    chfsi_ctx* c = b->ctx[i];
+    const int64_t ld4 = b->h_sys[i].ldr;
+    const size_t bytes = (size_t)c->mesh.ndofs * ld4 * 4 + 16;
+    if (c->mem_limit > 0 && c->dev_bytes + (int64_t)bytes > c->mem_limit) continue;
+    if (ensure_dbuf(b->T0[i], bytes) != cudaSuccess) {
+      cudaGetLastError();
+      continue;
+    }
+    BSys& sy = b->h_sys[i];
+    sy.Y[0] = (const float*)b->T0[i].ptr;
+    sy.ldY[0] = ld4;
+    sy.ncol = (int)ld4;
+  }
   return cudaMemcpyAsync(b->d_sys, b->h_sys.data(), n * sizeof(BSys), cudaMemcpyHostToDevice,
                          b->stream);
 }

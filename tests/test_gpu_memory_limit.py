@@ -8,7 +8,7 @@ import numpy as np
 import pytest
 import torch
 
-from paper_1903_10959_gb300 import Context, workloads as W
+from paper_1903_10959_gb300 import Batch, Context, workloads as W
 
 from gpu_util import gpu_context, rel_fro
 
@@ -161,3 +161,34 @@ def test_ragged_filter_without_its_copies(prec, lanes, n):
             assert torch.equal(X, ref)
         finally:
             ctx.destroy()
+
+
+@pytest.mark.parametrize("prec", ["bf16x3", "mixed"])
+@pytest.mark.parametrize("degree", [5, 6])
+def test_batch_without_padded_copies(prec, degree):
+    """Ragged members of a batch, one of them without room for its padded copy: the
+    same bits, nothing written outside the blocks."""
+    shapes = [(3, 21), (4, 40), (3, 7)]
+    out = []
+    for limited in (False, True):
+        ctxs, X = [], []
+        for k, (cells, n) in enumerate(shapes):
+            s = W.small_periodic(seed=370 + k, ncell=cells, p=4, L=2.0 * cells, n_wells=3, n_want=10)
+            c = gpu_context(s)
+            buf = torch.full((c.ndofs, n + 2), 7.0, dtype=torch.float32, device=DEV)
+            buf[:, 1:1 + n] = torch.tensor(W.start_block(k, c.ndofs, n), dtype=torch.float32, device=DEV)
+            ctxs.append(c)
+            X.append(buf)
+        batch = Batch(ctxs)
+        views = [x[:, 1:1 + n] for x, (_, n) in zip(X, shapes)]
+        for r in range(2):                             # the second call replays the graph
+            if limited:
+                ctxs[1].debug_memory_limit(ctxs[1].device_bytes())
+            batch.filter(views, degree, [3.0] * 3, [150.0] * 3, [-2.0] * 3, prec=prec)
+        out.append(X)
+        batch.destroy()
+        for c in ctxs:
+            c.destroy()
+    for a, b in zip(*out):
+        assert torch.equal(a, b)
+        assert bool((b[:, 0] == 7.0).all()) and bool((b[:, -1] == 7.0).all())
