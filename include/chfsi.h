@@ -681,9 +681,12 @@ chfsi_status chfsi_batch_solve(chfsi_batch* b, double* const* X, const int64_t* 
  * polish_iters > 0 (mixed precisions: the polished block, rounded to
  * binary32, is the next solve's start), and then chfsi_residuals on the
  * lowest n_check pairs.  Requests share no device data, so a request's
- * results do not depend on what else runs.  A request whose estimate exceeds
- * the whole budget completes with CHFSI_ERR_OOM; one that only has to wait
- * for memory stays queued.  chfsi_server_destroy lets running requests finish,
+ * results do not depend on what else runs.  The estimate includes what the
+ * default binary64 products take (digit words of the cell matrices, 8 B per
+ * entry, and their scratch) and padded copies of ragged filter blocks; a
+ * request that exceeds the whole budget only with these runs without them
+ * (chfsi_set_fp64_products 1), and one that exceeds it all the same completes
+ * with CHFSI_ERR_OOM.  One that only has to wait for memory stays queued.  chfsi_server_destroy lets running requests finish,
  * fails the ones still queued (CHFSI_ERR_STATE) and joins every thread. */
 #define CHFSI_MAX_SOLVES 16
 
@@ -733,7 +736,8 @@ chfsi_status chfsi_server_submit(chfsi_server* sv, const chfsi_request* req, uin
  * evals_host[k * n], (resolves + 1) * n doubles. */
 chfsi_status chfsi_server_poll(chfsi_server* sv, uint64_t ticket, int wait, chfsi_result* out,
                                double* evals_host);
-/* Device-memory estimate the server admits a request by (bytes). */
+/* Device-memory estimate the server admits a request by (bytes), when the budget
+ * is not smaller. */
 size_t       chfsi_server_estimate(const chfsi_request* req);
 chfsi_status chfsi_server_destroy(chfsi_server* sv);
 

@@ -597,7 +597,7 @@ chfsi_status filter_range(chfsi_ctx* ctx, void* X, int64_t ldx, int ncol, int de
     // column scales come with the block, nor a few steps, which the two copies
     // would cost.
     int ncs = nb;   // columns of the steps
-    bool pad = is_mixed(prec) && prec != CHFSI_MIXED_F16X2 && degree >= kPadDegree &&
+    bool pad = is_mixed(prec) && prec != CHFSI_MIXED_F16X2 && degree >= kPadDegree && !ctx->no_pad &&
                ((nb & 3) || (ldx & 3) || (reinterpret_cast<uintptr_t>(Xb) & 15));
     const std::string err = ctx->err;
     if (pad) {

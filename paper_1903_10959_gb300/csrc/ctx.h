@@ -69,6 +69,7 @@ struct chfsi_ctx {
   float* d_dof_c32 = nullptr;
   // grown scratch
   chfsi::DevBuf T1, T2, Wb, NLb, Zb, rot, Ssq, work, part, vec, lam, Rb;
+  bool no_pad = false;             // ragged filter blocks always in place
   bool pad_steps = false;          // a filter step on padded copies is under way (T2 in use)
   chfsi::DevBuf exb;               // digit slices: the block's words and scales
   chfsi::DevBuf pol;               // binary64 staging block of the polish

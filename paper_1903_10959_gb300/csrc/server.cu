@@ -38,6 +38,7 @@ struct Job {
   chfsi_request req{};
   std::vector<double> xyz, depth, width, depth_seq;
   size_t bytes = 0;
+  bool plain = false;              // admitted by the plain estimate, and run so
   Clock::time_point submitted;
   // results
   bool done = false;
@@ -73,8 +74,9 @@ namespace {
 // Device bytes a request will hold: what its context allocates (cell
 // matrices, their packed binary32 split copy, the mesh tables, the filter,
 // rotation and residual scratch, the Gram partial sums and the solver
-// workspace, at the default filter block of 200 columns) plus the block X.
-size_t estimate_bytes(const chfsi_request& r) {
+// workspace, at the default filter block of 200 columns) plus the block X.  plain:
+// without what only makes it faster (digit slices, padded copies).
+size_t estimate_bytes(const chfsi_request& r, bool plain = false) {
   const chfsi_mesh_desc& d = r.mesh;
   const size_t p = (size_t)d.p, ne = (p + 1) * (p + 1) * (p + 1);
   size_t ncells = 1, M = 1;
@@ -93,9 +95,12 @@ size_t estimate_bytes(const chfsi_request& r) {
   b += M * n * es;                                                  // X
   b += std::max(M * n * es, M * B * 16);                            // rotation / binary64 pair
   b += M * B * es + M * B * 8;                                      // filter block, binary64 apply
-  if (mixed) b += 2 * M * ((B + 3) / 4 * 4) * es;                   // padded copies of a ragged block
-  b += ncells * ne * ((B + 1) & ~(size_t)1) * 8;                    // dense cell blocks R_e (binary64 applications)
-  {                                                                 // digit words of the binary64 products
+  if (plain) {
+    if (mixed) b += ncells * ne * ((B + 3) / 4 * 4) * 4;            // dense cell blocks R_e
+  } else {
+    if (mixed) b += 2 * M * ((B + 3) / 4 * 4) * es;                 // padded copies of a ragged block
+    b += ncells * ne * ((B + 1) & ~(size_t)1) * 8;                  // dense cell blocks R_e (binary64 applications)
+    // digit words of the binary64 products
     size_t words = 0, scales = 0;
     chfsi::ex_cell_bytes((int64_t)ncells, (int)ne, &words, &scales);
     b += words + scales + chfsi::ex_cell_work_bytes((int64_t)ncells, (int)ne, (int)B);
@@ -129,6 +134,7 @@ void run_job(chfsi_server* sv, std::shared_ptr<Job> job) {
   if (s != CHFSI_OK) {
     finish(s, "create");
   } else {
+    ctx->fp64_alu = ctx->no_pad = J.plain;
     const int64_t M = chfsi_num_dofs(ctx);
     const int n = r.n;
     J.evals.assign((size_t)(r.resolves + 1) * n, 0.0);
@@ -254,6 +260,13 @@ chfsi_status chfsi_server_submit(chfsi_server* sv, const chfsi_request* r, uint6
     job->depth_seq.assign(r->depth_seq, r->depth_seq + (size_t)r->resolves * r->nwells);
   job->req.xyz = job->req.depth = job->req.width = job->req.depth_seq = nullptr;
   job->bytes = estimate_bytes(*r);
+  if (job->bytes > sv->budget) {   // (constant after creation)
+    const size_t plain = estimate_bytes(*r, true);
+    if (plain <= sv->budget) {
+      job->bytes = plain;
+      job->plain = true;
+    }
+  }
   job->submitted = Clock::now();
   std::lock_guard<std::mutex> lk(sv->mu);
   if (sv->stop) return CHFSI_ERR_STATE;

@@ -157,3 +157,26 @@ def test_warm_start_needs_fewer_iterations(small):
     assert max(r["max_gresidual"]) < 1e-8
     for j in range(len(seq) + 1):
         assert np.abs(r["evals"][j][:s.n_want] - exact[j][:s.n_want]).max() < 1e-10
+
+
+@pytest.mark.parametrize("prec,polish", [("fp64", 0), ("mixed", 0), ("bf16x3", 1)])
+def test_request_that_fits_the_budget_only_without_the_fast_forms(requests, prec, polish):
+    """A budget below the estimate but above what the request takes with binary64
+    products on the ALUs and without padded copies: it runs, within that budget,
+    and gives the values of the other form (the tolerances of the method: 1e-10 Ha
+    in binary64, 1e-7 in the mixed precisions, on the converged pairs)."""
+    s, seq = requests[0]
+    tol = 1e-10 if prec == "fp64" else 1e-7
+    full = _run([(s, seq)], max_active=1, prec=prec, polish=polish)[0]
+    assert full["status"] == 0
+    hi = full["est_bytes"] - 1
+    runs = {}
+    for budget in (hi, int(0.9 * hi), int(0.8 * hi), int(0.7 * hi)):
+        r = _run([(s, seq)], max_active=1, budget=budget, prec=prec, polish=polish)[0]
+        runs[budget] = r
+        if r["status"] != 0:
+            assert r["nsolves"] == 0 and "budget" in r["error"]
+            continue
+        assert r["used_bytes"] <= r["est_bytes"] <= budget
+        assert np.abs(r["evals"][:, :s.n_want] - full["evals"][:, :s.n_want]).max() <= tol
+    assert runs[hi]["status"] == 0
