@@ -7,13 +7,15 @@ namespace chfsi {
 
 constexpr uint64_t kZeroWord = 0x8080808080808080ull;   // eight digits 0, biased by 128
 
-__device__ __forceinline__ int expo(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
+// Exponent field of v as its scale: subnormal numbers have that of the smallest
+// normal ones (and no leading bit), and so have zeros.
+__device__ __forceinline__ int expo(double v) { return max((__double2hiint(v) >> 20) & 0x7ff, 1); }
+__device__ __forceinline__ bool nonzero(double v) { return ((__double2hiint(v) & 0x7fffffff) | __double2loint(v)) != 0; }
 
 // v as an integer of up to 62 bits under the scale s = (vector's exponent field - v's own).
 __device__ __forceinline__ int64_t fixed_of(double v, int s) {
   const int hi = __double2hiint(v);
-  if (!(hi & 0x7ff00000)) return 0;                 // zeros and subnormal numbers vanish
-  const uint64_t m = (uint64_t)(uint32_t)((hi & 0xfffff) | 0x100000) << 32 | (uint32_t)__double2loint(v);
+  const uint64_t m = (uint64_t)(uint32_t)((hi & 0xfffff) | (hi & 0x7ff00000 ? 0x100000 : 0)) << 32 | (uint32_t)__double2loint(v);
   const int64_t t = (int64_t)(m << 9);
   return (hi < 0 ? -t : t) >> min(s, 63);
 }

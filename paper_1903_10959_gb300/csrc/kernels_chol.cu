@@ -39,19 +39,21 @@ __device__ __forceinline__ void group_sync(int g) {
   asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "n"(GROUP) : "memory");
 }
 
-// 1 / d by a third-order Newton step on the binary32 reciprocal of d's
-// significand (relative error 2^-22; its cube lies below rounding).  Three
-// binary64 operations of 64 clocks each, a division takes as long as 5.5.
-__device__ __forceinline__ double reciprocal(double d) {
+// v / d by a third-order Newton step on the binary32 reciprocal of d's
+// significand (relative error 2^-22; its cube lies below rounding).  Four
+// binary64 operations of 64 clocks each, a division takes as long as 5.5 more;
+// it is left to pivots whose reciprocal is out of range (columns of norm below
+// 2^-511 have such squares).
+__device__ __forceinline__ double quotient(double v, double d) {
   const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
   const int e = (hi >> 20) & 0x7ff;
-  if (e < 2 || e > 2044) return 1.0 / d;
+  if (e < 2 || e > 2044) return v / d;
   const double m = __hiloint2double((int)((hi & 0xfffff) | 0x3ff00000), (int)lo);
   const uint32_t f = __float_as_uint(__fdividef(1.f, __uint_as_float(0x3f800000 | (hi & 0xfffff) << 3 | lo >> 29)));
   const double y = __hiloint2double((int)(((f >> 23) + 896) << 20 | (f >> 3 & 0xfffff)), (int)(f << 29));
   const double r = fma(-m, y, 1.0);
   const double z = fma(y, fma(r, r, r), y);
-  return __hiloint2double((__double2hiint(z) - ((e - 1023) << 20)) | (int)(hi & 0x80000000u), __double2loint(z));
+  return v * __hiloint2double((__double2hiint(z) - ((e - 1023) << 20)) | (int)(hi & 0x80000000u), __double2loint(z));
 }
 
 // The diagonal tile at o (nv columns): S minus the products with the 32 columns
@@ -93,7 +95,7 @@ __device__ void factor_tile(const double (*P)[NB + 1], double (*V)[NB + 1], doub
     }
     group_sync(0);
     if (top[0] <= j) continue;                               // this warp's rows are finished
-    const double s = -V[j][lane] * reciprocal(V[j][j]);
+    const double s = quotient(-V[j][lane], V[j][j]);
 #pragma unroll
     for (int i = 0; i < SLOTS; ++i) {
       if (top[i] > j) {

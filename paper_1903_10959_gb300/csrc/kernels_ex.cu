@@ -178,7 +178,12 @@ __device__ __forceinline__ double compose(int64_t v, int ex) {
   m += ((t & 0x7ff) + (m & 1)) > 0x400;              // to nearest, ties to even
   const int f = 63 - lz + ex - 1033 - SH;                 // exponent field
   const uint64_t sg = v < 0 ? 0x8000000000000000ull : 0ull;
-  if (f <= 0) return __longlong_as_double((long long)sg);
+  if (f <= 0) {                                      // units of 2^-1074
+    const int sh = 12 - f;
+    if (sh > 64) return __longlong_as_double((long long)sg);
+    const uint64_t q = sh > 63 ? 0 : t >> sh, h = 1ull << (sh - 1), r = t & (h | (h - 1));
+    return __longlong_as_double((long long)(sg | (q + (r > h || (r == h && (q & 1))))));
+  }
   if (f >= 2047) return __longlong_as_double((long long)(sg | 0x7ff0000000000000ull));
   return __longlong_as_double((long long)(sg | (((uint64_t)f << 52) + (m - (1ull << 52)))));
 }
@@ -587,7 +592,7 @@ __global__ void __launch_bounds__(256) ex_cell_words_kernel(const int32_t* __res
   if (c >= ncol) return;
 #pragma unroll
   for (int w = 0; w < 8; ++w) m = max(m, red[w][threadIdx.x]);
-  m >>= 20;
+  m = max(m >> 20, 1);
   if (threadIdx.y == 0) cexp[e * ncol + c] = (int16_t)m;
 #pragma unroll 8
   for (int l = threadIdx.y; l < nep; l += 8) {
@@ -611,7 +616,7 @@ __global__ void __launch_bounds__(256) ex_col_scale_kernel(const double* __restr
 #pragma unroll 8
     for (int64_t r = (int64_t)blockIdx.y * 8 + threadIdx.y; r < M; r += (int64_t)gridDim.y * 8) {
       const int e = expo(__ldg(X + r * ldx + c));
-      m = max(m, finite && e == 2047 ? 0 : e);
+      m = max(m, finite && e == 2047 ? 1 : e);
     }
   }
   __shared__ int red[8][32];
@@ -650,8 +655,9 @@ __global__ void __launch_bounds__(256) ex_row_scale_kernel(const double* __restr
   int m = kNoScale;
 #pragma unroll 4
   for (int k = lane; k < n; k += 32) {
-    const int e = expo(__ldg(X + r * ldx + k));
-    if (e) m = max(m, e == 2047 ? kNonFinite : e - __ldg(ecol + k));
+    const double v = __ldg(X + r * ldx + k);
+    const int e = expo(v);
+    if (nonzero(v)) m = max(m, e == 2047 ? kNonFinite : e - __ldg(ecol + k));
   }
   m = __reduce_max_sync(0xffffffffu, m);
   if (lane == 0) rexp[r] = m;
@@ -697,8 +703,9 @@ __global__ void __launch_bounds__(256) ex_u_scale_kernel(const double* __restric
   int m = kNoScale;
   const int kend = upper ? min(n1, j + 1) : n1;
   for (int k = lane; k < kend; k += 32) {
-    const int e = expo(trans ? U[j + (int64_t)k * ldu] : U[k + (int64_t)j * ldu]);
-    if (e) m = max(m, e == 2047 ? kNonFinite : e + ecol[k]);
+    const double v = trans ? U[j + (int64_t)k * ldu] : U[k + (int64_t)j * ldu];
+    const int e = expo(v);
+    if (nonzero(v)) m = max(m, e == 2047 ? kNonFinite : e + ecol[k]);
   }
   m = __reduce_max_sync(0xffffffffu, m);
   if (lane == 0) uexp[j] = m;
