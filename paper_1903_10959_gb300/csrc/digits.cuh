@@ -15,7 +15,8 @@ __device__ __forceinline__ bool nonzero(double v) { return ((__double2hiint(v) &
 // v as an integer of up to 62 bits under the scale s = (vector's exponent field - v's own).
 __device__ __forceinline__ int64_t fixed_of(double v, int s) {
   const int hi = __double2hiint(v);
-  const uint64_t m = (uint64_t)(uint32_t)((hi & 0xfffff) | (hi & 0x7ff00000 ? 0x100000 : 0)) << 32 | (uint32_t)__double2loint(v);
+  const uint32_t lead = min(hi & 0x7ff00000, 0x100000);
+  const uint64_t m = (uint64_t)((hi & 0xfffff) | lead) << 32 | (uint32_t)__double2loint(v);
   const int64_t t = (int64_t)(m << 9);
   return (hi < 0 ? -t : t) >> min(s, 63);
 }
