@@ -190,7 +190,8 @@ chfsi_status chfsi_set_cell_gather(chfsi_ctx* ctx, int mode);
  * and polish): 0 = the stored cell matrices H~_e (dense n_e x n_e products,
  * Sec. 3.3.1), evaluated on the tensor cores as exact products of 8-bit digit
  * slices (a library-owned copy of the matrices as 64-bit digit words, 8 B per
- * entry, made on first use; the ALUs take over when it does not fit); 1 =
+ * entry, made on first use; the ALUs take over when it does not fit, and take
+ * p = 1 and narrow blocks of p = 2 to 4); 1 =
  * matrix-free, H_e applied by sum factorisation over the tensor-product cell
  * (1-D mass / stiffness / Gauss-point factors, the alternative the paper notes
  * for the cell-level products), 3.2x (p = 6) to 5.5x (p = 8) fewer flops, on

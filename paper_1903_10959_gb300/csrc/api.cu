@@ -290,19 +290,41 @@ chfsi_status ensure_tc_data(chfsi_ctx* ctx, chfsi_precision prec) {
   return CHFSI_OK;
 }
 
-// Columns up to which a binary64 step stays on the matrix-free kernel: the
+// Whether a binary64 step stays on the ALUs because of its few columns: the
 // digit-slice kernel always computes 128-column tiles, so a narrow block wastes
 // them unless the whole launch is only a few tiles per SM (4^3 cells, p = 4, one
 // column: 0.045 ms against 0.168 ms in eight colour launches).  8^3 cells, p = 6:
 // matrix-free 0.42 ms (8 columns), 0.74 (12, 13), digit slices 0.51; 16^3 cells:
-// 2.9, 4.0, 5.0 against 3.8; 8^3 cells, p = 7: 0.62, 0.89, 1.72 (16) against 1.13.
-int narrow_columns(const chfsi_ctx* ctx) { return ctx->mesh.p >= 7 ? 15 : 12; }
-constexpr int64_t kFewTiles = 4 * 152;
-bool stays_matrix_free(const chfsi_ctx* ctx, int ncol) {
-  return use_matrix_free(ctx) &&
-         (ctx->fp64_op == 1 || (ncol <= narrow_columns(ctx) &&
-                                ex_cell_tiles(ctx->mesh.ncells, ctx->mesh.ne, ncol) > kFewTiles));
+// 2.9, 4.0, 5.0 against 3.8; 8^3 cells, p = 7: 0.62, 0.89, 1.72 (16) against 1.13
+// (p = 2 to 5 and 8 behave alike).
+//
+// Without the matrix-free form the alternative is the ALU kernel of the stored
+// matrices, n_e^2 products per column.  Against its 128 x 48 tiles of 16-deep chunks
+// small matrices count for little, so that p = 1 stays there at any width (8 of 48
+// rows; 31^3 cells, 1 and 200 columns: 0.17 and 1.23 ms against 1.16 and 3.00), p =
+// 2 up to 32 columns (33^3: 1.20 times as fast at 32, 1.02 at 48), p = 3 up to 16
+// (22^3: 1.15; 0.62 at 24), p = 4 up to two (17^3: 2.0 and 1.6; 0.51 at 4), p >= 7
+// for one (10^3, p = 7: 1.65), on a few thousand tiles about half of that (10^3, p =
+// 2: 1.03 to 1.06 from 4 to 12 columns, 0.77 at 32; 8^3, p = 4: 1.31, two columns
+// 0.94).  Up to 64 tiles per colour the launch of each colour costs more than the
+// tiles (8^3, p = 1, 8 colours: 1.06 times as fast, 6^3 0.8; 11^3, 27 colours: 0.55).
+bool narrow(const chfsi_ctx* ctx, int ncol) {
+  const HostMesh& m = ctx->mesh;
+  const int64_t tiles = ex_cell_tiles(m.ncells, m.ne, 1);
+  if (use_matrix_free(ctx)) return ncol <= (m.p >= 7 ? 15 : 12) && tiles > 4 * 152;
+  const bool many = tiles > 4096;
+  const int most = m.p == 1   ? ncol
+                   : m.p == 2 ? (many ? 32 : 16)
+                   : m.p == 3 ? (many ? 16 : 12)
+                   : m.p == 4 ? (many ? 2 : 1)
+                   : m.p >= 7 ? (many ? 1 : 0)
+                              : 0;
+  return ncol <= most && tiles > 64 * (int64_t)(m.colour_offsets.size() - 1);
 }
+bool stays_on_alus(const chfsi_ctx* ctx, int ncol) {
+  return (ctx->fp64_op == 1 && use_matrix_free(ctx)) || narrow(ctx, ncol);
+}
+constexpr int kNarrow = 32;   // no wider block of p >= 2 is a narrow one
 
 // The stream capture that s takes part in (0: none).
 uint64_t capture_id(cudaStream_t s) {
@@ -317,14 +339,14 @@ uint64_t capture_id(cudaStream_t s) {
 
 // Whether a binary64 step of ncol columns takes the digit-slice cell products
 // (kernels_ex.cu): the cell matrices are resident, the block is not one for the
-// matrix-free kernel, and the words of the matrices, of the block and its dense
+// ALUs, and the words of the matrices, of the block and its dense
 // cell blocks fit in memory.  Otherwise the colour-ordered ALU kernels run.
 // It takes its memory after the call's other buffers; a width whose scratch does not
 // fit stays on the ALUs until the next build or chfsi_autotune, and so does every
 // width once the words had to give way to another buffer.
 bool ensure_ex(chfsi_ctx* ctx, int ncol, int64_t* ldr) {
   const HostMesh& m = ctx->mesh;
-  if (!ctx->d_Ht || ctx->fp64_alu || ctx->ex_off || ncol >= ctx->ex_too_wide || stays_matrix_free(ctx, ncol)) return false;
+  if (!ctx->d_Ht || ctx->fp64_alu || ctx->ex_off || ncol >= ctx->ex_too_wide || stays_on_alus(ctx, ncol)) return false;
   *ldr = (ncol + 1) & ~1;
   if (!ctx->ex_ready) {
     ExCellData& d = ctx->ex;
@@ -349,10 +371,11 @@ bool ensure_ex(chfsi_ctx* ctx, int ncol, int64_t* ldr) {
       ctx->ex_ready = !capture;
     }
   }
-  // the partial sums of the narrow blocks that follow on the matrix-free kernel
-  // are allocated with the first block of any width, as one call always did
-  const int nw = std::min(ncol, narrow_columns(ctx));
-  if ((stays_matrix_free(ctx, nw) && !grow_optional(ctx, ctx->Wb, (size_t)m.ndofs * nw * sizeof(double))) ||
+  // the partial sums of the narrow blocks that follow on the ALUs are allocated with
+  // the first block of any width, as one call always did
+  int nw = std::min(ncol, kNarrow);
+  while (nw > 0 && !stays_on_alus(ctx, nw)) --nw;
+  if ((nw > 0 && !grow_optional(ctx, ctx->Wb, (size_t)m.ndofs * nw * sizeof(double))) ||
       !grow_optional(ctx, ctx->exb, ex_cell_work_bytes(m.ncells, m.ne, ncol)) ||
       !grow_optional(ctx, ctx->Rb, (size_t)m.ncells * m.ne * *ldr * sizeof(double))) {
     ctx->ex_too_wide = ncol;

@@ -125,3 +125,30 @@ def test_localised_columns():
         assert (np.abs(out["digits"] - out["alu"]) <= bound).all()
     finally:
         ctx.destroy()
+
+
+@pytest.mark.parametrize("p,cells,ncol,op,alu", [
+    (1, 14, 1, "default", True), (1, 14, 200, "default", True), (1, 5, 40, "default", False),
+    (2, 17, 32, "cells", True), (2, 17, 33, "cells", False), (2, 10, 16, "cells", True), (2, 10, 17, "cells", False),
+    (3, 17, 16, "cells", True), (3, 17, 17, "cells", False), (4, 12, 2, "cells", True), (4, 12, 3, "cells", False),
+    (5, 9, 1, "cells", False), (7, 8, 1, "cells", True), (7, 8, 2, "cells", False),
+    (4, 8, 12, "default", True), (4, 8, 13, "default", False)])
+def test_widths_that_stay_on_the_alus(p, cells, ncol, op, alu):
+    """Blocks for which the 128 x 48 tiles of the digit slices are a waste take the
+    same kernels as with the products on the ALUs, and so the same bits."""
+    ctx = Context(cells, 2.0 * cells, p)
+    ctx.set_potential_gaussians([[1.0, 2.0, 3.0]], [2.0], [0.9])
+    ctx.build()
+    try:
+        ctx.set_fp64_operator(op)
+        g = torch.Generator(DEV).manual_seed(6)
+        X = torch.randn((ctx.ndofs, ncol), device=DEV, generator=g, dtype=torch.float64)
+        Y, Z = torch.empty_like(X), torch.empty_like(X)
+        ctx.apply(X, Y)
+        ctx.set_fp64_products("alu")
+        ctx.apply(X, Z)
+        ctx.last_timings()
+        assert torch.equal(Y, Z) == alu
+        assert float((Y - Z).norm() / Z.norm()) <= 1e-13
+    finally:
+        ctx.destroy()
