@@ -2100,11 +2100,24 @@ static cudaError_t stream_launch(const RParams& P, cudaStream_t s) {
 // columns 520 and 587 us, but 12^3, p = 7, 1,100 columns 6.48 and 6.40 ms, and where
 // the projectors take more chunks than the nodes (6^3, p = 6) 87 and 83 ms, because
 // the rows of Z are looked up one chunk at a time.
-static int64_t stream_items(int64_t ncells, int ncol, int ne, int nt = 3, int64_t nl_chunks = 0) {
+// Cells of three row parts and more (p = 7, 8; the ring kernel has two or three)
+// stay with the ring kernel where the last of a few rounds of items is nearly empty
+// (5^3, p = 7, up to 128 columns, 2.5 items per SM: 82 us as rings, 92; 3^3, p = 8,
+// 330 columns, 2.1: 93 and 103) and where the second column tile is: a ring block of
+// few columns loads little, the stream kernel works a whole tile (FP16x2, 6^3, p = 7:
+// 129 columns 163 and 177 us a step, 160 156 and 163, 180 161 and 163; BF16x3 only
+// with unaligned rows, 11^3, p = 8, 129 columns 1,517 and 1,724 us, aligned 0.92 of
+// the ring kernel's time).
+static int64_t stream_items(int64_t ncells, int ncol, int ne, bool aligned, int nt = 3, int64_t nl_chunks = 0) {
   const int tiles = (ncol + 127) / 128;
-  const int64_t items = ncells * tiles * stream_plan(ne, false, nt).np;
+  const int64_t items = ncells * tiles * stream_plan(ne, false, nt).np, sms = stream_grid(INT64_MAX);
   if (nl_chunks > 0 && (ne > 343 || nl_chunks > ncells * ((ne + BF_KC - 1) / BF_KC))) return 0;
-  return items >= 2 * (int64_t)stream_grid(INT64_MAX) && (ne > 128 || tiles > 1) ? items : 0;
+  if (ne > 343) {
+    const int64_t rounds = (items + sms - 1) / sms;
+    if (rounds <= 6 && 100 * items < 85 * rounds * sms) return 0;
+    if (tiles == 2 && (nt == 2 ? ncol <= 160 : ncol <= 144 && !aligned)) return 0;
+  }
+  return items >= 2 * sms && (ne > 128 || tiles > 1) ? items : 0;
 }
 
 // ----------------------------------------------------------------- BF16x3 cell kernel, several column tiles per CTA
@@ -2518,6 +2531,7 @@ cudaError_t tc_cell_bf16_launch(const TcCellData& d, const TcApplyArgs& a, cudaS
   if (B.np * B.nh > d.mt * 128) return cudaErrorInvalidValue;   // parts stay inside the packed rows
   RParams P{reinterpret_cast<const float*>(d.bf), a.dofmap, a.Yin, a.R, a.ld_in, a.ncol, d.ne, d.mt,
             nk16, 1, nullptr, 0, 0, a.ldr, 0};
+  const bool aligned = (reinterpret_cast<uintptr_t>(a.Yin) & 15) == 0 && a.ld_in % 4 == 0;   // 16-byte rows of Y
   if (a.Z) {   // projector chunks: only the ring kernels take them
     if (!d.nl || !tc_cell_bf16_nl_ok(a.gather)) return cudaErrorInvalidValue;
     P.nlA = d.nl;
@@ -2529,7 +2543,7 @@ cudaError_t tc_cell_bf16_launch(const TcCellData& d, const TcApplyArgs& a, cudaS
   if (a.kG) {   // the Bloch block: the ring kernel with two-column pairs
     if (a.Z || (a.ncol & 1) || (a.ld_in & 1)) return cudaErrorInvalidValue;
     P.nlA = a.kG;
-    if ((P.nitems = stream_items(a.ncells, a.ncol, d.ne)) > 0) return stream_launch<false, 3, false, true>(P, s);
+    if ((P.nitems = stream_items(a.ncells, a.ncol, d.ne, aligned)) > 0) return stream_launch<false, 3, false, true>(P, s);
     static std::once_flag attrk;
     std::call_once(attrk, [] {
       cudaFuncSetAttribute(tc_cell_bf16_rings_kernel<2, 3, false, false, true>,
@@ -2544,7 +2558,7 @@ cudaError_t tc_cell_bf16_launch(const TcCellData& d, const TcApplyArgs& a, cudaS
     }
     return cudaGetLastError();
   }
-  if (a.gather == 2 && (P.nitems = stream_items(a.ncells, a.ncol, d.ne, 3, P.nlA ? d.nl_chunks : 0)) > 0)
+  if (a.gather == 2 && (P.nitems = stream_items(a.ncells, a.ncol, d.ne, aligned, 3, P.nlA ? d.nl_chunks : 0)) > 0)
     return P.nlA ? stream_launch<false, 3, true>(P, s) : stream_launch<false>(P, s);
   static std::once_flag attr;
   std::call_once(attr, [] {
@@ -2614,7 +2628,7 @@ cudaError_t tc_cell_f16_launch(const TcCellData& d, const TcApplyArgs& a, const 
   if (B.np * B.nh > d.mt * 128) return cudaErrorInvalidValue;
   RParams P{reinterpret_cast<const float*>(d.f16), a.dofmap, a.Yin, a.R, a.ld_in, a.ncol, d.ne, d.mt,
             nk16, 1, nullptr, 0, 0, a.ldr, 0, cmax, d.f16_inv};
-  if ((P.nitems = stream_items(a.ncells, a.ncol, d.ne, 2)) > 0) return stream_launch<false, 2>(P, s);
+  if ((P.nitems = stream_items(a.ncells, a.ncol, d.ne, true, 2)) > 0) return stream_launch<false, 2>(P, s);
   static std::once_flag attr;
   std::call_once(attr, [] {
     cudaFuncSetAttribute(tc_cell_bf16_rings_kernel<2, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
