@@ -2809,9 +2809,11 @@ __global__ void __launch_bounds__(256) tc_assemble_kernel(AssembleParams P) {
 // 8) takes 128 columns (a quad per lane) of every 8-th row group; each thread
 // keeps its quad's maximum over its rows, the block reduces over its 8 row
 // lanes and adds one atomicMax per column (binary32 bits of a non-negative
-// value order as unsigned integers).
+// value order as unsigned integers).  Bound by the loads in flight: eight blocks
+// share an SM (32 registers; the grid of cmax_row_blocks then runs at once), which
+// takes 72 us for 9^3 cells, p = 8, 20 columns where six (38 registers) take 112.
 template <bool NL>
-__global__ void __launch_bounds__(256) tc_assemble_cmax_kernel(AssembleParams P, uint32_t* __restrict__ cmax) {
+__global__ void __launch_bounds__(256, NL ? 6 : 8) tc_assemble_cmax_kernel(AssembleParams P, uint32_t* __restrict__ cmax) {
   const int nq = (P.ncol + 3) / 4;
   const int qd = blockIdx.x * 32 + threadIdx.x;
   float m[4] = {0.f, 0.f, 0.f, 0.f};
