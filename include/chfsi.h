@@ -311,7 +311,7 @@ chfsi_status chfsi_filter(chfsi_ctx* ctx, void* X, int64_t ldx, int ncol, int de
 /* CholGS (Algorithm CholGS): S = X^T X, S = L L^T, X <- X L^{-T}, in place on
  * X (M x n).  Returns CHFSI_ERR_NOT_SPD and leaves X unchanged when the
  * Cholesky factorisation (binary64, the library's own) meets a pivot that is
- * not positive. */
+ * not positive and finite. */
 chfsi_status chfsi_cholgs(chfsi_ctx* ctx, void* X, int64_t ldx, int n, chfsi_precision prec);
 
 /* Rayleigh-Ritz (Sec. 3.5): H^ = X^T H~ X, H^ Q = Q D (ascending, binary64

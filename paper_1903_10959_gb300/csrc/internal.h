@@ -247,7 +247,7 @@ cudaError_t launch_axpy2(double* w, const double* v, const double* vp, int64_t M
 cudaError_t launch_scal_copy(double* v, const double* w, int64_t M, double sc, cudaStream_t s);
 // S = L L^T (S: n x n column-major, lower triangle; L replaces it) and X = L^{-1}
 // (n x n, zero above the diagonal).  *info (device): 0, or the 1-based index of the
-// first pivot that is not positive (L and X are then undefined).
+// first pivot that is not positive and finite (L and X are then undefined).
 cudaError_t launch_chol_inverse(double* S, int n, double* X, int* info, cudaStream_t s);
 
 // nonlocal: Z (nproj x ncol) = C~ Y ; NL (M x ncol) = C~^T h Z

@@ -106,7 +106,7 @@ __device__ void factor_tile(const double (*P)[NB + 1], double (*V)[NB + 1], doub
   }
   const double d = V[lane][lane], rs = rsqrt(d);
   if (w == 0) {
-    const uint32_t bad = __ballot_sync(0xffffffffu, lane < nv && !(d > 0.0));
+    const uint32_t bad = __ballot_sync(0xffffffffu, lane < nv && (!(d > 0.0) || isinf(d)));
     if (lane == 0 && bad && *info == 0) *info = o + __ffs(bad);
   }
 #pragma unroll
