@@ -2086,7 +2086,8 @@ template <bool MULTI, int NT = 3, bool NLC = false, bool KPT = false>
 static cudaError_t stream_launch(const RParams& P, cudaStream_t s) {
   if (P.nitems <= 0) return cudaSuccess;
   const StreamPlan B = stream_plan(P.ne, MULTI, NT);
-  if (B.sy < stream_sets(MULTI)) return stream_launch_own<MULTI, NT, NLC, KPT, true>(P, B.total, s);
+  if constexpr (!MULTI)   // a batch has two sets, and every plan has two stages and more
+    if (B.sy < stream_sets(MULTI)) return stream_launch_own<MULTI, NT, NLC, KPT, true>(P, B.total, s);
   return stream_launch_own<MULTI, NT, NLC, KPT, false>(P, B.total, s);
 }
 

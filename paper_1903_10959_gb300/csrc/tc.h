@@ -54,8 +54,9 @@ struct TcApplyArgs {
   int ncol;
   const float* Yin;
   int64_t ld_in;
-  float* R;                 // dense cell blocks, rows of stride ldr (the ring kernel writes whole 16-byte
-  int64_t ldr;              //   quads when ldr is a multiple of 4: ldr >= ncol rounded up)
+  float* R;                 // dense cell blocks, rows of stride ldr >= ncol; with ldr a multiple of 4 the
+  int64_t ldr;              //   columns from ncol to the next one may hold anything (the assembly reads a
+                            //   ragged last quad whole and stores none of them)
   int split3;
   int tile = 64;            // columns per CTA of the cell kernel: 64 or 128
   int gather = 2;           // BF16x3: 2 = decoupled matrix / Y rings (with two items per SM and more the kernel
