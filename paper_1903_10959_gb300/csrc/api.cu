@@ -482,7 +482,7 @@ chfsi_status apply_step(chfsi_ctx* ctx, chfsi_precision prec, const void* Yin, i
     if (nl_in_cells && ctx->tc.pj) {
       if ((st = grow(ctx, ctx->pjb, (size_t)ctx->tc.pj_rows * ncol * sizeof(float))) != CHFSI_OK) return st;
       CK(tc_nl_project_cells(ctx->tc, ctx->d_dofmap, m.ncells, ctx->hproj.nsite, (const float*)Yin, ld_in,
-                             ncol, (float*)ctx->pjb.ptr, (float*)ctx->Zb.ptr, ctx->stream));
+                             ncol, (float*)ctx->pjb.ptr, (float*)ctx->Zb.ptr, ctx->watch.status, ctx->stream));
     } else {
       CK(tc_nl_project(ctx->d_site_ptr, ctx->d_site_dof, ctx->d_site_c32, ctx->hproj.nsite,
                        (const float*)Yin, ld_in, ncol, (float*)ctx->Zb.ptr, ctx->stream));
@@ -513,6 +513,7 @@ chfsi_status apply_step(chfsi_ctx* ctx, chfsi_precision prec, const void* Yin, i
   ra.ld_in = ld_in;
   ra.R = (float*)ctx->Rb.ptr;
   ra.ldr = ldr4;
+  ra.status = ctx->watch.status;
   ra.split3 = prec == CHFSI_MIXED_TF32X3;
   ra.tile = ctx->cell_tile;
   ra.gather = ctx->cell_gather;
@@ -577,9 +578,7 @@ chfsi_status check_x(chfsi_ctx* ctx, const void* X, int64_t ldx, int ncol, chfsi
 
 // Device-side bounded waits report through a status word; map it to an error.
 chfsi_status check_device_status(chfsi_ctx* ctx, chfsi_precision prec) {
-  const int v = is_mixed(prec) ? tc_read_status(ctx->stream) : 0;
-  if (v) return fail(ctx, CHFSI_ERR_TIMEOUT, "device wait timed out (site " + std::to_string(v) + ")");
-  if (ctx->ex_used) {
+  if (is_mixed(prec) || ctx->ex_used) {
     ctx->ex_used = false;
     CK(cudaStreamSynchronize(ctx->stream));
   }
@@ -788,7 +787,7 @@ chfsi_status gram_impl(chfsi_ctx* ctx, chfsi_precision prec, const void* A, int6
   if ((st = grow(ctx, ctx->part, want)) != CHFSI_OK) return st;
   CK(tc_gram_mixed((const float*)A, lda, (const float*)Bm, ldb, m.ndofs, n1, n2, C, ldc, lower,
                    ctx->diag_block, split3_of(prec), ctx->part.ptr, ctx->part.bytes,
-                   ctx->stream));
+                   ctx->watch.status, ctx->stream));
   return CHFSI_OK;
 }
 
@@ -826,7 +825,7 @@ chfsi_status rotate_impl(chfsi_ctx* ctx, chfsi_precision prec, void* X, int64_t 
     if ((st = grow(ctx, ctx->work, tc_tallgemm_work_bytes(n, n))) != CHFSI_OK) return st;
     CK(tc_tallgemm_mixed((const float*)X, ldx, U, n, m.ndofs, n, n, (float*)ctx->rot.ptr, n, upper,
                          trans, ctx->diag_block, split3_of(prec), ctx->work.ptr,
-                         ctx->stream, ctx->tall_kernel));
+                         ctx->watch.status, ctx->stream, ctx->tall_kernel));
   }
   CK(cudaMemcpy2DAsync(X, ldx * es, ctx->rot.ptr, n * es, n * es, m.ndofs, cudaMemcpyDeviceToDevice,
                        ctx->stream));
@@ -1677,7 +1676,7 @@ chfsi_status chfsi_rayleigh_ritz_split(chfsi_ctx* ctx, const void* X, int64_t ld
   } else {
     if ((st = grow(ctx, ctx->work, tc_tallgemm_work_bytes(n, n_fr))) != CHFSI_OK) return st;
     CK(tc_tallgemm_mixed((const float*)X, ldx, Hh, n, m.ndofs, n, n_fr, (float*)Xfr, ldfr, 0, 0, 0,
-                         split3_of(prec), ctx->work.ptr, ctx->stream, ctx->tall_kernel));
+                         split3_of(prec), ctx->work.ptr, ctx->watch.status, ctx->stream, ctx->tall_kernel));
   }
   toc(ctx, 2);
   return check_device_status(ctx, prec);

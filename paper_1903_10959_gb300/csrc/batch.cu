@@ -22,7 +22,6 @@ using namespace chfsi;
 
 namespace chfsi {
 
-__device__ int g_batch_status = 0;
 
 using BSys = TcBatchSys;
 
@@ -31,6 +30,7 @@ struct BParams {
   int nsys;
   int64_t nitems;
   int ne, mt, nk, split3, S, parity;
+  int* status;              // where a bounded wait that gives up reports
 };
 
 template <int BN>
@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(320, 1) tc_cell_batched_kernel(BParams P) {
         for (int i = 0; i < nk; ++i, ++gi) {
           const int s = (int)(gi % S);
           if (gi >= S && !mbar_wait(em(s), (uint32_t)((gi / S) - 1) & 1)) {
-            atomicExch(&g_batch_status, 1);
+            report_timeout(P.status, 1);
             *(volatile int*)abort_flag = 1;
             break;
           }
@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(320, 1) tc_cell_batched_kernel(BParams P) {
       for (int64_t it = 0; it < my_items && ok; ++it) {
         const int b = (int)(it & 1);
         if (it >= 2 && !mbar_wait(acce(b), (uint32_t)((it / 2) - 1) & 1)) {
-          atomicExch(&g_batch_status, 2);
+          report_timeout(P.status, 2);
           *(volatile int*)abort_flag = 1;
           break;
         }
@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(320, 1) tc_cell_batched_kernel(BParams P) {
           const int s = (int)(gi % S);
           const uint32_t par = (uint32_t)(gi / S) & 1;
           if (!mbar_wait(fa(s), par) || !mbar_wait(fy(s), par) || *(volatile int*)abort_flag) {
-            atomicExch(&g_batch_status, 3);
+            report_timeout(P.status, 3);
             *(volatile int*)abort_flag = 1;
             ok = false;
             break;
@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(320, 1) tc_cell_batched_kernel(BParams P) {
       if (more) load_chunk(gi + 4, vb);
       const int s = (int)(gi % S);
       if (gi >= S && !mbar_wait(em(s), (uint32_t)((gi / S) - 1) & 1)) {
-        atomicExch(&g_batch_status, 4);
+        report_timeout(P.status, 4);
         *(volatile int*)abort_flag = 1;
       }
       if (*(volatile int*)abort_flag) break;
@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(320, 1) tc_cell_batched_kernel(BParams P) {
       const int bne = I.ncv <= 16 ? 16 : (I.ncv + 15) / 16 * 16;
       const bool okw = !*(volatile int*)abort_flag && mbar_wait(accf(b), (uint32_t)(it / 2) & 1);
       if (!okw) {
-        atomicExch(&g_batch_status, 5);
+        report_timeout(P.status, 5);
         *(volatile int*)abort_flag = 1;
       }
       tc_fence_after();
@@ -428,6 +428,8 @@ struct chfsi_batch {
   // tile choice: BN (32 / 64) and stages; set by the autotuner
   int bn = 64, S = -1;             // S < 0: the non-persistent multi-system kernel
   int nsm = 0;
+  int* h_status = nullptr;      // where the bounded waits report (pinned), and the device's view of it
+  int* d_status = nullptr;
   std::string err;
 };
 
@@ -451,7 +453,7 @@ cudaError_t ensure_dbuf(DevBuf& d, size_t bytes) {
 
 template <int BN>
 cudaError_t launch_batched_cell(chfsi_batch* b, int split3, int S, int parity, cudaStream_t s) {
-  BParams P{b->d_sys, (int)b->ctx.size(), b->nitems, b->ne, b->mt, b->nk, split3, S, parity};
+  BParams P{b->d_sys, (int)b->ctx.size(), b->nitems, b->ne, b->mt, b->nk, split3, S, parity, b->d_status};
   const BLayout<BN> L = b_layout<BN>(b->mt, split3, S);
   const int grid = (int)std::min<int64_t>(b->nitems, b->nsm);
   note_launch();
@@ -554,9 +556,9 @@ cudaError_t batch_enqueue(chfsi_batch* b, float* const* X, const int* ncol, int 
   for (int k = 1; k <= degree; ++k) {
     const int parity = (k - 1) & 1;
     if (split3 == kBatchBf16x3)
-      e = tc_cell_bf16_multi_launch(b->d_sys, n, b->nitems, b->ne, b->mt, parity, b->stream);
+      e = tc_cell_bf16_multi_launch(b->d_sys, n, b->nitems, b->ne, b->mt, parity, b->d_status, b->stream);
     else if (S < 0)
-      e = tc_cell_multi_launch(b->d_sys, n, b->nitems, b->ne, b->mt, b->nk, split3, parity, b->stream);
+      e = tc_cell_multi_launch(b->d_sys, n, b->nitems, b->ne, b->mt, b->nk, split3, parity, b->d_status, b->stream);
     else
       e = bn == 64 ? launch_batched_cell<64>(b, split3, S, parity, b->stream)
                    : launch_batched_cell<32>(b, split3, S, parity, b->stream);
@@ -651,22 +653,12 @@ chfsi_status batch_prepare(chfsi_batch* b, float* const* X, const int64_t* ldx, 
   return CHFSI_OK;
 }
 
-int batch_read_status_persistent(cudaStream_t s);
-// Status words of both cell kernels (persistent batched, multi-system).
-int batch_read_status(cudaStream_t s) {
-  const int a = batch_read_status_persistent(s);
-  const int c = tc_read_status(s);
-  return a ? a : c;
-}
-int batch_read_status_persistent(cudaStream_t s) {
-  int v = 0;
-  cudaMemcpyFromSymbolAsync(&v, g_batch_status, sizeof(int), 0, cudaMemcpyDeviceToHost, s);
-  cudaStreamSynchronize(s);
-  if (v) {
-    int z = 0;
-    cudaMemcpyToSymbolAsync(g_batch_status, &z, sizeof(int), 0, cudaMemcpyHostToDevice, s);
-    cudaStreamSynchronize(s);
-  }
+// Read and clear the status word of the bounded waits (0: no timeout).
+int batch_read_status(chfsi_batch* b) {
+  cudaStreamSynchronize(b->stream);
+  volatile int* w = b->h_status;
+  const int v = *w;
+  if (v) *w = 0;
   return v;
 }
 
@@ -713,10 +705,14 @@ chfsi_status chfsi_batch_create(int n, chfsi_ctx* const* ctxs, void* stream, chf
   int dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&b->nsm, cudaDevAttrMultiProcessorCount, dev);
-  if (cudaMalloc(&b->d_sys, n * sizeof(BSys)) != cudaSuccess) {
-    delete b;
+  if (cudaMalloc(&b->d_sys, n * sizeof(BSys)) != cudaSuccess ||
+      cudaHostAlloc((void**)&b->h_status, sizeof(int), cudaHostAllocMapped) != cudaSuccess ||
+      cudaHostGetDevicePointer((void**)&b->d_status, b->h_status, 0) != cudaSuccess) {
+    cudaGetLastError();
+    chfsi_batch_destroy(b);
     return CHFSI_ERR_OOM;
   }
+  *(volatile int*)b->h_status = 0;
   *out = b;
   return CHFSI_OK;
 }
@@ -731,6 +727,7 @@ chfsi_status chfsi_batch_destroy(chfsi_batch* b) {
   if (b->d_sys) cudaFree(b->d_sys);
   if (b->d_coef) cudaFree(b->d_coef);
   if (b->h_coef) cudaFreeHost(b->h_coef);
+  if (b->h_status) cudaFreeHost(b->h_status);
   if (b->own_stream) cudaStreamDestroy(b->stream);
   delete b;
   return CHFSI_OK;
@@ -796,7 +793,7 @@ chfsi_status chfsi_batch_filter(chfsi_batch* b, float* const* X, const int64_t* 
   }
   cudaError_t e = cudaGraphLaunch(b->gexec, b->stream);
   if (e != cudaSuccess) return bfail(b, CHFSI_ERR_CUDA, cudaGetErrorString(e));
-  if (batch_read_status(b->stream)) return bfail(b, CHFSI_ERR_TIMEOUT, "device wait timed out");
+  if (batch_read_status(b)) return bfail(b, CHFSI_ERR_TIMEOUT, "device wait timed out");
   return CHFSI_OK;
 }
 
@@ -852,7 +849,7 @@ chfsi_status chfsi_batch_autotune(chfsi_batch* b, float* const* X, const int64_t
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (st != CHFSI_OK) return st;
-  if (batch_read_status(b->stream)) return bfail(b, CHFSI_ERR_TIMEOUT, "device wait timed out");
+  if (batch_read_status(b)) return bfail(b, CHFSI_ERR_TIMEOUT, "device wait timed out");
   b->bn = cand[bi].first;
   b->S = cand[bi].second;
   batch_free_graph(b);

@@ -324,10 +324,7 @@ __global__ void __launch_bounds__(EX_THREADS, 1) ex_kernel(const __grid_constant
   const int seg = MODE == EX_CELL && *P.hsum <= (1 << 24) - (1 << 18) ? 1 << 20 : SEG;   // chunks per segment
   // A role whose wait gives up records it and leaves; the waits of the roles
   // that depend on it then run out in turn, so that every warp reaches the end.
-  auto give_up = [&](int site) {
-    *(volatile int*)P.watch.status = site;
-    __threadfence_system();
-  };
+  auto give_up = [&](int site) { report_timeout(P.watch.status, site); };
 
   if (warp < 8) {
     // ---- drain: lane quarter warp % 4, N columns HN (warp / 4) ..

@@ -41,7 +41,6 @@ namespace chfsi {
 
 using namespace ptx;
 
-__device__ int g_tc_status = 0;   // nonzero after a bounded wait gave up
 // Test hook of the bounded waits (0 = off, the default): when set, gather warp
 // 0 of the first CTA of the BF16x3 cell kernel (the shared-ring and the
 // decoupled-ring forms) withholds its arrival on the first chunk's full
@@ -594,6 +593,7 @@ struct RParams {
   int pj_npmax;
   int tpc;                  // multi-tile kernel: column tiles per CTA
   int64_t nitems;           // stream kernel: (cell, column tile, row part) items
+  int* status;              // where a bounded wait that gives up reports
 };
 
 template <int BN, bool MULTI>
@@ -666,7 +666,7 @@ __global__ void __launch_bounds__(CELL_THREADS, 1) tc_cell_r_kernel(RParams P) {
       for (int i = 0; i < nk; ++i) {
         const int s = i % S;
         if (i >= S && !mbar_wait(em(s), ((i / S) - 1) & 1)) {
-          atomicExch(&g_tc_status, 21);
+          report_timeout(P.status, 21);
           *(volatile int*)abort_flag = 1;
           break;
         }
@@ -685,7 +685,7 @@ __global__ void __launch_bounds__(CELL_THREADS, 1) tc_cell_r_kernel(RParams P) {
         const int s = i % S;
         if (!mbar_wait(fa(s), (i / S) & 1) || !mbar_wait(fy(s), (i / S) & 1) ||
             *(volatile int*)abort_flag) {
-          atomicExch(&g_tc_status, 22);
+          report_timeout(P.status, 22);
           *(volatile int*)abort_flag = 1;
           break;
         }
@@ -749,7 +749,7 @@ __global__ void __launch_bounds__(CELL_THREADS, 1) tc_cell_r_kernel(RParams P) {
         const int s = i % S;
         load_chunk(i, v);
         if (i >= S && !mbar_wait(em(s), ((i / S) - 1) & 1)) {
-          atomicExch(&g_tc_status, 23);
+          report_timeout(P.status, 23);
           *(volatile int*)abort_flag = 1;
         }
         if (*(volatile int*)abort_flag) break;
@@ -774,7 +774,7 @@ __global__ void __launch_bounds__(CELL_THREADS, 1) tc_cell_r_kernel(RParams P) {
     // epilogue: TMEM row -> R row (16-byte stores only)
     const bool okacc = mbar_wait(accb, 0);
     if (!okacc) {
-      atomicExch(&g_tc_status, 24);
+      report_timeout(P.status, 24);
       *(volatile int*)abort_flag = 1;
     }
     tc_fence_after();
@@ -816,6 +816,7 @@ cudaError_t tc_cell_r_launch(const TcCellData& d, const TcApplyArgs& a, cudaStre
   const int bn = a.tile == 128 ? 128 : 64;
   RParams P{d.hi, a.dofmap, a.Yin, a.R, a.ld_in, a.ncol, d.ne, d.mt, d.kt / CELL_KC, a.split3,
             nullptr, 0, 0, a.ldr, 0};
+  P.status = a.status;
   tc_cell_prepare();
   const CellSmem L = cell_smem(d.mt, a.split3, bn);
   for (int64_t e0 = 0; e0 < a.ncells; e0 += 65535) {   // grid y is limited to 65535
@@ -841,10 +842,11 @@ void tc_cell_prepare() {
 }
 
 cudaError_t tc_cell_multi_launch(const TcBatchSys* d_sys, int nsys, int64_t nitems, int ne, int mt,
-                                 int nk, int split3, int parity, cudaStream_t s) {
+                                 int nk, int split3, int parity, int* status, cudaStream_t s) {
   if (nitems == 0 || nsys == 0) return cudaSuccess;
   if (nitems > 0x7fffffff) return cudaErrorInvalidValue;
   RParams P{nullptr, nullptr, nullptr, nullptr, 0, 0, ne, mt, nk, split3, d_sys, nsys, parity, 0, 0};
+  P.status = status;
   tc_cell_prepare();
   const CellSmem L = cell_smem(mt, split3, 64);
   note_launch();
@@ -971,7 +973,7 @@ __global__ void __launch_bounds__(CELL_THREADS, 2) tc_cell_bf16_kernel(RParams P
       for (int i = 0; i < nk; ++i) {
         const int s = i % S;
         if (i >= S && !mbar_wait(em(s), ((i / S) - 1) & 1)) {
-          atomicExch(&g_tc_status, 31);
+          report_timeout(P.status, 31);
           *(volatile int*)abort_flag = 1;
           break;
         }
@@ -993,7 +995,7 @@ __global__ void __launch_bounds__(CELL_THREADS, 2) tc_cell_bf16_kernel(RParams P
         const int s = i % S;
         if (!mbar_wait(fa(s), (i / S) & 1) || !mbar_wait(fy(s), (i / S) & 1) ||
             *(volatile int*)abort_flag) {
-          atomicExch(&g_tc_status, 32);
+          report_timeout(P.status, 32);
           *(volatile int*)abort_flag = 1;
           break;
         }
@@ -1038,7 +1040,7 @@ __global__ void __launch_bounds__(CELL_THREADS, 2) tc_cell_bf16_kernel(RParams P
         }
       }
       if (i >= S && !mbar_wait(em(s), ((i / S) - 1) & 1)) {
-        atomicExch(&g_tc_status, 33);
+        report_timeout(P.status, 33);
         *(volatile int*)abort_flag = 1;
       }
       if (*(volatile int*)abort_flag) break;
@@ -1061,7 +1063,7 @@ __global__ void __launch_bounds__(CELL_THREADS, 2) tc_cell_bf16_kernel(RParams P
     // for each row the warp's lanes store 32 consecutive floats
     const bool okacc = mbar_wait(accb, 0);
     if (!okacc) {
-      atomicExch(&g_tc_status, 34);
+      report_timeout(P.status, 34);
       *(volatile int*)abort_flag = 1;
     }
     tc_fence_after();
@@ -1175,7 +1177,7 @@ __global__ void __launch_bounds__(BFA_THREADS, 2) tc_cell_bf16_async_kernel(RPar
       if (lane == 0 && i >= SY) ok = mbar_wait(se(s), ((i / SY) - 1) & 1);
       ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
       if (!ok && lane == 0) {
-        atomicExch(&g_tc_status, 35);
+        report_timeout(P.status, 35);
         *(volatile int*)abort_flag = 1;
       }
       if (__shfl_sync(0xffffffffu, *(volatile int*)abort_flag, 0)) break;
@@ -1199,7 +1201,7 @@ __global__ void __launch_bounds__(BFA_THREADS, 2) tc_cell_bf16_async_kernel(RPar
       for (int i = 0; i < nk; ++i) {
         const int s = i % ST;
         if (i >= ST && !mbar_wait(em(s), ((i / ST) - 1) & 1)) {
-          atomicExch(&g_tc_status, 31);
+          report_timeout(P.status, 31);
           *(volatile int*)abort_flag = 1;
           break;
         }
@@ -1222,7 +1224,7 @@ __global__ void __launch_bounds__(BFA_THREADS, 2) tc_cell_bf16_async_kernel(RPar
         const int s = i % ST;
         if (!mbar_wait(fa(s), (i / ST) & 1) || !mbar_wait(fy(s), (i / ST) & 1) ||
             *(volatile int*)abort_flag) {
-          atomicExch(&g_tc_status, 32);
+          report_timeout(P.status, 32);
           *(volatile int*)abort_flag = 1;
           break;
         }
@@ -1256,7 +1258,7 @@ __global__ void __launch_bounds__(BFA_THREADS, 2) tc_cell_bf16_async_kernel(RPar
       bool ok = mbar_wait(sf(sl), (i / SY) & 1);
       if (ok && i >= ST) ok = mbar_wait(em(s), ((i / ST) - 1) & 1);
       if (!ok) {
-        atomicExch(&g_tc_status, 33);
+        report_timeout(P.status, 33);
         *(volatile int*)abort_flag = 1;
       }
       if (*(volatile int*)abort_flag) break;
@@ -1299,7 +1301,7 @@ __global__ void __launch_bounds__(BFA_THREADS, 2) tc_cell_bf16_async_kernel(RPar
     // epilogue (as tc_cell_bf16_kernel)
     const bool okacc = mbar_wait(accb, 0);
     if (!okacc) {
-      atomicExch(&g_tc_status, 34);
+      report_timeout(P.status, 34);
       *(volatile int*)abort_flag = 1;
     }
     tc_fence_after();
@@ -1445,7 +1447,7 @@ __global__ void __launch_bounds__((2 * NPAIR + 2) * 32, 2) tc_cell_bf16_rings_ke
       for (int i = 0; i < nkt; ++i) {
         const int s = i % SM;
         if (i >= SM && !mbar_wait(ea(s), ((i / SM) - 1) & 1)) {
-          atomicExch(&g_tc_status, 41);
+          report_timeout(P.status, 41);
           *(volatile int*)abort_flag = 1;
           break;
         }
@@ -1468,7 +1470,7 @@ __global__ void __launch_bounds__((2 * NPAIR + 2) * 32, 2) tc_cell_bf16_rings_ke
         const int sa = i % SM, sy = i % SY;
         if (!mbar_wait(fa(sa), (i / SM) & 1) || !mbar_wait(fy(sy), (i / SY) & 1) ||
             *(volatile int*)abort_flag) {
-          atomicExch(&g_tc_status, 42);
+          report_timeout(P.status, 42);
           *(volatile int*)abort_flag = 1;
           break;
         }
@@ -1534,7 +1536,7 @@ __global__ void __launch_bounds__((2 * NPAIR + 2) * 32, 2) tc_cell_bf16_rings_ke
         }
       }
       if (i >= SY && !mbar_wait(ey(s), ((i / SY) - 1) & 1)) {
-        atomicExch(&g_tc_status, 43);
+        report_timeout(P.status, 43);
         *(volatile int*)abort_flag = 1;
       }
       if (*(volatile int*)abort_flag) return false;
@@ -1567,7 +1569,7 @@ __global__ void __launch_bounds__((2 * NPAIR + 2) * 32, 2) tc_cell_bf16_rings_ke
     if (warp < 4) {
     const bool okacc = mbar_wait(accb, 0);
     if (!okacc) {
-      atomicExch(&g_tc_status, 44);
+      report_timeout(P.status, 44);
       *(volatile int*)abort_flag = 1;
     }
     tc_fence_after();
@@ -1716,7 +1718,7 @@ __global__ void __launch_bounds__(stream_threads(MULTI), 1) tc_cell_bf16_stream_
   const uint32_t tmem_y = tmem + 2 * B.nh;
   const int64_t term_bytes = (int64_t)P.mt * 4096;
   auto give_up = [&](int code) {
-    atomicExch(&g_tc_status, code);
+    report_timeout(P.status, code);
     *(volatile int*)abort_flag = 1;
   };
   int ib = 0, iph = 0;                       // item buffer, its phase
@@ -2204,7 +2206,7 @@ __global__ void __launch_bounds__((2 * NPAIR + 6) * 32, NACC == 1 ? 2 : 1) tc_ce
       for (int g = 0; g < G; ++g) {
         const int q = g % SM, i = g % nk;
         if (g >= SM && !mbar_wait(ea(q), ((g / SM) - 1) & 1)) {
-          atomicExch(&g_tc_status, 51);
+          report_timeout(P.status, 51);
           *(volatile int*)abort_flag = 1;
           break;
         }
@@ -2226,7 +2228,7 @@ __global__ void __launch_bounds__((2 * NPAIR + 6) * 32, NACC == 1 ? 2 : 1) tc_ce
       for (int t = 0; t < nt && ok; ++t) {
         const int b = t % NACC;   // accumulator of tile t
         if (t >= NACC && !mbar_wait(tmeb(b), ((t / NACC) - 1) & 1)) {   // drained tile t - NACC
-          atomicExch(&g_tc_status, 52);
+          report_timeout(P.status, 52);
           *(volatile int*)abort_flag = 1;
           break;
         }
@@ -2237,7 +2239,7 @@ __global__ void __launch_bounds__((2 * NPAIR + 6) * 32, NACC == 1 ? 2 : 1) tc_ce
           const int sa = g % SM, sy = g % SY;
           if (!mbar_wait(fa(sa), (g / SM) & 1) || !mbar_wait(fy(sy), (g / SY) & 1) ||
               *(volatile int*)abort_flag) {
-            atomicExch(&g_tc_status, 53);
+            report_timeout(P.status, 53);
             *(volatile int*)abort_flag = 1;
             ok = false;
             break;
@@ -2284,7 +2286,7 @@ __global__ void __launch_bounds__((2 * NPAIR + 6) * 32, NACC == 1 ? 2 : 1) tc_ce
         }
       }
       if (g >= SY && !mbar_wait(ey(s), ((g / SY) - 1) & 1)) {
-        atomicExch(&g_tc_status, 54);
+        report_timeout(P.status, 54);
         *(volatile int*)abort_flag = 1;
       }
       if (*(volatile int*)abort_flag) break;
@@ -2310,7 +2312,7 @@ __global__ void __launch_bounds__((2 * NPAIR + 6) * 32, NACC == 1 ? 2 : 1) tc_ce
       const int b = t % NACC;
       const bool okacc = mbar_wait(accb(b), (t / NACC) & 1);
       if (!okacc) {
-        atomicExch(&g_tc_status, 55);
+        report_timeout(P.status, 55);
         *(volatile int*)abort_flag = 1;
       }
       tc_fence_after();
@@ -2418,7 +2420,7 @@ __global__ void __launch_bounds__(BFW_THREADS, 1) tc_cell_bf16_whole_kernel(RPar
       for (int i = 0; i < nk; ++i) {
         const int s = i % SM;
         if (i >= SM && !mbar_wait(ea(s), ((i / SM) - 1) & 1)) {
-          atomicExch(&g_tc_status, 51);
+          report_timeout(P.status, 51);
           *(volatile int*)abort_flag = 1;
           break;
         }
@@ -2440,7 +2442,7 @@ __global__ void __launch_bounds__(BFW_THREADS, 1) tc_cell_bf16_whole_kernel(RPar
         const int sa = i % SM, sy = i % SY;
         if (!mbar_wait(fa(sa), (i / SM) & 1) || !mbar_wait(fy(sy), (i / SY) & 1) ||
             *(volatile int*)abort_flag) {
-          atomicExch(&g_tc_status, 52);
+          report_timeout(P.status, 52);
           *(volatile int*)abort_flag = 1;
           break;
         }
@@ -2486,7 +2488,7 @@ __global__ void __launch_bounds__(BFW_THREADS, 1) tc_cell_bf16_whole_kernel(RPar
         }
       }
       if (i >= SY && !mbar_wait(ey(s), ((i / SY) - 1) & 1)) {
-        atomicExch(&g_tc_status, 53);
+        report_timeout(P.status, 53);
         *(volatile int*)abort_flag = 1;
       }
       if (*(volatile int*)abort_flag) break;
@@ -2508,7 +2510,7 @@ __global__ void __launch_bounds__(BFW_THREADS, 1) tc_cell_bf16_whole_kernel(RPar
     // epilogue: part h = warp / 4, TMEM lane quarter = warp % 4 (column c0 + 32 (warp % 4) + lane)
     const bool okacc = mbar_wait(accb, 0);
     if (!okacc) {
-      atomicExch(&g_tc_status, 54);
+      report_timeout(P.status, 54);
       *(volatile int*)abort_flag = 1;
     }
     tc_fence_after();
@@ -2532,6 +2534,7 @@ cudaError_t tc_cell_bf16_launch(const TcCellData& d, const TcApplyArgs& a, cudaS
   if (B.np * B.nh > d.mt * 128) return cudaErrorInvalidValue;   // parts stay inside the packed rows
   RParams P{reinterpret_cast<const float*>(d.bf), a.dofmap, a.Yin, a.R, a.ld_in, a.ncol, d.ne, d.mt,
             nk16, 1, nullptr, 0, 0, a.ldr, 0};
+  P.status = a.status;
   const bool aligned = (reinterpret_cast<uintptr_t>(a.Yin) & 15) == 0 && a.ld_in % 4 == 0;   // 16-byte rows of Y
   if (a.Z) {   // projector chunks: only the ring kernels take them
     if (!d.nl || !tc_cell_bf16_nl_ok(a.gather)) return cudaErrorInvalidValue;
@@ -2629,6 +2632,7 @@ cudaError_t tc_cell_f16_launch(const TcCellData& d, const TcApplyArgs& a, const 
   if (B.np * B.nh > d.mt * 128) return cudaErrorInvalidValue;
   RParams P{reinterpret_cast<const float*>(d.f16), a.dofmap, a.Yin, a.R, a.ld_in, a.ncol, d.ne, d.mt,
             nk16, 1, nullptr, 0, 0, a.ldr, 0, cmax, d.f16_inv};
+  P.status = a.status;
   if ((P.nitems = stream_items(a.ncells, a.ncol, d.ne, true, 2)) > 0) return stream_launch<false, 2>(P, s);
   static std::once_flag attr;
   std::call_once(attr, [] {
@@ -2646,12 +2650,14 @@ cudaError_t tc_cell_f16_launch(const TcCellData& d, const TcApplyArgs& a, const 
 }
 
 cudaError_t tc_nl_project_cells(const TcCellData& d, const int32_t* dofmap, int64_t ncells, int nsite,
-                                const float* Y, int64_t ldy, int ncol, float* part, float* Z, cudaStream_t s) {
+                                const float* Y, int64_t ldy, int ncol, float* part, float* Z, int* status,
+                                cudaStream_t s) {
   if (ncells == 0 || ncol == 0 || nsite == 0) return cudaSuccess;
   if (!d.pj) return cudaErrorInvalidValue;
   const int nk16 = (d.ne + BF_KC - 1) / BF_KC;
   RParams P{reinterpret_cast<const float*>(d.pj), dofmap, Y, part, ldy, ncol, d.ne, d.mt, nk16, 1, nullptr, 0, 0,
             ncol, 0};
+  P.status = status;
   P.pj_np = d.pj_np;
   P.pj_off = d.pj_off;
   P.pj_row = d.pj_row;
@@ -2680,11 +2686,12 @@ cudaError_t tc_nl_project_cells(const TcCellData& d, const int32_t* dofmap, int6
 int tc_bf16_parts(int ne) { return stream_plan(ne, true).np; }
 
 cudaError_t tc_cell_bf16_multi_launch(const TcBatchSys* d_sys, int nsys, int64_t nitems, int ne, int mt,
-                                      int parity, cudaStream_t s) {
+                                      int parity, int* status, cudaStream_t s) {
   if (nitems == 0 || nsys == 0) return cudaSuccess;
   if (nitems > 0x7fffffff) return cudaErrorInvalidValue;
   const int nk16 = (ne + BF_KC - 1) / BF_KC;
   RParams P{nullptr, nullptr, nullptr, nullptr, 0, 0, ne, mt, nk16, 1, d_sys, nsys, parity, 0, 0};
+  P.status = status;
   P.nitems = nitems;
   return stream_launch<true>(P, s);
 }
@@ -2931,18 +2938,6 @@ cudaError_t tc_set_withhold(int on, cudaStream_t s) {
   return e;
 }
 
-int tc_read_status(cudaStream_t s) {
-  int v = 0;
-  cudaMemcpyFromSymbolAsync(&v, g_tc_status, sizeof(int), 0, cudaMemcpyDeviceToHost, s);
-  cudaStreamSynchronize(s);
-  if (v) {
-    int z = 0;
-    cudaMemcpyToSymbolAsync(g_tc_status, &z, sizeof(int), 0, cudaMemcpyHostToDevice, s);
-    cudaStreamSynchronize(s);
-  }
-  return v;
-}
-
 // ----------------------------------------------------------------- Gram (A^T B)
 constexpr int GR_T = 128, GR_KC = 8, GR_THREADS = 160, GR_S = 6;
 static_assert(GR_S >= 4, "parity waits of the 4 producer warps need at least 4 stages");
@@ -2958,6 +2953,7 @@ struct GramParams {
   int n1, n2, lower, split3;
   int64_t rows_per_split;
   double* partial;
+  int* status;
 };
 
 // (row n, K index k) of a 128 x 8 operand block, K-major core matrices:
@@ -3045,7 +3041,7 @@ __global__ void __launch_bounds__(GR_THREADS, 1) tc_gram_kernel(GramParams P) {
       for (int i = 0; i < nk; ++i) {
         const int s = i % S;
         if (!mbar_wait(full(s), (i / S) & 1) || *(volatile int*)abort_flag) {
-          atomicExch(&g_tc_status, 5);
+          report_timeout(P.status, 5);
           *(volatile int*)abort_flag = 1;
           break;
         }
@@ -3081,7 +3077,7 @@ __global__ void __launch_bounds__(GR_THREADS, 1) tc_gram_kernel(GramParams P) {
     auto fill_stage = [&](int i, const float (&va)[2][4][4], const float (&vb)[2][4][4]) -> bool {
       const int s = i % S;
       if (i >= S && !mbar_wait(emp(s), ((i / S) - 1) & 1)) {
-        atomicExch(&g_tc_status, 6);
+        report_timeout(P.status, 6);
         *(volatile int*)abort_flag = 1;
       }
       if (*(volatile int*)abort_flag) return false;
@@ -3106,7 +3102,7 @@ __global__ void __launch_bounds__(GR_THREADS, 1) tc_gram_kernel(GramParams P) {
     bool okacc = true;
     if (nk > 0) {
       okacc = mbar_wait(accb, 0);
-      if (!okacc) atomicExch(&g_tc_status, 7);
+      if (!okacc) report_timeout(P.status, 7);
     }
     tc_fence_after();
     // epilogue: thread row i = ti*128 + warp*32 + lane; consecutive lanes write
@@ -3281,7 +3277,7 @@ int64_t tc_gram_splits(int64_t tiles, int64_t max_split, int64_t slots) {
 
 cudaError_t tc_gram_mixed(const float* A, int64_t lda, const float* B, int64_t ldb, int64_t M,
                           int n1, int n2, double* C, int64_t ldc, int lower, int diag_block,
-                          int split3, void* partial, size_t partial_bytes, cudaStream_t s) {
+                          int split3, void* partial, size_t partial_bytes, int* status, cudaStream_t s) {
   if (n1 == 0 || n2 == 0) return cudaSuccess;
   const int t1 = (n1 + GR_T - 1) / GR_T, t2 = (n2 + GR_T - 1) / GR_T;
   const int64_t tiles = lower ? (int64_t)t1 * (t1 + 1) / 2 : (int64_t)t1 * t2;
@@ -3291,7 +3287,7 @@ cudaError_t tc_gram_mixed(const float* A, int64_t lda, const float* B, int64_t l
   int64_t nsplit = tc_gram_splits(tiles, max_split, 2 * 152);
   int64_t rps = ((M + nsplit - 1) / nsplit + GR_KC - 1) / GR_KC * GR_KC;
   nsplit = (M + rps - 1) / rps;
-  GramParams P{A, B, lda, ldb, M, n1, n2, lower, split3, rps, (double*)partial};
+  GramParams P{A, B, lda, ldb, M, n1, n2, lower, split3, rps, (double*)partial, status};
   const int smem = GR_S * gram_stage_bytes(0) + 1024;
   static std::once_flag attr;
   std::call_once(attr, [&] {
@@ -3420,6 +3416,7 @@ struct TallParams {
   int n1, n2, upper, trans, bd, split3;
   float* C;
   int64_t ldc;
+  int* status;
 };
 
 __global__ void __launch_bounds__(TG_THREADS, 1) tc_tall_kernel(TallParams P) {
@@ -3466,7 +3463,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1) tc_tall_kernel(TallParams P) {
       for (int i = 0; i < nk; ++i) {
         const int s = i % S;
         if (!mbar_wait(full(s), (i / S) & 1) || *(volatile int*)abort_flag) {
-          atomicExch(&g_tc_status, 8);
+          report_timeout(P.status, 8);
           *(volatile int*)abort_flag = 1;
           break;
         }
@@ -3517,7 +3514,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1) tc_tall_kernel(TallParams P) {
         }
       }
       if (i >= S && !mbar_wait(emp(s), ((i / S) - 1) & 1)) {
-        atomicExch(&g_tc_status, 9);
+        report_timeout(P.status, 9);
         *(volatile int*)abort_flag = 1;
       }
       if (*(volatile int*)abort_flag) break;
@@ -3556,7 +3553,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1) tc_tall_kernel(TallParams P) {
     bool okacc = true;
     if (nk > 0) {
       okacc = mbar_wait(accb, 0);
-      if (!okacc) atomicExch(&g_tc_status, 10);
+      if (!okacc) report_timeout(P.status, 10);
     }
     tc_fence_after();
     const bool run = __all_sync(0xffffffffu, okacc && !*(volatile int*)abort_flag);
@@ -3727,7 +3724,7 @@ __global__ void __launch_bounds__(TW_THREADS, 1) tc_tall_wide_kernel(TallParams 
       for (int i = 0; i < nk; ++i) {
         const int s = i % S;
         if (!mbar_wait(full(s), (i / S) & 1) || *(volatile int*)abort_flag) {
-          atomicExch(&g_tc_status, 11);
+          report_timeout(P.status, 11);
           *(volatile int*)abort_flag = 1;
           break;
         }
@@ -3786,7 +3783,7 @@ __global__ void __launch_bounds__(TW_THREADS, 1) tc_tall_wide_kernel(TallParams 
     auto fill_stage = [&](int i, const float4 (&av)[4][2]) -> bool {
       const int s = i % S;
       if (i >= S && !mbar_wait(emp(s), ((i / S) - 1) & 1)) {
-        atomicExch(&g_tc_status, 12);
+        report_timeout(P.status, 12);
         *(volatile int*)abort_flag = 1;
       }
       if (*(volatile int*)abort_flag) return false;
@@ -3835,7 +3832,7 @@ __global__ void __launch_bounds__(TW_THREADS, 1) tc_tall_wide_kernel(TallParams 
     bool okacc = true;
     if (nk > 0) {
       okacc = mbar_wait(accb, 0);
-      if (!okacc) atomicExch(&g_tc_status, 13);
+      if (!okacc) report_timeout(P.status, 13);
     }
     tc_fence_after();
     const bool run = __all_sync(0xffffffffu, okacc && !*(volatile int*)abort_flag);
@@ -3895,7 +3892,7 @@ __global__ void __launch_bounds__(TW_THREADS, 1) tc_tall_wide_kernel(TallParams 
 
 cudaError_t tc_tallgemm_mixed(const float* A, int64_t lda, const double* U, int64_t ldu, int64_t M,
                               int n1, int n2, float* C, int64_t ldc, int upper, int trans,
-                              int diag_block, int split3, void* work, cudaStream_t s, int kernel) {
+                              int diag_block, int split3, void* work, int* status, cudaStream_t s, int kernel) {
   if (M == 0 || n2 == 0) return cudaSuccess;
   const int nkc = (n1 + TG_KC - 1) / TG_KC;
   const int ntile = (n2 + TG_T - 1) / TG_T;
@@ -3916,7 +3913,7 @@ cudaError_t tc_tallgemm_mixed(const float* A, int64_t lda, const double* U, int6
     note_launch();
     tc_splitu_w_kernel<<<(unsigned)((totw + 255) / 256), 256, 0, s>>>(U, ldu, n1, n2, upper, trans, bd, bw,
                                                                      Us);
-    TallParams P{A, lda, M, Us, Ud, ldu, n1, n2, upper, trans, bd, split3, C, ldc};
+    TallParams P{A, lda, M, Us, Ud, ldu, n1, n2, upper, trans, bd, split3, C, ldc, status};
     const int smem = TW_S * tw_stage_bytes(256) + 1024;
     static std::once_flag attrw;
     std::call_once(attrw, [&] {
@@ -3930,7 +3927,7 @@ cudaError_t tc_tallgemm_mixed(const float* A, int64_t lda, const double* U, int6
   const int64_t tot = (int64_t)ntile * nkc * TG_T * TG_KC;
   note_launch();
   tc_splitu_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(U, ldu, n1, n2, upper, trans, bd, Us);
-  TallParams P{A, lda, M, Us, Ud, ldu, n1, n2, upper, trans, bd, split3, C, ldc};
+  TallParams P{A, lda, M, Us, Ud, ldu, n1, n2, upper, trans, bd, split3, C, ldc, status};
   const int smem = TG_S * (2 * TG_T * TG_KC * 4 * 2) + 1024;
   static std::once_flag attr;
   std::call_once(attr, [&] {

@@ -228,6 +228,7 @@ chfsi_status kapply_mixed(chfsi_ctx* ctx, const float* Yin, int64_t ld_in, float
   ra.ld_in = ld_in;
   ra.R = (float*)ctx->kY.ptr;
   ra.ldr = ldr;
+  ra.status = ctx->watch.status;
   ra.split3 = 1;
   ra.gather = 2;
   ra.kG = ctx->kgbf;
@@ -599,8 +600,8 @@ chfsi_status chfsi_solve_kpoint_prec(chfsi_ctx* ctx, double* X, int64_t ldx, int
     if ((st = kcholgs(ctx, X, ldx, n)) != CHFSI_OK) return st;
     if ((st = krr(ctx, X, ldx, n, D.data())) != CHFSI_OK) return st;
   }
-  if (tc_read_status(ctx->stream)) return kfail(ctx, CHFSI_ERR_TIMEOUT, "device wait timed out");
   KK(cudaStreamSynchronize(ctx->stream));
+  if ((st = late_timeout(ctx)) != CHFSI_OK) return st;
   std::memcpy(evals_host, D.data(), (size_t)n * 8);
   return CHFSI_OK;
 }

@@ -58,6 +58,8 @@ struct TcApplyArgs {
   int64_t ldr;              //   columns from ncol to the next one may hold anything (the assembly reads a
                             //   ragged last quad whole and stores none of them)
   int split3;
+  int* status;              // where a bounded wait that gives up reports: a word of the context's (or batch's)
+                            // own in host memory that the device can write
   int tile = 64;            // columns per CTA of the cell kernel: 64 or 128
   int gather = 2;           // BF16x3: 2 = decoupled matrix / Y rings (with two items per SM and more the kernel
                             // of one block per SM), 0 = one shared ring, 1 = rows staged by
@@ -88,7 +90,8 @@ cudaError_t tc_pack_proj(TcCellData& d, int64_t ncells, int nsite, const int32_t
 // tensor cores: per cell the partial sums of its owned rows (a ring-kernel
 // launch into part, pj_rows x ncol), then the per-site sums in a fixed order.
 cudaError_t tc_nl_project_cells(const TcCellData& d, const int32_t* dofmap, int64_t ncells, int nsite,
-                                const float* Y, int64_t ldy, int ncol, float* part, float* Z, cudaStream_t s);
+                                const float* Y, int64_t ldy, int ncol, float* part, float* Z, int* status,
+                                cudaStream_t s);
 // Pack the projector chunks (from build_nl_cells: nnz entries at nz_pos) into d.nl.
 cudaError_t tc_pack_nl(TcCellData& d, const int32_t* chunk_off, int64_t ncells, const int32_t* zrow,
                        const int64_t* nz_pos, const double* nz_val, int64_t nnz, cudaStream_t s,
@@ -114,12 +117,12 @@ struct TcBatchSys {
 // batch in one launch (items of system s start at sys[s].item0, tiles fastest);
 // Y[parity] of each system is the input.  All systems share n_e / mt / nk.
 cudaError_t tc_cell_multi_launch(const TcBatchSys* d_sys, int nsys, int64_t nitems, int ne, int mt,
-                                 int nk, int split3, int parity, cudaStream_t s);
+                                 int nk, int split3, int parity, int* status, cudaStream_t s);
 // The BF16x3 cell kernel over the (cell, 128-column tile, row part) items of
 // every system (A = each system's packed BF16x3 copy, tiles = column tiles x
 // tc_bf16_parts(ne)); Y[parity] is the input.
 cudaError_t tc_cell_bf16_multi_launch(const TcBatchSys* d_sys, int nsys, int64_t nitems, int ne, int mt,
-                                      int parity, cudaStream_t s);
+                                      int parity, int* status, cudaStream_t s);
 int tc_bf16_parts(int ne);
 // Set the cell kernels' shared-memory attributes (before any stream capture).
 void tc_cell_prepare();
@@ -170,8 +173,6 @@ cudaError_t tc_cell_bf16_launch(const TcCellData& d, const TcApplyArgs& a, cudaS
 // Split the binary64 device cell matrices into the TF32 hi / lo operand layout.
 cudaError_t tc_pack_from_device(TcCellData& d, const double* dHt, cudaStream_t s,
                                 int64_t* dev_bytes);
-// Read and clear the device status word of the bounded waits (0: no timeout).
-int tc_read_status(cudaStream_t s);
 // Test hook: withhold one gather arrival in the BF16x3 cell kernel (see kernels_tc.cu).
 cudaError_t tc_set_withhold(int on, cudaStream_t s);
 size_t tc_tallgemm_work_bytes(int n1, int n2);
@@ -179,11 +180,12 @@ void tc_free(TcCellData& d);
 size_t tc_gram_partial_bytes(int64_t M, int n1, int n2);
 cudaError_t tc_gram_mixed(const float* A, int64_t lda, const float* B, int64_t ldb, int64_t M,
                           int n1, int n2, double* C, int64_t ldc, int lower, int diag_block,
-                          int split3, void* partial, size_t partial_bytes, cudaStream_t s);
+                          int split3, void* partial, size_t partial_bytes, int* status, cudaStream_t s);
 // kernel: -1 chooses by size, 0 the 128 x 128 tile kernel, 1 the 256-row tile kernel.
 cudaError_t tc_tallgemm_mixed(const float* A, int64_t lda, const double* U, int64_t ldu, int64_t M,
                               int n1, int n2, float* C, int64_t ldc, int upper, int trans,
-                              int diag_block, int split3, void* work, cudaStream_t s, int kernel = -1);
+                              int diag_block, int split3, void* work, int* status, cudaStream_t s,
+                              int kernel = -1);
 cudaError_t tc_nl_project(const int64_t* site_ptr, const int32_t* site_dof, const float* site_c,
                           int nsite, const float* Y, int64_t ldy, int ncol, float* Z,
                           cudaStream_t s);

@@ -61,6 +61,12 @@ __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
+// Reports a wait that gave up to the host: `word` is host memory that the device
+// can write.
+__device__ __forceinline__ void report_timeout(int* word, int site) {
+  *(volatile int*)word = site;
+  __threadfence_system();
+}
 // Bounded wait on the phase with the given parity.  Returns false on timeout.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
   if (mbar_try_wait(bar, parity)) return true;

@@ -1,11 +1,14 @@
-"""Bounded device waits of the binary64 digit-slice kernels: a withheld arrival
-(test hook chfsi_debug_withhold_arrival) makes the waits of one launch run out
-after 2 s; the kernel drains and frees its tensor memory, and the context it ran
-for, and no other, reports CHFSI_ERR_TIMEOUT and stays usable.
+"""Bounded device waits of contexts side by side, in the binary64 digit-slice
+kernels and in the mixed precisions: a withheld arrival (test hook
+chfsi_debug_withhold_arrival) makes the waits of one launch run out after 2 s; the
+kernel drains and frees its tensor memory, and the context it ran for, and no
+other, reports CHFSI_ERR_TIMEOUT and stays usable.
 
 Tolerances: 1e-13 for a binary64 application against the oracle, as the other
 binary64 tests have it; equal bits for the same launches on the same data.
 """
+import threading
+
 import pytest
 import torch
 
@@ -104,3 +107,37 @@ def test_synchronous_calls(pair, call):
     b.apply(X, Y)
     b.last_timings()
     assert rel_fro(Y.cpu().numpy(), ref) <= 1e-13
+
+
+def test_mixed_precisions_beside_another_context(pair):
+    """A BF16x3 application whose wait runs out in one thread; a context in another
+    keeps applying 3xTF32 products, which synchronise and check."""
+    a, b, X, ref = pair
+    x = X.float()
+    y, z = torch.empty_like(x), torch.empty_like(x)
+    b.apply(x, y, prec="bf16x3")                     # packs the cell data
+    a.apply(x, z, prec="mixed")
+    raised = []
+
+    def wait_in_vain():
+        try:
+            b.apply(x, y, prec="bf16x3")
+        except ChfsiError as e:
+            raised.append(e.status)
+
+    b.debug_withhold_arrival(True)
+    t = threading.Thread(target=wait_in_vain)
+    try:
+        t.start()
+        calls = 0
+        while t.is_alive():
+            a.apply(x, z, prec="mixed")              # no error of the other context's
+            calls += 1
+    finally:
+        t.join()
+        b.debug_withhold_arrival(False)
+    a.apply(x, z, prec="mixed")
+    assert raised == [TIMEOUT] and calls > 10
+    b.apply(x, y, prec="bf16x3")
+    assert rel_fro(y.double().cpu().numpy(), ref) < 1e-5
+    assert rel_fro(z.double().cpu().numpy(), ref) < 1e-5
