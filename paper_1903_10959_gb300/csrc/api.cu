@@ -326,17 +326,6 @@ bool stays_on_alus(const chfsi_ctx* ctx, int ncol) {
 }
 constexpr int kNarrow = 32;   // no wider block of p >= 2 is a narrow one
 
-// The stream capture that s takes part in (0: none).
-uint64_t capture_id(cudaStream_t s) {
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  unsigned long long id = 0;
-  if (cudaStreamGetCaptureInfo(s, &cs, &id) != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
-  return cs == cudaStreamCaptureStatusActive ? (uint64_t)id + 1 : 0;
-}
-
 // Whether a binary64 step of ncol columns takes the digit-slice cell products
 // (kernels_ex.cu): the cell matrices are resident, the block is not one for the
 // ALUs, and the words of the matrices, of the block and its dense
@@ -1063,6 +1052,16 @@ cudaError_t noalloc_scratch(chfsi_ctx* ctx, void** out) {
 
 // ===================================================================== C ABI
 namespace chfsi {
+uint64_t capture_id(cudaStream_t s) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  unsigned long long id = 0;
+  if (cudaStreamGetCaptureInfo(s, &cs, &id) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return cs == cudaStreamCaptureStatusActive ? (uint64_t)id + 1 : 0;
+}
+
 bool give_way(chfsi_ctx* ctx) {
   const int64_t before = ctx->dev_bytes;
   cudaDeviceSynchronize();   // the context's stream, and those of the filter lanes

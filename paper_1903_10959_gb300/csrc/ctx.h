@@ -87,6 +87,7 @@ struct chfsi_ctx {
   uint16_t* kgbf = nullptr;        // G~, one block
   size_t kbf_bytes = 0, kgbf_bytes = 0;
   bool kpack_valid = false;
+  uint64_t kpack_capture = 0;      // stream capture in which the packing was recorded
   bool scf_setup = false;          // scfb holds the load of 1 and the weights
   double scf_msum = 0.0;           // sum_j int N_j (the box volume)
   chfsi::DevBuf Db;                // density tables: M^{-1/2}, basis at Gauss points, weights
@@ -121,6 +122,8 @@ chfsi_status rayleigh_ritz_internal(chfsi_ctx* ctx, void* X, int64_t ldx, int n,
 // CHFSI_ERR_TIMEOUT (once) when a bounded wait of the context's digit-slice kernels
 // gave up in work that has run by now; does not synchronise.
 chfsi_status late_timeout(chfsi_ctx* ctx);
+// The stream capture that s takes part in (0: none).
+uint64_t capture_id(cudaStream_t s);
 // Frees the buffers of the context that only make products faster and hold nothing
 // that a call in progress still reads: the digit words of the cell matrices with
 // their scratch, the dense cell blocks of the last application, the padded copies

@@ -192,7 +192,9 @@ chfsi_status kfilter(chfsi_ctx* ctx, double* X, int64_t ldx, int n, int degree, 
 
 // Pack the mixed-path blocks for the current k (after a rebuild or a new k).
 chfsi_status kpack_mixed(chfsi_ctx* ctx) {
-  if (ctx->kpack_valid) return CHFSI_OK;
+  // recorded in a stream capture, the packing is still due for calls outside the graph
+  const uint64_t capture = ctx->kpack_valid ? 0 : capture_id(ctx->stream);
+  if (ctx->kpack_valid || (capture && capture == ctx->kpack_capture)) return CHFSI_OK;
   const HostMesh& m = ctx->mesh;
   if (!ctx->d_kA || !ctx->d_kG)
     return kfail(ctx, CHFSI_ERR_ARG, "mixed k-points need every cell to share the M^{-1/2} pattern");
@@ -204,7 +206,8 @@ chfsi_status kpack_mixed(chfsi_ctx* ctx) {
   KK(tc_pack_bf16_matrices(ctx->d_kG, nullptr, 1, m.ne, &ctx->kgbf, &ctx->kgbf_bytes, ctx->stream));
   if (fresh_a) ctx->dev_bytes += (int64_t)ctx->kbf_bytes;
   if (fresh_g) ctx->dev_bytes += (int64_t)ctx->kgbf_bytes;
-  ctx->kpack_valid = true;
+  ctx->kpack_capture = capture;
+  ctx->kpack_valid = !capture;
   return CHFSI_OK;
 }
 

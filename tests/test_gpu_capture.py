@@ -60,3 +60,35 @@ def test_application_recorded_after_a_rebuild(replay_first, block):
         torch.cuda.synchronize()
         ctx.destroy()
         other.destroy()
+
+
+def test_bloch_application_recorded_after_a_new_wavevector():
+    """The mixed-precision Bloch blocks are packed on first use after set_kpoint."""
+    st = torch.cuda.Stream()
+    _, ctx = system(st)
+    _, other = system()
+    try:
+        g = torch.Generator(DEV).manual_seed(5)
+        X = torch.view_as_complex(torch.randn((ctx.ndofs, 20, 2), device=DEV, generator=g))
+        Y, G, ref = torch.empty_like(X), torch.empty_like(X), torch.empty_like(X)
+        torch.cuda.synchronize()
+        ctx.set_kpoint([0.3, -0.2, 0.1])
+        ctx.apply_kpoint_mixed(X, Y)
+        for c in (ctx, other):
+            c.set_kpoint([-0.1, 0.25, 0.2])
+        other.apply_kpoint_mixed(X, ref)
+        graph = torch.cuda.CUDAGraph()
+        st.synchronize()
+        with torch.cuda.graph(graph, stream=st):
+            ctx.apply_kpoint_mixed(X, G)
+        torch.cuda.synchronize()
+        ctx.apply_kpoint_mixed(X, Y)
+        torch.cuda.synchronize()
+        assert torch.equal(Y, ref)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(G, ref)
+    finally:
+        torch.cuda.synchronize()
+        ctx.destroy()
+        other.destroy()
