@@ -302,13 +302,30 @@ FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
 MMA_PASSES = {"bf16x3": 6, "f16x2": 3, "mixed": 3, "tf32": 1, "fp64": 35}
 # Cell-matrix bytes per element each precision's cell kernel reads.
 CELL_MATRIX_BYTES = {"bf16x3": 6, "f16x2": 4, "mixed": 8, "tf32": 4, "fp64": 8}
-CELL_KERNEL = {"bf16x3": "tc_cell_bf16_kernel", "f16x2": "tc_cell_bf16_stream_kernel<0, 2>",
-               "mixed": "tc_cell_r_kernel",
-               "tf32": "tc_cell_r_kernel", "fp64": "ex_kernel<0>"}
-# The BF16x3 cell kernel each gather mode launches (rings: for two items per SM and more).
+CELL_KERNEL = {"mixed": "tc_cell_r_kernel", "tf32": "tc_cell_r_kernel", "fp64": "ex_kernel<0>"}
+# The BF16x3 cell kernel each gather mode launches (rings: by the size of the launch).
 BF16_KERNEL = {"registers": "tc_cell_bf16_kernel", "async": "tc_cell_bf16_async_kernel",
-               "rings": "tc_cell_bf16_stream_kernel", "rings4": "tc_cell_bf16_rings_kernel",
-               "whole": "tc_cell_bf16_whole_kernel"}
+               "rings4": "tc_cell_bf16_rings_kernel", "whole": "tc_cell_bf16_whole_kernel"}
+
+
+def cell_kernel(prec, gather, s, width, sms=152):
+    """Name of the kernel that a cell launch of `width` columns takes (the rule of
+    stream_items in kernels_tc.cu, for aligned blocks; of the projectors only that
+    p >= 7 with any stays with the ring kernel)."""
+    if prec not in ("bf16x3", "f16x2"):
+        return CELL_KERNEL[prec]
+    if prec == "bf16x3" and gather in BF16_KERNEL:
+        return BF16_KERNEL[gather]
+    nt = 3 if prec == "bf16x3" else 2
+    ne, tiles = (s.p + 1) ** 3, -(-width // 128)
+    items = s.ncell ** 3 * tiles * -(-ne // ((512 - 16 * nt) // 32 * 16))
+    rounds = -(-items // sms)
+    ring = items < 2 * sms or (ne <= 128 and tiles == 1)
+    if ne > 343:
+        ring = (ring or (rounds <= 6 and 100 * items < 85 * rounds * sms)
+                or (tiles == 2 and nt == 2 and width <= 160) or (nt == 3 and len(s.nl_centres) > 0))
+    name = "tc_cell_bf16_rings_kernel" if ring else "tc_cell_bf16_stream_kernel"
+    return name + ("" if nt == 3 else " (FP16x2)")
 
 
 def load_peaks():
@@ -367,7 +384,7 @@ def rooflines(prec, s, n, M, peaks, col_steps, steps_blocks, nblocks, cell_ms, c
     alg_flops = col_steps * ncells * 2 * ne * ne
     peak, note = dtype_peak(prec, peaks)
     achieved = alg_flops / (cell_ms / 1e3) / 1e12
-    kern = BF16_KERNEL.get(gather, CELL_KERNEL[prec]) if prec == "bf16x3" else CELL_KERNEL[prec]
+    kern = cell_kernel(prec, gather, s, -(-n // nblocks))
     roof = {"bound": "alu" if prec == "fp64" else "tensor", "achieved": achieved, "peak": peak,
             "unit": "TFLOP/s", "frac": achieved / peak,
             "traffic": profiled_traffic(kern, s, n) if prec != "fp64" else None,

@@ -49,3 +49,23 @@ def test_assembly_bytes_match_a_launch_by_launch_count(block, gather, nl):
     assert roof["flops_per_launch"] * launches == pytest.approx(s.ncell ** 3 * 2 * ne * ne * n * steps_blocks,
                                                                  rel=1e-12)
     assert roof["frac"] == pytest.approx(roof["achieved"] / peaks["bf16_tflops_sustained"])
+
+
+def test_cell_kernel_names():
+    """The roofline names the kernel the launch takes: the stream kernel for two items
+    per SM and more, the ring kernel below and for p = 7 with projectors."""
+    import bench
+    from types import SimpleNamespace as S
+
+    def name(ncell, p, width, prec="bf16x3", gather="rings", sites=0):
+        return bench.cell_kernel(prec, gather, S(ncell=ncell, p=p, nl_centres=[0] * sites), width)
+
+    assert name(16, 6, 1100) == "tc_cell_bf16_stream_kernel"
+    assert name(20, 7, 1100, sites=1000) == "tc_cell_bf16_rings_kernel"
+    assert name(20, 7, 1100) == "tc_cell_bf16_stream_kernel"
+    assert name(4, 7, 110) == "tc_cell_bf16_rings_kernel"
+    assert name(5, 7, 128) == "tc_cell_bf16_rings_kernel"       # 2.5 items per SM
+    assert name(11, 4, 22) == "tc_cell_bf16_rings_kernel"       # one column tile of small cells
+    assert name(16, 6, 1100, gather="whole") == "tc_cell_bf16_whole_kernel"
+    assert name(16, 6, 1100, prec="f16x2").startswith("tc_cell_bf16_stream_kernel")
+    assert name(16, 6, 1100, prec="mixed") == "tc_cell_r_kernel"
