@@ -418,6 +418,7 @@ struct chfsi_batch {
   float* h_coef = nullptr;      // pinned
   int coef_cap = 0;
   int64_t nitems = 0, nq = 0;
+  bool rings = false;           // BF16x3 products by the ring kernel
   // graph of the last filter configuration
   cudaGraphExec_t gexec = nullptr;
   std::vector<const void*> g_x;
@@ -476,6 +477,12 @@ cudaError_t batch_describe(chfsi_batch* b, float* const* X, const int64_t* ldx, 
   b->h_sys.assign(n, BSys{});
   b->ldx.assign(ldx, ldx + n);
   int64_t item = 0, q = 0;
+  b->rings = false;
+  if (mode == kBatchBf16x3) {
+    int64_t tiles = 0;
+    for (int i = 0; i < n; ++i) tiles += b->ctx[i]->mesh.ncells * ((ncol[i] + 127) / 128);
+    b->rings = tc_bf16_batch_rings(b->ne, tiles * tc_bf16_parts(b->ne, false), tiles * tc_bf16_parts(b->ne, true));
+  }
   // what a system needs: the padded copies of earlier calls and what the member
   // contexts can do without make room for it
   auto need = [&](DevBuf& d, size_t bytes) {
@@ -510,7 +517,7 @@ cudaError_t batch_describe(chfsi_batch* b, float* const* X, const int64_t* ldx, 
     sy.node_ent = c->d_node_ent;
     sy.ncells = m.ncells;
     sy.M = m.ndofs;
-    sy.tiles = mode == kBatchBf16x3 ? (ncol[i] + 127) / 128 * tc_bf16_parts(b->ne) : (ncol[i] + bn - 1) / bn;
+    sy.tiles = mode == kBatchBf16x3 ? (ncol[i] + 127) / 128 * tc_bf16_parts(b->ne, b->rings) : (ncol[i] + bn - 1) / bn;
     sy.item0 = item;
     sy.q0 = q;
     item += m.ncells * sy.tiles;
@@ -556,7 +563,7 @@ cudaError_t batch_enqueue(chfsi_batch* b, float* const* X, const int* ncol, int 
   for (int k = 1; k <= degree; ++k) {
     const int parity = (k - 1) & 1;
     if (split3 == kBatchBf16x3)
-      e = tc_cell_bf16_multi_launch(b->d_sys, n, b->nitems, b->ne, b->mt, parity, b->d_status, b->stream);
+      e = tc_cell_bf16_multi_launch(b->d_sys, n, b->nitems, b->ne, b->mt, parity, b->rings, b->d_status, b->stream);
     else if (S < 0)
       e = tc_cell_multi_launch(b->d_sys, n, b->nitems, b->ne, b->mt, b->nk, split3, parity, b->d_status, b->stream);
     else

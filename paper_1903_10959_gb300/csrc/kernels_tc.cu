@@ -1370,24 +1370,47 @@ __host__ __device__ inline BfrPlan bfr_plan(int ne, int npair, int nt = 3, int p
 // M^{-1/2}, the same for every cell of the uniform periodic mesh), the rows
 // of Y gathered with each (real, imaginary) column pair swapped and the new
 // imaginary part negated, so R holds T~_e Y_r + G~ Y_i, T~_e Y_i - G~ Y_r.
-template <int NPAIR, int NT = 3, bool NLC = false, bool PROJ = false, bool KPT = false>
+// MULTI: grid x runs over the (system, cell, column tile, row part) items of a
+// batch (TcBatchSys: A = the system's packed BF16x3 copy, tiles = column tiles x
+// parts, items of system s from item0), all systems of one degree.
+template <int NPAIR, int NT = 3, bool NLC = false, bool PROJ = false, bool KPT = false, bool MULTI = false>
 __global__ void __launch_bounds__((2 * NPAIR + 2) * 32, 2) tc_cell_bf16_rings_kernel(RParams P) {
   static_assert(NT == 3 || NT == 2, "BF16x3 or FP16x2");
   static_assert(!NLC || NT == 3, "projector chunks: BF16x3");
   static_assert(!PROJ || (NT == 3 && !NLC), "projection: BF16x3");
   static_assert(!KPT || (NT == 3 && !NLC && !PROJ), "Bloch term: BF16x3");
+  static_assert(!MULTI || (NT == 3 && !NLC && !PROJ && !KPT), "batches: BF16x3");
   constexpr int NTHR = (2 * NPAIR + 2) * 32;
   constexpr int WPROD = 2 * NPAIR, WMMA = 2 * NPAIR + 1;
   constexpr int YT = NT * 128 * BF_KC * 2;   // Y stage bytes
   extern __shared__ __align__(1024) unsigned char smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int64_t e = P.e_off + blockIdx.y;
+  int64_t e = P.e_off + blockIdx.y;
   const int ne = P.ne, nk = P.nk;
   const BfrPlan B = bfr_plan(ne, NPAIR, NT, PROJ ? P.pj_npmax : 0);
+  int part = blockIdx.x;                        // (column tile, row part) of the cell
+  if (MULTI) {   // binary search over the systems' first items
+    int lo = 0, hi = P.nsys - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (P.sys[mid].item0 <= blockIdx.x) lo = mid; else hi = mid - 1;
+    }
+    const TcBatchSys& sy = P.sys[lo];
+    const int64_t li = blockIdx.x - sy.item0;
+    e = li / sy.tiles;
+    part = (int)(li - e * sy.tiles);
+    P.A = sy.A;
+    P.dofmap = sy.dofmap;
+    P.Yin = sy.Y[P.parity];
+    P.ld_in = sy.ldY[P.parity];
+    P.R = sy.R;
+    P.ncol = sy.ncol;
+    P.ldr = sy.ldr;
+  }
   const int nrow = PROJ ? P.pj_np[e] : B.nh;   // B-operand rows of this CTA
   if (PROJ && nrow == 0) return;                // a cell owning no projector rows: nothing to do
-  const int h = blockIdx.x % B.np;
-  const int c0 = (blockIdx.x / B.np) * 128;
+  const int h = part % B.np;
+  const int c0 = (part / B.np) * 128;
   const int ncv = min(128, P.ncol - c0);
   const int r0 = h * B.nh;
   const int SM = B.sm, SY = B.sy;
@@ -2683,17 +2706,40 @@ cudaError_t tc_nl_project_cells(const TcCellData& d, const int32_t* dofmap, int6
   return cudaGetLastError();
 }
 
-int tc_bf16_parts(int ne) { return stream_plan(ne, true).np; }
+int tc_bf16_parts(int ne, bool rings) { return rings ? bf_plan(ne).np : stream_plan(ne, true).np; }
+
+// A batch of few items per SM leaves the last round of the stream kernel's thread
+// blocks half empty, where the ring kernel keeps two or more blocks on an SM.  12 steps,
+// ring and stream kernel: 4^3 cells, p = 7, 128 columns (1.3 stream items per SM) 503 and
+// 662 us; 3 + 4 + 3 cells, p = 7, 100 columns (2.3) 714 and 936; 5^3, p = 6, 100 columns
+// (1.6) 454 and 552; 4 + 6 cells, p = 5, 100 columns (1.8) 471 and 543, p = 4 241 and
+// 251.  Past two ring items per SM (p = 4, 5) or four (p = 6, 7) the stream kernel is the
+// faster in most: 4^3 + 5^3 + 4^3, p = 4, 200 columns (3.3) 390 and 367; 5^3 and 6^3, p =
+// 6, 128 columns (4.5) 1,361 and 1,287.  Up to one item per SM it takes 0.69 to 0.85 of
+// the ring kernel's time.
+bool tc_bf16_batch_rings(int ne, int64_t stream_items, int64_t ring_items) {
+  const int64_t sms = stream_grid(INT64_MAX);
+  return ne > 64 && stream_items > sms && ring_items <= (ne > 216 ? 4 : 2) * sms;
+}
 
 cudaError_t tc_cell_bf16_multi_launch(const TcBatchSys* d_sys, int nsys, int64_t nitems, int ne, int mt,
-                                      int parity, int* status, cudaStream_t s) {
+                                      int parity, bool rings, int* status, cudaStream_t s) {
   if (nitems == 0 || nsys == 0) return cudaSuccess;
   if (nitems > 0x7fffffff) return cudaErrorInvalidValue;
   const int nk16 = (ne + BF_KC - 1) / BF_KC;
   RParams P{nullptr, nullptr, nullptr, nullptr, 0, 0, ne, mt, nk16, 1, d_sys, nsys, parity, 0, 0};
   P.status = status;
   P.nitems = nitems;
-  return stream_launch<true>(P, s);
+  if (!rings) return stream_launch<true>(P, s);
+  static std::once_flag attr;
+  std::call_once(attr, [] {
+    cudaFuncSetAttribute(tc_cell_bf16_rings_kernel<2, 3, false, false, false, true>,
+                         cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  });
+  note_launch();
+  tc_cell_bf16_rings_kernel<2, 3, false, false, false, true>
+      <<<(unsigned)nitems, 6 * 32, bfr_plan(ne, 2).total, s>>>(P);
+  return cudaGetLastError();
 }
 
 // Each thread: one unknown j, 4 consecutive columns.  Sums the cell rows

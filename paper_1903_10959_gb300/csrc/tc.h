@@ -120,10 +120,12 @@ cudaError_t tc_cell_multi_launch(const TcBatchSys* d_sys, int nsys, int64_t nite
                                  int nk, int split3, int parity, int* status, cudaStream_t s);
 // The BF16x3 cell kernel over the (cell, 128-column tile, row part) items of
 // every system (A = each system's packed BF16x3 copy, tiles = column tiles x
-// tc_bf16_parts(ne)); Y[parity] is the input.
+// tc_bf16_parts(ne, rings)); Y[parity] is the input.  rings: by the ring kernel, which
+// tc_bf16_batch_rings chooses by the batch's counts of items.
 cudaError_t tc_cell_bf16_multi_launch(const TcBatchSys* d_sys, int nsys, int64_t nitems, int ne, int mt,
-                                      int parity, int* status, cudaStream_t s);
-int tc_bf16_parts(int ne);
+                                      int parity, bool rings, int* status, cudaStream_t s);
+int tc_bf16_parts(int ne, bool rings);
+bool tc_bf16_batch_rings(int ne, int64_t stream_items, int64_t ring_items);
 // Set the cell kernels' shared-memory attributes (before any stream capture).
 void tc_cell_prepare();
 // Owner-computes assembly fused with the Chebyshev update:
